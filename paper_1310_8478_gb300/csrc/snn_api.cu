@@ -50,6 +50,7 @@ void *g_alloc_ctx = nullptr;
         if (r_ != SNN_OK) return r_;                                                     \
     } while (0)
 
+constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
 // Device staging of snn_read_synapses_noalloc: target, weight and sd words,
@@ -140,6 +141,7 @@ struct snn_net {
     int dense_grid = 0;             // blocks of the dense pass (at most one wave of resident blocks)
     int staged_grid = 0;            // blocks of the column-staged delivery (likewise)
     int ordered_grid = 0;           // blocks of the column-ordered delivery (likewise)
+    int stdp_grid = 0;              // blocks of a plasticity window's pass (likewise); 0: no windows
     uint64_t version = 0;           // bumped whenever captured launches go stale
     // stimulus
     size_t stim_cap = 0;
@@ -166,7 +168,7 @@ struct snn_net {
 
 // kinds of step kernel a batch launches once per step for all of its nets
 enum BatchKind { kBLtp, kBFold, kBDeriv, kBOrdered, kBRing, kBStaged, kBDense, kBNeuron32, kBNeuron64, kBProbe,
-                 kBKinds };
+                 kBWinOpen, kBTrain, kBStdp, kBKinds };
 
 struct snn_batch {
     std::vector<snn_net *> nets;
@@ -194,11 +196,15 @@ struct snn_batch {
 
 namespace {
 
+void drop_windows(snn_net *net);
+
 int dalloc(snn_net *net, size_t bytes, void **out)
 {
     *out = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~size_t(255);
+    // the plasticity windows' arrays are optional: they make room
+    if (net->budget && net->bytes_held + bytes > net->budget) drop_windows(net);
     if (net->budget && net->bytes_held + bytes > net->budget) {
         set_error("device budget exceeded: %zu + %zu > %zu bytes", net->bytes_held, bytes, net->budget);
         return SNN_ENOMEM;
@@ -206,6 +212,10 @@ int dalloc(snn_net *net, size_t bytes, void **out)
     void *p = nullptr;
     if (net->alloc) {
         p = net->alloc(bytes, (void *)net->stream, net->alloc_ctx);
+        if (!p && net->dn.win) {
+            drop_windows(net);
+            p = net->alloc(bytes, (void *)net->stream, net->alloc_ctx);
+        }
         if (!p) {
             set_error("allocator hook failed for %zu bytes", bytes);
             return SNN_ENOMEM;
@@ -217,6 +227,11 @@ int dalloc(snn_net *net, size_t bytes, void **out)
         }
     } else {
         cudaError_t e = cudaMalloc(&p, bytes);
+        if (e != cudaSuccess && net->dn.win) {
+            cudaGetLastError();
+            drop_windows(net);
+            e = cudaMalloc(&p, bytes);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             set_error("cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -262,6 +277,25 @@ void drop_graphs(snn_net *net)
     }
     net->graphs_dirty = true;
     net->version++;
+}
+
+// the arrays of the plasticity windows go back (no window is open between
+// two calls): the net's steps apply their STDP at once from here on
+void drop_windows(snn_net *net)
+{
+    DevNet &dn = net->dn;
+    if (!dn.win) return;
+    if (net->stream) cudaStreamSynchronize(net->stream);
+    dfree(net, dn.win);
+    dfree(net, dn.hl0);
+    dfree(net, dn.spk);
+    dfree(net, dn.train);
+    dn.win = nullptr;
+    dn.hl0 = nullptr;
+    dn.spk = nullptr;
+    dn.train = nullptr;
+    net->stdp_grid = 0;
+    drop_graphs(net);
 }
 
 int check_config(const snn_config *c)
@@ -532,6 +566,75 @@ int setup_dense(snn_net *net)
     return SNN_OK;
 }
 
+// no window open (its steps are counted from a clock that a restart sets back)
+int clear_window(snn_net *net)
+{
+    if (!net->dn.win) return SNN_OK;
+    const DevWindow none{0, -1, kNoDefer, 0u, 0u};
+    SNN_CUDA(cudaMemcpyAsync(net->dn.win, &none, sizeof none, cudaMemcpyHostToDevice, net->stream));
+    return SNN_OK;
+}
+
+// Plasticity windows (snn_window.cu): nets with compact targets whose 13
+// columns of train words fit shared memory, with STDP and delivery on, and
+// not tiles.  From 8 M plastic synapses on: a window costs three launches
+// (about 30 us with the change of the shared-memory split, 0.6 us per step;
+// the one-column workload ran 1.7 us per step slower with windows) and a dense
+// step of such a net saves 8 bytes per synapse, about 10 us.  Their arrays (24 bytes per neuron) are taken only where the
+// budget and the device have room; without them every step applies its STDP
+// at once.
+int setup_windows(snn_net *net)
+{
+    DevNet &dn = net->dn;
+    net->stdp_grid = 0;
+    const size_t bytes = stdp_smem_bytes(dn.npc, kStdpBlock);
+    int optin = 0;
+    SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
+    if (!net->tgt16 || dn.tile || (net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) ||
+        net->n_rin < kWinMinSynapses || bytes + 1024 > (size_t)optin) {
+        drop_windows(net);
+        return SNN_OK;
+    }
+    if (!dn.win) {
+        dn.spk_words = (net->N + 31u) / 32u;
+        const size_t words = (size_t)kWinSlots * dn.spk_words;
+        const size_t need = (size_t)net->N * 16 + words * 4 + 4096;
+        if (net->budget && net->bytes_held + need > net->budget) return SNN_OK;
+        DevWindow *win = nullptr;
+        if (dalloc_t(net, (size_t)net->N, &dn.hl0) != SNN_OK || dalloc_t(net, (size_t)net->N, &dn.train) != SNN_OK ||
+            dalloc_t(net, words, &dn.spk) != SNN_OK || dalloc_t(net, 1, &win) != SNN_OK) {
+            dfree(net, dn.hl0);
+            dfree(net, dn.train);
+            dfree(net, dn.spk);
+            dn.hl0 = nullptr;
+            dn.train = nullptr;
+            dn.spk = nullptr;
+            return SNN_OK;
+        }
+        dn.win = win;
+        SNN_TRY(clear_window(net));
+    }
+    SNN_CUDA(cudaFuncSetAttribute(k_stdp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    int per_sm = 0;
+    SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stdp, (int)kStdpBlock, bytes));
+    if (per_sm < 1) {
+        drop_windows(net);
+        return SNN_OK;
+    }
+    // about four work units per resident block, of at least 32 rows (a row
+    // per warp, which pays for staging the 13 columns' trains)
+    const uint64_t want = 4ull * per_sm * net->sm_count;
+    uint32_t chunks = (uint32_t)std::max<uint64_t>(1, (want + dn.C - 1) / dn.C);
+    chunks = std::min(chunks, std::max(1u, dn.ne / 32u));
+    dn.stdp_rows = (dn.ne + chunks - 1) / chunks;
+    const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
+    net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
+    // the deferral starts with the dense pass: its steps then move 6 bytes per
+    // synapse instead of 14
+    dn.defer_min_spikes = dn.dense_min_spikes;
+    return SNN_OK;
+}
+
 // in-degrees -> overflow check -> reverse index -> LUTs -> initial state
 int finish_build(snn_net *net)
 {
@@ -618,6 +721,7 @@ int finish_build(snn_net *net)
     SNN_CUDA(cudaStreamSynchronize(s));
     SNN_TRY(setup_dense(net));
     if (!net->dense_ok) net->dn.dense_min_spikes = 0xffffffffu;
+    SNN_TRY(setup_windows(net));
     return SNN_OK;
 }
 
@@ -714,7 +818,7 @@ void launch_flush(snn_net *net)
     const int32_t t = net->t;
     const int *t_now = &net->ctr->t_slot[t & 1];
     k_ltp<<<grid_for(net, net->launch.ltp_blocks_per_sm), net->launch.ltp_block, 0, s>>>(dn, t_now, 1);
-    k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, 1);
+    k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, kFoldForce);
     cudaMemsetAsync(&net->ctr->fold_cursor, 0, sizeof(unsigned), s);      // no step closes after this fold
     const uint32_t P = net->cfg.deriv_period_ms;
     if (P && t > 0 && (uint32_t)t % P == 0)
@@ -768,7 +872,7 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     // folded into sd first, both passes read sd afterwards
     if (closes) {
         mark(3, s);
-        k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, 0);
+        k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, kFoldStep);
         k_deriv<<<sized_grid(net, 8, (int64_t)dn.C * dn.ne, L.deriv_block / 32), L.deriv_block, 0, s>>>(dn, t_now, 0);
         launched += 2;
         mark(3, s);
@@ -810,11 +914,46 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     if (prof) net->prof_kernels += launched;
 }
 
+// a window's graphs fit the window
 uint32_t effective_graph_len(const snn_net *net)
 {
-    const uint32_t L = net->launch.graph_steps;
+    uint32_t L = net->launch.graph_steps;
     if (net->profile || L < 2) return 0;
+    if (net->stdp_grid) L = std::min<uint32_t>(L, kWinSteps);
     return L & ~1u;
+}
+
+// The next steps of a call as a plasticity window, at most to the end of the
+// period (the window's pass then runs the long-term update); 0: no window
+// (fewer than four steps could not share the pass with an immediate first
+// one; while profiling, every step's kernels do their own work).
+uint32_t window_steps(const snn_net *net, uint32_t left)
+{
+    if (!net->stdp_grid || net->profile) return 0;
+    const uint32_t P = net->cfg.deriv_period_ms;
+    uint32_t n = std::min<uint32_t>(left, kWinSteps);
+    if (P) n = std::min<uint32_t>(n, P - (uint32_t)net->t % P);
+    return n >= 4 ? n : 0;
+}
+
+void open_window(snn_net *net, uint32_t steps)
+{
+    const int *t_now = &net->ctr->t_slot[net->t & 1];
+    k_win_open<<<sized_grid(net, 8, net->N, 1024), 256, 0, net->stream>>>(net->dn, t_now, (int)steps);
+}
+
+// after the window's last step; the kernels return at once when no step left
+// its STDP to the window
+void close_window(snn_net *net)
+{
+    const DevNet &dn = net->dn;
+    cudaStream_t s = net->stream;
+    const int *t_now = &net->ctr->t_slot[net->t & 1];
+    const uint32_t P = net->cfg.deriv_period_ms;
+    if (P && (uint32_t)net->t % P == 0)
+        k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, kFoldWindow);
+    k_train<<<sized_grid(net, 8, dn.spk_words, 64), 256, 0, s>>>(dn, t_now);
+    k_stdp<<<net->stdp_grid, kStdpBlock, stdp_smem_bytes(dn.npc, kStdpBlock), s>>>(dn, t_now);
 }
 
 // one chunk of L steps starting at an even step (only the parity of t is
@@ -886,11 +1025,15 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
     }
     uint32_t left = n_ms;
     const uint32_t P = net->cfg.deriv_period_ms;
+    uint32_t window = 0;                       // steps left of the open window
     while (left > 0) {
         const int32_t t = net->t;
+        if (!window && (window = window_steps(net, left)) != 0) open_window(net, window);
+        const uint32_t ahead = window ? window : left;
         // the first step from t on that closes a period (t' > 0, t' % P == 0)
         const int64_t closing = P ? std::max<int64_t>((int64_t)P, ((int64_t)t + P - 1) / P * P) : INT64_MAX;
-        if (L >= 2 && (t & 1) == 0 && left >= L && closing >= (int64_t)t + L) {
+        const uint32_t before = left;
+        if (L >= 2 && (t & 1) == 0 && ahead >= L && closing >= (int64_t)t + L) {
             if (net->graphs_dirty) {
                 for (int i = 0; i < 2; ++i)
                     if (net->graph[i]) { cudaGraphExecDestroy(net->graph[i]); net->graph[i] = nullptr; }
@@ -907,6 +1050,10 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             net->t += 1;
             left -= 1;
             net->ltp_owed = true;
+        }
+        if (window && (window -= before - left) == 0) {
+            close_window(net);
+            SNN_CUDA(cudaGetLastError());
         }
     }
     return finish_run(net);
@@ -1274,6 +1421,7 @@ int snn_set_tile(snn_net *net, uint32_t first_col, uint32_t n_cols)
     net->dn.dense_min_spikes = dense_threshold(net->N, net->launch.dense_permille);
     SNN_TRY(setup_dense(net));
     if (!net->dense_ok) net->dn.dense_min_spikes = 0xffffffffu;
+    SNN_TRY(setup_windows(net));
     drop_graphs(net);
     return SNN_OK;
 }
@@ -1346,6 +1494,7 @@ int snn_set_launch(snn_net *net, const snn_launch *launch)
     net->dn.dense_min_spikes = dense_threshold(net->N, L.dense_permille);
     SNN_TRY(setup_dense(net));
     if (!net->dense_ok) net->dn.dense_min_spikes = 0xffffffffu;
+    SNN_TRY(setup_windows(net));
     drop_graphs(net);
     return SNN_OK;
 }
@@ -1596,6 +1745,21 @@ int batch_tables(snn_batch *b)
     }
     b->kind[kBNeuron32].block = b->kind[kBNeuron64].block = L.neuron_block;
     b->kind[kBProbe].block = 256;
+    // plasticity windows
+    size_t smem_w = 0;
+    for (int k : {kBWinOpen, kBTrain, kBStdp}) cnt[k].assign(nn, 0);
+    for (size_t i = 0; i < nn; ++i) {
+        const snn_net *n = b->nets[i];
+        if (!n->stdp_grid) continue;
+        smem_w = std::max(smem_w, stdp_smem_bytes(n->dn.npc, kStdpBlock));
+        cnt[kBWinOpen][i] = (uint32_t)sized_grid(n, 8, n->N, 1024);
+        cnt[kBTrain][i] = (uint32_t)sized_grid(n, 8, n->dn.spk_words, 64);
+        cnt[kBStdp][i] = (uint32_t)n->stdp_grid;
+    }
+    b->kind[kBWinOpen].block = b->kind[kBTrain].block = 256;
+    b->kind[kBStdp].block = kStdpBlock;
+    b->kind[kBStdp].smem = smem_w;
+    if (smem_w) SNN_CUDA(cudaFuncSetAttribute(k_stdp_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
     // one device buffer: DevNet[nn], parity[nn], then per kind first[nn],
     // count[nn] and net_of[grid]
     size_t bytes = ((nn * sizeof(DevNet) + nn + 255) & ~size_t(255));
@@ -1672,7 +1836,12 @@ void batch_launch_step(snn_batch *b, uint32_t k)
     };
     // [S4(t-1) S5(t-1) S1(t)] then [S2(t) S3(t)], as launch_step
     go(kBLtp, k_ltp_b);
-    go(kBFold, k_fold_b);
+    if (b->kind[kBFold].grid) {
+        const snn_batch::Kind &x = b->kind[kBFold];
+        BatchLaunch bl = x.bl;
+        bl.k = k;
+        k_fold_b<<<x.grid, x.block, x.smem, s>>>(bl, kFoldStep);
+    }
     go(kBDeriv, k_deriv_b);
     go(kBOrdered, k_deliver_ordered_b);
     go(kBRing, k_deliver_b);
@@ -1681,6 +1850,40 @@ void batch_launch_step(snn_batch *b, uint32_t k)
     go(kBNeuron32, k_neuron_f32_b);
     go(kBNeuron64, k_neuron_f64_b);
     go(kBProbe, k_probe_b);
+}
+
+// The chunks of the next plasticity window of the batch: all of them inside
+// every net's period (0: the next chunk runs without a window).
+uint32_t batch_window_chunks(const snn_batch *b, uint32_t left)
+{
+    if (!b->kind[kBStdp].grid || b->L > (uint32_t)kWinSteps) return 0;
+    uint32_t steps = std::min<uint32_t>(left, kWinSteps);
+    for (const snn_net *n : b->nets) {
+        const uint32_t P = n->cfg.deriv_period_ms;
+        if (n->stdp_grid && P) steps = std::min<uint32_t>(steps, P - (uint32_t)n->t % P);
+    }
+    return steps >= 4 ? steps / b->L : 0;
+}
+
+// the chunks are an even number of steps, so the nets' parities are the ones
+// of the graph at both ends of a window
+void batch_open_window(snn_batch *b, uint32_t steps)
+{
+    const snn_batch::Kind &x = b->kind[kBWinOpen];
+    if (x.grid) k_win_open_b<<<x.grid, x.block, 0, b->main>>>(x.bl, (int)steps);
+}
+
+void batch_close_window(snn_batch *b)
+{
+    bool closes = false;
+    for (const snn_net *n : b->nets) {
+        const uint32_t P = n->cfg.deriv_period_ms;
+        closes |= n->stdp_grid && P && (uint32_t)n->t % P == 0;
+    }
+    const snn_batch::Kind &f = b->kind[kBFold], &x = b->kind[kBTrain], &y = b->kind[kBStdp];
+    if (closes && f.grid) k_fold_b<<<f.grid, f.block, f.smem, b->main>>>(f.bl, kFoldWindow);
+    if (x.grid) k_train_b<<<x.grid, x.block, 0, b->main>>>(x.bl);
+    if (y.grid) k_stdp_b<<<y.grid, y.block, y.smem, b->main>>>(y.bl);
 }
 
 // a chunk of L steps of every net as one graph: per step one launch per kind
@@ -1727,6 +1930,7 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
     }
     const uint32_t L = b->L;
     uint32_t left = n_ms;
+    uint32_t window = 0;                       // chunks left of the open window
     while (left > 0) {
         if (L >= 2 && left >= L) {
             // the graph holds each net's launches for its step parity at capture
@@ -1734,9 +1938,14 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
             for (size_t i = 0; !stale && i < b->nets.size(); ++i)
                 stale = b->versions[i] != b->nets[i]->version || b->parity[i] != (b->nets[i]->t & 1);
             if (stale) SNN_TRY(batch_capture(b));
+            if (!window && (window = batch_window_chunks(b, left)) != 0) batch_open_window(b, window * L);
             SNN_CUDA(cudaGraphLaunch(b->graph, b->main));
             for (snn_net *n : b->nets) n->t += (int32_t)L;
             left -= L;
+            if (window && --window == 0) {
+                batch_close_window(b);
+                SNN_CUDA(cudaGetLastError());
+            }
         } else {
             batch_enqueue(b, 1, true);
             SNN_CUDA(cudaGetLastError());
@@ -1874,6 +2083,7 @@ int snn_autotune(snn_net *net, uint32_t probe_ms, snn_launch *best)
         net->dn.dense_min_spikes = dense_threshold(net->N, cand[i].dense_permille);
         if ((rc = setup_dense(net)) != SNN_OK) break;
         if (!net->dense_ok) net->dn.dense_min_spikes = 0xffffffffu;
+        if ((rc = setup_windows(net)) != SNN_OK) break;
         drop_graphs(net);
         if ((rc = snn_reset(net)) != SNN_OK) break;
         cudaEventRecord(e0, net->stream);
@@ -1891,6 +2101,7 @@ int snn_autotune(snn_net *net, uint32_t probe_ms, snn_launch *best)
     net->dn.dense_min_spikes = dense_threshold(net->N, net->launch.dense_permille);
     SNN_TRY(setup_dense(net));
     if (!net->dense_ok) net->dn.dense_min_spikes = 0xffffffffu;
+    SNN_TRY(setup_windows(net));
     drop_graphs(net);
     SNN_TRY(snn_reset(net));
     if (best) *best = net->launch;
@@ -1912,6 +2123,7 @@ int snn_reset(snn_net *net)
     SNN_CUDA(cudaMemcpyAsync(net->ctr, &hc, sizeof hc, cudaMemcpyHostToDevice, s));
     SNN_CUDA(cudaMemsetAsync(net->dn.ring_cnt, 0, (size_t)2 * net->cfg.max_delay_ms * 4, s));
     if (net->dn.raster_step_off) SNN_CUDA(cudaMemsetAsync(net->dn.raster_step_off, 0, 8, s));
+    SNN_TRY(clear_window(net));
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(s));
     net->t = 0;
@@ -2308,6 +2520,7 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     hc.fold_cursor = 0;
     SNN_CUDA(cudaMemcpyAsync(net->ctr, &hc, sizeof hc, cudaMemcpyHostToDevice, s));
     if (dn.raster_step_off) SNN_CUDA(cudaMemsetAsync(dn.raster_step_off, 0, 8, s));
+    SNN_TRY(clear_window(net));
     SNN_CUDA(cudaStreamSynchronize(s));
     dn.raster_t0 = h.t;
     drop_graphs(net);

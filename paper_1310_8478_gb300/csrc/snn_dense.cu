@@ -38,17 +38,6 @@ constexpr uint32_t kDepMask = 0x7fffu;
 // between LTP and delivery) -- excitatory rows only.
 constexpr int kPrefetchAhead = 1;   // segments of 256 synapses between a warp's loads and its prefetches
 
-// The 256 synapses from position k (a multiple of 8) into L2: targets, and
-// weights and derivatives when asked.
-__device__ __forceinline__ void prefetch_segment(const DevNet &n, int64_t k, bool w, bool sd)
-{
-    if (k >= n.S) return;
-    const uint32_t cnt = (uint32_t)min((int64_t)256, n.S - k);
-    prefetch_l2(n.tgt16 + k, cnt * 2u);
-    if (w) prefetch_l2(n.w + k, cnt * 4u);
-    if (sd) prefetch_l2(n.sd + k, cnt * 4u);
-}
-
 template <bool kExc, bool kDeriv>
 __device__ __forceinline__ void dense_row_walk(const DevNet &n, int64_t base, int m, int D, float scale, uint32_t fbits,
                                                bool stdp, bool ltp_on, const int32_t *w_off, const int32_t *w_amt,
@@ -165,6 +154,134 @@ __device__ __forceinline__ void dense_row_walk(const DevNet &n, int64_t base, in
     }
 }
 
+// The deliver flags of the 32 positions from q0 < m (bit i: the source fired
+// d ms before t, d being the delay bucket of position q0 + i).
+__device__ __forceinline__ uint32_t word_flags(int q0, int m, int D, float scale, uint32_t fbits, const int32_t *w_off)
+{
+    int d = min(D, 1 + (int)((float)q0 * scale));
+    while (w_off[d] <= q0) ++d;           // bucket D ends at m > q0
+    while (w_off[d - 1] > q0) --d;        // w_off[0] = 0 <= q0
+    const int end = min(32, m - q0);
+    uint32_t f = 0;
+    for (int a = 0; a < end; ++d) {
+        const int b = min(w_off[d] - q0, end);
+        if ((fbits >> d) & 1u) f |= (0xffffffffu >> (32 - b)) & (0xffffffffu << a);   // a < 32, 0 < b <= 32
+        a = b;
+    }
+    return f;
+}
+
+// The rows [r0, r1) of column col in a dense step whose STDP is left to the
+// window's pass: targets and, on excitatory rows, weights -- no derivatives,
+// no post-spike words.  Bound by instruction issue before HBM, so
+//   - the next 256 synapses are loaded into registers while this pass's are
+//     added (the bulk prefetches of the fused pass cost a third of the
+//     instructions here, and without derivatives there are registers to spare);
+//   - the delay buckets are looked up once per 1024 synapses, each lane the
+//     flags of 32 positions, and not at all when the source fired in each of
+//     the last D steps;
+//   - inside a chunk that has a due position the others add 0: a condition
+//     around each addition costs a branch and a reconvergence, several times
+//     the addition.
+struct Segment {
+    uint4 t;
+    int4 a, b;
+};
+
+// a lane's 8 synapses: chunk c of the row (none at or past its end)
+__device__ __forceinline__ void load_segment(const DevNet &n, Segment &x, const uint4 *t4, const int4 *w4, int c,
+                                             int chunks, bool exc)
+{
+    if (c >= chunks || out_of_range(n, (const uint16_t *)(t4 + c + 1) <= n.tgt16 + n.S)) return;
+    x.t = t4[c];
+    if (exc) {
+        x.a = w4[2 * c];
+        x.b = w4[2 * c + 1];
+    }
+}
+
+__device__ __forceinline__ void dense_deliver_rows(const DevNet &n, uint32_t col, uint32_t r0, uint32_t r1,
+                                                   uint32_t dmask, int32_t *w_off, int32_t *s_in,
+                                                   unsigned long long &ev_all, unsigned long long &ev_exc)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int D = (int)n.D, m = (int)n.canon_m, chunks = (m + 7) >> 3, nseg = (chunks + 31) >> 5;
+    const float scale = (float)D / (float)m;
+    const uint32_t in0 = (uint32_t)__cvta_generic_to_shared(s_in);
+    if (r0 + warp >= r1) return;
+    const uint32_t p0 = col * n.npc + r0 + warp;
+    uint32_t hist_next = n.hl[p0].x;
+    int off_next = lane <= D ? (int)n.doff[(size_t)p0 * kDoffStride + lane] : 0;
+    const uint4 *t4 = reinterpret_cast<const uint4 *>(n.tgt16 + row_base(n, p0));
+    const int4 *w4 = reinterpret_cast<const int4 *>(n.w + row_base(n, p0));
+    const size_t row4 = (size_t)nwarps * n.uniform_m / 8;           // chunks between a warp's rows
+    Segment cur{};
+    load_segment(n, cur, t4, w4, lane, chunks, r0 + warp < n.ne);
+    auto add = [&](uint32_t v, int32_t w) {
+        if (!out_of_range(n, v < kSlots * n.npc)) red_shared(in0 + 4u * v, w);
+    };
+    for (uint32_t r = r0 + warp; r < r1; r += nwarps, t4 += row4, w4 += 2 * row4) {
+        const uint32_t p = col * n.npc + r;
+        const bool exc = r < n.ne, next_exc = r + nwarps < n.ne;
+        const int next_chunks = r + nwarps < r1 ? chunks : 0;
+        const uint32_t due = exc ? dmask : 2u;         // inhibitory rows: delay 1 alone
+        const uint32_t fbits = (hist_next << 1) & due;
+        const int hi = off_next;
+        if (next_chunks) {
+            hist_next = n.hl[p + nwarps].x;
+            off_next = lane <= D ? (int)n.doff[(size_t)(p + nwarps) * kDoffStride + lane] : 0;
+        }
+        if (!fbits) {
+            load_segment(n, cur, t4 + row4, w4 + 2 * row4, lane, next_chunks, next_exc);
+            continue;
+        }
+        const bool full = fbits == due;                // the whole row is due
+        int events = m;
+        if (!full) {
+            const int lo = __shfl_up_sync(0xffffffffu, hi, 1);
+            w_off[lane] = hi;                          // lane d: end of bucket d, lane 0: 0
+            events = __reduce_add_sync(0xffffffffu, (lane && ((fbits >> lane) & 1u)) ? hi - lo : 0);
+            __syncwarp();
+        }
+        if (lane == 0) {
+            ev_all += (unsigned long long)events;
+            if (exc) ev_exc += (unsigned long long)events;
+        }
+        uint32_t flags = 0;
+        for (int s = 0; s < nseg; ++s) {
+            const Segment x = cur;
+            if (s + 1 < nseg) load_segment(n, cur, t4, w4, 32 * (s + 1) + lane, chunks, exc);
+            else load_segment(n, cur, t4 + row4, w4 + 2 * row4, lane, next_chunks, next_exc);
+            const uint32_t tw[4] = {x.t.x, x.t.y, x.t.z, x.t.w};
+            int32_t wv[8] = {x.a.x, x.a.y, x.a.z, x.a.w, x.b.x, x.b.y, x.b.z, x.b.w};
+            if (!exc) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) wv[u] = n.w_inh;
+            }
+            const int left = m - 8 * (32 * s + lane);
+            uint32_t fmask = left >= 8 ? 0xffu : left > 0 ? (1u << left) - 1u : 0u;
+            if (!full) {
+                if (!(s & 3)) {
+                    const int q0 = 256 * s + 32 * lane;
+                    flags = q0 < m ? word_flags(q0, m, D, scale, fbits, w_off) : 0u;
+                }
+                const uint32_t word = __shfl_sync(0xffffffffu, flags, 8 * (s & 3) + (lane >> 2));
+                fmask &= word >> (8 * (lane & 3));
+            }
+            if (full && s + 1 < nseg) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) add((u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu), wv[u]);
+            } else if (fmask) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    add((u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu), (fmask >> u) & 1u ? wv[u] : 0);
+            }
+        }
+        __syncwarp();
+    }
+}
+
 __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, const Part &g)
 {
     extern __shared__ int4 smem_i4[];
@@ -180,9 +297,10 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
     uint16_t *s_x = reinterpret_cast<uint16_t *>(s_amt + nwarps * 32);   // [kSlots * npc] packed words
     __shared__ uint32_t s_col[kSlots];
 
-    const bool stdp = !(n.flags & SNN_STDP_OFF);
+    const bool defer = deferring(n, t);      // the window's pass does the STDP of this step
+    const bool stdp = !(n.flags & SNN_STDP_OFF) && !defer;
     const bool deliver_on = !(n.flags & SNN_DELIVERY_OFF);
-    const bool owed = n.ctr->ltp_pending == t - 1;
+    const bool owed = n.ctr->ltp_pending == t - 1 && !defer;
     const bool ltp_on = owed && stdp;
     const bool deriv_on = owed && n.deriv_period && (t % (int)n.deriv_period) == 0;
     const uint32_t chunks = (npc + n.dense_rows - 1) / n.dense_rows;
@@ -206,13 +324,15 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
         const uint32_t r1 = min(npc, r0 + n.dense_rows);
         if (threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
         // every warp's first row starts streaming into L2 while the block stages
-        if (lane == 0 && r0 + warp < r1) {
+        if (lane == 0 && r0 + warp < r1 && !defer) {
             const int64_t b = row_base(n, col * npc + r0 + warp);
             for (int sgm = 0; sgm < kPrefetchAhead; ++sgm)
                 prefetch_segment(n, b + sgm * 256, true, r0 + warp < n.ne);
         }
         __syncthreads();
-        for (int sl = 0; sl < kSlots; ++sl) {
+        if (defer)
+            for (uint32_t k = threadIdx.x; k < kSlots * npc; k += blockDim.x) s_in[k] = 0;
+        for (int sl = 0; sl < kSlots && !defer; ++sl) {
             const int32_t *ls = n.last_spike + (size_t)s_col[sl] * npc;
             uint16_t *x_row = s_x + sl * npc;
             int32_t *in_row = s_in + sl * npc;
@@ -223,16 +343,17 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
             }
         }
         __syncthreads();
+        if (defer) dense_deliver_rows(n, col, r0, r1, dmask, w_off, s_in, ev_all, ev_exc);
         // row metadata goes out one row ahead: the spike-history word and, in lane
         // d <= D, the end of delay bucket d
         uint2 hv_next = make_uint2(0u, 0u);
         int off_next = 0;
-        if (r0 + warp < r1) {
+        if (r0 + warp < r1 && !defer) {
             const uint32_t p = col * npc + r0 + warp;
             hv_next = n.hl[p];
             off_next = (lane <= D) ? (int)n.doff[(size_t)p * kDoffStride + lane] : 0;
         }
-        for (uint32_t r = r0 + warp; r < r1; r += nwarps) {
+        for (uint32_t r = r0 + warp; r < r1 && !defer; r += nwarps) {
             const uint32_t p = col * npc + r;
             const bool exc = r < n.ne;
             const uint2 hv = hv_next;
@@ -334,7 +455,7 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
         if (g.bid == 0) {
             // potentiation visits: every incoming excitatory synapse of the
             // neurons that fired at t - 1 (counted when those spikes closed)
-            if (ltp_on) n.ctr->dense_l_exc += n.ctr->l_exc_last;
+            if (ltp_on || defer) n.ctr->dense_l_exc += n.ctr->l_exc_last;
             n.ctr->dense_steps += 1;
             if (deriv_on) n.ctr->dense_deriv_steps += 1;
         }

@@ -22,6 +22,11 @@ constexpr uint32_t kMinCompactNpc = 2;       // the slot reciprocal ceil(2^32 / 
 constexpr uint32_t kDenseMaxNpc = 2800;      // staged columns must fit in shared memory
 static_assert(kSlots * kMaxCompactNpc <= 65536, "compact targets must fit 16 bits");
 constexpr int kUnroll = 4;                   // event-driven walks: synapses per lane in flight
+constexpr int kWinSteps = 50;                // most steps of a plasticity window
+constexpr int kWinBits = 56;                 // spike bits of a train word (the top 8 bits hold a lag)
+constexpr int kWinSlots = 64;                // steps of spike bits kept
+constexpr int kNoDefer = 0x7fffffff;         // DevWindow::defer_from while the plasticity is immediate
+static_assert(kWinSteps <= kWinBits && kWinBits <= kWinSlots, "a window's steps must fit its train words");
 
 // Device counters and per-step bookkeeping (one struct, device memory).
 struct DevCounters {
@@ -42,6 +47,17 @@ struct DevCounters {
     unsigned fold_cursor;            // chunks of reverse entries handed out by the current fold
     int sd_rev_dirty;                // the event-driven potentiation wrote sd_rev since the last fold
     unsigned fold_done;              // blocks of the current fold finished (the last one clears the flag)
+};
+
+// A plasticity window: steps [p0, p1] of one call whose STDP may be put
+// together by one pass over the synapses after step p1 (snn_window.cu).  The
+// weights do not change inside a period and the derivatives are sums of
+// integers, so the order of the additions cannot be seen.
+struct DevWindow {
+    int p0, p1;                      // first and last step (p1 < p0: none open)
+    int defer_from;                  // from this step on the step kernels leave the STDP to the window
+    unsigned cursor;                 // work units of the pass handed out
+    unsigned done;                   // blocks of the pass finished
 };
 
 // Everything a step kernel needs, passed by value.
@@ -112,6 +128,15 @@ struct DevNet {
     // owners (snn_inject_spikes).  A whole net owns every column (tile = 0).
     uint32_t own_c0, own_c1;
     int tile;
+    // plasticity windows (NULL / 0 on nets without them)
+    DevWindow *win;
+    uint2 *hl0;                      // [N] the spike-history words before step p0
+    uint32_t *spk;                   // [kWinSlots][spk_words] bit i of step t's words: neuron i fired at t
+    unsigned long long *train;       // [N] bits 0..55: fired at p0 + k; bits 56..63: p0 - the latest
+                                     //     spike before p0, at most 255
+    uint32_t spk_words;
+    uint32_t defer_min_spikes;       // a step whose spikes reach this starts the deferral after it
+    uint32_t stdp_rows;              // source rows per work unit of the window's pass
 };
 
 __device__ __forceinline__ bool owned_column(const DevNet &n, uint32_t col)
@@ -294,6 +319,13 @@ __device__ __forceinline__ bool dense_selected(const DevNet &n, int t)
     return (uint32_t)(n.ring_cnt[2 * slot] + n.ring_cnt[2 * slot + 1]) >= n.dense_min_spikes;
 }
 
+// the STDP of step t (depression at its arrivals, potentiation owed by step
+// t - 1) is left to the window's pass
+__device__ __forceinline__ bool deferring(const DevNet &n, int t)
+{
+    return n.win && n.win->defer_from <= t;
+}
+
 // Checked builds (-DSNN_CHECKED) verify every computed index before use: a
 // bad one sets the device error word to SNN_EBOUNDS (first error kept) and the
 // caller skips the access.  Other builds compile the checks out.
@@ -383,6 +415,12 @@ __device__ __forceinline__ void red_add(int32_t *p, int32_t v)
     asm volatile("red.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Adds v into the shared-memory word at `addr` (a 32-bit shared address).
+__device__ __forceinline__ void red_shared(uint32_t addr, int32_t v)
+{
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T block_sum(T x)
 {
@@ -423,6 +461,17 @@ __device__ __forceinline__ void prefetch_inside(const void *p, size_t bytes)
 {
     const uintptr_t a = ((uintptr_t)p + 15u) & ~(uintptr_t)15u, b = ((uintptr_t)p + bytes) & ~(uintptr_t)15u;
     if (b > a) prefetch_l2(reinterpret_cast<const void *>(a), (uint32_t)(b - a));
+}
+
+// Up to `most` (a multiple of 8) synapses from position k (a multiple of 8)
+// into L2: targets, and weights and derivatives when asked.
+__device__ __forceinline__ void prefetch_segment(const DevNet &n, int64_t k, bool w, bool sd, int64_t most = 256)
+{
+    if (k >= n.S) return;
+    const uint32_t cnt = (uint32_t)min(most, n.S - k);
+    prefetch_l2(n.tgt16 + k, cnt * 2u);
+    if (w) prefetch_l2(n.w + k, cnt * 4u);
+    if (sd) prefetch_l2(n.sd + k, cnt * 4u);
 }
 
 // thalamic drive (thal_per_col events per column, Philox keyed by (t, col))
@@ -466,6 +515,9 @@ __global__ void k_ltp(DevNet n, const int *t_now, int force);
 __global__ void k_deriv(DevNet n, const int *t_now, int force);
 __global__ void k_fold(DevNet n, const int *t_now, int force);
 __global__ void k_inject(DevNet n, int t, const int32_t *gid, uint32_t count);
+__global__ void k_win_open(DevNet n, const int *t_now, int steps);
+__global__ void k_train(DevNet n, const int *t_now);
+__global__ void k_stdp(DevNet n, const int *t_now);
 
 // the same kernels for every net of a batch in one launch (BatchLaunch)
 __global__ void k_deliver_b(BatchLaunch b);
@@ -477,7 +529,10 @@ __global__ void k_neuron_f64_b(BatchLaunch b);
 __global__ void k_probe_b(BatchLaunch b);
 __global__ void k_ltp_b(BatchLaunch b);
 __global__ void k_deriv_b(BatchLaunch b);
-__global__ void k_fold_b(BatchLaunch b);
+__global__ void k_fold_b(BatchLaunch b, int mode);
+__global__ void k_win_open_b(BatchLaunch b, int steps);
+__global__ void k_train_b(BatchLaunch b);
+__global__ void k_stdp_b(BatchLaunch b);
 
 // net, part and step slots of a block of a batched launch
 struct BatchBlock {
@@ -501,6 +556,11 @@ __device__ __forceinline__ BatchBlock batch_block(const BatchLaunch &b)
 size_t dense_smem_bytes(uint32_t npc, uint32_t block);
 size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
+size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
+constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's pass
+// k_fold: as the step that closes a period runs it / always / before a
+// window's pass that closes a period
+enum FoldMode { kFoldStep = 0, kFoldForce = 1, kFoldWindow = 2 };
 constexpr uint32_t kStagedBlock = 512;      // threads per block of the column-staged delivery
 // the column-ordered delivery is compiled for five resident blocks of at most
 // this many threads per SM (47 registers; the measured optimum): a launch

@@ -11,7 +11,9 @@
 //   [S4(t-1) S5(t-1) S1(t)] then [S2(t) S3(t)]
 // i.e. the potentiation owed by the previous step travels with this step's
 // delivery, so that one pass over the synapses can do both.  Two
-// interchangeable implementations of the first bracket exist:
+// interchangeable implementations of the first bracket exist (a call that
+// runs many busy steps can also leave S4, S5 and the LTD to one pass at the
+// end of a window of steps, see snn_window.cu):
 //   sparse (event driven): k_ltp (reverse index of the spikers of t-1; the
 //       amounts accumulate in sd_rev, laid out like the reverse index so the
 //       updates of one target are contiguous), k_fold (sd += sd_rev before a
@@ -54,7 +56,7 @@ __device__ __forceinline__ void deliver_ring(const DevNet &n, const int *t_now, 
     __shared__ uint32_t s_tile_info[32 * 32];    // per warp: kind and source column of each item
     const int t = *t_now;
     if (!ring_selected(n, t)) return;
-    const bool stdp = !(n.flags & SNN_STDP_OFF);
+    const bool stdp = !(n.flags & SNN_STDP_OFF) && !deferring(n, t);
     const int nl = (int)(n.D + n.D_inh);
     for (int i = threadIdx.x; i < kLut; i += blockDim.x) s_lut[i] = n.lut_m[i];
     if (threadIdx.x == 0) {
@@ -219,7 +221,9 @@ size_t ordered_smem_bytes(uint32_t npc, uint32_t block)
 // s_amt: kStage -> uint16 LTD amounts of the 13 staged columns;
 //        otherwise int32 LTD amounts of the source column's own neurons.
 // s_hist: the history words (bit k: fired at t - k) of the column's rows.
-template <bool kStage>
+// kStdp: depression at the arrivals (not in steps that leave their STDP to a
+// window's pass).
+template <bool kStage, bool kStdp>
 __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_lut, int32_t *s_in, int32_t *s_tile,
                                              void *s_amt, uint32_t *s_hist, const Part &g, uint32_t *s_inh = nullptr)
 {
@@ -231,7 +235,6 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
     int32_t *s_ltd = reinterpret_cast<int32_t *>(s_amt);
     const uint32_t npc = n.npc;
     const uint32_t ngroups = (npc + 31) / 32;
-    const bool stdp = !(n.flags & SNN_STDP_OFF);
     const bool deliver_on = !(n.flags & SNN_DELIVERY_OFF);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kLut; i += blockDim.x) s_lut[i] = n.lut_m[i];
@@ -280,7 +283,7 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                     const uint32_t loc = base + q * blockDim.x;
                     if (loc < npc) {
                         s_hist[loc] = hv[q];
-                        s_ltd[loc] = stdp ? s_lut[min(t - lv[q], kLut - 1)] : 0;
+                        s_ltd[loc] = kStdp ? s_lut[min(t - lv[q], kLut - 1)] : 0;
                         s_in[loc] = 0;
                     }
                 }
@@ -294,7 +297,7 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                 uint16_t *x_row = s_x + sl * npc;
                 int32_t *in_row = s_in + sl * npc;
                 for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                    x_row[loc] = stdp ? (uint16_t)s_lut[min(t - ls[loc], kLut - 1)] : (uint16_t)0;
+                    x_row[loc] = kStdp ? (uint16_t)s_lut[min(t - ls[loc], kLut - 1)] : (uint16_t)0;
                     in_row[loc] = 0;
                 }
             }
@@ -369,7 +372,7 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                     if (out_of_range(n, v < kSlots * npc)) continue;
                     if (kStage) {
                         atomicAdd(&s_in[v], wk[u]);
-                        am[u] = (ex && stdp) ? (int32_t)s_x[v] : 0;
+                        am[u] = (ex && kStdp) ? (int32_t)s_x[v] : 0;
                     } else {
                         const uint32_t slot = __umulhi(v, n.npc_recip);
                         const uint32_t loc = v - slot * npc;
@@ -377,11 +380,11 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                         if (n.tile) ++tile_ev;
                         if (slot == 0) {
                             atomicAdd(&s_in[loc], wk[u]);
-                            am[u] = (ex && stdp) ? s_ltd[loc] : 0;
+                            am[u] = (ex && kStdp) ? s_ltd[loc] : 0;
                         } else {
                             const uint32_t gid = s_col[slot] * npc + loc;        // target gid
                             red_add(&n.I[gid], wk[u]);
-                            if (ex && stdp) {
+                            if (ex && kStdp) {
                                 am[u] = n.last_spike[gid];
                                 remote |= 1u << u;
                             }
@@ -392,7 +395,7 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                     ev_all += (unsigned long long)tile_ev;
                     if (ex) ev_exc += (unsigned long long)tile_ev;
                 }
-                if (ex && stdp) {
+                if (ex && kStdp) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         if (!((mask >> u) & 1u)) continue;
@@ -543,7 +546,8 @@ __device__ __forceinline__ void deliver_staged(const DevNet &n, const int *t_now
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_in + kSlots * npc);   // [npc]
     int32_t *s_tile = reinterpret_cast<int32_t *>(s_hist + npc);         // [nwarps][kTileWords]
     uint16_t *s_x = reinterpret_cast<uint16_t *>(s_tile + nwarps * kTileWords);   // [kSlots * npc]
-    deliver_cols<true>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
+    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_cols<true, true>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
+    else deliver_cols<true, false>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
 }
 
 __device__ __forceinline__ void deliver_ordered(const DevNet &n, const int *t_now, const Part &g)
@@ -558,7 +562,10 @@ __device__ __forceinline__ void deliver_ordered(const DevNet &n, const int *t_no
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_ltd + npc);        // [npc]
     uint32_t *s_inh = s_hist + npc;                                      // [npc]
     int32_t *s_tile = reinterpret_cast<int32_t *>(s_inh + npc);          // [nwarps][kTileWords]
-    deliver_cols<false>(n, t, s_lut, s_in, s_tile, s_ltd, s_hist, g, s_inh);
+    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t))
+        deliver_cols<false, true>(n, t, s_lut, s_in, s_tile, s_ltd, s_hist, g, s_inh);
+    else
+        deliver_cols<false, false>(n, t, s_lut, s_in, s_tile, s_ltd, s_hist, g, s_inh);
 }
 
 // One target's reverse entries [lo, hi), walked by a warp, kUnroll entries
@@ -647,7 +654,7 @@ __device__ __forceinline__ void ltp_body(const DevNet &n, const int *t_now, int 
     const int t = *t_now;
     const int tp = t - 1;
     if (n.ctr->ltp_pending != tp || (n.flags & SNN_STDP_OFF)) return;
-    if (!force && dense_selected(n, t)) return;
+    if (!force && (dense_selected(n, t) || deferring(n, t))) return;
     const int slot = tp % (int)n.D;
     const int ce = n.ring_cnt[2 * slot], ci = n.ring_cnt[2 * slot + 1];
     const int total = ce + ci;
@@ -718,11 +725,12 @@ __device__ __forceinline__ void ltp_body(const DevNet &n, const int *t_now, int 
 // fold the event-driven LTP accumulated in reverse order into the forward
 // derivatives (each forward excitatory synapse has exactly one reverse entry)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void fold_body(const DevNet &n, const int *t_now, int force, const Part &g)
+__device__ __forceinline__ void fold_body(const DevNet &n, const int *t_now, int mode, const Part &g)
 {
-    if (!force) {
+    if (mode != kFoldForce) {
         const int t = *t_now;        // only before a long-term update (t closes a period)
         if (!n.deriv_period || t <= 0 || (t % (int)n.deriv_period) != 0) return;
+        if (mode == kFoldWindow && !deferring(n, t - 1)) return;   // step t's own kernels do it
     }
     // Chunks of kFoldTargets consecutive targets are handed out in order, so
     // the targets in flight form a narrow band of the torus and so do the
@@ -903,6 +911,12 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     F *const sv = state_v<F>(n);
     F *const su = state_u<F>(n);
     const int t = *t_now;
+    bool win_open = false, may_defer = false;
+    if (n.win) {
+        const int p0 = n.win->p0, p1 = n.win->p1;
+        win_open = t >= p0 && t <= p1;
+        may_defer = win_open && t + 3 <= p1 && n.win->defer_from == kNoDefer;
+    }
     const int par = t & 1;
     const uint32_t tile = blockDim.x * kNeuronsPerThread;
     const uint32_t first = g.bid * tile;
@@ -951,6 +965,17 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
         if (!(((fe | fi) >> it) & 1u)) continue;
         const uint32_t i = first + it * blockDim.x + threadIdx.x;
         indeg += (unsigned long long)(n.rin_off[i + 1] - n.rin_off[i]);
+    }
+    // the step's spike bits, kept while a plasticity window is open: a warp's
+    // 32 neurons are one word (an eighth of a byte per neuron and step)
+    if (win_open) {
+        uint32_t *bits = n.spk + (size_t)(t & (kWinSlots - 1)) * n.spk_words;
+#pragma unroll
+        for (int it = 0; it < kNeuronsPerThread; ++it) {
+            const uint32_t word = __ballot_sync(0xffffffffu, ((fe | fi) >> it) & 1u);
+            const uint32_t i = first + it * blockDim.x + threadIdx.x;
+            if ((threadIdx.x & 31) == 0 && i < n.N) bits[i >> 5] = word;
+        }
     }
     // block-wide exclusive prefix of the per-thread counts (exc, inh)
     __shared__ int s_w[2][32];
@@ -1033,6 +1058,10 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     c->fold_cursor = 0;
     c->ltp_pending = t;
     c->done_blocks = 0;
+    // from a busy step on, the rest of an open window leaves its STDP to one
+    // pass at the window's end, when at least three steps share it
+    if (may_defer && (uint32_t)total >= n.defer_min_spikes)
+        n.win->defer_from = t + 1;
     *t_next = t + 1;
 }
 
@@ -1076,9 +1105,9 @@ __global__ void __launch_bounds__(1024) k_ltp(DevNet n, const int *t_now, int fo
     ltp_body(n, t_now, force, whole_grid());
 }
 
-__global__ void __launch_bounds__(1024) k_fold(DevNet n, const int *t_now, int force)
+__global__ void __launch_bounds__(1024) k_fold(DevNet n, const int *t_now, int mode)
 {
-    fold_body(n, t_now, force, whole_grid());
+    fold_body(n, t_now, mode, whole_grid());
 }
 
 __global__ void __launch_bounds__(1024) k_deriv(DevNet n, const int *t_now, int force)
@@ -1126,11 +1155,11 @@ __global__ void __launch_bounds__(1024) k_ltp_b(BatchLaunch b)
     ltp_body(n, x.t_now, 0, x.part);
 }
 
-__global__ void __launch_bounds__(1024) k_fold_b(BatchLaunch b)
+__global__ void __launch_bounds__(1024) k_fold_b(BatchLaunch b, int mode)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
-    fold_body(n, x.t_now, 0, x.part);
+    fold_body(n, x.t_now, mode, x.part);
 }
 
 __global__ void __launch_bounds__(1024) k_deriv_b(BatchLaunch b)
