@@ -370,6 +370,13 @@ int sized_grid(const snn_net *net, uint32_t blocks_per_sm, int64_t units, int64_
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)grid_for(net, blocks_per_sm)));
 }
 
+// blocks of the neuron update: one tile of 4 neurons per thread each, at most
+// one resident wave (32 warps per SM at the kernel's registers), which loops
+int neuron_blocks(const snn_net *net, uint32_t block)
+{
+    return sized_grid(net, std::max(1u, 1024u / block), net->N, (int64_t)block * kNeuronsPerThread);
+}
+
 // whether the reverse index takes 4-byte entries: compact targets and rows of
 // at most kRin32MaxRow stored slots
 bool rin32_ok(const snn_config *c, bool explicit_net)
@@ -900,8 +907,7 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     }
     if (fork) cudaStreamWaitEvent(s, net->ev_join, 0);
     // [S2(t) S3(t)]
-    const int nb_neuron = (int)((net->N + L.neuron_block * kNeuronsPerThread - 1) /
-                                (L.neuron_block * kNeuronsPerThread));
+    const int nb_neuron = neuron_blocks(net, L.neuron_block);
     mark(1, s);
     if (dn.vd) k_neuron_f64<<<nb_neuron, L.neuron_block, 0, s>>>(dn, t_now, t_next);
     else k_neuron_f32<<<nb_neuron, L.neuron_block, 0, s>>>(dn, t_now, t_next);
@@ -1739,7 +1745,7 @@ int batch_tables(snn_batch *b)
     for (int k : {kBNeuron32, kBNeuron64, kBProbe}) cnt[k].assign(nn, 0);
     for (size_t i = 0; i < nn; ++i) {
         const snn_net *n = b->nets[i];
-        const uint32_t nb = (n->N + L.neuron_block * kNeuronsPerThread - 1) / (L.neuron_block * kNeuronsPerThread);
+        const uint32_t nb = (uint32_t)neuron_blocks(n, L.neuron_block);
         cnt[n->dn.vd ? kBNeuron64 : kBNeuron32][i] = nb;
         cnt[kBProbe][i] = (n->dn.probe_n + 255) / 256;
     }

@@ -12,7 +12,7 @@ namespace snn {
 constexpr int kLut = 256;            // STDP amounts for lags 0..255 (the rest are 0)
 constexpr int kDoffStride = 32;      // uint16 delay offsets per source row: [0..D], D <= 31
 constexpr int32_t kNever = -(1 << 30);  // "no spike yet" time stamp
-constexpr int kNeuronsPerThread = 8; // S2/S3: neurons handled by one thread
+constexpr int kNeuronsPerThread = 4; // S2/S3: consecutive neurons handled by one thread (16-byte loads)
 constexpr int kKinds = 5;            // profiled kernel kinds: deliver, neuron, ltp, deriv, dense
 constexpr int kSlots = 13;           // own column + 3 rings of 4 neighbour columns
 constexpr int kSlotStride = 16;      // entries per column in the neighbour table

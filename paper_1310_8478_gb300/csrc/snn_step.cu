@@ -831,7 +831,7 @@ __device__ __forceinline__ void deriv_body(const DevNet &n, const int *t_now, in
 // ---------------------------------------------------------------------------
 // S2 + S3: Izhikevich update (paper Sec. 2 "Spiking neuron model"; v in two
 // 0.5 ms Euler substeps, u in one 1 ms step, Sec. 3) of kNeuronsPerThread
-// neurons per thread, one block-wide compaction of the neurons that fired
+// consecutive neurons per thread, one block-wide compaction of the neurons that fired
 // into ring slot t % D (exc ids from the front, inh ids from the back) and
 // into the raster.  The last block to finish closes the step: ring counts,
 // counters, raster step offset, LTP owed for step t, next time stamp.
@@ -905,122 +905,204 @@ template <typename F> __device__ __forceinline__ F *state_u(const DevNet &n);
 template <> __device__ __forceinline__ float *state_u<float>(const DevNet &n) { return n.u; }
 template <> __device__ __forceinline__ double *state_u<double>(const DevNet &n) { return n.ud; }
 
+// kNeuronsPerThread consecutive values from index i (a multiple of 4) of an
+// array of n: 16-byte accesses where they are all inside it
+template <typename T>
+__device__ __forceinline__ void load4(const T *p, uint32_t i, uint32_t n, T (&x)[4])
+{
+    if (i + 4 <= n) {
+        constexpr int kWords = (int)sizeof(T);       // 16-byte words: 4 * sizeof(T) / 16
+        const uint4 *q = reinterpret_cast<const uint4 *>(p + i);
+        uint4 *o = reinterpret_cast<uint4 *>(x);
+#pragma unroll
+        for (int k = 0; k < kWords / 4; ++k) o[k] = q[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k < n) x[k] = p[i + k];
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void store4(T *p, uint32_t i, uint32_t n, const T (&x)[4])
+{
+    if (i + 4 <= n) {
+        uint4 *q = reinterpret_cast<uint4 *>(p + i);
+        const uint4 *o = reinterpret_cast<const uint4 *>(x);
+#pragma unroll
+        for (int k = 0; k < (int)sizeof(T) / 4; ++k) q[k] = o[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k < n) p[i + k] = x[k];
+    }
+}
+
+// a warp's spikes not yet in the ring and raster
+constexpr int kWarpSpikes = 256;
+
 template <typename F>
 __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, int *t_next, const Part &g)
 {
+    static_assert(kNeuronsPerThread == 4, "one 16-byte access per 4-byte array");
+    __shared__ int32_t s_spk[32][kWarpSpikes];       // per warp: exc ids from the front, inh ids from the back
+    __shared__ unsigned long long s_cnt[32];         // per warp: exc | inh << 32, then their block-wide prefix
+    __shared__ unsigned long long s_base;
+    __shared__ bool s_last;
     F *const sv = state_v<F>(n);
     F *const su = state_u<F>(n);
     const int t = *t_now;
+    const int par = t & 1;
     bool win_open = false, may_defer = false;
     if (n.win) {
         const int p0 = n.win->p0, p1 = n.win->p1;
         win_open = t >= p0 && t <= p1;
         may_defer = win_open && t + 3 <= p1 && n.win->defer_from == kNoDefer;
     }
-    const int par = t & 1;
-    const uint32_t tile = blockDim.x * kNeuronsPerThread;
-    const uint32_t first = g.bid * tile;
-    uint32_t fe = 0, fi = 0;          // bit it: neuron first + it * blockDim + tid fired
-    unsigned long long indeg = 0;     // excitatory in-degree of the neurons that fired
-    // all loads of the thread's neurons first, then the updates and stores
-    int32_t iq[kNeuronsPerThread];
-    F vv[kNeuronsPerThread], uu[kNeuronsPerThread];
-    uint2 hh[kNeuronsPerThread];
-#pragma unroll
-    for (int it = 0; it < kNeuronsPerThread; ++it) {
-        const uint32_t i = first + it * blockDim.x + threadIdx.x;
-        if (i < n.N) {
-            iq[it] = n.I[i];
-            vv[it] = sv[i];
-            uu[it] = su[i];
-            hh[it] = n.hl[i];
-        }
-    }
-#pragma unroll
-    for (int it = 0; it < kNeuronsPerThread; ++it) {
-        const uint32_t i = first + it * blockDim.x + threadIdx.x;
-        if (i >= n.N) break;
-        const bool exc = (i % n.npc) < n.ne;
-        F v = vv[it], u = uu[it];
-        // a tile leaves the neurons of other columns to their owners (their
-        // spikes of this step are injected afterwards)
-        const bool mine = !n.tile || owned_column(n, i / n.npc);
-        const bool fired = mine && izhikevich_step(v, u, iq[it], exc);
-        n.I[i] = 0;
-        if (mine) {
-            sv[i] = v;
-            su[i] = u;
-        }
-        uint2 h = hh[it];
-        if (h.x & 0x80000000u) h.y = (uint32_t)(t - 32);
-        h.x = (h.x << 1) | (fired ? 1u : 0u);
-        n.hl[i] = h;
-        if (fired) {
-            n.last_spike[i] = t;
-            if (exc) fe |= 1u << it; else fi |= 1u << it;
-        }
-    }
-#pragma unroll
-    for (int it = 0; it < kNeuronsPerThread; ++it) {
-        if (!(((fe | fi) >> it) & 1u)) continue;
-        const uint32_t i = first + it * blockDim.x + threadIdx.x;
-        indeg += (unsigned long long)(n.rin_off[i + 1] - n.rin_off[i]);
-    }
-    // the step's spike bits, kept while a plasticity window is open: a warp's
-    // 32 neurons are one word (an eighth of a byte per neuron and step)
-    if (win_open) {
-        uint32_t *bits = n.spk + (size_t)(t & (kWinSlots - 1)) * n.spk_words;
-#pragma unroll
-        for (int it = 0; it < kNeuronsPerThread; ++it) {
-            const uint32_t word = __ballot_sync(0xffffffffu, ((fe | fi) >> it) & 1u);
-            const uint32_t i = first + it * blockDim.x + threadIdx.x;
-            if ((threadIdx.x & 31) == 0 && i < n.N) bits[i >> 5] = word;
-        }
-    }
-    // block-wide exclusive prefix of the per-thread counts (exc, inh)
-    __shared__ int s_w[2][32];
-    __shared__ int s_base[3];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int ce = __popc(fe), ci = __popc(fi);
-    int ie = ce, ii = ci;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int ye = __shfl_up_sync(0xffffffffu, ie, o);
-        const int yi = __shfl_up_sync(0xffffffffu, ii, o);
-        if (lane >= o) { ie += ye; ii += yi; }
-    }
-    if (lane == 31) { s_w[0][warp] = ie; s_w[1][warp] = ii; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int se = 0, si = 0;
-        for (int k = 0; k < nw; ++k) {
-            const int a = s_w[0][k], b = s_w[1][k];
-            s_w[0][k] = se; s_w[1][k] = si;
-            se += a; si += b;
-        }
-        s_base[0] = se ? atomicAdd(&n.ctr->step_cnt[par][0], se) : 0;
-        s_base[1] = si ? atomicAdd(&n.ctr->step_cnt[par][1], si) : 0;
-        s_base[2] = (se + si) ? atomicAdd(&n.ctr->step_cnt[par][2], se + si) : 0;
-    }
-    __syncthreads();
-    if (fe | fi) {
-        int pe = s_base[0] + s_w[0][warp] + ie - ce;
-        int pi = s_base[1] + s_w[1][warp] + ii - ci;
+    unsigned long long *const counts = reinterpret_cast<unsigned long long *>(&n.ctr->step_cnt[par][0]);
+    int32_t *const list = s_spk[warp];
+    int we = 0, wi = 0;               // the warp's pending spikes
+    unsigned long long indeg = 0;     // excitatory in-degree of the neurons that fired
+    // the warp's pending spikes into the ring and the raster, at the positions
+    // that `base` (exc | inh << 32 of the step so far) gives
+    auto emit = [&](unsigned long long base) {
+        const int be = (int)(base & 0xffffffffull), bi = (int)(base >> 32);
         int32_t *ring = n.ring_ids + (size_t)(t % (int)n.D) * n.N;
-        const unsigned long long rbase = n.ctr->raster_total;
-        int pr = s_base[2] + (s_w[0][warp] + ie - ce) + (s_w[1][warp] + ii - ci);
+        const unsigned long long rbase = n.ctr->raster_total + (unsigned long long)(be + bi);
+        for (int q = lane; q < we + wi; q += 32) {
+            const bool e = q < we;
+            const int32_t id = e ? list[q] : list[kWarpSpikes - 1 - (q - we)];
+            const int pos = e ? be + q : (int)n.N - 1 - (bi + q - we);
+            if (!out_of_range(n, pos >= 0 && pos < (int)n.N)) ring[pos] = id;
+            const unsigned long long r = rbase + (unsigned long long)q;
+            if (r < n.raster_cap) n.raster_gid[r] = id;
+            n.last_spike[id] = t;
+            indeg += (unsigned long long)(n.rin_off[id + 1] - n.rin_off[id]);
+        }
+    };
+    // A block takes tiles of 4 neurons per thread, the next tile's state loaded
+    // while this one is updated (not in double: the registers spill, and the
+    // FP64 units are the bound); its spikes collect in shared memory and leave
+    // with one atomic per block.  HBM bound: 40 bytes per neuron, 4.1 M
+    // neurons in 29 us (41 us with a block per 2048 neurons, each waiting for
+    // its loads, its prefix, its atomics and its fence in turn).
+    constexpr bool kAhead = sizeof(F) == 4;
+    const uint32_t stride = part_threads(g) * 4u;
+    __align__(16) int32_t iq[4], iq_n[4];
+    __align__(16) F vv[4], uu[4], vv_n[4], uu_n[4];
+    __align__(16) uint2 hh[4], hh_n[4];
+    uint32_t i0 = part_tid(g) * 4u;
+    if (i0 < n.N) {
+        load4(n.I, i0, n.N, iq);
+        load4(sv, i0, n.N, vv);
+        load4(su, i0, n.N, uu);
+        load4(n.hl, i0, n.N, hh);
+    }
+    for (uint32_t w0 = i0 - 4u * lane; w0 < n.N; w0 += stride, i0 += stride) {    // warp-uniform
+        const uint32_t i_n = i0 + stride;
+        if (kAhead && i_n < n.N) {
+            load4(n.I, i_n, n.N, iq_n);
+            load4(sv, i_n, n.N, vv_n);
+            load4(su, i_n, n.N, uu_n);
+            load4(n.hl, i_n, n.N, hh_n);
+        }
+        uint32_t fe = 0, fi = 0;          // bit k: neuron i0 + k fired
+        if (i0 < n.N) {
+            uint32_t col = i0 / n.npc, loc = i0 - col * n.npc;
 #pragma unroll
-        for (int it = 0; it < kNeuronsPerThread; ++it) {
-            const uint32_t i = first + it * blockDim.x + threadIdx.x;
-            const bool e = (fe >> it) & 1u, q = (fi >> it) & 1u;
-            if (!(e || q)) continue;
-            const int pos = e ? pe++ : (int)n.N - 1 - (pi++);
-            if (!out_of_range(n, pos >= 0 && pos < (int)n.N)) ring[pos] = (int32_t)i;
-            const unsigned long long r = rbase + (unsigned long long)(pr++);
-            if (r < n.raster_cap) n.raster_gid[r] = (int32_t)i;
+            for (int k = 0; k < 4; ++k) {
+                const bool exc = loc < n.ne;
+                // a tile leaves the neurons of other columns to their owners
+                // (their spikes of this step are injected afterwards)
+                const bool mine = !n.tile || owned_column(n, col);
+                F v = vv[k], u = uu[k];
+                const bool fired = izhikevich_step(v, u, iq[k], exc) && mine && i0 + k < n.N;
+                if (mine) {
+                    vv[k] = v;
+                    uu[k] = u;
+                }
+                iq[k] = 0;
+                if (hh[k].x & 0x80000000u) hh[k].y = (uint32_t)(t - 32);
+                hh[k].x = (hh[k].x << 1) | (fired ? 1u : 0u);
+                if (fired) {
+                    if (exc) fe |= 1u << k; else fi |= 1u << k;
+                }
+                if (++loc == n.npc) {
+                    loc = 0;
+                    ++col;
+                }
+            }
+            store4(n.I, i0, n.N, iq);
+            store4(sv, i0, n.N, vv);
+            store4(su, i0, n.N, uu);
+            store4(n.hl, i0, n.N, hh);
+        }
+        // the step's spike bits, kept while a plasticity window is open: 8
+        // lanes' neurons are one word (an eighth of a byte per neuron and step)
+        if (win_open) {
+            uint32_t word = (fe | fi) << (4 * (lane & 7));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
+            if (!(lane & 7) && i0 < n.N) n.spk[(size_t)(t & (kWinSlots - 1)) * n.spk_words + (i0 >> 5)] = word;
+        }
+        if (__any_sync(0xffffffffu, (fe | fi) != 0)) {
+            const uint32_t own = (uint32_t)__popc(fe) | ((uint32_t)__popc(fi) << 16);
+            uint32_t incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t sum = __shfl_sync(0xffffffffu, incl, 31);
+            const int se = (int)(sum & 0xffffu), si = (int)(sum >> 16);
+            if (we + wi + se + si > kWarpSpikes) {       // no room: the pending ones leave now
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(counts, (unsigned long long)we | ((unsigned long long)wi << 32));
+                emit(__shfl_sync(0xffffffffu, base, 0));
+                we = wi = 0;
+                __syncwarp();
+            }
+            int pe = we + (int)((incl - own) & 0xffffu), pi = wi + (int)((incl - own) >> 16);
+            for (uint32_t f = fe | fi; f; f &= f - 1u) {
+                const int k = __ffs(f) - 1;
+                if ((fe >> k) & 1u) list[pe++] = (int32_t)(i0 + k);
+                else list[kWarpSpikes - 1 - pi++] = (int32_t)(i0 + k);
+            }
+            we += se;
+            wi += si;
+            __syncwarp();
+        }
+        if constexpr (kAhead) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                iq[k] = iq_n[k];
+                vv[k] = vv_n[k];
+                uu[k] = uu_n[k];
+                hh[k] = hh_n[k];
+            }
+        } else if (i_n < n.N) {
+            load4(n.I, i_n, n.N, iq);
+            load4(sv, i_n, n.N, vv);
+            load4(su, i_n, n.N, uu);
+            load4(n.hl, i_n, n.N, hh);
         }
     }
+    if (lane == 0) s_cnt[warp] = (unsigned long long)we | ((unsigned long long)wi << 32);
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long own = lane < nw ? s_cnt[lane] : 0ull;
+        unsigned long long incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane < nw) s_cnt[lane] = incl - own;
+        if (lane == 31) s_base = incl ? atomicAdd(counts, incl) : 0ull;
+    }
+    __syncthreads();
+    if (we | wi) emit(s_base + s_cnt[warp]);
     const unsigned long long bdeg = block_sum(indeg);
     if (threadIdx.x == 0) {
         if (bdeg) atomicAdd(&n.ctr->l_exc, bdeg);
