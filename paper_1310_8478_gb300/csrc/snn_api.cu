@@ -51,6 +51,7 @@ void *g_alloc_ctx = nullptr;
     } while (0)
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
+constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
 // Device staging of snn_read_synapses_noalloc: target, weight and sd words,
@@ -2195,36 +2196,68 @@ int snn_read_synapses(snn_net *net, uint32_t first, uint32_t count, int32_t *hos
     if (n_out) *n_out = (size_t)total;
     if ((size_t)total > cap) { set_error("need %lld entries", (long long)total); return SNN_ETRUNC; }
     if (total == 0) return SNN_OK;
-    // chunks of rows of at most ~64 M synapses through device scratch
-    const int64_t chunk_syn = 64ll << 20;
-    uint32_t r0 = first;
-    while (r0 < first + count) {
-        // find r1 with row_off[r1] - row_off[r0] <= chunk_syn (rows hold <= 65535)
-        uint32_t r1 = std::min<uint32_t>(first + count, r0 + (uint32_t)std::max<int64_t>(1, chunk_syn / 65536));
+    // chunks of rows of at most kReadChunk synapses through device scratch
+    // taken once per call (12.8 M synapses, weight and derivative, into touched
+    // pages: 1 ms, where 1024 rows per chunk with a thread per row, an
+    // allocation and a synchronisation each took 71 ms); where there is no room for that much, 1024 rows at a time (rows hold at most 65535)
+    const int64_t row_max = net->dn.uniform_m ? (int64_t)net->dn.canon_m : 65535;
+    const uint32_t few = std::min<uint32_t>(count, 1024u);
+    uint32_t rows = total <= kReadChunk
+                        ? count
+                        : (uint32_t)std::min<int64_t>(count, std::max<int64_t>(few, kReadChunk / row_max));
+    struct Scratch {
+        snn_net *net;
+        int32_t *t = nullptr, *w = nullptr, *s = nullptr;
+        uint8_t *d = nullptr;
+        ~Scratch() { drop(); }
+        void drop()
+        {
+            dfree(net, t);
+            dfree(net, d);
+            dfree(net, w);
+            dfree(net, s);
+            t = w = s = nullptr;
+            d = nullptr;
+        }
+    } x{net};
+    auto take = [&](size_t n) {
+        int r = SNN_OK;
+        if (host_tgt) r = dalloc_t(net, n, &x.t);
+        if (r == SNN_OK && host_delay) r = dalloc_t(net, n, &x.d);
+        if (r == SNN_OK && host_w) r = dalloc_t(net, n, &x.w);
+        if (r == SNN_OK && host_sd) r = dalloc_t(net, n, &x.s);
+        return r;
+    };
+    auto room = [&](size_t n) {          // without pushing anything else out of the budget
+        const size_t bytes = n * ((host_tgt ? 4 : 0) + (host_delay ? 1 : 0) + (host_w ? 4 : 0) + (host_sd ? 4 : 0)) + 1024;
+        return !net->budget || net->bytes_held + bytes <= net->budget;
+    };
+    const size_t big = (size_t)std::min<int64_t>(total, (int64_t)rows * row_max);
+    const bool once = rows > few && room(big) && take(big) == SNN_OK;
+    if (!once) {
+        x.drop();
+        rows = few;
+    }
+    for (uint32_t r0 = first; r0 < first + count;) {
+        const uint32_t r1 = std::min<uint32_t>(first + count, r0 + rows);
         int64_t a = 0, b = 0;
         SNN_TRY(canon_offset(net, r0, &a));
         SNN_TRY(canon_offset(net, r1, &b));
         const int64_t n = b - a;
         if (n > 0) {
-            int32_t *dt = nullptr, *dw = nullptr, *ds = nullptr;
-            uint8_t *dd = nullptr;
-            if (host_tgt) SNN_TRY(dalloc_t(net, (size_t)n, &dt));
-            if (host_delay) SNN_TRY(dalloc_t(net, (size_t)n, &dd));
-            if (host_w) SNN_TRY(dalloc_t(net, (size_t)n, &dw));
-            if (host_sd) SNN_TRY(dalloc_t(net, (size_t)n, &ds));
-            k_read_rows<<<grid_for(net, 8), 128, 0, net->stream>>>(net->dn, net->gen, net->canon_delay, r0, r1 - r0,
-                                                                   a, dt, dd, dw, ds);
+            if (!once) {
+                x.drop();
+                SNN_TRY(take((size_t)n));
+            }
+            k_read_rows<<<sized_grid(net, 8, r1 - r0, 8), 256, 0, net->stream>>>(net->dn, net->gen, net->canon_delay, r0,
+                                                                              r1 - r0, a, x.t, x.d, x.w, x.s);
             SNN_CUDA(cudaGetLastError());
             const size_t o = (size_t)(a - ro[0]);
-            if (dt) SNN_CUDA(cudaMemcpyAsync(host_tgt + o, dt, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
-            if (dd) SNN_CUDA(cudaMemcpyAsync(host_delay + o, dd, (size_t)n, cudaMemcpyDeviceToHost, net->stream));
-            if (dw) SNN_CUDA(cudaMemcpyAsync(host_w + o, dw, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
-            if (ds) SNN_CUDA(cudaMemcpyAsync(host_sd + o, ds, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
+            if (x.t) SNN_CUDA(cudaMemcpyAsync(host_tgt + o, x.t, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
+            if (x.d) SNN_CUDA(cudaMemcpyAsync(host_delay + o, x.d, (size_t)n, cudaMemcpyDeviceToHost, net->stream));
+            if (x.w) SNN_CUDA(cudaMemcpyAsync(host_w + o, x.w, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
+            if (x.s) SNN_CUDA(cudaMemcpyAsync(host_sd + o, x.s, (size_t)n * 4, cudaMemcpyDeviceToHost, net->stream));
             SNN_CUDA(cudaStreamSynchronize(net->stream));
-            dfree(net, dt);
-            dfree(net, dd);
-            dfree(net, dw);
-            dfree(net, ds);
         }
         r0 = r1;
     }
@@ -2259,8 +2292,8 @@ int snn_read_synapses_noalloc(snn_net *net, uint32_t first, uint32_t count, int3
     int32_t *ds = host_sd ? base + 2 * M : nullptr;
     uint8_t *dd = host_delay ? reinterpret_cast<uint8_t *>(base + 3 * M) : nullptr;
     // every staged entry of the range is written by the kernel: nothing to clear
-    k_read_rows<<<grid_for(net, 8), 128, 0, net->stream>>>(net->dn, net->gen, net->canon_delay, first, count, a,
-                                                           dt, dd, dw, ds);
+    k_read_rows<<<sized_grid(net, 8, count, 8), 256, 0, net->stream>>>(net->dn, net->gen, net->canon_delay, first, count,
+                                                                    a, dt, dd, dw, ds);
     SNN_CUDA(cudaGetLastError());
     if (dt) SNN_CUDA(cudaMemcpyAsync(host_tgt, dt, (size_t)total * 4, cudaMemcpyDeviceToHost, net->stream));
     if (dd) SNN_CUDA(cudaMemcpyAsync(host_delay, dd, (size_t)total, cudaMemcpyDeviceToHost, net->stream));

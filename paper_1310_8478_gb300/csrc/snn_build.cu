@@ -246,34 +246,54 @@ __global__ void k_init_state(DevNet n)
     }
 }
 
-// Canonical-order read-back: thread per source row recovers the ordinal of
-// every stored synapse from the canonical delays (regenerated, or kept for
-// explicit nets) and the stable delay order.
+// Canonical-order read-back: a warp per source row recovers the stored
+// position of 32 ordinals at a time from the canonical delays (regenerated,
+// or kept for explicit nets) and the stable delay order -- the synapses of the
+// same delay before this ordinal, counted by lane d for delay d over the
+// earlier passes and by a match inside this one.  The reads stay inside the
+// row, the writes are consecutive.
 __global__ void k_read_rows(DevNet n, GenParams g, const uint8_t *canon_delay, uint32_t first,
                             uint32_t count, int64_t out_base, int32_t *o_tgt, uint8_t *o_delay,
                             int32_t *o_w, int32_t *o_sd)
 {
-    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < count; r += gridDim.x * blockDim.x) {
+    __shared__ int s_count[32][32];                    // per warp: this pass's synapses of every delay
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = lanemask_lt();
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    s_count[warp][lane] = 0;
+    __syncwarp();
+    for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < count; r += warps) {
         const uint32_t p = first + r;
         const int64_t lo = row_base(n, p), len = row_len(n, p), cb = canon_base(n, p);
-        const uint16_t *off = n.doff + (size_t)p * kDoffStride;
-        uint16_t used[kDoffStride];
-        for (int d = 0; d < kDoffStride; ++d) used[d] = 0;
-        for (int64_t j = 0; j < len; ++j) {
-            uint32_t d;
-            if (canon_delay) {
-                d = canon_delay[cb + j];
-            } else {
-                uint32_t t, sl;
-                gen_synapse(g, p, (uint32_t)j, t, d, sl);
+        // lane d: where the next synapse of delay d is stored
+        int next = (lane >= 1 && lane <= (int)n.D) ? (int)n.doff[(size_t)p * kDoffStride + lane - 1] : 0;
+        for (int64_t j0 = 0; j0 < len; j0 += 32) {
+            const int64_t j = j0 + lane;
+            uint32_t d = 0;                            // 0: no synapse in this lane
+            if (j < len) {
+                if (canon_delay) {
+                    d = canon_delay[cb + j];
+                } else {
+                    uint32_t t, sl;
+                    gen_synapse(g, p, (uint32_t)j, t, d, sl);
+                }
             }
-            const int64_t pos = lo + off[d - 1] + used[d];
-            used[d]++;
-            const int64_t o = cb - out_base + j;
-            if (o_tgt) o_tgt[o] = (int32_t)target_gid(n, p / n.npc, pos);
-            if (o_delay) o_delay[o] = (uint8_t)d;
-            if (o_w) o_w[o] = n.w[pos];
-            if (o_sd) o_sd[o] = n.sd[pos];
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const int start = __shfl_sync(0xffffffffu, next, (int)d);
+            if (!(peers & lt)) s_count[warp][d] = __popc(peers);   // the first lane of every delay
+            __syncwarp();
+            next += s_count[warp][lane];
+            __syncwarp();
+            s_count[warp][lane] = 0;
+            __syncwarp();
+            if (j < len) {
+                const int64_t pos = lo + start + __popc(peers & lt);
+                const int64_t o = cb - out_base + j;
+                if (o_tgt) o_tgt[o] = (int32_t)target_gid(n, p / n.npc, pos);
+                if (o_delay) o_delay[o] = (uint8_t)d;
+                if (o_w) o_w[o] = n.w[pos];
+                if (o_sd) o_sd[o] = n.sd[pos];
+            }
         }
     }
 }
