@@ -1166,35 +1166,55 @@ int set_stimulus_impl(snn_net *net, const snn_stimulus *ev, size_t n)
     return SNN_OK;
 }
 
-int raster_window(snn_net *net, int32_t t0, int32_t t1, std::vector<snn_spike> &out, bool &truncated)
+// The spikes of steps [t0, t1), sorted by step and neuron: *total of them, the
+// first `cap` into buf (may be NULL, to count them).  The device sorts each
+// step in place while its bits fit shared memory; the ids travel into the
+// upper half of buf and are expanded from its front, so that no second host
+// buffer is needed.  (1.06 M spikes: 13 ms when the host sorted them into a
+// vector and copied that.)
+int raster_window(snn_net *net, int32_t t0, int32_t t1, snn_spike *buf, size_t cap, size_t *total, bool *truncated)
 {
-    out.clear();
-    truncated = false;
+    *total = 0;
+    *truncated = false;
     DevNet &dn = net->dn;
     if (!dn.raster_gid) { set_error("the net keeps no raster (raster_capacity = 0)"); return SNN_ESTATE; }
     const int32_t lo = std::max(t0, dn.raster_t0), hi = std::min(t1, net->t);
-    if (t0 < dn.raster_t0) truncated = true;
+    if (t0 < dn.raster_t0) *truncated = true;
     if (hi <= lo) return SNN_OK;
+    cudaStream_t s = net->stream;
+    const int64_t *dev_off = dn.raster_step_off + (lo - dn.raster_t0);
     std::vector<int64_t> off((size_t)(hi - lo) + 1);
-    SNN_CUDA(cudaMemcpyAsync(off.data(), dn.raster_step_off + (lo - dn.raster_t0), off.size() * 8,
-                             cudaMemcpyDeviceToHost, net->stream));
-    SNN_CUDA(cudaStreamSynchronize(net->stream));
-    const int64_t a = off.front(), b = off.back();
-    std::vector<int32_t> gid((size_t)(b - a));
-    if (b > a) {
-        SNN_CUDA(cudaMemcpyAsync(gid.data(), dn.raster_gid + a, (size_t)(b - a) * 4, cudaMemcpyDeviceToHost,
-                                 net->stream));
-        SNN_CUDA(cudaStreamSynchronize(net->stream));
-    }
-    out.resize(gid.size());
-    for (int32_t t = lo; t < hi; ++t) {
-        const int64_t s0 = off[(size_t)(t - lo)] - a, s1 = off[(size_t)(t - lo) + 1] - a;
-        std::sort(gid.begin() + s0, gid.begin() + s1);
-        for (int64_t k = s0; k < s1; ++k) out[(size_t)k] = snn_spike{t, gid[(size_t)k]};
-    }
     DevCounters hc{};
+    SNN_CUDA(cudaMemcpyAsync(off.data(), dev_off, off.size() * 8, cudaMemcpyDeviceToHost, s));
     SNN_TRY(read_counters_raw(net, &hc));
-    if (hc.raster_dropped && hi > hc.raster_first_drop_t) truncated = true;
+    if (hc.raster_dropped && hi > hc.raster_first_drop_t) *truncated = true;
+    const int64_t a = off.front();
+    const size_t n = (size_t)(off.back() - a);
+    *total = n;
+    const size_t k = buf ? std::min(cap, n) : 0;
+    if (k == 0) return SNN_OK;
+    const bool on_device = net->N <= kSortMaxNeurons;
+    std::vector<int32_t> all;
+    int32_t *gid = reinterpret_cast<int32_t *>(buf) + k;
+    if (on_device) {
+        const size_t smem = sort_smem_bytes(net->N);
+        SNN_CUDA(cudaFuncSetAttribute(k_sort_raster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_sort_raster<<<sized_grid(net, 4, hi - lo, 1), kSortBlock, smem, s>>>(dev_off, (uint32_t)(hi - lo), net->N,
+                                                                              dn.raster_gid);
+        SNN_CUDA(cudaGetLastError());
+        SNN_CUDA(cudaMemcpyAsync(gid, dn.raster_gid + a, k * 4, cudaMemcpyDeviceToHost, s));
+    } else {
+        all.resize(n);
+        gid = all.data();
+        SNN_CUDA(cudaMemcpyAsync(gid, dn.raster_gid + a, n * 4, cudaMemcpyDeviceToHost, s));
+    }
+    SNN_CUDA(cudaStreamSynchronize(s));
+    for (int32_t t = lo; t < hi; ++t) {
+        const size_t s0 = (size_t)(off[(size_t)(t - lo)] - a), s1 = (size_t)(off[(size_t)(t - lo) + 1] - a);
+        if (s0 >= k) break;
+        if (!on_device) std::sort(gid + s0, gid + s1);
+        for (size_t q = s0; q < std::min(s1, k); ++q) buf[q] = snn_spike{t, gid[q]};
+    }
     return SNN_OK;
 }
 
@@ -1542,14 +1562,12 @@ int snn_run_host(snn_net *net, uint32_t n_ms, const snn_stimulus *host_stimulus,
     if (!net->dn.raster_gid) { set_error("snn_run_host needs raster_capacity > 0"); return SNN_ESTATE; }
     if (net->dn.raster_t0 != t0) SNN_TRY(raster_reset_impl(net));
     SNN_TRY(run_steps(net, n_ms));
-    std::vector<snn_spike> out;
+    size_t total = 0;
     bool trunc = false;
-    SNN_TRY(raster_window(net, t0, t0 + (int32_t)n_ms, out, trunc));
-    if (n_out) *n_out = out.size();
-    const size_t k = std::min(cap, out.size());
-    if (k && host_spikes) std::memcpy(host_spikes, out.data(), k * sizeof(snn_spike));
+    SNN_TRY(raster_window(net, t0, t0 + (int32_t)n_ms, host_spikes, cap, &total, &trunc));
+    if (n_out) *n_out = total;
     SNN_TRY(raster_reset_impl(net));
-    if (trunc || out.size() > cap) { set_error("raster window truncated"); return SNN_ETRUNC; }
+    if (trunc || total > cap) { set_error("raster window truncated"); return SNN_ETRUNC; }
     return SNN_OK;
 }
 
@@ -2167,13 +2185,11 @@ int snn_thalamic_events(const snn_config *cfg, int32_t t0, uint32_t n_ms, snn_st
 int snn_read_raster(snn_net *net, int32_t t0, int32_t t1, snn_spike *host_buf, size_t cap, size_t *n_out)
 {
     if (!net) { set_error("net is NULL"); return SNN_EINVAL; }
-    std::vector<snn_spike> out;
+    size_t total = 0;
     bool trunc = false;
-    SNN_TRY(raster_window(net, t0, t1, out, trunc));
-    if (n_out) *n_out = out.size();
-    const size_t k = std::min(cap, out.size());
-    if (k && host_buf) std::memcpy(host_buf, out.data(), k * sizeof(snn_spike));
-    if (trunc || out.size() > cap) { set_error("raster window truncated"); return SNN_ETRUNC; }
+    SNN_TRY(raster_window(net, t0, t1, host_buf, cap, &total, &trunc));
+    if (n_out) *n_out = total;
+    if (trunc || total > cap) { set_error("raster window truncated"); return SNN_ETRUNC; }
     return SNN_OK;
 }
 

@@ -246,6 +246,59 @@ __global__ void k_init_state(DevNet n)
     }
 }
 
+// ---------------------------------------------------------------------------
+// The raster's entries of each step in ascending order, in place: a block per
+// step sets a bit per spike in shared memory (a neuron fires once a step at
+// most) and writes the set bits back in order, a warp 32 words at a time.
+// step_off: raster index of the first entry of steps 0..steps.  1.06 M spikes
+// of 200 steps of 256 000 neurons sort in about 30 us beside the copy.
+// ---------------------------------------------------------------------------
+size_t sort_smem_bytes(uint32_t n) { return (size_t)((n + 31) / 32) * 4; }
+
+__global__ void __launch_bounds__(kSortBlock) k_sort_raster(const int64_t *step_off, uint32_t steps, uint32_t n,
+                                                            int32_t *gid)
+{
+    extern __shared__ uint32_t s_bits[];
+    __shared__ uint32_t s_start[kSortBlock / 32];
+    const uint32_t words = (n + 31) / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr uint32_t kWarps = kSortBlock / 32;
+    // warp w takes words [w0, w1), a multiple of 32 but for the last
+    const uint32_t per = ((words + kWarps - 1) / kWarps + 31) & ~31u;
+    const uint32_t w0 = min(words, warp * per), w1 = min(words, w0 + per);
+    for (uint32_t s = blockIdx.x; s < steps; s += gridDim.x) {
+        const int64_t lo = step_off[s], hi = step_off[s + 1];
+        if (hi - lo < 2) continue;
+        for (uint32_t w = threadIdx.x; w < words; w += kSortBlock) s_bits[w] = 0;
+        __syncthreads();
+        for (int64_t e = lo + threadIdx.x; e < hi; e += kSortBlock) {
+            const uint32_t g = (uint32_t)gid[e];
+            if (g < n) atomicOr(&s_bits[g >> 5], 1u << (g & 31));
+        }
+        __syncthreads();
+        uint32_t count = 0;
+        for (uint32_t w = w0 + lane; w < w1; w += 32) count += __popc(s_bits[w]);
+        count = __reduce_add_sync(0xffffffffu, count);
+        if (lane == 0) s_start[warp] = count;
+        __syncthreads();
+        int64_t out = lo;
+        for (uint32_t k = 0; k < warp; ++k) out += s_start[k];
+        for (uint32_t b = w0; b < w1; b += 32) {
+            uint32_t x = b + lane < w1 ? s_bits[b + lane] : 0u;
+            const uint32_t own = __popc(x);
+            uint32_t incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            int64_t at = out + incl - own;
+            for (; x; x &= x - 1u) gid[at++] = (int32_t)((b + lane) * 32 + __ffs(x) - 1);
+            out += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        __syncthreads();
+    }
+}
+
 // Canonical-order read-back: a warp per source row recovers the stored
 // position of 32 ordinals at a time from the canonical delays (regenerated,
 // or kept for explicit nets) and the stable delay order -- the synapses of the

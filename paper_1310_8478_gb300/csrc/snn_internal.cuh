@@ -504,6 +504,11 @@ __global__ void k_read_rows(DevNet n, GenParams g, const uint8_t *canon_delay, u
                             uint32_t count, int64_t out_base, int32_t *o_tgt, uint8_t *o_delay,
                             int32_t *o_w, int32_t *o_sd);
 
+constexpr uint32_t kSortBlock = 512;
+constexpr uint32_t kSortMaxNeurons = 1750000;    // their bits fit the shared memory of a block
+size_t sort_smem_bytes(uint32_t n);
+__global__ void k_sort_raster(const int64_t *step_off, uint32_t steps, uint32_t n, int32_t *gid);
+
 __global__ void k_deliver(DevNet n, const int *t_now);
 __global__ void k_dense(DevNet n, const int *t_now);
 __global__ void k_deliver_cols(DevNet n, const int *t_now);
