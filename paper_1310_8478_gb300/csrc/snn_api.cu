@@ -52,6 +52,7 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
+constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
 // Device staging of snn_read_synapses_noalloc: target, weight and sd words,
@@ -82,6 +83,19 @@ int noalloc_lookup(int device, int32_t **out)
     g_noalloc_ptr[device] = (int32_t *)ptr;
     *out = (int32_t *)ptr;
     return SNN_OK;
+}
+
+// Lets a kernel take `bytes` of dynamic shared memory.  The limit is the
+// process's, so it is only ever raised: nets of other sizes launch the same
+// kernels.
+std::mutex g_smem_mutex;
+cudaError_t allow_smem(const void *kernel, size_t bytes)
+{
+    std::lock_guard<std::mutex> lock(g_smem_mutex);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 __global__ void k_fill_row_off(int64_t *row_off, uint32_t n, uint32_t m)
@@ -143,6 +157,8 @@ struct snn_net {
     int staged_grid = 0;            // blocks of the column-staged delivery (likewise)
     int ordered_grid = 0;           // blocks of the column-ordered delivery (likewise)
     int stdp_grid = 0;              // blocks of a plasticity window's pass (likewise); 0: no windows
+    bool step_windows = false;      // the step kernels' steps take windows
+    int res_grid = 0;               // blocks of the resident grid that runs this net's windows; 0: none does
     uint64_t version = 0;           // bumped whenever captured launches go stale
     // stimulus
     size_t stim_cap = 0;
@@ -287,10 +303,10 @@ void drop_windows(snn_net *net)
     DevNet &dn = net->dn;
     if (!dn.win) return;
     if (net->stream) cudaStreamSynchronize(net->stream);
-    dfree(net, dn.win);
-    dfree(net, dn.hl0);
-    dfree(net, dn.spk);
-    dfree(net, dn.train);
+    dfree(net, dn.win);                  // the block that holds all of them
+    dn.I2 = nullptr;
+    net->res_grid = 0;
+    net->step_windows = false;
     dn.win = nullptr;
     dn.hl0 = nullptr;
     dn.spk = nullptr;
@@ -519,7 +535,7 @@ int setup_dense(snn_net *net)
         int per_sm = 0;
         const uint32_t ob = ordered_block(net->launch.deliver_block);
         const size_t obytes = ordered_smem_bytes(net->cfg.neurons_per_col, ob);
-        SNN_CUDA(cudaFuncSetAttribute(k_deliver_ordered, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)obytes));
+        SNN_CUDA(allow_smem((const void *)k_deliver_ordered, obytes));
         SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deliver_ordered, (int)ob, obytes));
         per_sm = std::min<int>(per_sm, (int)std::max(1u, net->launch.deliver_blocks_per_sm));
         if (per_sm >= 1) {
@@ -541,7 +557,7 @@ int setup_dense(snn_net *net)
     SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
     const size_t sbytes = staged_smem_bytes(net->cfg.neurons_per_col, kStagedBlock);
     if (sbytes + 1024 <= (size_t)optin) {
-        SNN_CUDA(cudaFuncSetAttribute(k_deliver_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes));
+        SNN_CUDA(allow_smem((const void *)k_deliver_cols, sbytes));
         int per_sm = 0;
         SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deliver_cols, (int)kStagedBlock, sbytes));
         if (per_sm >= 1 && net->launch.staged_permille != 0xffffffffu) {
@@ -553,7 +569,7 @@ int setup_dense(snn_net *net)
     }
     const size_t bytes = dense_smem_bytes(net->cfg.neurons_per_col, net->launch.dense_block);
     if (bytes + 1024 > (size_t)optin) return SNN_OK;
-    SNN_CUDA(cudaFuncSetAttribute(k_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    SNN_CUDA(allow_smem((const void *)k_dense, bytes));
     int per_sm = 0;
     SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dense, (int)net->launch.dense_block, bytes));
     if (per_sm < 1) return SNN_OK;
@@ -578,51 +594,96 @@ int setup_dense(snn_net *net)
 int clear_window(snn_net *net)
 {
     if (!net->dn.win) return SNN_OK;
-    const DevWindow none{0, -1, kNoDefer, 0u, 0u};
+    DevWindow none{};
+    none.p1 = -1;
+    none.defer_from = kNoDefer;
     SNN_CUDA(cudaMemcpyAsync(net->dn.win, &none, sizeof none, cudaMemcpyHostToDevice, net->stream));
     return SNN_OK;
 }
 
+// Resident grids (snn_resident.cu) run the windows of nets whose blocks all
+// fit the GPU at once, with the device's own choice of pass: as many blocks
+// per column as fit, up to kResMaxParts and down to slices of 32 neurons (us
+// per step with 1, 2, 4, 8 and 16 blocks per column: 4x4 torus of the paper's
+// columns 9.5, 7.7, 6.6, 6.5, 6.9; 2x2 with M = 300 8.7, 7.1, 6.1, 5.8, 5.6;
+// one column in FP64 12.3, 9.0, 6.5, 5.7, 5.8).  A net of one block needs no
+// grid barrier, so one column in FP32 stays with it (4.3 us, else 4.6 or
+// more).
+int resident_grid(snn_net *net, int *parts_out)
+{
+    const DevNet &dn = net->dn;
+    const snn_launch &L = net->launch;
+    if (L.dense_permille != 250 || L.staged_permille != 0xffffffffu || L.ring_permille != 0) return 0;
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, net->device) != cudaSuccess || !coop) return 0;
+    const bool f64 = dn.vd != nullptr;
+    const void *kernel = f64 ? (const void *)k_resident_f64 : (const void *)k_resident_f32;
+    int parts = kResMaxParts;
+    if (dn.C == 1 && !f64) parts = 1;
+    for (; parts >= 1; --parts) {
+        if (parts > 1 && (dn.npc + parts - 1) / parts < 32) continue;
+        const size_t bytes = resident_smem_bytes(dn.npc, (uint32_t)parts, f64);
+        int per_sm = 0;
+        if (allow_smem(kernel, bytes) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, (int)kResBlock, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if ((int64_t)dn.C * parts <= (int64_t)per_sm * net->sm_count) {
+            *parts_out = parts;
+            return (int)dn.C * parts;
+        }
+    }
+    return 0;
+}
+
 // Plasticity windows (snn_window.cu): nets with compact targets whose 13
 // columns of train words fit shared memory, with STDP and delivery on, and
-// not tiles.  From 8 M plastic synapses on: a window costs three launches
-// (about 30 us with the change of the shared-memory split, 0.6 us per step;
-// the one-column workload ran 1.7 us per step slower with windows) and a dense
-// step of such a net saves 8 bytes per synapse, about 10 us.  Their arrays (24 bytes per neuron) are taken only where the
-// budget and the device have room; without them every step applies its STDP
-// at once.
+// not tiles.  The step kernels take them from 8 M plastic synapses on: a
+// window costs three launches (about 30 us with the change of the
+// shared-memory split, 0.6 us per step; the one-column workload ran 1.7 us
+// per step slower with windows) and a dense step of such a net saves 8 bytes
+// per synapse, about 10 us.  Resident grids take them at any size.  The
+// arrays (24 or 28 bytes per neuron) are taken only where the budget and the device
+// have room; without them every step applies its STDP at once.
 int setup_windows(snn_net *net)
 {
     DevNet &dn = net->dn;
     net->stdp_grid = 0;
+    net->res_grid = 0;
+    net->step_windows = false;
     const size_t bytes = stdp_smem_bytes(dn.npc, kStdpBlock);
-    int optin = 0;
+    int optin = 0, parts = 1;
     SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
-    if (!net->tgt16 || dn.tile || (net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) ||
-        net->n_rin < kWinMinSynapses || bytes + 1024 > (size_t)optin) {
+    const bool can = net->tgt16 && !dn.tile && !(net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) &&
+                     bytes + 1024 <= (size_t)optin;
+    if (can && dn.win && !dn.I2 && resident_grid(net, &parts)) drop_windows(net);   // (a shape that lets one run now)
+    const int res = can ? resident_grid(net, &parts) : 0;
+    if (!can || (!res && net->n_rin < kWinMinSynapses)) {
         drop_windows(net);
         return SNN_OK;
     }
     if (!dn.win) {
         dn.spk_words = (net->N + 31u) / 32u;
         const size_t words = (size_t)kWinSlots * dn.spk_words;
-        const size_t need = (size_t)net->N * 16 + words * 4 + 4096;
+        const size_t need = (size_t)net->N * (res ? 20 : 16) + words * 4 + 8192;
         if (net->budget && net->bytes_held + need > net->budget) return SNN_OK;
-        DevWindow *win = nullptr;
-        if (dalloc_t(net, (size_t)net->N, &dn.hl0) != SNN_OK || dalloc_t(net, (size_t)net->N, &dn.train) != SNN_OK ||
-            dalloc_t(net, words, &dn.spk) != SNN_OK || dalloc_t(net, 1, &win) != SNN_OK) {
-            dfree(net, dn.hl0);
-            dfree(net, dn.train);
-            dfree(net, dn.spk);
-            dn.hl0 = nullptr;
-            dn.train = nullptr;
-            dn.spk = nullptr;
-            return SNN_OK;
-        }
+        // one block: window, histories, trains, spike bits, step inputs
+        auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+        const size_t N8 = up((size_t)net->N * 8), N4 = up((size_t)net->N * 4), bits = up(words * 4);
+        char *block = nullptr;
+        if (dalloc_t(net, up(sizeof(DevWindow)) + 2 * N8 + bits + (res ? N4 : 0), &block) != SNN_OK) return SNN_OK;
+        DevWindow *win = reinterpret_cast<DevWindow *>(block);
+        block += up(sizeof(DevWindow));
+        dn.hl0 = reinterpret_cast<uint2 *>(block);
+        dn.train = reinterpret_cast<unsigned long long *>(block + N8);
+        dn.spk = reinterpret_cast<uint32_t *>(block + 2 * N8);
+        if (res) dn.I2 = reinterpret_cast<int32_t *>(block + 2 * N8 + bits);
         dn.win = win;
+        if (res) SNN_CUDA(cudaMemsetAsync(dn.I2, 0, (size_t)net->N * 4, net->stream));
         SNN_TRY(clear_window(net));
     }
-    SNN_CUDA(cudaFuncSetAttribute(k_stdp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    SNN_CUDA(allow_smem((const void *)k_stdp, bytes));
     int per_sm = 0;
     SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stdp, (int)kStdpBlock, bytes));
     if (per_sm < 1) {
@@ -637,9 +698,16 @@ int setup_windows(snn_net *net)
     dn.stdp_rows = (dn.ne + chunks - 1) / chunks;
     const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
     net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
-    // the deferral starts with the dense pass: its steps then move 6 bytes per
-    // synapse instead of 14
-    dn.defer_min_spikes = dn.dense_min_spikes;
+    net->step_windows = net->n_rin >= kWinMinSynapses;
+    net->res_grid = res;
+    dn.res_parts = (uint32_t)parts;
+    // a step starts the deferral when the rest of its window, at its rate, will
+    // see half a spike per neuron: the pass then costs less than the
+    // potentiation and depression of the single steps (us per step at a
+    // threshold of 0.5, 1 and never: 64x64 torus of the paper's columns, 1 to
+    // 2 % firing, 152, 160, 160; 32x32 with M = 300, 4 to 8 %, 142, 143, 177;
+    // dense steps: less than half)
+    dn.defer_visits = std::max<uint32_t>(1, net->N / 2);
     return SNN_OK;
 }
 
@@ -926,7 +994,7 @@ uint32_t effective_graph_len(const snn_net *net)
 {
     uint32_t L = net->launch.graph_steps;
     if (net->profile || L < 2) return 0;
-    if (net->stdp_grid) L = std::min<uint32_t>(L, kWinSteps);
+    if (net->step_windows) L = std::min<uint32_t>(L, kWinSteps);
     return L & ~1u;
 }
 
@@ -936,7 +1004,7 @@ uint32_t effective_graph_len(const snn_net *net)
 // one; while profiling, every step's kernels do their own work).
 uint32_t window_steps(const snn_net *net, uint32_t left)
 {
-    if (!net->stdp_grid || net->profile) return 0;
+    if (!net->step_windows || net->profile) return 0;
     const uint32_t P = net->cfg.deriv_period_ms;
     uint32_t n = std::min<uint32_t>(left, kWinSteps);
     if (P) n = std::min<uint32_t>(n, P - (uint32_t)net->t % P);
@@ -949,6 +1017,14 @@ void open_window(snn_net *net, uint32_t steps)
     k_win_open<<<sized_grid(net, 8, net->N, 1024), 256, 0, net->stream>>>(net->dn, t_now, (int)steps);
 }
 
+// the window's pass (a resident grid has written the trains itself)
+void launch_stdp(snn_net *net, bool trains)
+{
+    const DevNet &dn = net->dn;
+    if (!trains) k_train<<<sized_grid(net, 8, dn.spk_words, 64), 256, 0, net->stream>>>(dn);
+    k_stdp<<<net->stdp_grid, kStdpBlock, stdp_smem_bytes(dn.npc, kStdpBlock), net->stream>>>(dn);
+}
+
 // after the window's last step; the kernels return at once when no step left
 // its STDP to the window
 void close_window(snn_net *net)
@@ -959,8 +1035,33 @@ void close_window(snn_net *net)
     const uint32_t P = net->cfg.deriv_period_ms;
     if (P && (uint32_t)net->t % P == 0)
         k_fold<<<sized_grid(net, 8, net->n_rin, 4096), 256, 0, s>>>(dn, t_now, kFoldWindow);
-    k_train<<<sized_grid(net, 8, dn.spk_words, 64), 256, 0, s>>>(dn, t_now);
-    k_stdp<<<net->stdp_grid, kStdpBlock, stdp_smem_bytes(dn.npc, kStdpBlock), s>>>(dn, t_now);
+    launch_stdp(net, false);
+}
+
+// the steps of a call on a resident grid: false when the net takes the step
+// kernels (no such grid, a profile, a probe, or a call of fewer than four
+// steps, which would pay for a window's pass each)
+bool resident_call(const snn_net *net, uint32_t left)
+{
+    return net->res_grid && !net->profile && !net->dn.probe_n && left >= 4;
+}
+
+// `steps` more steps from t0 as one window on the resident grid (it runs as
+// far as its steps stay sparse, and not at all when an earlier window of the
+// call stopped before t0)
+int launch_resident(snn_net *net, int32_t t0, uint32_t steps)
+{
+    DevNet &dn = net->dn;
+    cudaStream_t s = net->stream;
+    const bool f64 = dn.vd != nullptr;
+    int n_steps = (int)steps;
+    void *args[] = {&dn, &t0, &n_steps};
+    SNN_CUDA(cudaLaunchCooperativeKernel(f64 ? (const void *)k_resident_f64 : (const void *)k_resident_f32,
+                                         dim3((unsigned)net->res_grid), dim3(kResBlock), args,
+                                         resident_smem_bytes(dn.npc, dn.res_parts, f64), s));
+    k_emit<<<dim3((dn.spk_words + kEmitWords - 1) / kEmitWords, steps), kEmitBlock, 0, s>>>(dn);
+    launch_stdp(net, true);
+    return SNN_OK;
 }
 
 // one chunk of L steps starting at an even step (only the parity of t is
@@ -994,10 +1095,12 @@ int read_counters_raw(snn_net *net, DevCounters *hc)
 
 // end of a run: the counters are copied out behind the steps and read after
 // the one synchronisation (the device error word decides the return code)
-int finish_run(snn_net *net)
+int finish_run(snn_net *net, bool copied)
 {
-    SNN_CUDA(cudaMemcpyAsync(&net->host_ctr[1], net->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, net->stream));
-    SNN_CUDA(cudaStreamSynchronize(net->stream));
+    if (!copied) {
+        SNN_CUDA(cudaMemcpyAsync(&net->host_ctr[1], net->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, net->stream));
+        SNN_CUDA(cudaStreamSynchronize(net->stream));
+    }
     SNN_CUDA(cudaGetLastError());
     if (net->profile && net->ev_used) {
         for (size_t i = 0; i + 1 < net->ev_used; i += 2) {
@@ -1033,8 +1136,40 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
     uint32_t left = n_ms;
     const uint32_t P = net->cfg.deriv_period_ms;
     uint32_t window = 0;                       // steps left of the open window
+    const bool resident = resident_call(net, left);
+    int64_t resident_from = net->t;            // the step from which the resident grid is tried
+    bool copied = false;                       // the counters have been read behind the last step
     while (left > 0) {
         const int32_t t = net->t;
+        copied = false;
+        if (resident && !window && t >= resident_from) {
+            // every window of the call at once; the one synchronisation says
+            // how far they came
+            if (net->ltp_owed) {
+                launch_flush(net);
+                net->ltp_owed = false;
+            }
+            for (uint32_t ahead = 0; ahead < left;) {
+                const uint32_t at = (uint32_t)t + ahead;
+                uint32_t n = std::min<uint32_t>(left - ahead, kWinSteps);
+                if (P) n = std::min<uint32_t>(n, P - at % P);
+                SNN_TRY(launch_resident(net, (int32_t)at, n));
+                ahead += n;
+            }
+            SNN_CUDA(cudaGetLastError());
+            SNN_CUDA(cudaMemcpyAsync(&net->host_ctr[1], net->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, net->stream));
+            SNN_CUDA(cudaStreamSynchronize(net->stream));
+            const DevCounters &hc = net->host_ctr[1];
+            if (hc.error) return finish_run(net, true);
+            const int32_t now = std::max(t, hc.t_slot[(hc.t_slot[0] < hc.t_slot[1]) ? 1 : 0]);
+            left -= (uint32_t)(now - t);
+            net->t = now;
+            // a busy net goes on with the step kernels, 200 steps until the
+            // next try
+            resident_from = (int64_t)now + 200;
+            copied = true;
+            continue;
+        }
         if (!window && (window = window_steps(net, left)) != 0) open_window(net, window);
         const uint32_t ahead = window ? window : left;
         // the first step from t on that closes a period (t' > 0, t' % P == 0)
@@ -1063,7 +1198,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             SNN_CUDA(cudaGetLastError());
         }
     }
-    return finish_run(net);
+    return finish_run(net, copied);
 }
 
 // canonical (unpadded, source-major) index of the first synapse of row p
@@ -1198,7 +1333,7 @@ int raster_window(snn_net *net, int32_t t0, int32_t t1, snn_spike *buf, size_t c
     int32_t *gid = reinterpret_cast<int32_t *>(buf) + k;
     if (on_device) {
         const size_t smem = sort_smem_bytes(net->N);
-        SNN_CUDA(cudaFuncSetAttribute(k_sort_raster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SNN_CUDA(allow_smem((const void *)k_sort_raster, smem));
         k_sort_raster<<<sized_grid(net, 4, hi - lo, 1), kSortBlock, smem, s>>>(dev_off, (uint32_t)(hi - lo), net->N,
                                                                               dn.raster_gid);
         SNN_CUDA(cudaGetLastError());
@@ -1721,7 +1856,7 @@ int batch_tables(snn_batch *b)
     b->kind[kBOrdered].smem = smem_o;
     if (smem_o) {
         if (smem_o + 1024 > (size_t)optin) { set_error("batch: ordered delivery needs too much shared memory"); return SNN_EINVAL; }
-        SNN_CUDA(cudaFuncSetAttribute(k_deliver_ordered_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_o));
+        SNN_CUDA(allow_smem((const void *)k_deliver_ordered_b, smem_o));
     }
     share_blocks(w, cap, sms * batch_occupancy((const void *)k_deliver_ordered_b, ordered_block(L.deliver_block), smem_o,
                                                L.deliver_blocks_per_sm), cnt[kBOrdered]);
@@ -1743,7 +1878,7 @@ int batch_tables(snn_batch *b)
     b->kind[kBStaged].smem = smem_s;
     if (smem_s) {
         if (smem_s + 1024 > (size_t)optin) { set_error("batch: staged delivery needs too much shared memory"); return SNN_EINVAL; }
-        SNN_CUDA(cudaFuncSetAttribute(k_deliver_cols_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_s));
+        SNN_CUDA(allow_smem((const void *)k_deliver_cols_b, smem_s));
     }
     share_blocks(w, cap, sms * batch_occupancy((const void *)k_deliver_cols_b, kStagedBlock, smem_s, 64), cnt[kBStaged]);
     // dense pass (nets where it may run), work units of dense_rows rows
@@ -1757,7 +1892,7 @@ int batch_tables(snn_batch *b)
     b->kind[kBDense].smem = smem_d;
     if (smem_d) {
         if (smem_d + 1024 > (size_t)optin) { set_error("batch: dense pass needs too much shared memory"); return SNN_EINVAL; }
-        SNN_CUDA(cudaFuncSetAttribute(k_dense_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d));
+        SNN_CUDA(allow_smem((const void *)k_dense_b, smem_d));
     }
     share_blocks(w, cap, sms * batch_occupancy((const void *)k_dense_b, L.dense_block, smem_d, 64), cnt[kBDense]);
     // neuron update and probes: exact block counts
@@ -1775,7 +1910,7 @@ int batch_tables(snn_batch *b)
     for (int k : {kBWinOpen, kBTrain, kBStdp}) cnt[k].assign(nn, 0);
     for (size_t i = 0; i < nn; ++i) {
         const snn_net *n = b->nets[i];
-        if (!n->stdp_grid) continue;
+        if (!n->step_windows) continue;
         smem_w = std::max(smem_w, stdp_smem_bytes(n->dn.npc, kStdpBlock));
         cnt[kBWinOpen][i] = (uint32_t)sized_grid(n, 8, n->N, 1024);
         cnt[kBTrain][i] = (uint32_t)sized_grid(n, 8, n->dn.spk_words, 64);
@@ -1784,7 +1919,7 @@ int batch_tables(snn_batch *b)
     b->kind[kBWinOpen].block = b->kind[kBTrain].block = 256;
     b->kind[kBStdp].block = kStdpBlock;
     b->kind[kBStdp].smem = smem_w;
-    if (smem_w) SNN_CUDA(cudaFuncSetAttribute(k_stdp_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
+    if (smem_w) SNN_CUDA(allow_smem((const void *)k_stdp_b, smem_w));
     // one device buffer: DevNet[nn], parity[nn], then per kind first[nn],
     // count[nn] and net_of[grid]
     size_t bytes = ((nn * sizeof(DevNet) + nn + 255) & ~size_t(255));
@@ -1885,7 +2020,7 @@ uint32_t batch_window_chunks(const snn_batch *b, uint32_t left)
     uint32_t steps = std::min<uint32_t>(left, kWinSteps);
     for (const snn_net *n : b->nets) {
         const uint32_t P = n->cfg.deriv_period_ms;
-        if (n->stdp_grid && P) steps = std::min<uint32_t>(steps, P - (uint32_t)n->t % P);
+        if (n->step_windows && P) steps = std::min<uint32_t>(steps, P - (uint32_t)n->t % P);
     }
     return steps >= 4 ? steps / b->L : 0;
 }
@@ -1903,7 +2038,7 @@ void batch_close_window(snn_batch *b)
     bool closes = false;
     for (const snn_net *n : b->nets) {
         const uint32_t P = n->cfg.deriv_period_ms;
-        closes |= n->stdp_grid && P && (uint32_t)n->t % P == 0;
+        closes |= n->step_windows && P && (uint32_t)n->t % P == 0;
     }
     const snn_batch::Kind &f = b->kind[kBFold], &x = b->kind[kBTrain], &y = b->kind[kBStdp];
     if (closes && f.grid) k_fold_b<<<f.grid, f.block, f.smem, b->main>>>(f.bl, kFoldWindow);

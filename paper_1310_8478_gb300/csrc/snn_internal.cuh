@@ -58,6 +58,11 @@ struct DevWindow {
     int defer_from;                  // from this step on the step kernels leave the STDP to the window
     unsigned cursor;                 // work units of the pass handed out
     unsigned done;                   // blocks of the pass finished
+    // a window run by a resident grid (snn_resident.cu)
+    int steps_done;                  // steps it ran
+    unsigned bar;                    // arrivals at the grid barrier (0 between two grids)
+    unsigned long long cnt[kWinSlots];   // spikes of step p0 + k: exc | inh << 32
+    unsigned long long last_deg;     // in-degrees of the last step's spikes (0 between two grids)
 };
 
 // Everything a step kernel needs, passed by value.
@@ -135,8 +140,11 @@ struct DevNet {
     unsigned long long *train;       // [N] bits 0..55: fired at p0 + k; bits 56..63: p0 - the latest
                                      //     spike before p0, at most 255
     uint32_t spk_words;
-    uint32_t defer_min_spikes;       // a step whose spikes reach this starts the deferral after it
+    unsigned long long defer_visits; // a step whose spikes, times the steps left in the window, reach
+                                     //     this starts the deferral after it
     uint32_t stdp_rows;              // source rows per work unit of the window's pass
+    int32_t *I2;                     // [N] resident grids: the input of every other step (the others: I)
+    uint32_t res_parts;              // resident grids: blocks per column
 };
 
 __device__ __forceinline__ bool owned_column(const DevNet &n, uint32_t col)
@@ -449,6 +457,70 @@ __device__ __forceinline__ int32_t deriv_sd(const DevNet &n, int32_t s)
     return (int32_t)(((long long)s * n.deriv_decay + 32768) >> 16);
 }
 
+// One step of a neuron (paper Sec. 2 "Spiking neuron model"): v in two 0.5 ms
+// Euler substeps, u in one 1 ms step; whether it fired.
+__device__ __forceinline__ bool izhikevich_step(float &v, float &u, int32_t iq, bool exc)
+{
+    const float a = exc ? 0.02f : 0.1f;
+    const float b = 0.2f;
+    const float c = -65.0f;
+    const float d = exc ? 8.0f : 2.0f;
+    const float cur = __fmul_rn(__int2float_rn(iq), 0x1p-16f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float x = __fmul_rn(0.04f, v);
+        x = __fadd_rn(x, 5.0f);
+        x = __fmul_rn(x, v);
+        x = __fadd_rn(x, 140.0f);
+        x = __fsub_rn(x, u);
+        x = __fadd_rn(x, cur);
+        x = __fmul_rn(0.5f, x);
+        v = __fadd_rn(v, x);
+    }
+    float y = __fmul_rn(b, v);
+    y = __fsub_rn(y, u);
+    y = __fmul_rn(a, y);
+    u = __fadd_rn(u, y);
+    if (v >= 30.0f) {
+        v = c;
+        u = __fadd_rn(u, d);
+        return true;
+    }
+    return false;
+}
+
+// the same scheme in double (SNN_FP64): identical operation order, decimal
+// parameters
+__device__ __forceinline__ bool izhikevich_step(double &v, double &u, int32_t iq, bool exc)
+{
+    const double a = exc ? 0.02 : 0.1;
+    const double b = 0.2;
+    const double c = -65.0;
+    const double d = exc ? 8.0 : 2.0;
+    const double cur = __dmul_rn(__int2double_rn(iq), 0x1p-16);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        double x = __dmul_rn(0.04, v);
+        x = __dadd_rn(x, 5.0);
+        x = __dmul_rn(x, v);
+        x = __dadd_rn(x, 140.0);
+        x = __dsub_rn(x, u);
+        x = __dadd_rn(x, cur);
+        x = __dmul_rn(0.5, x);
+        v = __dadd_rn(v, x);
+    }
+    double y = __dmul_rn(b, v);
+    y = __dsub_rn(y, u);
+    y = __dmul_rn(a, y);
+    u = __dadd_rn(u, y);
+    if (v >= 30.0) {
+        v = c;
+        u = __dadd_rn(u, d);
+        return true;
+    }
+    return false;
+}
+
 // Bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
 // multiple of 16); nothing waits on it.
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
@@ -521,8 +593,11 @@ __global__ void k_deriv(DevNet n, const int *t_now, int force);
 __global__ void k_fold(DevNet n, const int *t_now, int force);
 __global__ void k_inject(DevNet n, int t, const int32_t *gid, uint32_t count);
 __global__ void k_win_open(DevNet n, const int *t_now, int steps);
-__global__ void k_train(DevNet n, const int *t_now);
-__global__ void k_stdp(DevNet n, const int *t_now);
+__global__ void k_train(DevNet n);
+__global__ void k_stdp(DevNet n);
+__global__ void k_resident_f32(DevNet n, int t0, int steps);
+__global__ void k_resident_f64(DevNet n, int t0, int steps);
+__global__ void k_emit(DevNet n);
 
 // the same kernels for every net of a batch in one launch (BatchLaunch)
 __global__ void k_deliver_b(BatchLaunch b);
@@ -562,6 +637,10 @@ size_t dense_smem_bytes(uint32_t npc, uint32_t block);
 size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
+size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64);
+constexpr uint32_t kResBlock = 512;         // threads per block of a resident grid
+constexpr uint32_t kEmitBlock = 512;
+constexpr uint32_t kEmitWords = 2048;       // words of a step's spike bits per block
 constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's pass
 // k_fold: as the step that closes a period runs it / always / before a
 // window's pass that closes a period

@@ -836,68 +836,6 @@ __device__ __forceinline__ void deriv_body(const DevNet &n, const int *t_now, in
 // into the raster.  The last block to finish closes the step: ring counts,
 // counters, raster step offset, LTP owed for step t, next time stamp.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool izhikevich_step(float &v, float &u, int32_t iq, bool exc)
-{
-    const float a = exc ? 0.02f : 0.1f;
-    const float b = 0.2f;
-    const float c = -65.0f;
-    const float d = exc ? 8.0f : 2.0f;
-    const float cur = __fmul_rn(__int2float_rn(iq), 0x1p-16f);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float x = __fmul_rn(0.04f, v);
-        x = __fadd_rn(x, 5.0f);
-        x = __fmul_rn(x, v);
-        x = __fadd_rn(x, 140.0f);
-        x = __fsub_rn(x, u);
-        x = __fadd_rn(x, cur);
-        x = __fmul_rn(0.5f, x);
-        v = __fadd_rn(v, x);
-    }
-    float y = __fmul_rn(b, v);
-    y = __fsub_rn(y, u);
-    y = __fmul_rn(a, y);
-    u = __fadd_rn(u, y);
-    if (v >= 30.0f) {
-        v = c;
-        u = __fadd_rn(u, d);
-        return true;
-    }
-    return false;
-}
-
-// the same scheme in double (SNN_FP64): identical operation order, decimal
-// parameters
-__device__ __forceinline__ bool izhikevich_step(double &v, double &u, int32_t iq, bool exc)
-{
-    const double a = exc ? 0.02 : 0.1;
-    const double b = 0.2;
-    const double c = -65.0;
-    const double d = exc ? 8.0 : 2.0;
-    const double cur = __dmul_rn(__int2double_rn(iq), 0x1p-16);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        double x = __dmul_rn(0.04, v);
-        x = __dadd_rn(x, 5.0);
-        x = __dmul_rn(x, v);
-        x = __dadd_rn(x, 140.0);
-        x = __dsub_rn(x, u);
-        x = __dadd_rn(x, cur);
-        x = __dmul_rn(0.5, x);
-        v = __dadd_rn(v, x);
-    }
-    double y = __dmul_rn(b, v);
-    y = __dsub_rn(y, u);
-    y = __dmul_rn(a, y);
-    u = __dadd_rn(u, y);
-    if (v >= 30.0) {
-        v = c;
-        u = __dadd_rn(u, d);
-        return true;
-    }
-    return false;
-}
-
 template <typename F> __device__ __forceinline__ F *state_v(const DevNet &n);
 template <> __device__ __forceinline__ float *state_v<float>(const DevNet &n) { return n.v; }
 template <> __device__ __forceinline__ double *state_v<double>(const DevNet &n) { return n.vd; }
@@ -953,11 +891,12 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     F *const su = state_u<F>(n);
     const int t = *t_now;
     const int par = t & 1;
-    bool win_open = false, may_defer = false;
+    bool win_open = false;
+    int may_defer = 0;                // steps of the open window behind this one that could defer
     if (n.win) {
         const int p0 = n.win->p0, p1 = n.win->p1;
         win_open = t >= p0 && t <= p1;
-        may_defer = win_open && t + 3 <= p1 && n.win->defer_from == kNoDefer;
+        if (win_open && n.win->defer_from == kNoDefer) may_defer = p1 - t;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned long long *const counts = reinterpret_cast<unsigned long long *>(&n.ctr->step_cnt[par][0]);
@@ -1141,8 +1080,8 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     c->ltp_pending = t;
     c->done_blocks = 0;
     // from a busy step on, the rest of an open window leaves its STDP to one
-    // pass at the window's end, when at least three steps share it
-    if (may_defer && (uint32_t)total >= n.defer_min_spikes)
+    // pass at the window's end, when at least two steps share it
+    if (may_defer >= 2 && (unsigned long long)total * may_defer >= n.defer_visits)
         n.win->defer_from = t + 1;
     *t_next = t + 1;
 }

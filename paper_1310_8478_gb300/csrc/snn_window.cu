@@ -17,59 +17,97 @@
 // pass, 7.5 ms per 50 steps (bound by instruction issue: two sums over 50-bit
 // trains per synapse).  A train is a 64-bit word: 56 step bits and, in the top 8, the lag of
 // the latest event before the window (255: none that matters).
+#include <type_traits>
+
 #include "snn_internal.cuh"
 
 namespace snn {
 
 constexpr unsigned long long kTrainMask = (1ull << kWinBits) - 1ull;
 
+constexpr int kSpikeCap = 96;          // spikes of a row that arrive in a window: at most 31 + kWinSteps
+constexpr int kAmounts = 96;           // steps -31 .. kWinSteps of a row's potentiation amounts
+constexpr int kFewSpikes = 14;         // up to here a row's arrivals are taken one by one
+
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block)
 {
     return (size_t)kSlots * npc * 8            // trains of the 13 columns the rows reach
            + (size_t)(block / 32) * 32 * 8     // per warp: arrival trains, one per delay
            + (size_t)(block / 32) * 32 * 4     // per warp: bucket ends
+           + (size_t)(block / 32) * kSpikeCap  // per warp: the row's spike times
+           + (size_t)(block / 32) * kAmounts * 4   // per warp: the row's potentiation amounts
            + 2 * kLut * 4;                     // amounts
 }
 
-__device__ __forceinline__ int top_bit(unsigned long long x) { return 63 - __clzll((long long)x); }
-
 // Sum of lut[lag] over the set bits k of `at`: lag to the latest bit of
-// `of` at or before k - `gap` (gap 0 or 1), else k + before (the lag of the
-// latest event before the window), beyond the table 0.  Few bits are taken
-// one by one; many are counted lag by lag, which ends after the longest
-// gap between two bits of `of`.
-__device__ __forceinline__ int32_t nearest_sum(unsigned long long at, unsigned long long of, int gap, int before,
-                                               const int32_t *lut)
+// `of` at or before k - gap (gap 0 or 1), else k + before (the lag of the
+// latest event before the window), beyond the table 0.  Counted lag by lag,
+// which ends after the longest gap between two bits of `of`: for trains with
+// many bits.
+__device__ __forceinline__ int32_t lag_sum(unsigned long long at, unsigned long long of, int gap, int before,
+                                           const int32_t *lut)
 {
-    int32_t sum = 0;
-    if (__popcll(at) > 6) {
-        const unsigned long long first = (of & (0ull - of)) << gap;      // first bit that has a predecessor
-        unsigned long long early = of ? at & (first - 1ull) : at;
-        at ^= early;
-        unsigned long long s = of << gap;
-        for (int lag = gap; at; ++lag, s <<= 1) {
-            const unsigned long long hit = at & s;
-            if (hit) {
-                sum += lut[lag] * __popcll(hit);
-                at ^= hit;
-            }
+    // two saturated trains end here or one lag on
+    unsigned long long s = of << gap;
+    int32_t sum = lut[gap] * __popcll(at & s);
+    at &= ~s;
+    s <<= 1;
+    sum += lut[gap + 1] * __popcll(at & s);
+    at &= ~s;
+    if (!at) return sum;
+    const unsigned long long first = (of & (0ull - of)) << gap;      // first bit that has a predecessor
+    unsigned long long early = of ? at & (first - 1ull) : at;
+    at ^= early;
+    for (int lag = gap + 2; at; ++lag) {
+        s <<= 1;
+        const unsigned long long hit = at & s;
+        if (hit) {
+            sum += lut[lag] * __popcll(hit);
+            at ^= hit;
         }
-        at = early;
-        while (at) {
-            const int lag = __ffsll((long long)at) - 1 + before;
-            if (lag >= kLut - 1) break;
-            sum += lut[lag];
-            at &= at - 1ull;
-        }
-        return sum;
     }
-    while (at) {
-        const int k = __ffsll((long long)at) - 1;
-        at &= at - 1ull;
-        const unsigned long long m = of & ((1ull << (k + 1 - gap)) - 1ull);
-        const int lag = m ? k - top_bit(m) : min(k + before, kLut - 1);
+    for (; early; early &= early - 1ull) {
+        const int lag = __ffsll((long long)early) - 1 + before;
+        if (lag >= kLut - 1) break;
         sum += lut[lag];
     }
+    return sum;
+}
+
+// What the window adds to a synapse's derivative: x the arrivals, y the post
+// spikes (train words), for a source with many spikes.  A target with many
+// too is counted lag by lag; else the events are taken one by one in time
+// order with the latest arrival and post spike at hand (an arrival comes
+// before a post spike of its step).
+// Only the amounts of `arrivals` and `posts` count (the first steps of a window
+// may have applied theirs at once).
+__device__ __forceinline__ int32_t window_delta(unsigned long long x, unsigned long long y, unsigned long long posts,
+                                                unsigned long long arrivals, const int32_t *lutp, const int32_t *lutm)
+{
+    constexpr uint32_t kHigh = (uint32_t)(kTrainMask >> 32);
+    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32) & kHigh, y0 = (uint32_t)y, y1 = (uint32_t)(y >> 32) & kHigh;
+    const int before_x = (int)(x >> kWinBits), before_y = (int)(y >> kWinBits);
+    if (__popc(y0) + __popc(y1) >= 12)
+        return lag_sum(y & posts, x & kTrainMask, 0, before_x, lutp) - lag_sum(x & arrivals, y & kTrainMask, 1, before_y, lutm);
+    int32_t sum = 0;
+    int arrived = -before_x, fired = -before_y;           // steps of the latest ones
+    auto half = [&](uint32_t xs, uint32_t ys, uint32_t am, uint32_t pm, int k0) {
+        for (uint32_t u = xs | ys; u;) {
+            const uint32_t bit = u & (0u - u);
+            const int k = k0 + 31 - __clz((int)bit);
+            u ^= bit;
+            if (xs & bit) {
+                if (am & bit) sum -= lutm[min(k - fired, kLut - 1)];
+                arrived = k;
+            }
+            if (ys & bit) {
+                if (pm & bit) sum += lutp[min(k - arrived, kLut - 1)];
+                fired = k;
+            }
+        }
+    };
+    half(x0, y0, (uint32_t)arrivals, (uint32_t)posts, 0);
+    half(x1, y1, (uint32_t)(arrivals >> 32), (uint32_t)(posts >> 32), 32);
     return sum;
 }
 
@@ -90,10 +128,10 @@ __device__ __forceinline__ void win_open_body(const DevNet &n, const int *t_now,
 // The window's spike bits (a word of 32 neurons per step) turned into one
 // train word per neuron.  A warp takes 8 words: its loads are full sectors,
 // 32 ballots turn 32 steps of 32 neurons.
-__device__ __forceinline__ void train_body(const DevNet &n, const int *t_now, const Part &g)
+__device__ __forceinline__ void train_body(const DevNet &n, const Part &g)
 {
     __shared__ uint32_t s_bits[8][kWinSlots][8];
-    if (!n.win || !deferring(n, *t_now)) return;
+    if (!n.win || n.win->defer_from > n.win->p1) return;
     const int p0 = n.win->p0, steps = n.win->p1 - p0 + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t warps = part_threads(g) >> 5, nw = (n.N + 31u) / 32u;
@@ -128,16 +166,26 @@ __device__ __forceinline__ void train_body(const DevNet &n, const int *t_now, co
 }
 
 // One row: the lane takes 4 synapses per pass.
-template <bool kDeriv>
+//   kFew: the row has few spikes, at times w_j[0..ns) relative to the window
+//   (an arrival is delay d later).  A post spike at step k adds w_q[k - d]:
+//   the potentiation depends on the source and on k - d alone, so a row has
+//   one table of it for all of its delays.  The depression of its arrivals is
+//   looked up by all lanes in turn, at the lag to the target's latest post
+//   spike before each.  (246 M plastic synapses at 2 to 3 spikes per neuron
+//   and window: 3.7 ms; 6.1 ms with both kinds of events taken per synapse in
+//   time order, as window_delta does.)
+template <bool kDeriv, bool kFew>
 __device__ __forceinline__ void stdp_row(const DevNet &n, int64_t base, int m, int D, const int32_t *w_off,
-                                         const unsigned long long *w_x, const unsigned long long *s_y,
-                                         const int32_t *s_lutp, const int32_t *s_lutm, unsigned long long posts,
+                                         const unsigned long long *w_x, const signed char *w_j, int ns,
+                                         const unsigned long long *s_y, const int32_t *w_q, const int32_t *s_lutp,
+                                         const int32_t *s_lutm, int steps, unsigned long long posts,
                                          unsigned long long arrivals, int lane)
 {
     const uint2 *rt2 = reinterpret_cast<const uint2 *>(n.tgt16 + base);
     int4 *rs4 = reinterpret_cast<int4 *>(n.sd + base);
     int4 *rw4 = reinterpret_cast<int4 *>(n.w + base);
     const float scale = (float)D / (float)m;
+    const int a_min = arrivals ? __ffsll((long long)arrivals) - 1 : steps;
     for (int c = lane; c * 4 < m; c += 32) {
         const int k0 = c * 4;
         if (out_of_range(n, base + k0 + 4 <= n.S)) continue;
@@ -145,44 +193,72 @@ __device__ __forceinline__ void stdp_row(const DevNet &n, int64_t base, int m, i
         const int4 sa = rs4[c];
         int4 wa = make_int4(0, 0, 0, 0);
         if (kDeriv) wa = rw4[c];
-        int d = min(D, 1 + (int)((float)k0 * scale));
-        while (w_off[d] <= k0) ++d;       // bucket D ends at m > k0
-        while (w_off[d - 1] > k0) --d;    // w_off[0] = 0 <= k0
+        int b = min(D, 1 + (int)((float)k0 * scale));
+        while (w_off[b] <= k0) ++b;       // bucket D ends at m > k0
+        while (w_off[b - 1] > k0) --b;    // w_off[0] = 0 <= k0
         const uint32_t tw[2] = {tv.x, tv.y};
-        int32_t sv[4] = {sa.x, sa.y, sa.z, sa.w};
-        int32_t wv[4] = {wa.x, wa.y, wa.z, wa.w};
-        bool dirty = kDeriv;
+        int32_t delta[4];
+        int d[4];
+        uint32_t y0[4], y1[4];            // post spikes of steps 0..31, 32..55
+        int before0[4], before1[4];       // a - the latest post spike before step 0 (32): a + this
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (k0 + u >= m) continue;    // the row's padding
-            while (k0 + u >= w_off[d]) ++d;
+            delta[u] = 0;
             const uint32_t v = (u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu);
-            if (out_of_range(n, v < kSlots * n.npc)) continue;
-            const unsigned long long x = w_x[d], y = s_y[v];
-            const unsigned long long xb = x & kTrainMask, yb = y & kTrainMask;
-            const int32_t delta = nearest_sum(yb & posts, xb, 0, (int)(x >> kWinBits), s_lutp) -
-                                  nearest_sum(xb & arrivals, yb, 1, (int)(y >> kWinBits), s_lutm);
-            if (delta) {
-                sv[u] += delta;
-                dirty = true;
+            const bool in = k0 + u < m && !out_of_range(n, v < kSlots * n.npc);     // not the row's padding
+            if (in)
+                while (k0 + u >= w_off[b]) ++b;
+            d[u] = in ? b : -kSpikeCap;   // padding: every arrival lies before the window
+            const unsigned long long y = in ? s_y[v] : 0ull;
+            if (!kFew) {
+                if (in) delta[u] = window_delta(w_x[b], y, posts, arrivals, s_lutp, s_lutm);
+                continue;
             }
-            if (kDeriv) {
+            y0[u] = (uint32_t)y;
+            y1[u] = (uint32_t)(y >> 32) & (uint32_t)(kTrainMask >> 32);
+            before0[u] = (int)(y >> kWinBits);
+            before1[u] = y0[u] ? __clz((int)y0[u]) - 31 : before0[u];
+            const int32_t *q = w_q + 31 - b;
+            for (uint32_t f = y0[u] & (uint32_t)posts; f; f &= f - 1u) delta[u] += q[__ffs((int)f) - 1];
+            for (uint32_t f = y1[u] & (uint32_t)(posts >> 32); f; f &= f - 1u) delta[u] += q[__ffs((int)f) + 31];
+        }
+        if (kFew) {
+            for (int i = 0; i < ns; ++i) {
+                const int j = w_j[i];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int a = j + d[u];
+                    if (a < a_min || a >= steps) continue;
+                    // post spikes of a's half of the window before a, the latest on top
+                    const uint32_t z = ((a < 32 ? y0[u] : y1[u]) << 1) << (31 - (a & 31));
+                    const int lag = z ? 1 + __clz((int)z) : a + (a < 32 ? before0[u] : before1[u]);
+                    delta[u] -= s_lutm[min(lag, kLut - 1)];
+                }
+            }
+        }
+        const bool dirty = kDeriv || delta[0] || delta[1] || delta[2] || delta[3];
+        int32_t sv[4] = {sa.x + delta[0], sa.y + delta[1], sa.z + delta[2], sa.w + delta[3]};
+        if (kDeriv) {
+            int32_t wv[4] = {wa.x, wa.y, wa.z, wa.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (k0 + u >= m) continue;
                 wv[u] = deriv_w(n, wv[u], sv[u]);
                 sv[u] = deriv_sd(n, sv[u]);
             }
+            rw4[c] = make_int4(wv[0], wv[1], wv[2], wv[3]);
         }
         if (dirty) rs4[c] = make_int4(sv[0], sv[1], sv[2], sv[3]);
-        if (kDeriv) rw4[c] = make_int4(wv[0], wv[1], wv[2], wv[3]);
     }
 }
 
-__device__ __forceinline__ void stdp_body(const DevNet &n, const int *t_now, const Part &g)
+__device__ __forceinline__ void stdp_body(const DevNet &n, const Part &g)
 {
     extern __shared__ int4 smem_i4[];
-    const int t = *t_now;                  // the step after the window
     if (!n.win) return;
     DevWindow *win = n.win;
-    if (!deferring(n, t)) {
+    const int t = win->p1 + 1;             // the step after the window
+    if (win->defer_from > win->p1) {
         if (g.bid == 0 && threadIdx.x == 0) win->p1 = win->p0 - 1;   // closed, nothing was left to it
         return;
     }
@@ -190,8 +266,10 @@ __device__ __forceinline__ void stdp_body(const DevNet &n, const int *t_now, con
     unsigned long long *s_y = reinterpret_cast<unsigned long long *>(smem_i4);      // [kSlots * npc]
     unsigned long long *s_x = s_y + kSlots * npc;                                   // [nwarps][32]
     int32_t *s_off = reinterpret_cast<int32_t *>(s_x + nwarps * 32);                // [nwarps][32]
-    int32_t *s_lutp = s_off + nwarps * 32;
+    int32_t *s_q = s_off + nwarps * 32;                                             // [nwarps][kAmounts]
+    int32_t *s_lutp = s_q + nwarps * kAmounts;
     int32_t *s_lutm = s_lutp + kLut;
+    signed char *s_j = reinterpret_cast<signed char *>(s_lutm + kLut);              // [nwarps][kSpikeCap]
     __shared__ uint32_t s_col[kSlots];
     __shared__ uint32_t s_unit;
     const int p0 = win->p0, from = win->defer_from;
@@ -205,10 +283,12 @@ __device__ __forceinline__ void stdp_body(const DevNet &n, const int *t_now, con
     const int D = (int)n.D;
     unsigned long long *w_x = s_x + warp * 32;
     int32_t *w_off = s_off + warp * 32;
+    signed char *w_j = s_j + warp * kSpikeCap;
     for (int i = threadIdx.x; i < kLut; i += blockDim.x) {
         s_lutp[i] = n.lut_p[i];
         s_lutm[i] = n.lut_m[i];
     }
+    int32_t *w_q = s_q + warp * kAmounts;
     const uint32_t chunks = (n.ne + n.stdp_rows - 1) / n.stdp_rows;
     for (uint32_t unit = g.bid; unit < n.C * chunks;) {
         const uint32_t col = unit / chunks;
@@ -238,13 +318,47 @@ __device__ __forceinline__ void stdp_body(const DevNet &n, const int *t_now, con
             }
             w_x[lane] = x;
             w_off[lane] = end;
+            // the source's spikes that arrive in the window, in order: the
+            // last D steps before it and the window's own
+            const uint32_t pre = h.x & (0xffffffffu >> (32 - D));
+            const int npre = __popc(pre), ns = npre + __popcll(own);
+            if ((pre >> lane) & 1u) w_j[npre - __popc(pre & (0xffffffffu >> (31 - lane)))] = (signed char)(-1 - lane);
+#pragma unroll
+            for (int q = lane; q < 64; q += 32)
+                if ((own >> q) & 1ull) w_j[npre + __popcll(own & ((1ull << q) - 1ull))] = (signed char)q;
+            // what a post spike `tau` after a spike's own step, less the delay,
+            // adds: the amount at the lag to the source's latest spike
+            if (ns <= kFewSpikes) {
+#pragma unroll
+                for (int q = lane; q < kAmounts; q += 32) {
+                    const int tau = q - 31;
+                    int lag;
+                    if (tau >= 0) {
+                        const unsigned long long late = own & (tau < 63 ? (2ull << tau) - 1ull : ~0ull);
+                        lag = late ? tau - 63 + __clzll((long long)late) : tau + (h.x ? __ffs(h.x) : p0 - (int)h.y);
+                    } else {
+                        const uint32_t late = h.x & (0xffffffffu << (-1 - tau));
+                        lag = tau + (late ? __ffs(late) : p0 - (int)h.y);
+                    }
+                    w_q[q] = lag < kLut ? s_lutp[lag] : 0;
+                }
+            }
             // a source without an arrival inside any amount's reach changes nothing
             const bool live = (x & kTrainMask) || (lane >= 1 && lane <= D && (int)(x >> kWinBits) < kLut - 1);
             __syncwarp();
             if (closes || __any_sync(0xffffffffu, live)) {
                 const int64_t base = row_base(n, p);
-                if (closes) stdp_row<true>(n, base, m, D, w_off, w_x, s_y, s_lutp, s_lutm, posts, arrivals, lane);
-                else stdp_row<false>(n, base, m, D, w_off, w_x, s_y, s_lutp, s_lutm, posts, arrivals, lane);
+                auto row = [&](auto deriv, auto few) {
+                    stdp_row<decltype(deriv)::value, decltype(few)::value>(n, base, m, D, w_off, w_x, w_j, ns, s_y, w_q,
+                                                                          s_lutp, s_lutm, t - p0, posts, arrivals, lane);
+                };
+                if (ns <= kFewSpikes) {
+                    if (closes) row(std::true_type{}, std::true_type{});
+                    else row(std::false_type{}, std::true_type{});
+                } else {
+                    if (closes) row(std::true_type{}, std::false_type{});
+                    else row(std::false_type{}, std::false_type{});
+                }
             }
             __syncwarp();
         }
@@ -272,9 +386,9 @@ __global__ void __launch_bounds__(1024) k_win_open(DevNet n, const int *t_now, i
     win_open_body(n, t_now, steps, whole_grid());
 }
 
-__global__ void __launch_bounds__(256) k_train(DevNet n, const int *t_now) { train_body(n, t_now, whole_grid()); }
+__global__ void __launch_bounds__(256) k_train(DevNet n) { train_body(n, whole_grid()); }
 
-__global__ void __launch_bounds__(kStdpBlock) k_stdp(DevNet n, const int *t_now) { stdp_body(n, t_now, whole_grid()); }
+__global__ void __launch_bounds__(kStdpBlock) k_stdp(DevNet n) { stdp_body(n, whole_grid()); }
 
 __global__ void __launch_bounds__(1024) k_win_open_b(BatchLaunch b, int steps)
 {
@@ -287,14 +401,14 @@ __global__ void __launch_bounds__(256) k_train_b(BatchLaunch b)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
-    train_body(n, x.t_now, x.part);
+    train_body(n, x.part);
 }
 
 __global__ void __launch_bounds__(kStdpBlock) k_stdp_b(BatchLaunch b)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
-    stdp_body(n, x.t_now, x.part);
+    stdp_body(n, x.part);
 }
 
 }  // namespace snn

@@ -1,0 +1,131 @@
+"""Plasticity windows and resident grids against the oracle, where they can go
+wrong: columns that are no multiple of 32 neurons, slices, the shortest and
+longest delays, calls that end inside, at and behind a window or a period,
+external events, activity that stops a resident grid, FP64, and step kernels
+that start a window's deferral in its middle.  Everything is bit-exact."""
+import numpy as np
+import pytest
+
+import workloads
+from test_gpu_parity import assert_same_run, gpu_net
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def eng():
+    import paper_1310_8478_gb300 as e
+    e.build_engine()
+    return e
+
+
+def _cfg(gx, gy, npc, m, mix=(40, 30, 20, 10), **kw):
+    kw.setdefault("exc_per_col", max(1, npc * 4 // 5))
+    return workloads.custom(grid_x=gx, grid_y=gy, neurons_per_col=npc, fanout=m,
+                            pct_ring=mix if gx * gy > 1 else (100, 0, 0, 0), **kw)
+
+
+CASES = {
+    # calls of every remainder of a window, across two periods of 70 ms
+    "ragged_columns": (_cfg(3, 2, 333, 61, seed=61, deriv_period_ms=70), [4, 50, 3, 51, 1, 49, 101, 5]),
+    "one_column_odd": (_cfg(1, 1, 77, 40, seed=62, thal_per_col_per_ms=3, deriv_period_ms=60), [50, 7, 64, 99]),
+    # three neurons per column, a single excitatory one
+    "tiny_columns": (_cfg(5, 4, 3, 9, seed=63, exc_per_col=1, thal_per_col_per_ms=1), [60, 120]),
+    "longest_delay": (_cfg(2, 2, 100, 33, seed=64, max_delay_ms=31, thal_per_col_per_ms=2), [55, 130]),
+    "shortest_delay": (_cfg(2, 3, 65, 24, seed=65, max_delay_ms=1, w_exc0_q16=7 * 65536, thal_per_col_per_ms=2), [120]),
+    # thousands of drive events per column and window are not drawn ahead
+    "strong_drive": (_cfg(2, 1, 200, 20, seed=66, thal_per_col_per_ms=40, thal_amp_q16=4 * 65536), [53, 60]),
+    # runs away: the resident grid stops, the step kernels go on and defer
+    "runaway": (_cfg(2, 2, 400, 400, seed=67, w_exc0_q16=8 * 65536, thal_per_col_per_ms=2, deriv_period_ms=90), [40, 120, 70]),
+    # other STDP tables, the depression too wide for 15 bits
+    "wide_depression": (_cfg(2, 2, 100, 50, seed=68, a_minus_mv=1.0, tau_plus_ms=12.0, thal_per_col_per_ms=2), [75, 75]),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_calls_of_any_length_equal_the_oracle(eng, orc, name):
+    cfg, calls = CASES[name]
+    o = orc.Oracle(cfg)
+    with gpu_net(eng, cfg) as n:
+        for steps in calls:
+            o.run(steps)
+            n.run(steps)
+            assert_same_run(o, n)
+        assert n.counters()["spikes"] > 10          # something happened
+
+
+def test_fp64_and_events_inside_windows(eng, orc):
+    cfg = _cfg(2, 2, 90, 45, seed=69)
+    rng = np.random.default_rng(3)
+    t, g = rng.integers(0, 130, 300), rng.integers(0, 360, 300)
+    t.sort()
+    q = np.full(300, 25 * 65536)
+    o = orc.Oracle(cfg)
+    o.set_stimulus(t, g, q)
+    o.run(140)
+    with gpu_net(eng, cfg) as n:
+        n.set_stimulus(t, g, q)
+        n.run(140)
+        assert_same_run(o, n)
+    cfg["flags"] = eng.snn.FP64
+    o = orc.Oracle(cfg, flags=4)
+    o.run(140)
+    with gpu_net(eng, cfg) as n:
+        n.run(140)
+        ot, og = o.raster()
+        gt, gg = n.raster()
+        assert np.array_equal(gt, ot) and np.array_equal(gg, og)
+        s, x = o.neurons(), n.neurons_f64()
+        assert np.array_equal(x["v"], s["vd"]) and np.array_equal(x["u"], s["ud"])
+        w, sd = n.weights()
+        assert np.array_equal(w, o.synapses()["w"]) and np.array_equal(sd, o.synapses()["sd"])
+
+
+def test_resident_and_step_kernels_share_a_net(eng, orc):
+    """Windows of one call and single steps of the next, checkpoints between
+    them, and the spike lists that a later launch shape delivers from."""
+    cfg = _cfg(3, 3, 120, 60, seed=70, thal_per_col_per_ms=2, deriv_period_ms=110)
+    o = orc.Oracle(cfg)
+    o.run(300)
+    with gpu_net(eng, cfg) as n, gpu_net(eng, cfg) as other:
+        n.run(64)
+        for _ in range(20):
+            n.step()
+        n.run(50)
+        other.load_state(n.save_state())
+        for net in (n, other):
+            if net is other:
+                net.set_launch(dense_permille=1001, ring_permille=0xffffffff)
+            net.run(26)
+            net.set_launch(dense_permille=1001, ring_permille=0xffffffff)
+            net.run(40)
+            net.set_launch(dense_permille=250)
+            net.run(100)
+            s = o.synapses()
+            w, sd = net.weights()
+            assert np.array_equal(w, s["w"]) and np.array_equal(sd, s["sd"])
+            assert net.counters()["spikes"] == o.counters()["spikes"]
+            x = net.neurons()
+            assert np.array_equal(x["v"].view(np.int32), o.neurons()["v"].view(np.int32))
+        assert_same_run(o, n)
+
+
+@pytest.mark.parametrize("npc,m", [(1000, 300), (1250, 1125)])
+def test_step_kernels_defer_inside_a_window(eng, npc, m):
+    """A net too large for a resident grid: the windows of long calls against
+    single steps (which never defer), whose own results the parity tests hold
+    against the oracle on small nets."""
+    cfg = _cfg(20, 20, npc, m, seed=71, mix=(76, 12, 8, 4) if m == 300 else (40, 30, 20, 10), deriv_period_ms=60)
+    T = 150 if m == 300 else 75
+    with eng.Network(cfg, raster_capacity=0) as a, eng.Network(cfg, raster_capacity=0) as b:
+        a.run(T)
+        for _ in range(T // 3):
+            b.run(3)
+        ca, cb = a.counters(), b.counters()
+        assert ca == cb and ca["spikes"] > 400 * npc // 2
+        for first in (0, 7 * npc, 399 * npc):
+            x, y = a.synapses(first, npc, fields=("w", "sd")), b.synapses(first, npc, fields=("w", "sd"))
+            assert np.array_equal(x["w"], y["w"]) and np.array_equal(x["sd"], y["sd"])
+            assert np.count_nonzero(x["sd"]) > npc
+        x, y = a.neurons(), b.neurons()
+        assert np.array_equal(x["v"].view(np.int32), y["v"].view(np.int32))
