@@ -117,7 +117,7 @@ typedef struct {
 typedef struct {
     uint32_t deliver_block;          /* threads per block of the event-driven delivery (multiple of 32;
                                         the column-ordered delivery gives one column to each block
-                                        and takes at most 256 threads) */
+                                        of twice as many threads, 512 at most) */
     uint32_t deliver_blocks_per_sm;  /* resident blocks per SM of the event-driven delivery (at most) */
     uint32_t neuron_block;           /* threads per block of the neuron update */
     uint32_t ltp_block;              /* threads per block of the event-driven potentiation */

@@ -546,6 +546,184 @@ __device__ __forceinline__ void prefetch_segment(const DevNet &n, int64_t k, boo
     if (sd) prefetch_l2(n.sd + k, cnt * 4u);
 }
 
+// ---------------------------------------------------------------------------
+// event-driven walk of delay buckets by the column-ordered delivery: a block
+// lists its due (row, delay) items in shared memory, its warps take them 32 at
+// a time (the resident grids walk alike, but inside their step loop: through
+// these functions their steps took 5 % longer)
+// ---------------------------------------------------------------------------
+constexpr uint32_t kItems = 2048;            // items listed by a block
+constexpr int kFlight = 4;                   // buckets of a group of lanes in flight
+
+// Items of rows [r0, r1), whose due delays are the bits of (hist[row] << 1) &
+// dmask, appended to the list as (row0 + row) << 5 | delay; those beyond its
+// end are only counted.  Called by the whole block (of
+// `threads` threads, here and below).
+__device__ __forceinline__ void list_items(uint32_t threads, const uint32_t *hist, uint32_t r0, uint32_t r1, uint32_t row0, uint32_t dmask,
+                                           uint32_t *items, unsigned *count)
+{
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i = r0 + threadIdx.x; i - lane < r1; i += threads) {
+        uint32_t f = i < r1 ? (hist[i] << 1) & dmask : 0u;
+        if (!__any_sync(0xffffffffu, f != 0)) continue;
+        const uint32_t own = __popc(f);
+        uint32_t incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        unsigned at = 0;
+        if (lane == 31) at = atomicAdd(count, incl);
+        at = __shfl_sync(0xffffffffu, at, 31) + incl - own;
+        if (at + own > kItems) continue;
+        for (; f; f &= f - 1u) items[at++] = ((row0 + i) << 5) | (uint32_t)(__ffs(f) - 1);
+    }
+}
+
+// Rows [r0, r1) with bit 0 of their history set (fired at t - 1), appended to
+// the list as row0 + row.  Called by the whole block.
+__device__ __forceinline__ void list_fired(uint32_t threads, const uint32_t *hist, uint32_t r0, uint32_t r1, uint32_t row0, uint32_t *rows,
+                                           unsigned *count)
+{
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i = r0 + threadIdx.x; i - lane < r1; i += threads) {
+        const bool on = i < r1 && (hist[i] & 1u);
+        const uint32_t b = __ballot_sync(0xffffffffu, on);
+        if (!b) continue;
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(count, (unsigned)__popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & lanemask_lt());
+        if (on) rows[at] = row0 + i;
+    }
+}
+
+// Inhibitory rows that fired at t - 1 (generated nets): the whole row at
+// delay 1, one weight, targets of the own column; all threads share the
+// rows' 8-synapse chunks.  tg: targets of the column, in0: its input (shared).
+__device__ __forceinline__ void walk_inhibitory(uint32_t threads, const DevNet &n, const uint32_t *rows, uint32_t count, const uint16_t *tg,
+                                                int64_t col_syn, uint32_t in0)
+{
+    const uint4 *t4 = reinterpret_cast<const uint4 *>(tg);
+    const uint32_t m = n.canon_m, cpr = (m + 7u) / 8u, row_chunks = n.uniform_m / 8u;
+    for (uint32_t c = threadIdx.x; c < count * cpr; c += threads) {
+        const uint32_t q = c / cpr, ci = c - q * cpr;
+        const uint32_t at = rows[q] * row_chunks + ci;
+        if (out_of_range(n, 8 * (int64_t)at + 8 <= col_syn)) continue;
+        const uint4 tv = t4[at];
+        const uint32_t nv = min(8u, m - 8u * ci);
+        const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
+        if (nv == 8) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t v = (tw[u >> 1] >> (16 * (u & 1))) & 0xffffu;
+                if (!out_of_range(n, v < n.npc)) red_shared(in0 + 4u * v, n.w_inh);
+            }
+        } else {
+            for (uint32_t u = 0; u < nv; ++u) {
+                const uint32_t v = tg[8 * (int64_t)at + u];
+                if (!out_of_range(n, v < n.npc)) red_shared(in0 + 4u * v, n.w_inh);
+            }
+        }
+    }
+}
+
+// log2 of the lanes per bucket: the power of two that a mean bucket (M / D
+// synapses) fills best, 8 at least
+__device__ __forceinline__ int bucket_lanes(const DevNet &n)
+{
+    const uint32_t mean = n.canon_m / n.D;
+    return mean <= 6 ? 3 : mean <= 12 ? 4 : 5;
+}
+
+// The warp's share of a block's `items`, tile by tile: a lane fetches an
+// item's bucket, then a lane takes a synapse, a group of 2^lg lanes a bucket,
+// kFlight buckets of every group in flight.  (A lane per 8-synapse chunk, with
+// a branch per synapse, took 2.5 times the instructions at M = 200, whose
+// buckets of 10 fill 0.6 of their chunks.)  Per synapse: x = begin(target word,
+// weight), then, behind the other synapses in flight, end(x, position).
+// `first` runs once under the first fetch.  w_ab: 64 words of the warp's own.
+// Returns the synapses walked (lane 0).
+template <typename First, typename Begin, typename End>
+__device__ __forceinline__ unsigned walk_items(uint32_t threads, const DevNet &n, uint32_t col, const uint32_t *items, uint32_t count,
+                                               int32_t *w_ab, int lg, const uint16_t *tg, const int32_t *wt,
+                                               int64_t col_syn, First first, Begin begin, End end)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)(threads >> 5);
+    const int gl = lane & ((1 << lg) - 1), gi = lane >> lg, groups = 32 >> lg;
+    int32_t *w_a = w_ab, *w_b = w_ab + 32;
+    const uint32_t share = (count + warps - 1) / warps;
+    const uint32_t i_hi = min(count, (warp + 1) * share);
+    uint32_t i_lo = warp * share, row = 0;
+    unsigned walked = 0;
+    int a = 0, b = 0;
+    auto fetch = [&]() {
+        a = b = 0;
+        if (i_lo + lane < i_hi) {
+            const uint32_t it = items[i_lo + lane];
+            row = it >> 5;
+            const uint16_t *off = n.doff + (size_t)(col * n.npc + row) * kDoffStride + (it & 31u);
+            a = off[-1];
+            b = off[0];
+        }
+    };
+    fetch();
+    first();
+    while (i_lo < i_hi) {
+        const int tile = (int)min(32u, i_hi - i_lo);
+        walked += (unsigned)__reduce_add_sync(0xffffffffu, b - a);
+        const int base = (int)(row * n.uniform_m);
+        w_a[lane] = base + a;
+        w_b[lane] = base + b;
+        __syncwarp();
+        i_lo += 32;
+        fetch();                                 // the next tile's buckets, under this tile's walk
+        for (int q0 = 0; q0 < tile; q0 += kFlight * groups) {
+            int at[kFlight], stop[kFlight];
+            int left = 0;
+#pragma unroll
+            for (int h = 0; h < kFlight; ++h) {
+                const int q = q0 + h * groups + gi;
+                at[h] = q < tile ? w_a[q] + gl : 0;
+                stop[h] = q < tile ? w_b[q] : 0;
+                left |= at[h] < stop[h];
+            }
+            while (__any_sync(0xffffffffu, left)) {
+                uint32_t v[kFlight];
+                int32_t x[kFlight];
+                left = 0;
+#pragma unroll
+                for (int h = 0; h < kFlight; ++h) {
+                    v[h] = 0xffffffffu;
+                    if (at[h] < stop[h] && !out_of_range(n, at[h] >= 0 && at[h] < col_syn)) {
+                        v[h] = tg[at[h]];
+                        x[h] = wt[at[h]];
+                    }
+                    at[h] += 1 << lg;
+                    left |= at[h] < stop[h];
+                }
+#pragma unroll
+                for (int h = 0; h < kFlight; ++h)
+                    if (v[h] != 0xffffffffu) x[h] = out_of_range(n, v[h] < kSlots * n.npc) ? kNever : begin(v[h], x[h]);
+#pragma unroll
+                for (int h = 0; h < kFlight; ++h)
+                    if (v[h] != 0xffffffffu) end(x[h], at[h] - (1 << lg));
+            }
+        }
+        __syncwarp();
+    }
+    return walked;
+}
+
+// 4 bytes from global to shared memory, asynchronously
+__device__ __forceinline__ void copy4_async(void *shared, const void *global)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(shared)), "l"(global)
+                 : "memory");
+}
+
+__device__ __forceinline__ void wait_async() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // thalamic drive (thal_per_col events per column, Philox keyed by (t, col))
 // and the external events of step t, by the threads of a whole grid
 __device__ __forceinline__ void drive(const DevNet &n, int t, uint32_t gtid, uint32_t gthreads)
@@ -646,13 +824,12 @@ constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's
 // window's pass that closes a period
 enum FoldMode { kFoldStep = 0, kFoldForce = 1, kFoldWindow = 2 };
 constexpr uint32_t kStagedBlock = 512;      // threads per block of the column-staged delivery
-// the column-ordered delivery is compiled for five resident blocks of at most
-// this many threads per SM (47 registers; the measured optimum): a launch
-// shape asking for more threads per block is clamped to it
-constexpr uint32_t kOrderedMaxBlock = 256;
+// the column-ordered delivery takes twice a launch shape's delivery threads
+// per column, at most this many
+constexpr uint32_t kOrderedMaxBlock = 512;
 __host__ __device__ __forceinline__ uint32_t ordered_block(uint32_t deliver_block)
 {
-    return deliver_block < kOrderedMaxBlock ? deliver_block : kOrderedMaxBlock;
+    return 2 * deliver_block < kOrderedMaxBlock ? 2 * deliver_block : kOrderedMaxBlock;
 }
 
 }  // namespace snn

@@ -183,24 +183,16 @@ __device__ __forceinline__ void deliver_ring(const DevNet &n, const int *t_now, 
 // sparse S1, column by column (generated nets with compact targets).  A
 // persistent grid takes source columns from a step-wide cursor, so the
 // columns in flight form a narrow band of the torus and so do the targets
-// they reach.  Per column, every thread first issues its share of the loads
-// of the column's spike-history words and its neurons' last spikes (one
-// round of latency for the whole column).  Then the warps take 32-row groups
-// from a block cursor, the inhibitory groups first (an inhibitory spike
-// delivers its whole row at delay 1, an excitatory one a single delay
-// bucket: longest work first, so the warps finish the column together); a
-// warp turns every delay bucket d whose source fired at t - d into an item
-// and walks the 8-synapse chunks of 32 items with all lanes, one 16-byte
-// load of 8 targets (and of 4 weights / derivatives twice) per chunk.
-//   kStage (steps with many events): the input accumulators and LTD amounts
-//   of the 13 columns the block's synapses reach are staged in shared memory,
-//   so an event costs a shared atomic and a shared load; the input is flushed
-//   with one coalesced reduction per touched neuron.
-//   otherwise: only the source column's own neurons are staged (the targets
-//   of every inhibitory synapse and of the local share of the excitatory
-//   ones); an event on another column is an L2 reduction into the target's
-//   input and a gather of its last spike, both on the band of columns in
-//   flight, which stays in L2.
+// they reach.  Two forms:
+//   deliver_columns (the default): the source column's own neurons -- the
+//   targets of every inhibitory synapse and of the local share of the
+//   excitatory ones -- have their input and last spikes in shared memory.
+//   deliver_cols (13-column staging, for launch shapes that ask for it): the
+//   input accumulators and LTD amounts of all 13 columns the block's synapses
+//   reach are, so an event costs a shared atomic and a shared load.  Warps take
+//   32-row groups from a block cursor, turn every delay bucket d whose source
+//   fired at t - d into an item and walk the 8-synapse chunks of 32 items with
+//   all lanes.
 // ---------------------------------------------------------------------------
 constexpr int kItemCap = 96;                // per warp: pending (row, bucket) items
 // per warp: first chunk, chunk-count prefix, first / end synapse, kind of each
@@ -215,24 +207,20 @@ size_t staged_smem_bytes(uint32_t npc, uint32_t block)
 
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block)
 {
-    return (size_t)kLut * 4 + (size_t)npc * 16 + (size_t)(block / 32) * kTileWords * 4;
+    return (size_t)kLut * 4 + (size_t)npc * 24 + kItems * 4 + (size_t)(block / 32) * 64 * 4;
 }
 
-// s_amt: kStage -> uint16 LTD amounts of the 13 staged columns;
-//        otherwise int32 LTD amounts of the source column's own neurons.
+// s_x: LTD amounts of the 13 staged columns.
 // s_hist: the history words (bit k: fired at t - k) of the column's rows.
 // kStdp: depression at the arrivals (not in steps that leave their STDP to a
 // window's pass).
-template <bool kStage, bool kStdp>
+template <bool kStdp>
 __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_lut, int32_t *s_in, int32_t *s_tile,
-                                             void *s_amt, uint32_t *s_hist, const Part &g, uint32_t *s_inh = nullptr)
+                                             uint16_t *s_x, uint32_t *s_hist, const Part &g)
 {
     __shared__ uint32_t s_col[kSlots];
     __shared__ uint32_t s_unit[2];             // the next column, claimed while this one is walked
     __shared__ uint32_t s_grp;                 // row groups of the current column handed out
-    __shared__ uint32_t s_ninh;                // inhibitory rows of the column that fired at t - 1
-    uint16_t *s_x = reinterpret_cast<uint16_t *>(s_amt);
-    int32_t *s_ltd = reinterpret_cast<int32_t *>(s_amt);
     const uint32_t npc = n.npc;
     const uint32_t ngroups = (npc + 31) / 32;
     const bool deliver_on = !(n.flags & SNN_DELIVERY_OFF);
@@ -254,52 +242,22 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
         if (threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
         if (threadIdx.x == 0) {
             s_grp = 0;
-            s_ninh = 0;
             s_unit[par] = g.nblk + atomicAdd(&n.ctr->staged_cursor, 1u);
         }
-        if (kStage) __syncthreads();
-        // one round of loads for the whole column: history words, and the
-        // staged neurons' last spikes turned into LTD amounts at lag
-        // t - last_spike >= 1 (saturated at the table end, whose entry is 0)
-        if (!kStage) {
-            constexpr int kSetup = 8;                  // rows per thread in flight
-            const int32_t *ls = n.last_spike + (size_t)col * npc;
-            const uint2 *hl = n.hl + (size_t)col * npc;
-            for (uint32_t base = threadIdx.x; base < npc; base += kSetup * blockDim.x) {
-                uint32_t hv[kSetup];
-                int32_t lv[kSetup];
-#pragma unroll
-                for (int q = 0; q < kSetup; ++q) {
-                    const uint32_t loc = base + q * blockDim.x;
-                    hv[q] = 0;
-                    lv[q] = kNever;
-                    if (loc < npc) {
-                        if (deliver_on) hv[q] = hl[loc].x;
-                        lv[q] = ls[loc];
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < kSetup; ++q) {
-                    const uint32_t loc = base + q * blockDim.x;
-                    if (loc < npc) {
-                        s_hist[loc] = hv[q];
-                        s_ltd[loc] = kStdp ? s_lut[min(t - lv[q], kLut - 1)] : 0;
-                        s_in[loc] = 0;
-                    }
-                }
-            }
-        } else {
-            for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x)
-                s_hist[loc] = deliver_on ? n.hl[col * npc + loc].x : 0u;
-            // at most 15 bits per amount: the host checks the table
-            for (int sl = 0; sl < kSlots; ++sl) {
-                const int32_t *ls = n.last_spike + (size_t)s_col[sl] * npc;
-                uint16_t *x_row = s_x + sl * npc;
-                int32_t *in_row = s_in + sl * npc;
-                for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                    x_row[loc] = kStdp ? (uint16_t)s_lut[min(t - ls[loc], kLut - 1)] : (uint16_t)0;
-                    in_row[loc] = 0;
-                }
+        __syncthreads();
+        // history words, and the staged neurons' last spikes turned into LTD
+        // amounts at lag t - last_spike >= 1 (saturated at the table end, whose
+        // entry is 0)
+        for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x)
+            s_hist[loc] = deliver_on ? n.hl[col * npc + loc].x : 0u;
+        // at most 15 bits per amount: the host checks the table
+        for (int sl = 0; sl < kSlots; ++sl) {
+            const int32_t *ls = n.last_spike + (size_t)s_col[sl] * npc;
+            uint16_t *x_row = s_x + sl * npc;
+            int32_t *in_row = s_in + sl * npc;
+            for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
+                x_row[loc] = kStdp ? (uint16_t)s_lut[min(t - ls[loc], kLut - 1)] : (uint16_t)0;
+                in_row[loc] = 0;
             }
         }
         __syncthreads();
@@ -336,10 +294,8 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
             w_exc[lane] = exc;
             if (lane == 0) {
                 w_start[32] = total;
-                if (!n.tile) {                 // a tile counts the events on its own columns below
-                    ev_all += (unsigned long long)len_all;
-                    ev_exc += (unsigned long long)len_exc;
-                }
+                ev_all += (unsigned long long)len_all;
+                ev_exc += (unsigned long long)len_exc;
             }
             __syncwarp();
             int j = 0;
@@ -361,91 +317,29 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                 }
                 const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
                 const int32_t wk[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-                int tile_ev = 0;                                    // tiles: events on own columns
-                int32_t am[8];                                      // LTD amount, or (remote) last spike
-                uint32_t remote = 0;                                // bit u: target on another column
+                int32_t am[8];                                      // LTD amount
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     am[u] = 0;
                     if (!((mask >> u) & 1u)) continue;
                     const uint32_t v = (tw[u >> 1] >> (16 * (u & 1))) & 0xffffu;
                     if (out_of_range(n, v < kSlots * npc)) continue;
-                    if (kStage) {
-                        atomicAdd(&s_in[v], wk[u]);
-                        am[u] = (ex && kStdp) ? (int32_t)s_x[v] : 0;
-                    } else {
-                        const uint32_t slot = __umulhi(v, n.npc_recip);
-                        const uint32_t loc = v - slot * npc;
-                        if (n.tile && !owned_column(n, s_col[slot])) continue;   // another tile's target
-                        if (n.tile) ++tile_ev;
-                        if (slot == 0) {
-                            atomicAdd(&s_in[loc], wk[u]);
-                            am[u] = (ex && kStdp) ? s_ltd[loc] : 0;
-                        } else {
-                            const uint32_t gid = s_col[slot] * npc + loc;        // target gid
-                            red_add(&n.I[gid], wk[u]);
-                            if (ex && kStdp) {
-                                am[u] = n.last_spike[gid];
-                                remote |= 1u << u;
-                            }
-                        }
-                    }
-                }
-                if (n.tile) {
-                    ev_all += (unsigned long long)tile_ev;
-                    if (ex) ev_exc += (unsigned long long)tile_ev;
+                    atomicAdd(&s_in[v], wk[u]);
+                    am[u] = (ex && kStdp) ? (int32_t)s_x[v] : 0;
                 }
                 if (ex && kStdp) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        if (!((mask >> u) & 1u)) continue;
-                        int32_t x = am[u];
-                        if ((remote >> u) & 1u) {
-                            const int lag = t - x;                            // >= 1
-                            x = lag < kLut ? s_lut[lag] : 0;
-                        }
-                        if (x) red_add(&n.sd[cbase + k0 + u], -x);     // no load: most amounts are 0
+                        if (((mask >> u) & 1u) && am[u]) red_add(&n.sd[cbase + k0 + u], -am[u]);   // no load: most are 0
                     }
                 }
             }
             __syncwarp();
         };
-        // Without 13-column staging, the inhibitory rows that fired at t - 1
-        // are walked by the whole block first: such a row delivers all of its
-        // synapses at delay 1, with one weight, to excitatory neurons of its
-        // own column (generated nets), so the block lists them and spreads
-        // the concatenated rows' chunks over all threads -- an even share
-        // whatever the rows' distribution over the groups.
-        if (!kStage) {
-            const bool mine = deliver_on && (!n.tile || owned_column(n, col));
-            if (mine)
-                for (uint32_t r = n.ne + threadIdx.x; r < npc; r += blockDim.x)
-                    if (s_hist[r] & 1u) s_inh[atomicAdd(&s_ninh, 1u)] = r;
-            __syncthreads();
-            const uint32_t ninh = s_ninh;
-            const uint32_t m = n.canon_m, cpr = (m + 7u) / 8u;
-            for (uint32_t c = threadIdx.x; c < ninh * cpr; c += blockDim.x) {
-                const uint32_t it = c / cpr, ci = c - it * cpr;
-                const int64_t k0 = (int64_t)s_inh[it] * n.uniform_m + 8 * ci;   // column-relative
-                if (out_of_range(n, k0 + 8 <= col_syn && cbase + k0 + 8 <= n.S)) continue;
-                const uint4 tv = t4[k0 >> 3];
-                const uint32_t nv = min(8u, m - 8u * ci);
-                const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const uint32_t v = (tw[u >> 1] >> (16 * (u & 1))) & 0xffffu;
-                    if ((uint32_t)u < nv && !out_of_range(n, v < npc)) atomicAdd(&s_in[v], n.w_inh);
-                }
-            }
-            if (threadIdx.x == 0) ev_all += (unsigned long long)ninh * m;
-        }
         // Items (row << 5 | bucket) collect in the warp's buffer across row
         // groups and are walked 32 at a time, so that a tile is full even when
         // few rows of a group fired; a group with too many items for the
         // buffer is walked directly, one flagged bucket per lane and pass.
-        // (Without staging the inhibitory rows are done above: the groups
-        // cover the excitatory rows only.)
-        const uint32_t ngroups_w = kStage ? ngroups : (n.ne + 31u) / 32u;
         int cnt = 0;                                   // items in the buffer
         bool groups_left = true;                       // warp-uniform
         uint32_t fb = 0, r = 0;                        // a group walked directly: its remaining flags
@@ -470,13 +364,13 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
                 uint32_t grp = 0;
                 if (lane == 0) grp = atomicAdd(&s_grp, 1u);
                 grp = __shfl_sync(0xffffffffu, grp, 0);
-                if (grp >= ngroups_w) {
+                if (grp >= ngroups) {
                     groups_left = false;
                     continue;
                 }
-                r = (ngroups_w - 1u - grp) * 32u + lane;   // the last groups (inhibitory rows) first
+                r = (ngroups - 1u - grp) * 32u + lane;   // the last groups (inhibitory rows) first
                 uint32_t f = 0;                        // bit d: the row's source fired at t - d
-                if (r < npc && (kStage || r < n.ne)) f = (s_hist[r] << 1) & (r < n.ne ? dmask_e : dmask_i);
+                if (r < npc) f = (s_hist[r] << 1) & (r < n.ne ? dmask_e : dmask_i);
                 const int mine = __popc(f);
                 int incl = mine;
 #pragma unroll
@@ -507,24 +401,162 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
             tile(tr, td, tv);
         }
         __syncthreads();
-        if (kStage) {
-            for (int sl = 0; sl < kSlots; ++sl) {
-                int32_t *dst = n.I + (size_t)s_col[sl] * npc;
-                const int32_t *in_row = s_in + sl * npc;
-                for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                    const int32_t x = in_row[loc];
-                    if (x) red_add(&dst[loc], x);
-                }
-            }
-        } else {
-            int32_t *dst = n.I + (size_t)col * npc;
+        for (int sl = 0; sl < kSlots; ++sl) {
+            int32_t *dst = n.I + (size_t)s_col[sl] * npc;
+            const int32_t *in_row = s_in + sl * npc;
             for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                const int32_t x = s_in[loc];
+                const int32_t x = in_row[loc];
                 if (x) red_add(&dst[loc], x);
             }
         }
         __syncthreads();
         col = s_unit[par];
+    }
+    if (lane != 0) ev_all = ev_exc = 0;
+    const unsigned long long ba = block_sum(ev_all);
+    const unsigned long long be = block_sum(ev_exc);
+    if (threadIdx.x == 0 && ba) {
+        atomicAdd(&n.ctr->e_all, ba);
+        atomicAdd(&n.ctr->e_exc, be);
+    }
+}
+
+// The column-ordered delivery.  Per column a block lists the inhibitory rows
+// that fired at t - 1 and the due (row, delay) items, walks both with all of
+// its threads (walk_inhibitory, walk_items) and flushes the column's own input
+// with one coalesced reduction per touched neuron; a target on another column
+// is a reduction into its input and, with kStdp, a gather of its last spike,
+// both on the band of columns in flight, which stays in L2.  The next column is
+// claimed two columns ahead, and its histories and last spikes are copied into
+// shared memory while this one is walked.  Bound by latency and instruction
+// issue (half of it) at 64 registers and two blocks of 512 threads per SM; with
+// three at 40 registers it spilled (busy 32x32 net: 142 against 129 us per
+// step), and five of 256 threads left a wave of 1024 columns two thirds full
+// (with depression, per step: busy 32x32 net 119 -> 90 us, onset of the 64x32
+// benchmark torus 83 -> 68, 64x64 torus of the paper's columns 91 -> 88).
+template <bool kStdp>
+__device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Part &g)
+{
+    extern __shared__ int4 smem_i4[];
+    __shared__ uint32_t s_col[2][kSlotStride], s_next[2];
+    __shared__ unsigned s_items_n, s_inh_n;
+    const uint32_t npc = n.npc, ne = n.ne;
+    int32_t *const s_lut = reinterpret_cast<int32_t *>(smem_i4);
+    int32_t *const s_in = s_lut + kLut;                                   // [npc] input of the column
+    uint32_t *const s_hist = reinterpret_cast<uint32_t *>(s_in + npc);    // [2][npc] bit k: fired at t - 1 - k
+    int32_t *const s_last = reinterpret_cast<int32_t *>(s_hist + 2 * npc);   // [2][npc] last spikes
+    uint32_t *const s_inh = reinterpret_cast<uint32_t *>(s_last + 2 * npc);  // [npc]
+    uint32_t *const s_items = s_inh + npc;                                // [kItems]
+    int32_t *const w_ab = reinterpret_cast<int32_t *>(s_items + kItems) + (threadIdx.x >> 5) * 64;
+    const int lane = threadIdx.x & 31;
+    const uint32_t dmask = (2u << n.D) - 2u;
+    const int64_t col_syn = (int64_t)npc * n.uniform_m;
+    const int lg = bucket_lanes(n);
+    if (kStdp)
+        for (int i = threadIdx.x; i < kLut; i += blockDim.x) s_lut[i] = n.lut_m[i];
+    drive(n, t, part_tid(g), part_threads(g));
+    if (n.flags & SNN_DELIVERY_OFF) return;
+    auto copy = [&](uint32_t col, int b) {
+        if (threadIdx.x < kSlotStride) copy4_async(&s_col[b][threadIdx.x], n.nbr + col * kSlotStride + threadIdx.x);
+        for (uint32_t i = threadIdx.x; i < npc; i += blockDim.x) {
+            copy4_async(s_hist + b * npc + i, &n.hl[(size_t)col * npc + i].x);
+            if (kStdp) copy4_async(s_last + b * npc + i, n.last_spike + (size_t)col * npc + i);
+        }
+    };
+    uint32_t col = g.bid;
+    if (col < n.C) copy(col, 0);
+    for (uint32_t i = threadIdx.x; i < npc; i += blockDim.x) s_in[i] = 0;
+    if (threadIdx.x == 0) {
+        s_next[0] = g.nblk + atomicAdd(&n.ctr->staged_cursor, 1u);
+        s_items_n = s_inh_n = 0;
+    }
+    unsigned long long ev_all = 0, ev_exc = 0;
+    for (int b = 0; col < n.C; b ^= 1) {
+        wait_async();
+        __syncthreads();
+        const uint32_t next = s_next[b];
+        uint32_t claimed = n.C;
+        if (next < n.C) {
+            copy(next, b ^ 1);
+            if (threadIdx.x == 0) claimed = g.nblk + atomicAdd(&n.ctr->staged_cursor, 1u);
+        }
+        const uint32_t *hist = s_hist + b * npc, *cols = s_col[b];
+        const int32_t *last = s_last + b * npc;
+        const int64_t cbase = (int64_t)col * col_syn;                     // first synapse of the column (8-aligned)
+        const uint16_t *tg = n.tgt16 + cbase;
+        int32_t *const sd = n.sd + cbase;
+        // slots that lead back to the column (rings of a small torus)
+        const uint32_t local = __ballot_sync(0xffffffffu, lane < kSlots && cols[lane] == col);
+        const bool mine = !n.tile || owned_column(n, col);                // inhibitory targets lie in the column
+        if (mine) list_fired(blockDim.x, hist, ne, npc, 0, s_inh, &s_inh_n);
+        // excitatory rows: all of them at once in a sparse step; where their
+        // items do not fit the list, in ranges, halved until they do
+        uint32_t range = ne;
+        bool begun = false;
+        for (uint32_t r0 = 0; r0 < ne;) {
+            list_items(blockDim.x, hist, r0, min(ne, r0 + range), 0, dmask, s_items, &s_items_n);
+            __syncthreads();
+            const uint32_t items = s_items_n;
+            if (items > kItems) {
+                range = max(kItems / n.D, range / 2);
+                __syncthreads();
+                if (threadIdx.x == 0) s_items_n = 0;
+                __syncthreads();
+                continue;
+            }
+            unsigned seen = 0;                                            // a tile's events on its own columns
+            const unsigned walked = walk_items(
+                blockDim.x, n, col, s_items, items, w_ab, lg, tg, n.w + cbase, col_syn,
+                [&] {
+                    if (begun) return;
+                    walk_inhibitory(blockDim.x, n, s_inh, s_inh_n, tg, col_syn, (uint32_t)__cvta_generic_to_shared(s_in));
+                    if (threadIdx.x == 0) ev_all += (unsigned long long)s_inh_n * n.canon_m;
+                },
+                [&](uint32_t v, int32_t w) -> int32_t {
+                    const uint32_t slot = __umulhi(v, n.npc_recip), loc = v - slot * npc;
+                    if (n.tile) {
+                        if (!owned_column(n, cols[slot])) return kNever;  // another tile's target
+                        ++seen;
+                    }
+                    if ((local >> slot) & 1u) {
+                        atomicAdd(&s_in[loc], w);
+                        return kStdp ? last[loc] : 0;
+                    }
+                    const uint32_t gid = cols[slot] * npc + loc;
+                    red_add(&n.I[gid], w);
+                    return kStdp ? n.last_spike[gid] : 0;
+                },
+                [&](int32_t x, int at) {
+                    if (!kStdp) return;
+                    const int32_t amount = s_lut[min(t - x, kLut - 1)];   // lag >= 1
+                    if (amount) red_add(&sd[at], -amount);                // no load: most amounts are 0
+                });
+            if (n.tile) {
+                ev_all += seen;
+                ev_exc += seen;
+            } else if (lane == 0) {
+                ev_all += walked;
+                ev_exc += walked;
+            }
+            begun = true;
+            r0 += range;
+            __syncthreads();                                              // the items and the column's input are done
+            if (threadIdx.x == 0) s_items_n = 0;
+            if (r0 < ne) __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            s_next[b ^ 1] = claimed;
+            s_inh_n = 0;
+        }
+        int32_t *dst = n.I + (size_t)col * npc;
+        for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
+            const int32_t x = s_in[loc];
+            if (x) {
+                red_add(&dst[loc], x);
+                s_in[loc] = 0;
+            }
+        }
+        col = next;
     }
     if (lane != 0 && !n.tile) ev_all = ev_exc = 0;
     const unsigned long long ba = block_sum(ev_all);
@@ -546,26 +578,16 @@ __device__ __forceinline__ void deliver_staged(const DevNet &n, const int *t_now
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_in + kSlots * npc);   // [npc]
     int32_t *s_tile = reinterpret_cast<int32_t *>(s_hist + npc);         // [nwarps][kTileWords]
     uint16_t *s_x = reinterpret_cast<uint16_t *>(s_tile + nwarps * kTileWords);   // [kSlots * npc]
-    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_cols<true, true>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
-    else deliver_cols<true, false>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
+    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_cols<true>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
+    else deliver_cols<false>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
 }
 
 __device__ __forceinline__ void deliver_ordered(const DevNet &n, const int *t_now, const Part &g)
 {
-    extern __shared__ int4 smem_i4[];
     const int t = *t_now;
     if (!ordered_selected(n, t)) return;
-    const uint32_t npc = n.npc;
-    int32_t *s_lut = reinterpret_cast<int32_t *>(smem_i4);
-    int32_t *s_in = s_lut + kLut;                                        // [npc]
-    int32_t *s_ltd = s_in + npc;                                         // [npc]
-    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_ltd + npc);        // [npc]
-    uint32_t *s_inh = s_hist + npc;                                      // [npc]
-    int32_t *s_tile = reinterpret_cast<int32_t *>(s_inh + npc);          // [nwarps][kTileWords]
-    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t))
-        deliver_cols<false, true>(n, t, s_lut, s_in, s_tile, s_ltd, s_hist, g, s_inh);
-    else
-        deliver_cols<false, false>(n, t, s_lut, s_in, s_tile, s_ltd, s_hist, g, s_inh);
+    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_columns<true>(n, t, g);
+    else deliver_columns<false>(n, t, g);
 }
 
 // One target's reverse entries [lo, hi), walked by a warp, kUnroll entries
@@ -1116,7 +1138,7 @@ __global__ void __launch_bounds__(kStagedBlock) k_deliver_cols(DevNet n, const i
     deliver_staged(n, t_now, whole_grid());
 }
 
-__global__ void __launch_bounds__(kOrderedMaxBlock, 5) k_deliver_ordered(DevNet n, const int *t_now)
+__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered(DevNet n, const int *t_now)
 {
     deliver_ordered(n, t_now, whole_grid());
 }
@@ -1162,7 +1184,7 @@ __global__ void __launch_bounds__(kStagedBlock) k_deliver_cols_b(BatchLaunch b)
     deliver_staged(n, x.t_now, x.part);
 }
 
-__global__ void __launch_bounds__(kOrderedMaxBlock, 5) k_deliver_ordered_b(BatchLaunch b)
+__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered_b(BatchLaunch b)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
