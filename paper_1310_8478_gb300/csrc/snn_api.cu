@@ -149,6 +149,7 @@ struct snn_net {
     int64_t raster_steps_cap = 0;   // entries of dn.raster_step_off
     uint16_t *tgt16 = nullptr;
     int32_t *nbr = nullptr;
+    bool weights_moved = false;     // a checkpoint was loaded (or a run broke off) since the last reset
     bool ltp_owed = false;          // the last step's LTP has not been applied yet
     int32_t *noalloc_base = nullptr; // device address of the no-allocation staging array
     int32_t *inject_buf = nullptr;  // tiles: device copy of the spikes received for a step
@@ -1160,7 +1161,10 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             SNN_CUDA(cudaMemcpyAsync(&net->host_ctr[1], net->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, net->stream));
             SNN_CUDA(cudaStreamSynchronize(net->stream));
             const DevCounters &hc = net->host_ctr[1];
-            if (hc.error) return finish_run(net, true);
+            if (hc.error) {
+                net->weights_moved = true;     // how far the steps came is not known
+                return finish_run(net, true);
+            }
             const int32_t now = std::max(t, hc.t_slot[(hc.t_slot[0] < hc.t_slot[1]) ? 1 : 0]);
             left -= (uint32_t)(now - t);
             net->t = now;
@@ -2274,8 +2278,14 @@ int snn_reset(snn_net *net)
     if (net->explicit_net) { set_error("explicit nets keep no copy of their initial weights"); return SNN_ESTATE; }
     cudaStream_t s = net->stream;
     const int g = grid_for(net, 8);
-    k_reset_weights<<<g, 256, 0, s>>>(net->dn, net->gen.w_exc0, net->gen.w_inh0);
-    SNN_CUDA(cudaMemsetAsync(net->dn.sd_rev, 0, (size_t)std::max<int64_t>(net->n_rin, 1) * 4, s));
+    // Weights move in long-term updates and loaded checkpoints only, and the
+    // reverse accumulator is empty after a fold: what still holds its initial
+    // value is not written again (the rows of 2.9 G synapses after 25 steps:
+    // 21 of 32 GB).
+    const uint32_t P = net->cfg.deriv_period_ms;
+    if (net->weights_moved || (P && (uint32_t)net->t >= P)) k_reset_weights<<<g, 256, 0, s>>>(net->dn, net->gen.w_exc0);
+    SNN_CUDA(cudaMemsetAsync(net->sd, 0, (size_t)net->S_store * 4, s));
+    k_reset_rev<<<g, 256, 0, s>>>(net->dn);
     k_init_state<<<g, 256, 0, s>>>(net->dn);
     DevCounters hc{};
     hc.raster_first_drop_t = 0x7fffffff;
@@ -2287,6 +2297,7 @@ int snn_reset(snn_net *net)
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(s));
     net->t = 0;
+    net->weights_moved = false;
     net->ltp_owed = false;
     net->dn.raster_t0 = 0;
     net->dn.stim_t0 = net->dn.stim_t1 = 0;
@@ -2684,6 +2695,7 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     }
     cudaStream_t s = net->stream;
     DevNet &dn = net->dn;
+    net->weights_moved = true;
     void *sv = dn.vd ? (void *)dn.vd : (void *)dn.v;
     void *su = dn.ud ? (void *)dn.ud : (void *)dn.u;
     void *dst[] = {sv, su, dn.I, dn.hl, dn.last_spike, dn.ring_ids, dn.ring_cnt, net->w, net->sd, net->ctr};

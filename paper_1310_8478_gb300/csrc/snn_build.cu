@@ -218,15 +218,34 @@ __global__ void k_max2(const int32_t *a, const int32_t *b, uint32_t n, int32_t *
     }
 }
 
-// initial weights of a generated net (by source kind) and zero derivatives
-__global__ void k_reset_weights(DevNet n, int32_t w_exc0, int32_t w_inh0)
+// initial weights of a generated net's excitatory rows (inhibitory ones do
+// not change); a warp per row
+__global__ void k_reset_weights(DevNet n, int32_t w_exc0)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n.S; k += stride) {
-        const uint32_t p = (uint32_t)(k / n.uniform_m);
-        n.w[k] = ((p % n.npc) < n.ne) ? w_exc0 : w_inh0;
-        n.sd[k] = 0;
+    const int lane = threadIdx.x & 31;
+    const uint32_t rows = n.C * n.ne, warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += warps) {
+        const uint32_t p = (r / n.ne) * n.npc + r % n.ne;
+        int32_t *w = n.w + row_base(n, p);
+        const uint32_t m = n.canon_m;
+        if (n.uniform_m % 4 == 0)                    // compact rows: 16-byte aligned
+            for (uint32_t k = 4 * lane; k + 4 <= m; k += 128)
+                *reinterpret_cast<int4 *>(w + k) = make_int4(w_exc0, w_exc0, w_exc0, w_exc0);
+        const uint32_t done = n.uniform_m % 4 == 0 ? m & ~3u : 0u;
+        for (uint32_t k = done + lane; k < m; k += 32) w[k] = w_exc0;
     }
+}
+
+// Zeroes the event-driven potentiation when any was accumulated since the
+// last fold (16 bytes per thread and pass).
+__global__ void k_reset_rev(DevNet n)
+{
+    if (!n.ctr->sd_rev_dirty) return;
+    const int64_t quads = n.n_rin / 4, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int4 *p = reinterpret_cast<int4 *>(n.sd_rev);
+    for (int64_t k = tid; k < quads; k += stride) p[k] = make_int4(0, 0, 0, 0);
+    for (int64_t k = 4 * quads + tid; k < n.n_rin; k += stride) n.sd_rev[k] = 0;
 }
 
 // initial state: v = -65 mV, u = b v (b = 0.2 for both kinds), no history

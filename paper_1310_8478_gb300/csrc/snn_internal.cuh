@@ -749,7 +749,8 @@ __global__ void k_scan_write(const int32_t *in, uint32_t n, const long long *blo
 __global__ void k_fill_reverse(DevNet n, int32_t *cursor, uint64_t *rin, uint32_t *rin32);
 __global__ void k_max2(const int32_t *a, const int32_t *b, uint32_t n, int32_t *out2);
 __global__ void k_init_state(DevNet n);
-__global__ void k_reset_weights(DevNet n, int32_t w_exc0, int32_t w_inh0);
+__global__ void k_reset_weights(DevNet n, int32_t w_exc0);
+__global__ void k_reset_rev(DevNet n);
 __global__ void k_read_rows(DevNet n, GenParams g, const uint8_t *canon_delay, uint32_t first,
                             uint32_t count, int64_t out_base, int32_t *o_tgt, uint8_t *o_delay,
                             int32_t *o_w, int32_t *o_sd);

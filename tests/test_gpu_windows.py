@@ -129,3 +129,31 @@ def test_step_kernels_defer_inside_a_window(eng, npc, m):
             assert np.count_nonzero(x["sd"]) > npc
         x, y = a.neurons(), b.neurons()
         assert np.array_equal(x["v"].view(np.int32), y["v"].view(np.int32))
+
+
+@pytest.mark.parametrize("before", ["few_steps", "single_steps", "a_period", "a_checkpoint"])
+def test_reset_restores_whatever_moved(eng, before):
+    cfg = _cfg(3, 2, 130, 70, seed=72, thal_per_col_per_ms=2, deriv_period_ms=60)
+    with eng.Network(cfg, raster_capacity=1 << 18) as fresh, eng.Network(cfg, raster_capacity=1 << 18) as n:
+        if before == "few_steps":
+            n.run(40)
+        elif before == "single_steps":
+            for _ in range(40):
+                n.step()
+        elif before == "a_period":
+            n.run(61)
+        else:
+            other = eng.Network(cfg, raster_capacity=1 << 18)
+            other.run(100)
+            n.load_state(other.save_state())
+            other.close()
+            n.reset()
+            n.run(5)
+        n.reset()
+        for steps in (0, 75):
+            if steps:
+                n.run(steps)
+                fresh.run(steps)
+            for a, b in zip(n.weights() + n.raster(), fresh.weights() + fresh.raster()):
+                assert np.array_equal(a, b)
+            assert n.counters() == fresh.counters()
