@@ -52,6 +52,7 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
+constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
@@ -195,7 +196,9 @@ struct snn_batch {
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> join;
     uint32_t L = 0;
-    cudaGraphExec_t graph = nullptr;
+    // a chunk of steps, without and with the long-term update's kernels
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    bool fresh = false;                  // the tables are of the launch shape and the nets below
     std::vector<uint64_t> versions;      // the nets' versions when the graph was captured
     std::vector<int> parity;             // the nets' step parity when the graph was captured
     snn_launch launch{};                 // block sizes and resident blocks of the batched kernels
@@ -925,7 +928,9 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     const bool prof = net->profile;
     const uint32_t P = net->cfg.deriv_period_ms;
     const bool closes = exact_t && P && t > 0 && (uint32_t)t % P == 0;
-    const bool fork = !closes && !prof;
+    // (an explicit net's small steps end sooner one after another: 5000
+    // neurons of 100 synapses 32.5 us per step against 38.8)
+    const bool fork = !closes && !prof && (dn.tgt16 || net->N >= kForkMinExplicit);
     cudaStream_t sl = fork ? net->side : s;        // the potentiation's stream
     auto mark = [&](int kind, cudaStream_t on) {
         if (prof) cudaEventRecord(next_event(net, kind), on);
@@ -1710,11 +1715,19 @@ int snn_run_host(snn_net *net, uint32_t n_ms, const snn_stimulus *host_stimulus,
     return SNN_OK;
 }
 
+static void batch_drop_graphs(snn_batch *b)
+{
+    for (cudaGraphExec_t &g : b->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 void snn_batch_free(snn_batch *b)
 {
     if (!b) return;
     if (b->main) cudaStreamSynchronize(b->main);
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    batch_drop_graphs(b);
     if (b->tables) cudaFree(b->tables);
     for (cudaEvent_t e : b->join) cudaEventDestroy(e);
     if (b->fork) cudaEventDestroy(b->fork);
@@ -1828,7 +1841,10 @@ int batch_tables(snn_batch *b)
     for (size_t i = 0; i < nn; ++i) {
         const snn_net *n = b->nets[i];
         w[i] = (n->cfg.flags & SNN_STDP_OFF) ? 0.0 : work(i);
-        cap[i] = (n->N + L.ltp_block / 32 - 1) / (L.ltp_block / 32);
+        // a warp per 128 neurons: a pass serves 0.8 % firing, and a block costs
+        // a chain of five loads before it finds its spikers (24 nets of sides
+        // 1 to 16: 31 us per step; 57 with a warp per 8, 72 with one each)
+        cap[i] = (n->N + 4 * L.ltp_block - 1) / (4 * L.ltp_block);
     }
     b->kind[kBLtp].block = L.ltp_block;
     share_blocks(w, cap, sms * batch_occupancy((const void *)k_ltp_b, L.ltp_block, 0, L.ltp_blocks_per_sm), cnt[kBLtp]);
@@ -1988,7 +2004,7 @@ int batch_tables(snn_batch *b)
 }
 
 // one step (index k of the chunk) of every net: each kind of kernel once
-void batch_launch_step(snn_batch *b, uint32_t k)
+void batch_launch_step(snn_batch *b, uint32_t k, bool closes)
 {
     cudaStream_t s = b->main;
     auto go = [&](int kind, auto kernel) {
@@ -2000,13 +2016,13 @@ void batch_launch_step(snn_batch *b, uint32_t k)
     };
     // [S4(t-1) S5(t-1) S1(t)] then [S2(t) S3(t)], as launch_step
     go(kBLtp, k_ltp_b);
-    if (b->kind[kBFold].grid) {
+    if (closes && b->kind[kBFold].grid) {
         const snn_batch::Kind &x = b->kind[kBFold];
         BatchLaunch bl = x.bl;
         bl.k = k;
         k_fold_b<<<x.grid, x.block, x.smem, s>>>(bl, kFoldStep);
     }
-    go(kBDeriv, k_deriv_b);
+    if (closes) go(kBDeriv, k_deriv_b);
     go(kBOrdered, k_deliver_ordered_b);
     go(kBRing, k_deliver_b);
     go(kBStaged, k_deliver_cols_b);
@@ -2050,32 +2066,49 @@ void batch_close_window(snn_batch *b)
     if (y.grid) k_stdp_b<<<y.grid, y.block, y.smem, b->main>>>(y.bl);
 }
 
-// a chunk of L steps of every net as one graph: per step one launch per kind
-// of kernel for the whole batch
-int batch_capture(snn_batch *b)
+// whether a net closes a period in its next L steps (step t' > 0 with
+// t' % P == 0 applies the long-term update of the period before it)
+bool batch_closes(const snn_batch *b)
 {
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
+    for (const snn_net *n : b->nets) {
+        const int64_t P = n->cfg.deriv_period_ms, t = n->t;
+        if (P && std::max<int64_t>(P, (t + P - 1) / P * P) < t + (int64_t)b->L) return true;
     }
+    return false;
+}
+
+// the launch tables for the nets as they are; graphs of earlier ones go
+int batch_refresh(snn_batch *b)
+{
+    batch_drop_graphs(b);
     SNN_TRY(batch_tables(b));
-    cudaGraph_t g = nullptr;
-    SNN_CUDA(cudaStreamBeginCapture(b->main, cudaStreamCaptureModeThreadLocal));
-    for (uint32_t k = 0; k < b->L; ++k) batch_launch_step(b, k);
-    cudaError_t e = cudaStreamEndCapture(b->main, &g);
-    if (e != cudaSuccess) { set_error("batch capture failed: %s", cudaGetErrorString(e)); return SNN_ECUDA; }
-    e = cudaGraphInstantiate(&b->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        b->graph = nullptr;
-        set_error("batch graph instantiate failed: %s", cudaGetErrorString(e));
-        return SNN_ECUDA;
-    }
     b->versions.clear();
     b->parity.clear();
     for (snn_net *n : b->nets) {
         b->versions.push_back(n->version);
         b->parity.push_back(n->t & 1);
+    }
+    b->fresh = true;
+    return SNN_OK;
+}
+
+// a chunk of L steps of every net as one graph: per step one launch per kind
+// of kernel for the whole batch, those of the long-term update only in chunks
+// that hold a period's end (24 nets of sides 1 to 16: the two that return at
+// once took 70 us per step)
+int batch_capture(snn_batch *b, bool closes)
+{
+    cudaGraph_t g = nullptr;
+    SNN_CUDA(cudaStreamBeginCapture(b->main, cudaStreamCaptureModeThreadLocal));
+    for (uint32_t k = 0; k < b->L; ++k) batch_launch_step(b, k, closes);
+    cudaError_t e = cudaStreamEndCapture(b->main, &g);
+    if (e != cudaSuccess) { set_error("batch capture failed: %s", cudaGetErrorString(e)); return SNN_ECUDA; }
+    e = cudaGraphInstantiate(&b->graph[closes], g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        b->graph[closes] = nullptr;
+        set_error("batch graph instantiate failed: %s", cudaGetErrorString(e));
+        return SNN_ECUDA;
     }
     return SNN_OK;
 }
@@ -2097,13 +2130,15 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
     uint32_t window = 0;                       // chunks left of the open window
     while (left > 0) {
         if (L >= 2 && left >= L) {
-            // the graph holds each net's launches for its step parity at capture
-            bool stale = !b->graph;
+            // the graphs hold each net's launches for its step parity at capture
+            bool stale = !b->fresh;
             for (size_t i = 0; !stale && i < b->nets.size(); ++i)
                 stale = b->versions[i] != b->nets[i]->version || b->parity[i] != (b->nets[i]->t & 1);
-            if (stale) SNN_TRY(batch_capture(b));
+            if (stale) SNN_TRY(batch_refresh(b));
+            const bool closes = batch_closes(b);
+            if (!b->graph[closes]) SNN_TRY(batch_capture(b, closes));
             if (!window && (window = batch_window_chunks(b, left)) != 0) batch_open_window(b, window * L);
-            SNN_CUDA(cudaGraphLaunch(b->graph, b->main));
+            SNN_CUDA(cudaGraphLaunch(b->graph[closes], b->main));
             for (snn_net *n : b->nets) n->t += (int32_t)L;
             left -= L;
             if (window && --window == 0) {
@@ -2153,10 +2188,8 @@ int snn_batch_set_launch(snn_batch *b, const snn_launch *launch)
     b->launch = L;
     b->L = L.graph_steps & ~1u;
     b->launch.graph_steps = b->L;
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+    batch_drop_graphs(b);
+    b->fresh = false;
     return SNN_OK;
 }
 
