@@ -24,7 +24,7 @@ LIB_PATH = os.path.join(BUILD_DIR, "libsnn.so")
 CHECKED_DIR = os.path.join(BUILD_DIR, "checked")
 CHECKED_LIB_PATH = os.path.join(BUILD_DIR, "libsnn_checked.so")
 SOURCES = ["snn_build.cu", "snn_step.cu", "snn_dense.cu", "snn_window.cu", "snn_resident.cu", "snn_api.cu", "snn_microbench.cu"]
-HEADERS = ["snn_internal.cuh"]
+HEADERS = ["snn_internal.cuh", "snn_deliver.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-fmad=false", "-Xcompiler", "-fPIC,-ffp-contract=off",

@@ -52,6 +52,7 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
+constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
 constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
@@ -159,6 +160,8 @@ struct snn_net {
     int staged_grid = 0;            // blocks of the column-staged delivery (likewise)
     int ordered_grid = 0;           // blocks of the column-ordered delivery (likewise)
     int stdp_grid = 0;              // blocks of a plasticity window's pass (likewise); 0: no windows
+    int merged_grid = 0;            // blocks of the delivery and dense pass in one launch; 0: two launches
+    int light_grid = 0;             // blocks of a dense step that defers its STDP (likewise)
     bool step_windows = false;      // the step kernels' steps take windows
     int res_grid = 0;               // blocks of the resident grid that runs this net's windows; 0: none does
     uint64_t version = 0;           // bumped whenever captured launches go stale
@@ -187,7 +190,7 @@ struct snn_net {
 
 // kinds of step kernel a batch launches once per step for all of its nets
 enum BatchKind { kBLtp, kBFold, kBDeriv, kBOrdered, kBRing, kBStaged, kBDense, kBNeuron32, kBNeuron64, kBProbe,
-                 kBWinOpen, kBTrain, kBStdp, kBKinds };
+                 kBWinOpen, kBTrain, kBStdp, kBDenseLight, kBKinds };
 
 struct snn_batch {
     std::vector<snn_net *> nets;
@@ -528,6 +531,7 @@ int alloc_common(snn_net *net)
 int setup_dense(snn_net *net)
 {
     net->dense_ok = false;
+    net->merged_grid = 0;
     net->dn.staged_ok = 0;
     net->dn.staged_min_events = ~0ull;
     net->dn.ordered_ok = 0;
@@ -591,6 +595,19 @@ int setup_dense(snn_net *net)
     const int64_t units = (int64_t)net->dn.C * ((net->cfg.neurons_per_col + rows - 1) / rows);
     net->dense_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
     net->dense_ok = true;
+    // Small nets run the column-ordered delivery and the dense pass as one
+    // launch (a closed-loop step of one column: 80 -> 75 us).  Large ones do
+    // not: with the dense pass's shared memory the delivery loses its L1 (onset
+    // of the 64x32 benchmark torus 6.3 -> 7.4 ms).
+    if (net->N <= kMergeMaxNeurons && net->dn.ordered_ok && !net->dn.staged_ok &&
+        net->launch.dense_block == ordered_block(net->launch.deliver_block)) {
+        const uint32_t blk = net->launch.dense_block;
+        const size_t most = std::max(bytes, ordered_smem_bytes(net->cfg.neurons_per_col, blk));
+        SNN_CUDA(allow_smem((const void *)k_deliver_dense, most));
+        SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deliver_dense, (int)blk, most));
+        if (per_sm >= 2)
+            net->merged_grid = (int)std::min<int64_t>(std::max<int64_t>(net->dn.C, units), (int64_t)per_sm * net->sm_count);
+    }
     return SNN_OK;
 }
 
@@ -703,6 +720,13 @@ int setup_windows(snn_net *net)
     const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
     net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
     net->step_windows = net->n_rin >= kWinMinSynapses;
+    if (net->step_windows) {
+        const size_t light = dense_light_smem_bytes(dn.npc);
+        SNN_CUDA(allow_smem((const void *)k_dense_light, light));
+        SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dense_light, (int)kDenseLightBlock, light));
+        const int64_t dense_units = (int64_t)dn.C * ((dn.npc + dn.dense_rows - 1) / dn.dense_rows);
+        net->light_grid = (int)std::min<int64_t>(dense_units, (int64_t)std::max(1, per_sm) * net->sm_count);
+    }
     net->res_grid = res;
     dn.res_parts = (uint32_t)parts;
     // a step starts the deferral when the rest of its window, at its rate, will
@@ -960,7 +984,13 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
         mark(3, s);
     }
     mark(0, s);
-    if (dn.ordered_ok) {
+    const bool both = net->merged_grid && !prof;
+    if (both) {
+        k_deliver_dense<<<net->merged_grid, L.dense_block,
+                          std::max(ordered_smem_bytes(dn.npc, L.dense_block), dense_smem_bytes(dn.npc, L.dense_block)),
+                          s>>>(dn, t_now);
+        ++launched;
+    } else if (dn.ordered_ok) {
         k_deliver_ordered<<<net->ordered_grid, ordered_block(L.deliver_block),
                             ordered_smem_bytes(dn.npc, ordered_block(L.deliver_block)), s>>>(dn, t_now);
         ++launched;
@@ -976,8 +1006,12 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     mark(0, s);
     if (net->dense_ok) {
         mark(4, s);
-        k_dense<<<net->dense_grid, L.dense_block, dense_smem_bytes(dn.npc, L.dense_block), s>>>(dn, t_now);
-        ++launched;
+        if (!both) k_dense<<<net->dense_grid, L.dense_block, dense_smem_bytes(dn.npc, L.dense_block), s>>>(dn, t_now);
+        launched += both ? 0 : 1;
+        if (net->step_windows && !prof) {
+            k_dense_light<<<net->light_grid, kDenseLightBlock, dense_light_smem_bytes(dn.npc), s>>>(dn, t_now);
+            ++launched;
+        }
         mark(4, s);
     }
     if (fork) cudaStreamWaitEvent(s, net->ev_join, 0);
@@ -1927,7 +1961,8 @@ int batch_tables(snn_batch *b)
     b->kind[kBProbe].block = 256;
     // plasticity windows
     size_t smem_w = 0;
-    for (int k : {kBWinOpen, kBTrain, kBStdp}) cnt[k].assign(nn, 0);
+    size_t smem_l = 0;
+    for (int k : {kBWinOpen, kBTrain, kBStdp, kBDenseLight}) cnt[k].assign(nn, 0);
     for (size_t i = 0; i < nn; ++i) {
         const snn_net *n = b->nets[i];
         if (!n->step_windows) continue;
@@ -1935,7 +1970,13 @@ int batch_tables(snn_batch *b)
         cnt[kBWinOpen][i] = (uint32_t)sized_grid(n, 8, n->N, 1024);
         cnt[kBTrain][i] = (uint32_t)sized_grid(n, 8, n->dn.spk_words, 64);
         cnt[kBStdp][i] = (uint32_t)n->stdp_grid;
+        if (!n->dense_ok) continue;
+        smem_l = std::max(smem_l, dense_light_smem_bytes(n->dn.npc));
+        cnt[kBDenseLight][i] = (uint32_t)n->light_grid;
     }
+    b->kind[kBDenseLight].block = kDenseLightBlock;
+    b->kind[kBDenseLight].smem = smem_l;
+    if (smem_l) SNN_CUDA(allow_smem((const void *)k_dense_light_b, smem_l));
     b->kind[kBWinOpen].block = b->kind[kBTrain].block = 256;
     b->kind[kBStdp].block = kStdpBlock;
     b->kind[kBStdp].smem = smem_w;
@@ -2027,6 +2068,7 @@ void batch_launch_step(snn_batch *b, uint32_t k, bool closes)
     go(kBRing, k_deliver_b);
     go(kBStaged, k_deliver_cols_b);
     go(kBDense, k_dense_b);
+    go(kBDenseLight, k_dense_light_b);
     go(kBNeuron32, k_neuron_f32_b);
     go(kBNeuron64, k_neuron_f64_b);
     go(kBProbe, k_probe_b);

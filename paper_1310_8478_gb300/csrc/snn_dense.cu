@@ -6,11 +6,16 @@
 // every source row once: per synapse LTP(t-1) -> long-term update at a period
 // end -> delivery + LTD(t), in the same per-synapse order as the event-driven
 // kernels of snn_step.cu, so both give bit-identical results.
-#include "snn_internal.cuh"
+#include "snn_deliver.cuh"
 
 namespace snn {
 
 // ---------------------------------------------------------------------------
+size_t ordered_smem_bytes(uint32_t npc, uint32_t block)
+{
+    return (size_t)kLut * 4 + (size_t)npc * 24 + kItems * 4 + (size_t)(block / 32) * 64 * 4;
+}
+
 size_t dense_smem_bytes(uint32_t npc, uint32_t block)
 {
     const size_t warps = block / 32;
@@ -171,122 +176,11 @@ __device__ __forceinline__ uint32_t word_flags(int q0, int m, int D, float scale
     return f;
 }
 
-// The rows [r0, r1) of column col in a dense step whose STDP is left to the
-// window's pass: targets and, on excitatory rows, weights -- no derivatives,
-// no post-spike words.  Bound by instruction issue before HBM, so
-//   - the next 256 synapses are loaded into registers while this pass's are
-//     added (the bulk prefetches of the fused pass cost a third of the
-//     instructions here, and without derivatives there are registers to spare);
-//   - the delay buckets are looked up once per 1024 synapses, each lane the
-//     flags of 32 positions, and not at all when the source fired in each of
-//     the last D steps;
-//   - inside a chunk that has a due position the others add 0: a condition
-//     around each addition costs a branch and a reconvergence, several times
-//     the addition.
-struct Segment {
-    uint4 t;
-    int4 a, b;
-};
-
-// a lane's 8 synapses: chunk c of the row (none at or past its end)
-__device__ __forceinline__ void load_segment(const DevNet &n, Segment &x, const uint4 *t4, const int4 *w4, int c,
-                                             int chunks, bool exc)
-{
-    if (c >= chunks || out_of_range(n, (const uint16_t *)(t4 + c + 1) <= n.tgt16 + n.S)) return;
-    x.t = t4[c];
-    if (exc) {
-        x.a = w4[2 * c];
-        x.b = w4[2 * c + 1];
-    }
-}
-
-__device__ __forceinline__ void dense_deliver_rows(const DevNet &n, uint32_t col, uint32_t r0, uint32_t r1,
-                                                   uint32_t dmask, int32_t *w_off, int32_t *s_in,
-                                                   unsigned long long &ev_all, unsigned long long &ev_exc)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int D = (int)n.D, m = (int)n.canon_m, chunks = (m + 7) >> 3, nseg = (chunks + 31) >> 5;
-    const float scale = (float)D / (float)m;
-    const uint32_t in0 = (uint32_t)__cvta_generic_to_shared(s_in);
-    if (r0 + warp >= r1) return;
-    const uint32_t p0 = col * n.npc + r0 + warp;
-    uint32_t hist_next = n.hl[p0].x;
-    int off_next = lane <= D ? (int)n.doff[(size_t)p0 * kDoffStride + lane] : 0;
-    const uint4 *t4 = reinterpret_cast<const uint4 *>(n.tgt16 + row_base(n, p0));
-    const int4 *w4 = reinterpret_cast<const int4 *>(n.w + row_base(n, p0));
-    const size_t row4 = (size_t)nwarps * n.uniform_m / 8;           // chunks between a warp's rows
-    Segment cur{};
-    load_segment(n, cur, t4, w4, lane, chunks, r0 + warp < n.ne);
-    auto add = [&](uint32_t v, int32_t w) {
-        if (!out_of_range(n, v < kSlots * n.npc)) red_shared(in0 + 4u * v, w);
-    };
-    for (uint32_t r = r0 + warp; r < r1; r += nwarps, t4 += row4, w4 += 2 * row4) {
-        const uint32_t p = col * n.npc + r;
-        const bool exc = r < n.ne, next_exc = r + nwarps < n.ne;
-        const int next_chunks = r + nwarps < r1 ? chunks : 0;
-        const uint32_t due = exc ? dmask : 2u;         // inhibitory rows: delay 1 alone
-        const uint32_t fbits = (hist_next << 1) & due;
-        const int hi = off_next;
-        if (next_chunks) {
-            hist_next = n.hl[p + nwarps].x;
-            off_next = lane <= D ? (int)n.doff[(size_t)(p + nwarps) * kDoffStride + lane] : 0;
-        }
-        if (!fbits) {
-            load_segment(n, cur, t4 + row4, w4 + 2 * row4, lane, next_chunks, next_exc);
-            continue;
-        }
-        const bool full = fbits == due;                // the whole row is due
-        int events = m;
-        if (!full) {
-            const int lo = __shfl_up_sync(0xffffffffu, hi, 1);
-            w_off[lane] = hi;                          // lane d: end of bucket d, lane 0: 0
-            events = __reduce_add_sync(0xffffffffu, (lane && ((fbits >> lane) & 1u)) ? hi - lo : 0);
-            __syncwarp();
-        }
-        if (lane == 0) {
-            ev_all += (unsigned long long)events;
-            if (exc) ev_exc += (unsigned long long)events;
-        }
-        uint32_t flags = 0;
-        for (int s = 0; s < nseg; ++s) {
-            const Segment x = cur;
-            if (s + 1 < nseg) load_segment(n, cur, t4, w4, 32 * (s + 1) + lane, chunks, exc);
-            else load_segment(n, cur, t4 + row4, w4 + 2 * row4, lane, next_chunks, next_exc);
-            const uint32_t tw[4] = {x.t.x, x.t.y, x.t.z, x.t.w};
-            int32_t wv[8] = {x.a.x, x.a.y, x.a.z, x.a.w, x.b.x, x.b.y, x.b.z, x.b.w};
-            if (!exc) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) wv[u] = n.w_inh;
-            }
-            const int left = m - 8 * (32 * s + lane);
-            uint32_t fmask = left >= 8 ? 0xffu : left > 0 ? (1u << left) - 1u : 0u;
-            if (!full) {
-                if (!(s & 3)) {
-                    const int q0 = 256 * s + 32 * lane;
-                    flags = q0 < m ? word_flags(q0, m, D, scale, fbits, w_off) : 0u;
-                }
-                const uint32_t word = __shfl_sync(0xffffffffu, flags, 8 * (s & 3) + (lane >> 2));
-                fmask &= word >> (8 * (lane & 3));
-            }
-            if (full && s + 1 < nseg) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) add((u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu), wv[u]);
-            } else if (fmask) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    add((u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu), (fmask >> u) & 1u ? wv[u] : 0);
-            }
-        }
-        __syncwarp();
-    }
-}
-
 __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, const Part &g)
 {
     extern __shared__ int4 smem_i4[];
     const int t = *t_now;
-    if (!dense_selected(n, t)) return;
+    if (!dense_selected(n, t) || deferring(n, t)) return;
     const uint32_t npc = n.npc;
     const uint32_t nwarps = blockDim.x >> 5;
     int32_t *s_lutp = reinterpret_cast<int32_t *>(smem_i4);
@@ -297,10 +191,9 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
     uint16_t *s_x = reinterpret_cast<uint16_t *>(s_amt + nwarps * 32);   // [kSlots * npc] packed words
     __shared__ uint32_t s_col[kSlots];
 
-    const bool defer = deferring(n, t);      // the window's pass does the STDP of this step
-    const bool stdp = !(n.flags & SNN_STDP_OFF) && !defer;
+    const bool stdp = !(n.flags & SNN_STDP_OFF);
     const bool deliver_on = !(n.flags & SNN_DELIVERY_OFF);
-    const bool owed = n.ctr->ltp_pending == t - 1 && !defer;
+    const bool owed = n.ctr->ltp_pending == t - 1;
     const bool ltp_on = owed && stdp;
     const bool deriv_on = owed && n.deriv_period && (t % (int)n.deriv_period) == 0;
     const uint32_t chunks = (npc + n.dense_rows - 1) / n.dense_rows;
@@ -324,15 +217,13 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
         const uint32_t r1 = min(npc, r0 + n.dense_rows);
         if (threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
         // every warp's first row starts streaming into L2 while the block stages
-        if (lane == 0 && r0 + warp < r1 && !defer) {
+        if (lane == 0 && r0 + warp < r1) {
             const int64_t b = row_base(n, col * npc + r0 + warp);
             for (int sgm = 0; sgm < kPrefetchAhead; ++sgm)
                 prefetch_segment(n, b + sgm * 256, true, r0 + warp < n.ne);
         }
         __syncthreads();
-        if (defer)
-            for (uint32_t k = threadIdx.x; k < kSlots * npc; k += blockDim.x) s_in[k] = 0;
-        for (int sl = 0; sl < kSlots && !defer; ++sl) {
+        for (int sl = 0; sl < kSlots; ++sl) {
             const int32_t *ls = n.last_spike + (size_t)s_col[sl] * npc;
             uint16_t *x_row = s_x + sl * npc;
             int32_t *in_row = s_in + sl * npc;
@@ -343,17 +234,16 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
             }
         }
         __syncthreads();
-        if (defer) dense_deliver_rows(n, col, r0, r1, dmask, w_off, s_in, ev_all, ev_exc);
         // row metadata goes out one row ahead: the spike-history word and, in lane
         // d <= D, the end of delay bucket d
         uint2 hv_next = make_uint2(0u, 0u);
         int off_next = 0;
-        if (r0 + warp < r1 && !defer) {
+        if (r0 + warp < r1) {
             const uint32_t p = col * npc + r0 + warp;
             hv_next = n.hl[p];
             off_next = (lane <= D) ? (int)n.doff[(size_t)p * kDoffStride + lane] : 0;
         }
-        for (uint32_t r = r0 + warp; r < r1 && !defer; r += nwarps) {
+        for (uint32_t r = r0 + warp; r < r1; r += nwarps) {
             const uint32_t p = col * npc + r;
             const bool exc = r < n.ne;
             const uint2 hv = hv_next;
@@ -455,20 +345,188 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
         if (g.bid == 0) {
             // potentiation visits: every incoming excitatory synapse of the
             // neurons that fired at t - 1 (counted when those spikes closed)
-            if (ltp_on || defer) n.ctr->dense_l_exc += n.ctr->l_exc_last;
+            if (ltp_on) n.ctr->dense_l_exc += n.ctr->l_exc_last;
             n.ctr->dense_steps += 1;
             if (deriv_on) n.ctr->dense_deriv_steps += 1;
         }
     }
 }
 
+// ---------------------------------------------------------------------------
+// A dense step whose STDP is left to the window's pass: targets and, on
+// excitatory rows, weights -- no derivatives, no post-spike words.  Without
+// them a thread needs 32 registers, so two blocks of 1024 threads reside per
+// SM and their 64 warps hide the loads that the fused pass above prefetches
+// (its bulk prefetches would cost a third of the instructions here).  The
+// delay buckets are looked up once per 1024 synapses, each lane the flags of
+// 32 positions, and not at all when the source fired in each of the last D
+// steps; inside a chunk that has a due position the others add 0: a condition
+// around each addition costs a branch and a reconvergence, several times the
+// addition.  1.28 M neurons of 1125 synapses: 1.2 ms a step, 0.95 of the copy
+// bandwidth (1.5 ms inside the fused pass's kernel with 32 warps, 2.9 ms with
+// the STDP); 320 000: 0.34 ms, with the L1's shared-memory passes at 0.8.
+// ---------------------------------------------------------------------------
+size_t dense_light_smem_bytes(uint32_t npc)
+{
+    return (size_t)kSlots * npc * 4            // staged input
+           + (kDenseLightBlock / 32) * 32 * 4; // per-warp bucket offsets
+}
+
+__device__ __forceinline__ void light_row(const DevNet &n, int64_t base, bool exc, uint32_t fbits, uint32_t due,
+                                          const int32_t *w_off, uint32_t in0, int lane)
+{
+    const int D = (int)n.D, m = (int)n.canon_m;
+    const uint4 *t4 = reinterpret_cast<const uint4 *>(n.tgt16 + base) + lane;
+    const int4 *w4 = reinterpret_cast<const int4 *>(n.w + base) + 2 * lane;
+    const bool full = fbits == due;                // the whole row is due
+    const float scale = (float)D / (float)m;
+    uint32_t flags = 0;
+    for (int s = 0; 256 * s < m; ++s, t4 += 32, w4 += 64) {
+        const int left = m - 256 * s - 8 * lane;   // positions from the lane's chunk to the row's end
+        uint32_t fmask = left >= 8 ? 0xffu : left > 0 ? (1u << left) - 1u : 0u;
+        if (!full) {
+            if (!(s & 3)) {
+                const int q0 = 256 * s + 32 * lane;
+                flags = q0 < m ? word_flags(q0, m, D, scale, fbits, w_off) : 0u;
+            }
+            const uint32_t word = __shfl_sync(0xffffffffu, flags, 8 * (s & 3) + (lane >> 2));
+            fmask &= word >> (8 * (lane & 3));
+        }
+        if (!fmask || out_of_range(n, (const uint16_t *)(t4 + 1) <= n.tgt16 + n.S)) continue;
+        const uint4 tv = *t4;
+        int4 wa, wb;
+        if (exc) {
+            wa = w4[0];
+            wb = w4[1];
+        } else {
+            wa = wb = make_int4(n.w_inh, n.w_inh, n.w_inh, n.w_inh);
+        }
+        const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
+        const int32_t wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        const bool all = full && 256 * (s + 1) <= m;   // warp-uniform
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t v = (u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu);
+            if (out_of_range(n, v < kSlots * n.npc)) continue;
+            red_shared(in0 + 4u * v, all || ((fmask >> u) & 1u) ? wv[u] : 0);
+        }
+    }
+}
+
+__device__ __forceinline__ void dense_light_body(const DevNet &n, const int *t_now, const Part &g)
+{
+    extern __shared__ int4 smem_i4[];
+    __shared__ uint32_t s_col[kSlots];
+    __shared__ uint32_t s_unit;
+    const int t = *t_now;
+    if (!deferring(n, t) || !dense_selected(n, t)) return;
+    const uint32_t npc = n.npc, nwarps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, D = (int)n.D;
+    int32_t *s_in = reinterpret_cast<int32_t *>(smem_i4);       // [kSlots * npc]
+    int32_t *w_off = s_in + kSlots * npc + warp * 32;           // bucket end offsets
+    const uint32_t in0 = (uint32_t)__cvta_generic_to_shared(s_in);
+    const uint32_t chunks = (npc + n.dense_rows - 1) / n.dense_rows;
+    const uint32_t dmask = (2u << D) - 2u;
+    drive(n, t, part_tid(g), part_threads(g));
+    unsigned long long ev_all = 0, ev_exc = 0;
+    for (uint32_t unit = g.bid; unit < n.C * chunks;) {
+        const uint32_t col = unit / chunks;
+        const uint32_t r0 = (unit - col * chunks) * n.dense_rows;
+        const uint32_t r1 = min(npc, r0 + n.dense_rows);
+        if (threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
+        for (uint32_t k = threadIdx.x; k < kSlots * npc; k += blockDim.x) s_in[k] = 0;
+        __syncthreads();
+        for (uint32_t r = r0 + warp; r < r1; r += nwarps) {
+            const uint32_t p = col * npc + r;
+            const bool exc = r < n.ne;
+            const uint32_t due = exc ? dmask : 2u;         // inhibitory rows: delay 1 alone
+            const uint32_t fbits = (n.hl[p].x << 1) & due;
+            if (!fbits) continue;
+            int events = (int)n.canon_m;
+            if (fbits != due) {
+                const int hi = lane <= D ? (int)n.doff[(size_t)p * kDoffStride + lane] : 0;
+                const int lo = __shfl_up_sync(0xffffffffu, hi, 1);
+                __syncwarp();
+                w_off[lane] = hi;                          // lane d: end of bucket d, lane 0: 0
+                events = __reduce_add_sync(0xffffffffu, (lane && ((fbits >> lane) & 1u)) ? hi - lo : 0);
+                __syncwarp();
+            }
+            if (lane == 0) {
+                ev_all += (unsigned long long)events;
+                if (exc) ev_exc += (unsigned long long)events;
+            }
+            light_row(n, row_base(n, p), exc, fbits, due, w_off, in0, lane);
+        }
+        __syncthreads();
+        for (int sl = 0; sl < kSlots; ++sl) {
+            int32_t *dst = n.I + (size_t)s_col[sl] * npc;
+            const int32_t *in_row = s_in + sl * npc;
+            for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
+                const int32_t v = in_row[loc];
+                if (v) red_add(&dst[loc], v);
+            }
+        }
+        if (threadIdx.x == 0) s_unit = g.nblk + atomicAdd(&n.ctr->dense_cursor, 1u);
+        __syncthreads();
+        unit = s_unit;
+        __syncthreads();
+    }
+    if (lane != 0) ev_all = ev_exc = 0;
+    const unsigned long long ba = block_sum(ev_all);
+    const unsigned long long be = block_sum(ev_exc);
+    if (threadIdx.x == 0) {
+        if (ba) {
+            atomicAdd(&n.ctr->e_all, ba);
+            atomicAdd(&n.ctr->e_exc, be);
+            atomicAdd(&n.ctr->dense_e_all, ba);
+            atomicAdd(&n.ctr->dense_e_exc, be);
+        }
+        if (g.bid == 0) {
+            n.ctr->dense_l_exc += n.ctr->l_exc_last;       // visits that the window's pass makes
+            n.ctr->dense_steps += 1;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(1024) k_dense(DevNet n, const int *t_now) { dense_body(n, t_now, whole_grid()); }
+
+__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered(DevNet n, const int *t_now)
+{
+    deliver_ordered(n, t_now, whole_grid());
+}
+
+__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered_b(BatchLaunch b)
+{
+    const BatchBlock x = batch_block(b);
+    const DevNet n = b.nets[x.net];
+    deliver_ordered(n, x.t_now, x.part);
+}
+
+// Both in one launch, for shapes that give them the same blocks (a step takes
+// one of them; the other alone would be a launch that returns, 3 us).
+__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_dense(DevNet n, const int *t_now)
+{
+    if (ordered_selected(n, *t_now)) deliver_ordered(n, t_now, whole_grid());
+    else dense_body(n, t_now, whole_grid());
+}
 
 __global__ void __launch_bounds__(1024) k_dense_b(BatchLaunch b)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
     dense_body(n, x.t_now, x.part);
+}
+
+__global__ void __launch_bounds__(kDenseLightBlock, 2) k_dense_light(DevNet n, const int *t_now)
+{
+    dense_light_body(n, t_now, whole_grid());
+}
+
+__global__ void __launch_bounds__(kDenseLightBlock, 2) k_dense_light_b(BatchLaunch b)
+{
+    const BatchBlock x = batch_block(b);
+    const DevNet n = b.nets[x.net];
+    dense_light_body(n, x.t_now, x.part);
 }
 
 }  // namespace snn

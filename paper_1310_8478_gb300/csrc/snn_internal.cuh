@@ -762,6 +762,8 @@ __global__ void k_sort_raster(const int64_t *step_off, uint32_t steps, uint32_t 
 
 __global__ void k_deliver(DevNet n, const int *t_now);
 __global__ void k_dense(DevNet n, const int *t_now);
+__global__ void k_deliver_dense(DevNet n, const int *t_now);
+__global__ void k_dense_light(DevNet n, const int *t_now);
 __global__ void k_deliver_cols(DevNet n, const int *t_now);
 __global__ void k_deliver_ordered(DevNet n, const int *t_now);
 __global__ void k_neuron_f32(DevNet n, const int *t_now, int *t_next);
@@ -781,6 +783,7 @@ __global__ void k_emit(DevNet n);
 // the same kernels for every net of a batch in one launch (BatchLaunch)
 __global__ void k_deliver_b(BatchLaunch b);
 __global__ void k_dense_b(BatchLaunch b);
+__global__ void k_dense_light_b(BatchLaunch b);
 __global__ void k_deliver_cols_b(BatchLaunch b);
 __global__ void k_deliver_ordered_b(BatchLaunch b);
 __global__ void k_neuron_f32_b(BatchLaunch b);
@@ -817,6 +820,8 @@ size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
 size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64);
+size_t dense_light_smem_bytes(uint32_t npc);
+constexpr uint32_t kDenseLightBlock = 1024;  // threads per block of a dense step that defers its STDP
 constexpr uint32_t kResBlock = 512;         // threads per block of a resident grid
 constexpr uint32_t kEmitBlock = 512;
 constexpr uint32_t kEmitWords = 2048;       // words of a step's spike bits per block

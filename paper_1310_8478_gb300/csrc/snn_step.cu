@@ -34,7 +34,7 @@
 // by the host-side flush (k_ltp + k_deriv with force = 1) before any read.
 #include <type_traits>
 
-#include "snn_internal.cuh"
+#include "snn_deliver.cuh"
 
 namespace snn {
 
@@ -184,7 +184,7 @@ __device__ __forceinline__ void deliver_ring(const DevNet &n, const int *t_now, 
 // persistent grid takes source columns from a step-wide cursor, so the
 // columns in flight form a narrow band of the torus and so do the targets
 // they reach.  Two forms:
-//   deliver_columns (the default): the source column's own neurons -- the
+//   deliver_columns (snn_deliver.cuh, the default): the source column's own neurons -- the
 //   targets of every inhibitory synapse and of the local share of the
 //   excitatory ones -- have their input and last spikes in shared memory.
 //   deliver_cols (13-column staging, for launch shapes that ask for it): the
@@ -203,11 +203,6 @@ size_t staged_smem_bytes(uint32_t npc, uint32_t block)
 {
     return (size_t)kLut * 4 + (size_t)kSlots * npc * 4 + (size_t)npc * 4 + (size_t)(block / 32) * kTileWords * 4 +
            (((size_t)kSlots * npc * 2 + 15) & ~size_t(15));
-}
-
-size_t ordered_smem_bytes(uint32_t npc, uint32_t block)
-{
-    return (size_t)kLut * 4 + (size_t)npc * 24 + kItems * 4 + (size_t)(block / 32) * 64 * 4;
 }
 
 // s_x: LTD amounts of the 13 staged columns.
@@ -421,152 +416,6 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
     }
 }
 
-// The column-ordered delivery.  Per column a block lists the inhibitory rows
-// that fired at t - 1 and the due (row, delay) items, walks both with all of
-// its threads (walk_inhibitory, walk_items) and flushes the column's own input
-// with one coalesced reduction per touched neuron; a target on another column
-// is a reduction into its input and, with kStdp, a gather of its last spike,
-// both on the band of columns in flight, which stays in L2.  The next column is
-// claimed two columns ahead, and its histories and last spikes are copied into
-// shared memory while this one is walked.  Bound by latency and instruction
-// issue (half of it) at 64 registers and two blocks of 512 threads per SM; with
-// three at 40 registers it spilled (busy 32x32 net: 142 against 129 us per
-// step), and five of 256 threads left a wave of 1024 columns two thirds full
-// (with depression, per step: busy 32x32 net 119 -> 90 us, onset of the 64x32
-// benchmark torus 83 -> 68, 64x64 torus of the paper's columns 91 -> 88).
-template <bool kStdp>
-__device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Part &g)
-{
-    extern __shared__ int4 smem_i4[];
-    __shared__ uint32_t s_col[2][kSlotStride], s_next[2];
-    __shared__ unsigned s_items_n, s_inh_n;
-    const uint32_t npc = n.npc, ne = n.ne;
-    int32_t *const s_lut = reinterpret_cast<int32_t *>(smem_i4);
-    int32_t *const s_in = s_lut + kLut;                                   // [npc] input of the column
-    uint32_t *const s_hist = reinterpret_cast<uint32_t *>(s_in + npc);    // [2][npc] bit k: fired at t - 1 - k
-    int32_t *const s_last = reinterpret_cast<int32_t *>(s_hist + 2 * npc);   // [2][npc] last spikes
-    uint32_t *const s_inh = reinterpret_cast<uint32_t *>(s_last + 2 * npc);  // [npc]
-    uint32_t *const s_items = s_inh + npc;                                // [kItems]
-    int32_t *const w_ab = reinterpret_cast<int32_t *>(s_items + kItems) + (threadIdx.x >> 5) * 64;
-    const int lane = threadIdx.x & 31;
-    const uint32_t dmask = (2u << n.D) - 2u;
-    const int64_t col_syn = (int64_t)npc * n.uniform_m;
-    const int lg = bucket_lanes(n);
-    if (kStdp)
-        for (int i = threadIdx.x; i < kLut; i += blockDim.x) s_lut[i] = n.lut_m[i];
-    drive(n, t, part_tid(g), part_threads(g));
-    if (n.flags & SNN_DELIVERY_OFF) return;
-    auto copy = [&](uint32_t col, int b) {
-        if (threadIdx.x < kSlotStride) copy4_async(&s_col[b][threadIdx.x], n.nbr + col * kSlotStride + threadIdx.x);
-        for (uint32_t i = threadIdx.x; i < npc; i += blockDim.x) {
-            copy4_async(s_hist + b * npc + i, &n.hl[(size_t)col * npc + i].x);
-            if (kStdp) copy4_async(s_last + b * npc + i, n.last_spike + (size_t)col * npc + i);
-        }
-    };
-    uint32_t col = g.bid;
-    if (col < n.C) copy(col, 0);
-    for (uint32_t i = threadIdx.x; i < npc; i += blockDim.x) s_in[i] = 0;
-    if (threadIdx.x == 0) {
-        s_next[0] = g.nblk + atomicAdd(&n.ctr->staged_cursor, 1u);
-        s_items_n = s_inh_n = 0;
-    }
-    unsigned long long ev_all = 0, ev_exc = 0;
-    for (int b = 0; col < n.C; b ^= 1) {
-        wait_async();
-        __syncthreads();
-        const uint32_t next = s_next[b];
-        uint32_t claimed = n.C;
-        if (next < n.C) {
-            copy(next, b ^ 1);
-            if (threadIdx.x == 0) claimed = g.nblk + atomicAdd(&n.ctr->staged_cursor, 1u);
-        }
-        const uint32_t *hist = s_hist + b * npc, *cols = s_col[b];
-        const int32_t *last = s_last + b * npc;
-        const int64_t cbase = (int64_t)col * col_syn;                     // first synapse of the column (8-aligned)
-        const uint16_t *tg = n.tgt16 + cbase;
-        int32_t *const sd = n.sd + cbase;
-        // slots that lead back to the column (rings of a small torus)
-        const uint32_t local = __ballot_sync(0xffffffffu, lane < kSlots && cols[lane] == col);
-        const bool mine = !n.tile || owned_column(n, col);                // inhibitory targets lie in the column
-        if (mine) list_fired(blockDim.x, hist, ne, npc, 0, s_inh, &s_inh_n);
-        // excitatory rows: all of them at once in a sparse step; where their
-        // items do not fit the list, in ranges, halved until they do
-        uint32_t range = ne;
-        bool begun = false;
-        for (uint32_t r0 = 0; r0 < ne;) {
-            list_items(blockDim.x, hist, r0, min(ne, r0 + range), 0, dmask, s_items, &s_items_n);
-            __syncthreads();
-            const uint32_t items = s_items_n;
-            if (items > kItems) {
-                range = max(kItems / n.D, range / 2);
-                __syncthreads();
-                if (threadIdx.x == 0) s_items_n = 0;
-                __syncthreads();
-                continue;
-            }
-            unsigned seen = 0;                                            // a tile's events on its own columns
-            const unsigned walked = walk_items(
-                blockDim.x, n, col, s_items, items, w_ab, lg, tg, n.w + cbase, col_syn,
-                [&] {
-                    if (begun) return;
-                    walk_inhibitory(blockDim.x, n, s_inh, s_inh_n, tg, col_syn, (uint32_t)__cvta_generic_to_shared(s_in));
-                    if (threadIdx.x == 0) ev_all += (unsigned long long)s_inh_n * n.canon_m;
-                },
-                [&](uint32_t v, int32_t w) -> int32_t {
-                    const uint32_t slot = __umulhi(v, n.npc_recip), loc = v - slot * npc;
-                    if (n.tile) {
-                        if (!owned_column(n, cols[slot])) return kNever;  // another tile's target
-                        ++seen;
-                    }
-                    if ((local >> slot) & 1u) {
-                        atomicAdd(&s_in[loc], w);
-                        return kStdp ? last[loc] : 0;
-                    }
-                    const uint32_t gid = cols[slot] * npc + loc;
-                    red_add(&n.I[gid], w);
-                    return kStdp ? n.last_spike[gid] : 0;
-                },
-                [&](int32_t x, int at) {
-                    if (!kStdp) return;
-                    const int32_t amount = s_lut[min(t - x, kLut - 1)];   // lag >= 1
-                    if (amount) red_add(&sd[at], -amount);                // no load: most amounts are 0
-                });
-            if (n.tile) {
-                ev_all += seen;
-                ev_exc += seen;
-            } else if (lane == 0) {
-                ev_all += walked;
-                ev_exc += walked;
-            }
-            begun = true;
-            r0 += range;
-            __syncthreads();                                              // the items and the column's input are done
-            if (threadIdx.x == 0) s_items_n = 0;
-            if (r0 < ne) __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            s_next[b ^ 1] = claimed;
-            s_inh_n = 0;
-        }
-        int32_t *dst = n.I + (size_t)col * npc;
-        for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-            const int32_t x = s_in[loc];
-            if (x) {
-                red_add(&dst[loc], x);
-                s_in[loc] = 0;
-            }
-        }
-        col = next;
-    }
-    if (lane != 0 && !n.tile) ev_all = ev_exc = 0;
-    const unsigned long long ba = block_sum(ev_all);
-    const unsigned long long be = block_sum(ev_exc);
-    if (threadIdx.x == 0 && ba) {
-        atomicAdd(&n.ctr->e_all, ba);
-        atomicAdd(&n.ctr->e_exc, be);
-    }
-}
-
 __device__ __forceinline__ void deliver_staged(const DevNet &n, const int *t_now, const Part &g)
 {
     extern __shared__ int4 smem_i4[];
@@ -580,14 +429,6 @@ __device__ __forceinline__ void deliver_staged(const DevNet &n, const int *t_now
     uint16_t *s_x = reinterpret_cast<uint16_t *>(s_tile + nwarps * kTileWords);   // [kSlots * npc]
     if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_cols<true>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
     else deliver_cols<false>(n, t, s_lut, s_in, s_tile, s_x, s_hist, g);
-}
-
-__device__ __forceinline__ void deliver_ordered(const DevNet &n, const int *t_now, const Part &g)
-{
-    const int t = *t_now;
-    if (!ordered_selected(n, t)) return;
-    if (!(n.flags & SNN_STDP_OFF) && !deferring(n, t)) deliver_columns<true>(n, t, g);
-    else deliver_columns<false>(n, t, g);
 }
 
 // One target's reverse entries [lo, hi), walked by a warp, kUnroll entries
@@ -1138,11 +979,6 @@ __global__ void __launch_bounds__(kStagedBlock) k_deliver_cols(DevNet n, const i
     deliver_staged(n, t_now, whole_grid());
 }
 
-__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered(DevNet n, const int *t_now)
-{
-    deliver_ordered(n, t_now, whole_grid());
-}
-
 __global__ void __launch_bounds__(1024) k_ltp(DevNet n, const int *t_now, int force)
 {
     ltp_body(n, t_now, force, whole_grid());
@@ -1182,13 +1018,6 @@ __global__ void __launch_bounds__(kStagedBlock) k_deliver_cols_b(BatchLaunch b)
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
     deliver_staged(n, x.t_now, x.part);
-}
-
-__global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered_b(BatchLaunch b)
-{
-    const BatchBlock x = batch_block(b);
-    const DevNet n = b.nets[x.net];
-    deliver_ordered(n, x.t_now, x.part);
 }
 
 __global__ void __launch_bounds__(1024) k_ltp_b(BatchLaunch b)

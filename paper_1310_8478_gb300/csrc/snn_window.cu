@@ -13,9 +13,9 @@
 //   depression: for each arrival at p0 + k, the amount at the lag to the
 //       target's latest spike before it.
 // A dense step then moves 6 bytes per synapse (target and weight) instead of
-// 14: at 1.28 M neurons of 1125 synapses about 1.5 ms instead of 2.9, plus the
-// pass, 7.5 ms per 50 steps (bound by instruction issue: two sums over 50-bit
-// trains per synapse).  A train is a 64-bit word: 56 step bits and, in the top 8, the lag of
+// 14: at 1.28 M neurons of 1125 synapses 1.2 ms instead of 2.9, plus the pass,
+// 7 ms per 50 steps (bound by instruction issue: two sums over 50-bit trains
+// per synapse).  A train is a 64-bit word: 56 step bits and, in the top 8, the lag of
 // the latest event before the window (255: none that matters).
 #include <type_traits>
 
