@@ -52,6 +52,7 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
+constexpr size_t kReadStage = 256 << 10;           // bytes of a net's pinned memory for small read-backs
 constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
 constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
@@ -152,6 +153,7 @@ struct snn_net {
     uint16_t *tgt16 = nullptr;
     int32_t *nbr = nullptr;
     bool weights_moved = false;     // a checkpoint was loaded (or a run broke off) since the last reset
+    bool skip_ltp = false;          // no neuron fired in the step before a call's first one
     bool ltp_owed = false;          // the last step's LTP has not been applied yet
     int32_t *noalloc_base = nullptr; // device address of the no-allocation staging array
     int32_t *inject_buf = nullptr;  // tiles: device copy of the spikes received for a step
@@ -166,11 +168,13 @@ struct snn_net {
     int res_grid = 0;               // blocks of the resident grid that runs this net's windows; 0: none does
     uint64_t version = 0;           // bumped whenever captured launches go stale
     // stimulus
-    size_t stim_cap = 0;
-    int64_t stim_off_cap = 0;
+    size_t stim_cap = 0;            // bytes of the device copy (offsets, neurons, currents)
+    bool stim_in_flight = false;    // an upload that no synchronisation has followed yet
     // pinned host memory: the counters read after a run ([1]) and before one
     // ([0]), and the staging of a stimulus upload
     DevCounters *host_ctr = nullptr;
+    bool host_ctr_known = false;    // [1] is what the device holds
+    char *read_stage = nullptr;     // kReadStage bytes of small read-backs
     char *stim_stage = nullptr;
     size_t stim_stage_cap = 0;
     // host state
@@ -954,7 +958,9 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     const bool closes = exact_t && P && t > 0 && (uint32_t)t % P == 0;
     // (an explicit net's small steps end sooner one after another: 5000
     // neurons of 100 synapses 32.5 us per step against 38.8)
-    const bool fork = !closes && !prof && (dn.tgt16 || net->N >= kForkMinExplicit);
+    const bool idle = net->skip_ltp && !closes && !prof && exact_t;
+    net->skip_ltp = false;
+    const bool fork = !idle && !closes && !prof && (dn.tgt16 || net->N >= kForkMinExplicit);
     cudaStream_t sl = fork ? net->side : s;        // the potentiation's stream
     auto mark = [&](int kind, cudaStream_t on) {
         if (prof) cudaEventRecord(next_event(net, kind), on);
@@ -970,8 +976,10 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     const int g_ltp = sized_grid(net, L.ltp_blocks_per_sm, net->N, L.ltp_block / 32);
     const int g_del = sized_grid(net, L.deliver_blocks_per_sm, (int64_t)net->N * dn.D / 4, L.deliver_block);
     int launched = 0;
-    k_ltp<<<g_ltp, L.ltp_block, 0, sl>>>(dn, t_now, 0);
-    ++launched;
+    if (!idle) {
+        k_ltp<<<g_ltp, L.ltp_block, 0, sl>>>(dn, t_now, 0);
+        ++launched;
+    }
     mark(2, sl);
     if (fork) cudaEventRecord(net->ev_join, sl);
     // long-term update when t closes a period: the event-driven LTP is
@@ -1142,6 +1150,8 @@ int finish_run(snn_net *net, bool copied)
         SNN_CUDA(cudaStreamSynchronize(net->stream));
     }
     SNN_CUDA(cudaGetLastError());
+    net->host_ctr_known = true;
+    net->stim_in_flight = false;
     if (net->profile && net->ev_used) {
         for (size_t i = 0; i + 1 < net->ev_used; i += 2) {
             float ms = 0.f;
@@ -1165,9 +1175,16 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
 {
     if ((int64_t)net->t + n_ms > 0x7fff0000ll) { set_error("time limit reached"); return SNN_ESTATE; }
     SNN_TRY(ensure_raster_steps(net, (int64_t)net->t + n_ms + 2 - net->dn.raster_t0));
-    if (count_before)
+    if (count_before && net->host_ctr_known) net->host_ctr[0] = net->host_ctr[1];
+    else if (count_before)
         SNN_CUDA(cudaMemcpyAsync(&net->host_ctr[0], net->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost,
                                  net->stream));
+    // the last step of this net was a step kernel's, read back behind it, and
+    // nothing fired in it: nothing to potentiate in the first one
+    const int32_t *fired = net->host_ctr[1].step_cnt[(net->t - 1) & 1];
+    net->skip_ltp = net->host_ctr_known && net->host_ctr[1].ltp_pending == net->t - 1 && net->t > 0 && fired[0] == 0 &&
+                    fired[1] == 0 && !net->dn.tile;
+    net->host_ctr_known = false;
     const uint32_t L = effective_graph_len(net);
     if (L != net->graph_len) {
         drop_graphs(net);
@@ -1236,6 +1253,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             left -= 1;
             net->ltp_owed = true;
         }
+        net->skip_ltp = false;                 // true of the call's first step at most
         if (window && (window -= before - left) == 0) {
             close_window(net);
             SNN_CUDA(cudaGetLastError());
@@ -1260,6 +1278,7 @@ int canon_offset(snn_net *net, uint32_t p, int64_t *out)
 int flush_owed(snn_net *net)
 {
     if (!net->ltp_owed) return SNN_OK;
+    net->host_ctr_known = false;
     launch_flush(net);
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(net->stream));
@@ -1293,12 +1312,14 @@ int set_stimulus_impl(snn_net *net, const snn_stimulus *ev, size_t n)
     auto by_t = [](const snn_stimulus &a, const snn_stimulus &b) { return a.t < b.t; };
     if (!std::is_sorted(e.begin(), e.end(), by_t)) std::stable_sort(e.begin(), e.end(), by_t);
     const int32_t t0 = e.front().t, t1 = e.back().t + 1;
-    // staged in pinned host memory (the copies below run behind the caller;
-    // the stream is idle here, every run ends with a synchronisation, so the
-    // staging of an earlier upload is free)
+    // staged in pinned host memory as it will lie on the device -- offsets,
+    // neurons, currents -- and uploaded by one copy behind the caller (a run
+    // ends with a synchronisation; two uploads without a run between them wait
+    // here)
     const size_t n_off = (size_t)(t1 - t0) + 1;
     const size_t stage = e.size() * 8 + n_off * 8;
-    SNN_CUDA(cudaStreamSynchronize(net->stream));
+    if (net->stim_in_flight) SNN_CUDA(cudaStreamSynchronize(net->stream));
+    net->stim_in_flight = false;
     if (stage > net->stim_stage_cap) {
         if (net->stim_stage) cudaFreeHost(net->stim_stage);
         net->stim_stage = nullptr;
@@ -1316,28 +1337,20 @@ int set_stimulus_impl(snn_net *net, const snn_stimulus *ev, size_t n)
         off[(size_t)(e[i].t - t0) + 1]++;
     }
     for (size_t k = 1; k < n_off; ++k) off[k] += off[k - 1];
-    if (e.size() > net->stim_cap) {
-        dfree(net, (void *)dn.stim_gid);
-        dfree(net, (void *)dn.stim_q16);
-        dn.stim_gid = dn.stim_q16 = nullptr;
-        int32_t *a = nullptr, *b = nullptr;
-        SNN_TRY(dalloc_t(net, e.size(), &a));
-        SNN_TRY(dalloc_t(net, e.size(), &b));
-        dn.stim_gid = a;
-        dn.stim_q16 = b;
-        net->stim_cap = e.size();
-    }
-    if ((int64_t)n_off > net->stim_off_cap) {
+    if (stage > net->stim_cap) {
+        dn.stim_t0 = dn.stim_t1 = 0;
         dfree(net, (void *)dn.stim_off);
         dn.stim_off = nullptr;
-        int64_t *o = nullptr;
-        SNN_TRY(dalloc_t(net, n_off, &o));
-        dn.stim_off = o;
-        net->stim_off_cap = (int64_t)n_off;
+        net->stim_cap = 0;
+        char *p = nullptr;
+        SNN_TRY(dalloc_t(net, stage, &p));
+        dn.stim_off = reinterpret_cast<int64_t *>(p);
+        net->stim_cap = stage;
     }
-    SNN_CUDA(cudaMemcpyAsync((void *)dn.stim_gid, gid, e.size() * 4, cudaMemcpyHostToDevice, net->stream));
-    SNN_CUDA(cudaMemcpyAsync((void *)dn.stim_q16, q, e.size() * 4, cudaMemcpyHostToDevice, net->stream));
-    SNN_CUDA(cudaMemcpyAsync((void *)dn.stim_off, off, n_off * 8, cudaMemcpyHostToDevice, net->stream));
+    SNN_CUDA(cudaMemcpyAsync((void *)dn.stim_off, net->stim_stage, stage, cudaMemcpyHostToDevice, net->stream));
+    net->stim_in_flight = true;
+    dn.stim_gid = reinterpret_cast<const int32_t *>(dn.stim_off + n_off);
+    dn.stim_q16 = dn.stim_gid + e.size();
     dn.stim_t0 = t0;
     dn.stim_t1 = t1;
     drop_graphs(net);
@@ -1398,6 +1411,7 @@ int raster_window(snn_net *net, int32_t t0, int32_t t1, snn_spike *buf, size_t c
 
 int raster_reset_impl(snn_net *net)
 {
+    net->host_ctr_known = false;
     DevNet &dn = net->dn;
     if (!dn.raster_gid) return SNN_OK;
     DevCounters hc{};
@@ -1457,6 +1471,7 @@ void snn_free(snn_net *net)
     if (net->ev_join) cudaEventDestroy(net->ev_join);
     if (net->side) cudaStreamDestroy(net->side);
     if (net->stim_stage) cudaFreeHost(net->stim_stage);
+    if (net->read_stage) cudaFreeHost(net->read_stage);
     if (net->own_stream && net->stream) cudaStreamDestroy(net->stream);
     delete net;
 }
@@ -2163,6 +2178,8 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
     if (n_ms == 0) return SNN_OK;
     for (snn_net *n : b->nets) {
         if (n->profile) { set_error("a net of the batch is profiling"); return SNN_ESTATE; }
+        n->host_ctr_known = false;
+        n->skip_ltp = false;
         if ((int64_t)n->t + n_ms > 0x7fff0000ll) { set_error("time limit reached"); return SNN_ESTATE; }
         SNN_TRY(ensure_raster_steps(n, (int64_t)n->t + n_ms + 2 - n->dn.raster_t0));
         SNN_CUDA(cudaStreamSynchronize(n->stream));
@@ -2372,6 +2389,7 @@ int snn_reset(snn_net *net)
     SNN_CUDA(cudaGetLastError());
     SNN_CUDA(cudaStreamSynchronize(s));
     net->t = 0;
+    net->host_ctr_known = false;
     net->weights_moved = false;
     net->ltp_owed = false;
     net->dn.raster_t0 = 0;
@@ -2562,9 +2580,20 @@ int snn_read_neurons(snn_net *net, uint32_t first, uint32_t count, float *host_v
         }
         return SNN_OK;
     }
-    if (host_v) SNN_CUDA(cudaMemcpyAsync(host_v, net->dn.v + first, (size_t)count * 4, cudaMemcpyDeviceToHost, net->stream));
-    if (host_u) SNN_CUDA(cudaMemcpyAsync(host_u, net->dn.u + first, (size_t)count * 4, cudaMemcpyDeviceToHost, net->stream));
+    // small reads through pinned memory: a copy into pageable memory waits for
+    // the stream by itself, each
+    const size_t bytes = (size_t)count * 4;
+    char *stage = nullptr;
+    if (2 * bytes <= kReadStage) {
+        if (!net->read_stage) SNN_CUDA(cudaHostAlloc(&net->read_stage, kReadStage, cudaHostAllocDefault));
+        stage = net->read_stage;
+    }
+    void *to_v = stage ? (void *)stage : (void *)host_v, *to_u = stage ? (void *)(stage + bytes) : (void *)host_u;
+    if (host_v) SNN_CUDA(cudaMemcpyAsync(to_v, net->dn.v + first, bytes, cudaMemcpyDeviceToHost, net->stream));
+    if (host_u) SNN_CUDA(cudaMemcpyAsync(to_u, net->dn.u + first, bytes, cudaMemcpyDeviceToHost, net->stream));
     SNN_CUDA(cudaStreamSynchronize(net->stream));
+    if (stage && host_v) std::memcpy(host_v, to_v, bytes);
+    if (stage && host_u) std::memcpy(host_u, to_u, bytes);
     return SNN_OK;
 }
 
@@ -2771,6 +2800,7 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     cudaStream_t s = net->stream;
     DevNet &dn = net->dn;
     net->weights_moved = true;
+    net->host_ctr_known = false;
     void *sv = dn.vd ? (void *)dn.vd : (void *)dn.v;
     void *su = dn.ud ? (void *)dn.ud : (void *)dn.u;
     void *dst[] = {sv, su, dn.I, dn.hl, dn.last_spike, dn.ring_ids, dn.ring_cnt, net->w, net->sd, net->ctr};

@@ -157,3 +157,38 @@ def test_reset_restores_whatever_moved(eng, before):
             for a, b in zip(n.weights() + n.raster(), fresh.weights() + fresh.raster()):
                 assert np.array_equal(a, b)
             assert n.counters() == fresh.counters()
+
+
+@pytest.mark.parametrize("lists", [False, True], ids=["generated", "explicit"])
+def test_closed_loop_of_single_steps_equals_the_oracle(eng, orc, lists):
+    """One call per millisecond with that step's host events: quiet steps,
+    whose successor has nothing to potentiate, between single spikes; events of
+    changing number; a period's end on the way."""
+    cfg = _cfg(2, 1, 60, 30, seed=73, thal_per_col_per_ms=0, deriv_period_ms=50)
+    rng = np.random.default_rng(9)
+    explicit = None
+    if lists:
+        rows = rng.integers(20, 40, 120)
+        off = np.concatenate([[0], np.cumsum(rows)])
+        exc = np.repeat(np.arange(120) % 60 < 48, rows)
+        explicit = dict(row_off=off, tgt=rng.integers(0, 120, off[-1]),
+                        delay=np.where(exc, rng.integers(1, 21, off[-1]), 1),
+                        w=np.where(exc, 7 * 65536, -5 * 65536))
+    T = 130
+    counts = rng.integers(0, 6, T)
+    t = np.repeat(np.arange(T), counts)
+    g = rng.integers(0, 120, len(t))
+    q = rng.integers(10, 60, len(t)) * 65536
+    o = orc.Oracle(cfg, explicit=explicit)
+    o.set_stimulus(t, g, q)
+    o.run(T)
+    ev = np.zeros(len(t), eng.snn.STIM_DTYPE)
+    ev["t"], ev["gid"], ev["q16"] = t, g, q
+    with gpu_net(eng, cfg, explicit=explicit) as n:
+        total, quiet = 0, 0
+        for k in range(T):
+            got = n.run_host_counts(1, ev[t == k])
+            total += got
+            quiet += got == 0
+        assert_same_run(o, n)
+        assert total == o.counters()["spikes"] and quiet > 10 and total > 10
