@@ -56,6 +56,8 @@ constexpr size_t kReadStage = 256 << 10;           // bytes of a net's pinned me
 constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
 constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
+constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
+constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
 // Device staging of snn_read_synapses_noalloc: target, weight and sd words,
@@ -633,7 +635,15 @@ int clear_window(snn_net *net)
 // columns 9.5, 7.7, 6.6, 6.5, 6.9; 2x2 with M = 300 8.7, 7.1, 6.1, 5.8, 5.6;
 // one column in FP64 12.3, 9.0, 6.5, 5.7, 5.8).  A net of one block needs no
 // grid barrier, so one column in FP32 stays with it (4.3 us, else 4.6 or
-// more).
+// more).  Nets with target lists: one block per SM with slices of at least 32
+// neurons (5000 neurons, 500000 synapses: 10.3 us per step with 152 blocks,
+// 10.1 with 76, 11.7 with 50, 10.6 with 304).
+const void *resident_kernel(const snn_net *net)
+{
+    if (!net->tgt16) return net->dn.vd ? (const void *)k_resident_lists_f64 : (const void *)k_resident_lists_f32;
+    return net->dn.vd ? (const void *)k_resident_f64 : (const void *)k_resident_f32;
+}
+
 int resident_grid(snn_net *net, int *parts_out)
 {
     const DevNet &dn = net->dn;
@@ -642,12 +652,24 @@ int resident_grid(snn_net *net, int *parts_out)
     int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, net->device) != cudaSuccess || !coop) return 0;
     const bool f64 = dn.vd != nullptr;
-    const void *kernel = f64 ? (const void *)k_resident_f64 : (const void *)k_resident_f32;
+    const void *kernel = resident_kernel(net);
+    if (!net->tgt16) {
+        // target lists: slices of all neurons, one block per SM
+        if (dn.S > 0x7fffffffll || (uint64_t)dn.C * dn.thal_per_col > kResListsThal) return 0;
+        const uint32_t blocks = std::min<uint32_t>((uint32_t)net->sm_count, (dn.N + 31u) / 32u);
+        const size_t bytes = resident_smem_bytes(dn.N, blocks, f64, true);
+        int per_sm = 0;
+        if (allow_smem(kernel, bytes) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, (int)kResBlock, bytes) != cudaSuccess)
+            cudaGetLastError();
+        *parts_out = (int)blocks;
+        return per_sm >= 1 ? (int)blocks : 0;
+    }
     int parts = kResMaxParts;
     if (dn.C == 1 && !f64) parts = 1;
     for (; parts >= 1; --parts) {
         if (parts > 1 && (dn.npc + parts - 1) / parts < 32) continue;
-        const size_t bytes = resident_smem_bytes(dn.npc, (uint32_t)parts, f64);
+        const size_t bytes = resident_smem_bytes(dn.npc, (uint32_t)parts, f64, false);
         int per_sm = 0;
         if (allow_smem(kernel, bytes) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, (int)kResBlock, bytes) != cudaSuccess) {
@@ -668,7 +690,8 @@ int resident_grid(snn_net *net, int *parts_out)
 // window costs three launches (about 30 us with the change of the
 // shared-memory split, 0.6 us per step; the one-column workload ran 1.7 us
 // per step slower with windows) and a dense step of such a net saves 8 bytes
-// per synapse, about 10 us.  Resident grids take them at any size.  The
+// per synapse, about 10 us.  Resident grids take them at any size, also for
+// nets with target lists, which have a pass of their own.  The
 // arrays (24 or 28 bytes per neuron) are taken only where the budget and the device
 // have room; without them every step applies its STDP at once.
 int setup_windows(snn_net *net)
@@ -680,11 +703,12 @@ int setup_windows(snn_net *net)
     const size_t bytes = stdp_smem_bytes(dn.npc, kStdpBlock);
     int optin = 0, parts = 1;
     SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
-    const bool can = net->tgt16 && !dn.tile && !(net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) &&
-                     bytes + 1024 <= (size_t)optin;
+    const bool lists = !net->tgt16;
+    const bool can = !dn.tile && !(net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) &&
+                     (lists || bytes + 1024 <= (size_t)optin);
     if (can && dn.win && !dn.I2 && resident_grid(net, &parts)) drop_windows(net);   // (a shape that lets one run now)
     const int res = can ? resident_grid(net, &parts) : 0;
-    if (!can || (!res && net->n_rin < kWinMinSynapses)) {
+    if (!can || (!res && (lists || net->n_rin < kWinMinSynapses))) {
         drop_windows(net);
         return SNN_OK;
     }
@@ -707,6 +731,13 @@ int setup_windows(snn_net *net)
         dn.win = win;
         if (res) SNN_CUDA(cudaMemsetAsync(dn.I2, 0, (size_t)net->N * 4, net->stream));
         SNN_TRY(clear_window(net));
+    }
+    net->res_grid = res;
+    dn.res_parts = (uint32_t)parts;
+    if (lists) {
+        // a warp per row, one wave
+        net->stdp_grid = sized_grid(net, 2048 / kStdpListsBlock, (int64_t)dn.C * dn.ne, kStdpListsBlock / 32);
+        return SNN_OK;
     }
     SNN_CUDA(allow_smem((const void *)k_stdp, bytes));
     int per_sm = 0;
@@ -731,8 +762,6 @@ int setup_windows(snn_net *net)
         const int64_t dense_units = (int64_t)dn.C * ((dn.npc + dn.dense_rows - 1) / dn.dense_rows);
         net->light_grid = (int)std::min<int64_t>(dense_units, (int64_t)std::max(1, per_sm) * net->sm_count);
     }
-    net->res_grid = res;
-    dn.res_parts = (uint32_t)parts;
     // a step starts the deferral when the rest of its window, at its rate, will
     // see half a spike per neuron: the pass then costs less than the
     // potentiation and depression of the single steps (us per step at a
@@ -1069,6 +1098,10 @@ void open_window(snn_net *net, uint32_t steps)
 void launch_stdp(snn_net *net, bool trains)
 {
     const DevNet &dn = net->dn;
+    if (!net->tgt16) {
+        k_stdp_lists<<<net->stdp_grid, kStdpListsBlock, stdp_smem_bytes(0, kStdpListsBlock), net->stream>>>(dn);
+        return;
+    }
     if (!trains) k_train<<<sized_grid(net, 8, dn.spk_words, 64), 256, 0, net->stream>>>(dn);
     k_stdp<<<net->stdp_grid, kStdpBlock, stdp_smem_bytes(dn.npc, kStdpBlock), net->stream>>>(dn);
 }
@@ -1091,7 +1124,13 @@ void close_window(snn_net *net)
 // steps, which would pay for a window's pass each)
 bool resident_call(const snn_net *net, uint32_t left)
 {
-    return net->res_grid && !net->profile && !net->dn.probe_n && left >= 4;
+    if (!net->res_grid || net->profile || net->dn.probe_n || left < 4) return false;
+    if (net->tgt16) return true;
+    // with target lists nothing bounds the synapses: the passes (15 us per
+    // million synapses and window) must cost less than the steps save (20 us
+    // each)
+    const uint32_t P = net->cfg.deriv_period_ms;
+    return (uint64_t)std::min<uint32_t>({left, kWinSteps, P ? P : left}) * kResListsPass >= (uint64_t)net->dn.S;
 }
 
 // `steps` more steps from t0 as one window on the resident grid (it runs as
@@ -1104,9 +1143,9 @@ int launch_resident(snn_net *net, int32_t t0, uint32_t steps)
     const bool f64 = dn.vd != nullptr;
     int n_steps = (int)steps;
     void *args[] = {&dn, &t0, &n_steps};
-    SNN_CUDA(cudaLaunchCooperativeKernel(f64 ? (const void *)k_resident_f64 : (const void *)k_resident_f32,
-                                         dim3((unsigned)net->res_grid), dim3(kResBlock), args,
-                                         resident_smem_bytes(dn.npc, dn.res_parts, f64), s));
+    const bool lists = !net->tgt16;
+    SNN_CUDA(cudaLaunchCooperativeKernel(resident_kernel(net), dim3((unsigned)net->res_grid), dim3(kResBlock), args,
+                                         resident_smem_bytes(lists ? dn.N : dn.npc, dn.res_parts, f64, lists), s));
     k_emit<<<dim3((dn.spk_words + kEmitWords - 1) / kEmitWords, steps), kEmitBlock, 0, s>>>(dn);
     launch_stdp(net, true);
     return SNN_OK;

@@ -778,6 +778,9 @@ __global__ void k_train(DevNet n);
 __global__ void k_stdp(DevNet n);
 __global__ void k_resident_f32(DevNet n, int t0, int steps);
 __global__ void k_resident_f64(DevNet n, int t0, int steps);
+__global__ void k_resident_lists_f32(DevNet n, int t0, int steps);
+__global__ void k_resident_lists_f64(DevNet n, int t0, int steps);
+__global__ void k_stdp_lists(DevNet n);
 __global__ void k_emit(DevNet n);
 
 // the same kernels for every net of a batch in one launch (BatchLaunch)
@@ -819,13 +822,14 @@ size_t dense_smem_bytes(uint32_t npc, uint32_t block);
 size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
-size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64);
+size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists);
 size_t dense_light_smem_bytes(uint32_t npc);
 constexpr uint32_t kDenseLightBlock = 1024;  // threads per block of a dense step that defers its STDP
 constexpr uint32_t kResBlock = 512;         // threads per block of a resident grid
 constexpr uint32_t kEmitBlock = 512;
 constexpr uint32_t kEmitWords = 2048;       // words of a step's spike bits per block
 constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's pass
+constexpr uint32_t kStdpListsBlock = 256;   // ... of nets with target lists
 // k_fold: as the step that closes a period runs it / always / before a
 // window's pass that closes a period
 enum FoldMode { kFoldStep = 0, kFoldForce = 1, kFoldWindow = 2 };

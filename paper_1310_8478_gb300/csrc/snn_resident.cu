@@ -23,8 +23,17 @@
 // arrivals from earlier spikes while the barrier fills, with three inputs in
 // turn (8x8 10.1, one column 4.9).
 //
+// Nets with target lists have no columns in this sense: a block owns a slice of
+// all neurons, inhibitory rows are walked by delay like the others, and every
+// target outside the slice is a reduction (a checkpointed net of 5000 neurons
+// and 500000 synapses at 100 Hz, 49000 events per step: 10 us per step with its
+// pass, 31 with the step kernels).
+//
 // A grid runs while its steps stay sparse: from a step with enough spikes for
-// the dense pass on it stops, and the host goes on with the step kernels.
+// the dense pass on it stops, and the host goes on with the step kernels (nets
+// with lists have no dense pass and run to the window's end).
+#include <type_traits>
+
 #include "snn_internal.cuh"
 
 namespace snn {
@@ -37,14 +46,14 @@ constexpr int kBarrierPolls = 1 << 22;       // about two seconds, then the kern
 
 __host__ __device__ __forceinline__ uint32_t res_slice(uint32_t npc, uint32_t parts) { return (npc + parts - 1) / parts; }
 
-size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64)
+size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists)
 {
     const size_t ns = res_slice(npc, parts);
     return ns * (fp64 ? 16 : 8)                                // v, u
            + ns * 8                                            // spike train of the window
            + ns * 8                                            // history word, older spike
            + ns * 4                                            // inhibitory rows that fired
-           + (size_t)npc * 4                                   // input of the column
+           + (lists ? ns : (size_t)npc) * 4                    // input of the column (of the own neurons)
            + kResItems * 4                                     // items
            + (size_t)(kResBlock / 32) * 64 * 4;                // per warp: a tile's buckets
 }
@@ -69,7 +78,7 @@ __device__ __forceinline__ bool grid_barrier(DevWindow *win, unsigned target, in
     return *s_ok != 0;
 }
 
-template <typename F>
+template <typename F, bool kLists>
 __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps)
 {
     extern __shared__ int4 smem_i4[];
@@ -77,7 +86,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
     __shared__ unsigned s_items_n, s_inh_n;
     __shared__ int s_fired[2];                 // spikes of the step: exc, inh
     __shared__ int s_ok, s_stop;
-    __shared__ uint16_t s_thal[kResThal];
+    __shared__ std::conditional_t<kLists, uint32_t, uint16_t> s_thal[kResThal];
     DevWindow *const win = n.win;
     // not when the net's clock stands elsewhere (an earlier window of the call
     // stopped) or the first step is one for the dense pass
@@ -92,9 +101,9 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         }
     }
     if (!go) return;
-    const uint32_t npc = n.npc, parts = n.res_parts;
+    const uint32_t npc = kLists ? n.N : n.npc, parts = kLists ? gridDim.x : n.res_parts;
     const uint32_t ns_max = res_slice(npc, parts);
-    const uint32_t col = blockIdx.x / parts, part = blockIdx.x - col * parts;
+    const uint32_t col = kLists ? 0u : blockIdx.x / parts, part = blockIdx.x - col * parts;
     const uint32_t lo = min(npc, part * ns_max), hi = min(npc, lo + ns_max), ns = hi - lo;   // own neurons
     const uint32_t g0 = col * npc + lo;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -110,7 +119,8 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
     int32_t *const s_old = reinterpret_cast<int32_t *>(s_hist + ns_max);
     uint32_t *const s_inh = reinterpret_cast<uint32_t *>(s_old + ns_max);
     int32_t *const s_in = reinterpret_cast<int32_t *>(s_inh + ns_max);
-    uint32_t *const s_items = reinterpret_cast<uint32_t *>(s_in + npc);
+    const uint32_t in_lo = kLists ? lo : 0u, in_n = kLists ? ns_max : npc;      // the neurons that s_in covers
+    uint32_t *const s_items = reinterpret_cast<uint32_t *>(s_in + in_n);
     int32_t *const w_a = reinterpret_cast<int32_t *>(s_items + kResItems) + warp * 64;
     int32_t *const w_b = w_a + 32;
     F *const gv = sizeof(F) == 8 ? (F *)n.vd : (F *)n.v;
@@ -133,35 +143,43 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         for (uint32_t w = (g0 >> 5) + i % kWinSlots; ns && w <= (g0 + ns - 1) >> 5; w += kWinSlots)
             n.spk[(size_t)((p0 + k) & (kWinSlots - 1)) * n.spk_words + w] = 0;
     }
-    for (uint32_t i = threadIdx.x; i < npc; i += kResBlock) s_in[i] = 0;
-    if (threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
-    // the window's thalamic events of the column, drawn at once
-    const uint32_t thal = n.thal_per_col;
+    for (uint32_t i = threadIdx.x; i < in_n; i += kResBlock) s_in[i] = 0;
+    if (!kLists && threadIdx.x < kSlots) s_col[threadIdx.x] = (uint32_t)n.nbr[col * kSlotStride + threadIdx.x];
+    // the window's thalamic events of the column (of all columns), drawn at once
+    const uint32_t thal = kLists ? n.C * n.thal_per_col : n.thal_per_col;
+    auto target = [&](int t, uint32_t e) -> uint32_t {
+        if (!kLists) return draw_below(philox10(make_uint4((uint32_t)t, col, 1u, e), n.seed_lo, n.seed_hi).x, npc);
+        const uint32_t c = e / n.thal_per_col;
+        return c * n.npc +
+               draw_below(philox10(make_uint4((uint32_t)t, c, 1u, e - c * n.thal_per_col), n.seed_lo, n.seed_hi).x, n.npc);
+    };
     const bool drawn = (uint32_t)steps * thal <= kResThal;
     if (drawn)
         for (uint32_t e = threadIdx.x; e < (uint32_t)steps * thal; e += kResBlock) {
             const uint32_t k = e / thal;
-            const uint4 r = philox10(make_uint4((uint32_t)p0 + k, col, 1u, e - k * thal), n.seed_lo, n.seed_hi);
-            s_thal[e] = (uint16_t)draw_below(r.x, npc);
+            s_thal[e] = (std::conditional_t<kLists, uint32_t, uint16_t>)target(p0 + (int)k, e - k * thal);
         }
     if (threadIdx.x == 0) {
         s_stop = 0;
         s_fired[0] = s_fired[1] = 0;
     }
-    const int64_t cbase = (int64_t)col * npc * n.uniform_m;      // first synapse of the column (8-aligned)
+    const int64_t cbase = kLists ? 0 : (int64_t)col * npc * n.uniform_m;   // first synapse of the column (8-aligned)
     const uint16_t *const tg = n.tgt16 + cbase;
     const int32_t *const wt = n.w + cbase;
     const uint4 *const t4 = reinterpret_cast<const uint4 *>(tg);
-    const int64_t col_syn = (int64_t)npc * n.uniform_m;
+    const int64_t col_syn = kLists ? n.S : (int64_t)npc * n.uniform_m;
     const uint32_t row_chunks = n.uniform_m / 8u, m = n.canon_m, cpr = (m + 7u) / 8u;
-    const uint32_t e_hi = lo < n.ne ? min(hi, n.ne) - lo : 0u;   // own excitatory neurons: slice rows [0, e_hi)
+    // own excitatory neurons: slice rows [0, e_hi) (lists: rows of both kinds)
+    const uint32_t e_hi = kLists ? ns : lo < n.ne ? min(hi, n.ne) - lo : 0u;
+    auto excitatory = [&](uint32_t loc) { return kLists ? loc % n.npc < n.ne : loc < n.ne; };
+    const uint32_t dmask_i = (2u << n.D_inh) - 2u;
     // slots that lead back to the column (rings of a small torus)
     __syncthreads();
     uint32_t local = 0;
-    for (int q = 0; q < kSlots; ++q) local |= (s_col[q] == col ? 1u : 0u) << q;
+    for (int q = 0; q < kSlots && !kLists; ++q) local |= (s_col[q] == col ? 1u : 0u) << q;
     // lanes per bucket: the power of two that a mean bucket (M / D synapses)
     // fills best, 8 at least
-    const uint32_t mean = m / (uint32_t)D;
+    const uint32_t mean = kLists ? (uint32_t)(n.S / n.N) / (uint32_t)D : m / (uint32_t)D;
     const int lg = mean <= 6 ? 3 : mean <= 12 ? 4 : 5;
     const uint32_t gl = lane & ((1u << lg) - 1u), gi = lane >> lg, groups = 32u >> lg;
     // a net of one block has its whole input in shared memory, but for
@@ -191,10 +209,8 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         // thalamic drive of the own neurons, external events through the
         // step's input
         for (uint32_t e = threadIdx.x; e < thal; e += kResBlock) {
-            const uint32_t loc =
-                drawn ? s_thal[(uint32_t)k * thal + e]
-                      : draw_below(philox10(make_uint4((uint32_t)t, col, 1u, e), n.seed_lo, n.seed_hi).x, npc);
-            if (loc >= lo && loc < hi) atomicAdd(&s_in[loc], n.thal_amp);
+            const uint32_t loc = drawn ? s_thal[(uint32_t)k * thal + e] : target(t, e);
+            if (loc >= lo && loc < hi) atomicAdd(&s_in[loc - in_lo], n.thal_amp);
         }
         if (t >= n.stim_t0 && t < n.stim_t1) {
             const int64_t a = n.stim_off[t - n.stim_t0], b = n.stim_off[t - n.stim_t0 + 1];
@@ -207,7 +223,8 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         bool inh_left = true;
         for (uint32_t r0 = 0;;) {
             for (uint32_t i = r0 + threadIdx.x; i - lane < min(e_hi, r0 + range); i += kResBlock) {
-                uint32_t f = i < min(e_hi, r0 + range) ? (s_hist[i] << 1) & dmask : 0u;
+                uint32_t f = i < min(e_hi, r0 + range) ? s_hist[i] << 1 : 0u;
+                f &= !kLists || excitatory(lo + i) ? dmask : dmask_i;
                 if (!__any_sync(0xffffffffu, f != 0)) continue;
                 const uint32_t own = __popc(f);
                 uint32_t incl = own;
@@ -235,7 +252,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             const uint32_t share = (items + kWarps - 1) / kWarps;
             const uint32_t i_hi = min(items, (warp + 1) * share);
             uint32_t i_lo = warp * share;
-            int a = 0, b = 0;
+            int a = 0, b = 0, first = 0;
             uint32_t row = 0;
             auto fetch = [&]() {
                 a = b = 0;
@@ -245,10 +262,11 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
                     const uint16_t *off = n.doff + (size_t)(col * npc + row) * kDoffStride + (it & 31u);
                     a = off[-1];
                     b = off[0];
+                    if (kLists) first = (int)row_base(n, row);
                 }
             };
             fetch();
-            if (inh_left) {
+            if (!kLists && inh_left) {
                 // inhibitory rows that fired at t - 1: the whole row, one
                 // weight, targets of the own column; all threads share them
                 const uint32_t ninh = s_inh_n;
@@ -279,11 +297,12 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             while (i_lo < i_hi) {
                 const int tile = (int)min(32u, i_hi - i_lo);
                 const int events = __reduce_add_sync(0xffffffffu, b - a);
+                const int plastic = kLists ? __reduce_add_sync(0xffffffffu, b > a && excitatory(row) ? b - a : 0) : events;
                 if (lane == 0) {
                     ev_all += (unsigned long long)events;
-                    ev_exc += (unsigned long long)events;
+                    ev_exc += (unsigned long long)plastic;
                 }
-                const int base = (int)(row * n.uniform_m);
+                const int base = kLists ? first : (int)(row * n.uniform_m);
                 w_a[lane] = base + a;
                 w_b[lane] = base + b;
                 __syncwarp();
@@ -309,7 +328,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
                         for (int h = 0; h < kResFlight; ++h) {
                             v[h] = 0xffffffffu;
                             if (at[h] < end[h] && !out_of_range(n, at[h] >= 0 && at[h] < col_syn)) {
-                                v[h] = tg[at[h]];
+                                v[h] = kLists ? (uint32_t)n.tgt[at[h]] : tg[at[h]];
                                 w[h] = wt[at[h]];
                             }
                             at[h] += 1 << lg;
@@ -317,7 +336,12 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
                         }
 #pragma unroll
                         for (int h = 0; h < kResFlight; ++h) {
-                            if (v[h] == 0xffffffffu || out_of_range(n, v[h] < kSlots * npc)) continue;
+                            if (v[h] == 0xffffffffu || out_of_range(n, v[h] < (kLists ? n.N : kSlots * npc))) continue;
+                            if (kLists) {
+                                if (v[h] - lo < ns) atomicAdd(&s_in[v[h] - lo], w[h]);
+                                else red_add(&I[v[h]], w[h]);
+                                continue;
+                            }
                             const uint32_t slot = __umulhi(v[h], n.npc_recip), loc = v[h] - slot * npc;
                             if ((local >> slot) & 1u) atomicAdd(&s_in[loc], w[h]);
                             else red_add(&I[s_col[slot] * npc + loc], w[h]);
@@ -332,7 +356,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             if (threadIdx.x == 0) s_items_n = 0;
             __syncthreads();
         }
-        if (parts > 1) {                                 // the column's other slices
+        if (!kLists && parts > 1) {                      // the column's other slices
             for (uint32_t i = threadIdx.x; i < npc; i += kResBlock) {
                 if (i >= lo && i < hi) continue;
                 const int32_t x = s_in[i];
@@ -354,7 +378,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         }
         if (threadIdx.x == 0 && k > 0) {
             const unsigned long long c = __ldcg(&win->cnt[k - 1]);
-            s_stop = (c & 0xffffffffull) + (c >> 32) >= n.dense_min_spikes;
+            s_stop = !kLists && (c & 0xffffffffull) + (c >> 32) >= n.dense_min_spikes;
         }
         // ---- S2, S3 of the own neurons: threads on word boundaries of the
         // spike bits, the words at the slice's ends shared with its neighbours
@@ -366,14 +390,14 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             bool fired = false;
             if (own) {
                 const uint32_t loc = lo + q;
-                int32_t iq = s_in[loc];
-                s_in[loc] = 0;
+                int32_t iq = s_in[loc - in_lo];
+                s_in[loc - in_lo] = 0;
                 if (input || k == 0) {
                     iq += __ldcg(&I[g0 + q]);
                     I[g0 + q] = 0;
                 }
                 F v = s_v[q], u = s_u[q];
-                fired = izhikevich_step(v, u, iq, loc < n.ne);
+                fired = izhikevich_step(v, u, iq, excitatory(loc));
                 s_v[q] = v;
                 s_u[q] = u;
                 const uint32_t h = s_hist[q];
@@ -385,7 +409,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
                 }
             }
             const uint32_t word = __ballot_sync(0xffffffffu, fired);
-            const uint32_t exc = __ballot_sync(0xffffffffu, fired && lo + q < n.ne);
+            const uint32_t exc = __ballot_sync(0xffffffffu, fired && excitatory(lo + q));
             const uint32_t owned = __ballot_sync(0xffffffffu, own);
             if (lane == 0 && owned) {
                 uint32_t *p = bits + ((g0 + q) >> 5);
@@ -423,12 +447,23 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
 
 __global__ void __launch_bounds__(kResBlock, 2) k_resident_f32(DevNet n, int t0, int steps)
 {
-    resident_body<float>(n, t0, steps);
+    resident_body<float, false>(n, t0, steps);
 }
 
 __global__ void __launch_bounds__(kResBlock, 2) k_resident_f64(DevNet n, int t0, int steps)
 {
-    resident_body<double>(n, t0, steps);
+    resident_body<double, false>(n, t0, steps);
+}
+
+// nets with target lists (explicit ones, columns above 4096 neurons)
+__global__ void __launch_bounds__(kResBlock, 2) k_resident_lists_f32(DevNet n, int t0, int steps)
+{
+    resident_body<float, true>(n, t0, steps);
+}
+
+__global__ void __launch_bounds__(kResBlock, 2) k_resident_lists_f64(DevNet n, int t0, int steps)
+{
+    resident_body<double, true>(n, t0, steps);
 }
 
 // spikes of word w of a step's bits by kind: exc | inh << 16

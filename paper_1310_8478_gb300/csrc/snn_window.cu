@@ -252,6 +252,123 @@ __device__ __forceinline__ void stdp_row(const DevNet &n, int64_t base, int m, i
     }
 }
 
+// What a warp keeps of row p for its synapses: bucket ends, arrival trains by
+// delay, the source's spike times and, for few of those, the potentiation
+// amounts; m its synapses, ns its spikes.  False in every lane: the source has
+// no arrival inside any amount's reach.
+__device__ __forceinline__ bool row_spikes(const DevNet &n, uint32_t p, unsigned long long own, int p0, int lane,
+                                           int32_t *w_off, unsigned long long *w_x, signed char *w_j, int32_t *w_q,
+                                           const int32_t *s_lutp, int &m, int &ns)
+{
+    const int D = (int)n.D;
+    const uint2 h = n.hl0[p];
+                const int end = lane <= D ? (int)n.doff[(size_t)p * kDoffStride + lane] : 0;
+                m = __shfl_sync(0xffffffffu, end, D);
+                unsigned long long x = 0;
+                if (lane >= 1 && lane <= D) {
+                    // arrivals by delay `lane`: source spikes of the window, and
+                    // before it (bit j of h.x: fired at p0 - 1 - j)
+                    const uint32_t recent = h.x & (0xffffffffu << lane);
+                    const int lag = recent ? __ffs(recent) - lane : p0 - (int)h.y - lane;
+                    x = ((own << lane) | (unsigned long long)(__brev(h.x) >> (32 - lane))) & kTrainMask;
+                    x |= (unsigned long long)min(lag, kLut - 1) << kWinBits;
+                }
+                w_x[lane] = x;
+                w_off[lane] = end;
+                // the source's spikes that arrive in the window, in order: the
+                // last D steps before it and the window's own
+                const uint32_t pre = h.x & (0xffffffffu >> (32 - D));
+                const int npre = __popc(pre);
+    ns = npre + __popcll(own);
+                if ((pre >> lane) & 1u) w_j[npre - __popc(pre & (0xffffffffu >> (31 - lane)))] = (signed char)(-1 - lane);
+    #pragma unroll
+                for (int q = lane; q < 64; q += 32)
+                    if ((own >> q) & 1ull) w_j[npre + __popcll(own & ((1ull << q) - 1ull))] = (signed char)q;
+                // what a post spike `tau` after a spike's own step, less the delay,
+                // adds: the amount at the lag to the source's latest spike
+                if (ns <= kFewSpikes) {
+    #pragma unroll
+                    for (int q = lane; q < kAmounts; q += 32) {
+                        const int tau = q - 31;
+                        int lag;
+                        if (tau >= 0) {
+                            const unsigned long long late = own & (tau < 63 ? (2ull << tau) - 1ull : ~0ull);
+                            lag = late ? tau - 63 + __clzll((long long)late) : tau + (h.x ? __ffs(h.x) : p0 - (int)h.y);
+                        } else {
+                            const uint32_t late = h.x & (0xffffffffu << (-1 - tau));
+                            lag = tau + (late ? __ffs(late) : p0 - (int)h.y);
+                        }
+                        w_q[q] = lag < kLut ? s_lutp[lag] : 0;
+                    }
+                }
+                // a source without an arrival inside any amount's reach changes nothing
+                return (x & kTrainMask) || (lane >= 1 && lane <= D && (int)(x >> kWinBits) < kLut - 1);
+}
+
+// One row of a net with target lists (explicit targets: no alignment, no
+// slots): a lane per synapse, its target's train from memory.  The net's
+// trains are a few KB to a few MB and stay in L2.
+template <bool kDeriv>
+__device__ __forceinline__ void stdp_row_lists(const DevNet &n, int64_t base, int m, int D, const int32_t *w_off,
+                                               const unsigned long long *w_x, const signed char *w_j, int ns,
+                                               const int32_t *w_q, const int32_t *s_lutp, const int32_t *s_lutm,
+                                               int steps, unsigned long long posts, unsigned long long arrivals, int lane)
+{
+    const float scale = (float)D / (float)m;
+    const int a_min = arrivals ? __ffsll((long long)arrivals) - 1 : steps;
+    for (int k = lane; k < m; k += 32) {
+        if (out_of_range(n, base + k < n.S)) continue;
+        const uint32_t v = (uint32_t)n.tgt[base + k];
+        const int32_t sd = n.sd[base + k];
+        const int32_t w = kDeriv ? n.w[base + k] : 0;
+        if (out_of_range(n, v < n.N)) continue;
+        const unsigned long long y = n.train[v];
+        int b = min(D, 1 + (int)((float)k * scale));
+        while (w_off[b] <= k) ++b;        // bucket D ends at m > k
+        while (w_off[b - 1] > k) --b;     // w_off[0] = 0 <= k
+        int32_t delta = 0;
+        if (ns <= kFewSpikes) {           // as stdp_row: one table of the row's potentiation
+            const int32_t *q = w_q + 31 - b;
+            for (unsigned long long f = y & posts; f; f &= f - 1ull) delta += q[__ffsll((long long)f) - 1];
+            const int before = (int)(y >> kWinBits);
+            for (int i = 0; i < ns; ++i) {
+                const int a = (int)w_j[i] + b;
+                if (a < a_min || a >= steps) continue;
+                const unsigned long long z = y & ((1ull << a) - 1ull);      // post spikes before a (< kWinBits)
+                const int lag = z ? a - 63 + __clzll((long long)z) : a + before;
+                delta -= s_lutm[min(lag, kLut - 1)];
+            }
+        } else {
+            delta = window_delta(w_x[b], y, posts, arrivals, s_lutp, s_lutm);
+        }
+        if (kDeriv) {
+            n.w[base + k] = deriv_w(n, w, sd + delta);
+            n.sd[base + k] = deriv_sd(n, sd + delta);
+        } else if (delta) {
+            n.sd[base + k] = sd + delta;
+        }
+    }
+}
+
+// the last block of the pass closes the window: nothing is owed
+__device__ __forceinline__ void close_pass(const DevNet &n, uint32_t blocks)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        DevWindow *win = n.win;
+        if (atomicAdd(&win->done, 1u) == blocks - 1) {
+            // every block has read the window
+            win->p1 = win->p0 - 1;
+            win->defer_from = kNoDefer;
+            win->cursor = 0;
+            win->done = 0;
+            n.ctr->ltp_pending = kNoPending;
+            n.ctr->fold_cursor = 0;
+        }
+    }
+}
+
 __device__ __forceinline__ void stdp_body(const DevNet &n, const Part &g)
 {
     extern __shared__ int4 smem_i4[];
@@ -304,47 +421,8 @@ __device__ __forceinline__ void stdp_body(const DevNet &n, const Part &g)
         for (uint32_t r = r0 + warp; r < r1; r += nwarps) {
             const uint32_t p = col * npc + r;
             const unsigned long long own = s_y[r] & kTrainMask;          // slot 0 is the row's own column
-            const uint2 h = n.hl0[p];
-            const int end = lane <= D ? (int)n.doff[(size_t)p * kDoffStride + lane] : 0;
-            const int m = __shfl_sync(0xffffffffu, end, D);
-            unsigned long long x = 0;
-            if (lane >= 1 && lane <= D) {
-                // arrivals by delay `lane`: source spikes of the window, and
-                // before it (bit j of h.x: fired at p0 - 1 - j)
-                const uint32_t recent = h.x & (0xffffffffu << lane);
-                const int lag = recent ? __ffs(recent) - lane : p0 - (int)h.y - lane;
-                x = ((own << lane) | (unsigned long long)(__brev(h.x) >> (32 - lane))) & kTrainMask;
-                x |= (unsigned long long)min(lag, kLut - 1) << kWinBits;
-            }
-            w_x[lane] = x;
-            w_off[lane] = end;
-            // the source's spikes that arrive in the window, in order: the
-            // last D steps before it and the window's own
-            const uint32_t pre = h.x & (0xffffffffu >> (32 - D));
-            const int npre = __popc(pre), ns = npre + __popcll(own);
-            if ((pre >> lane) & 1u) w_j[npre - __popc(pre & (0xffffffffu >> (31 - lane)))] = (signed char)(-1 - lane);
-#pragma unroll
-            for (int q = lane; q < 64; q += 32)
-                if ((own >> q) & 1ull) w_j[npre + __popcll(own & ((1ull << q) - 1ull))] = (signed char)q;
-            // what a post spike `tau` after a spike's own step, less the delay,
-            // adds: the amount at the lag to the source's latest spike
-            if (ns <= kFewSpikes) {
-#pragma unroll
-                for (int q = lane; q < kAmounts; q += 32) {
-                    const int tau = q - 31;
-                    int lag;
-                    if (tau >= 0) {
-                        const unsigned long long late = own & (tau < 63 ? (2ull << tau) - 1ull : ~0ull);
-                        lag = late ? tau - 63 + __clzll((long long)late) : tau + (h.x ? __ffs(h.x) : p0 - (int)h.y);
-                    } else {
-                        const uint32_t late = h.x & (0xffffffffu << (-1 - tau));
-                        lag = tau + (late ? __ffs(late) : p0 - (int)h.y);
-                    }
-                    w_q[q] = lag < kLut ? s_lutp[lag] : 0;
-                }
-            }
-            // a source without an arrival inside any amount's reach changes nothing
-            const bool live = (x & kTrainMask) || (lane >= 1 && lane <= D && (int)(x >> kWinBits) < kLut - 1);
+            int m, ns;
+            const bool live = row_spikes(n, p, own, p0, lane, w_off, w_x, w_j, w_q, s_lutp, m, ns);
             __syncwarp();
             if (closes || __any_sync(0xffffffffu, live)) {
                 const int64_t base = row_base(n, p);
@@ -367,18 +445,48 @@ __device__ __forceinline__ void stdp_body(const DevNet &n, const Part &g)
         unit = s_unit;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&win->done, 1u) == g.nblk - 1) {
-            // every block has read the window: it closes, nothing is owed
-            win->p1 = win->p0 - 1;
-            win->defer_from = kNoDefer;
-            win->cursor = 0;
-            win->done = 0;
-            n.ctr->ltp_pending = kNoPending;
-            n.ctr->fold_cursor = 0;
-        }
+    close_pass(n, g.nblk);
+}
+
+__device__ __forceinline__ void stdp_lists_body(const DevNet &n)
+{
+    extern __shared__ int4 smem_i4[];
+    if (!n.win) return;
+    DevWindow *win = n.win;
+    const int t = win->p1 + 1;             // the step after the window
+    if (win->defer_from > win->p1) return; // (a resident grid defers all steps of a window or ran none)
+    const int nwarps = (int)(blockDim.x >> 5), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long *w_x = reinterpret_cast<unsigned long long *>(smem_i4) + warp * 32;
+    int32_t *s_off = reinterpret_cast<int32_t *>(smem_i4) + nwarps * 64;            // behind [nwarps][32] 8-byte trains
+    int32_t *w_off = s_off + warp * 32;
+    int32_t *w_q = s_off + nwarps * 32 + warp * kAmounts;
+    int32_t *s_lutp = s_off + nwarps * (32 + kAmounts), *s_lutm = s_lutp + kLut;
+    signed char *w_j = reinterpret_cast<signed char *>(s_lutm + kLut) + warp * kSpikeCap;
+    const int p0 = win->p0, from = win->defer_from;
+    const unsigned long long arrivals = ((1ull << (t - p0)) - 1ull) & ~((1ull << (from - p0)) - 1ull);
+    const unsigned long long posts = kTrainMask & ~((1ull << max(0, from - 1 - p0)) - 1ull);
+    const bool closes = n.deriv_period && (t % (int)n.deriv_period) == 0;
+    for (int i = threadIdx.x; i < kLut; i += blockDim.x) {
+        s_lutp[i] = n.lut_p[i];
+        s_lutm[i] = n.lut_m[i];
     }
+    __syncthreads();
+    for (uint32_t r = blockIdx.x * nwarps + warp; r < n.C * n.ne; r += gridDim.x * nwarps) {
+        const uint32_t col = r / n.ne, p = col * n.npc + (r - col * n.ne);
+        int m, ns;
+        const bool live = row_spikes(n, p, n.train[p] & kTrainMask, p0, lane, w_off, w_x, w_j, w_q, s_lutp, m, ns);
+        __syncwarp();
+        if (closes || __any_sync(0xffffffffu, live)) {
+            auto row = [&](auto deriv) {
+                stdp_row_lists<decltype(deriv)::value>(n, row_base(n, p), m, (int)n.D, w_off, w_x, w_j, ns, w_q, s_lutp,
+                                                       s_lutm, t - p0, posts, arrivals, lane);
+            };
+            if (closes) row(std::true_type{});
+            else row(std::false_type{});
+        }
+        __syncwarp();
+    }
+    close_pass(n, gridDim.x);
 }
 
 __global__ void __launch_bounds__(1024) k_win_open(DevNet n, const int *t_now, int steps)
@@ -389,6 +497,8 @@ __global__ void __launch_bounds__(1024) k_win_open(DevNet n, const int *t_now, i
 __global__ void __launch_bounds__(256) k_train(DevNet n) { train_body(n, whole_grid()); }
 
 __global__ void __launch_bounds__(kStdpBlock) k_stdp(DevNet n) { stdp_body(n, whole_grid()); }
+
+__global__ void __launch_bounds__(kStdpListsBlock) k_stdp_lists(DevNet n) { stdp_lists_body(n); }
 
 __global__ void __launch_bounds__(1024) k_win_open_b(BatchLaunch b, int steps)
 {

@@ -192,3 +192,80 @@ def test_closed_loop_of_single_steps_equals_the_oracle(eng, orc, lists):
             quiet += got == 0
         assert_same_run(o, n)
         assert total == o.counters()["spikes"] and quiet > 10 and total > 10
+
+
+def _explicit(rng, cfg, rows_lo, rows_hi, w_exc):
+    """Random rows of both kinds with individual delays and weights; some rows
+    empty, some targets repeated or the source itself."""
+    n, npc = cfg["grid_x"] * cfg["grid_y"] * cfg["neurons_per_col"], cfg["neurons_per_col"]
+    rows = rng.integers(rows_lo, rows_hi, n)
+    rows[rng.random(n) < 0.1] = 0
+    off = np.concatenate([[0], np.cumsum(rows)])
+    src = np.repeat(np.arange(n), rows)
+    exc = src % npc < cfg["exc_per_col"]
+    tgt = rng.integers(0, n, off[-1])
+    tgt[rng.integers(0, off[-1], min(200, off[-1] // 50))] = 0     # (a Q16 input holds some 500 at wmax)
+    tgt = np.where(rng.random(off[-1]) < 0.02, src, tgt)
+    D = cfg["max_delay_ms"]
+    return dict(row_off=off, tgt=tgt, delay=np.where(exc, rng.integers(1, D + 1, off[-1]), rng.integers(1, 4, off[-1])),
+                w=np.where(exc, (w_exc * 65536 * (0.5 + rng.random(off[-1]))).astype(np.int64), -rng.integers(2, 6, off[-1]) * 65536))
+
+
+LISTS = {
+    # one block: no grid barrier; two, the second with a single neuron
+    "one_block": (_cfg(1, 1, 31, 0, seed=81, thal_per_col_per_ms=1, deriv_period_ms=70), (5, 25), 8, [4, 50, 51, 3, 90]),
+    "two_blocks": (_cfg(1, 1, 33, 0, seed=82, thal_per_col_per_ms=1, deriv_period_ms=60), (5, 25), 8, [64, 99]),
+    # columns of odd size, slices across columns, the longest delay
+    "ragged": (_cfg(3, 2, 111, 0, seed=83, thal_per_col_per_ms=1, deriv_period_ms=70, max_delay_ms=31), (10, 50), 6, [53, 120]),
+    # runs away: trains with many spikes, drive events that are not drawn ahead
+    "runaway": (_cfg(5, 4, 800, 0, seed=84, thal_per_col_per_ms=30, deriv_period_ms=40), (30, 70), 9, [30, 45]),
+    # forced spikes in every neuron: more pending rows than a block lists at once
+    "all_fire": (_cfg(2, 1, 45000, 0, seed=86, max_delay_ms=31), (2, 8), 3, [60]),
+}
+
+
+@pytest.mark.parametrize("fp64", [False, True], ids=["fp32", "fp64"])
+@pytest.mark.parametrize("name", sorted(LISTS))
+def test_resident_grids_of_target_lists_equal_the_oracle(eng, orc, name, fp64):
+    cfg, rows, w_exc, calls = LISTS[name]
+    cfg = dict(cfg, fanout=1)
+    rng = np.random.default_rng(cfg["seed"])
+    ex = _explicit(rng, cfg, *rows, w_exc)
+    N, T = len(ex["row_off"]) - 1, sum(calls)
+    t, g, q = np.sort(rng.integers(0, T, 200)), rng.integers(0, N, 200), np.full(200, 30 * 65536)
+    if name == "all_fire":
+        t, g, q = np.repeat(np.arange(4, 44, 4), N), np.tile(np.arange(N), 10), np.full(10 * N, 250 * 65536)
+    if fp64:
+        cfg["flags"] = eng.snn.FP64
+    o = orc.Oracle(cfg, explicit=ex, **(dict(flags=4) if fp64 else {}))
+    o.set_stimulus(t, g, q)
+    with gpu_net(eng, cfg, explicit=ex) as n:
+        n.set_stimulus(t, g, q)
+        for k, steps in enumerate(calls):
+            o.run(steps)
+            n.run(steps)
+            if k == 0:
+                n.step()
+                o.run(1)
+        for a, b in zip(n.raster(), o.raster()):
+            assert np.array_equal(a, b)
+        s, x = o.synapses(), n.neurons_f64() if fp64 else n.neurons()
+        w, sd = n.weights()
+        assert np.array_equal(w, s["w"]) and np.array_equal(sd, s["sd"]) and np.count_nonzero(sd) > 10
+        v = "vd" if fp64 else "v"
+        assert np.array_equal(o.neurons()[v], x["v"])
+        for key in ("spikes", "e_all", "e_exc", "l_exc"):
+            assert n.counters()[key] == o.counters()[key], key
+        assert n.counters()["spikes"] > 100
+
+
+def test_resident_grid_of_a_big_column_equals_the_oracle(eng, orc):
+    """Columns above 4096 neurons are generated with target lists."""
+    cfg = _cfg(2, 1, 4200, 24, seed=85, thal_per_col_per_ms=20, thal_amp_q16=30 * 65536, deriv_period_ms=50, w_exc0_q16=8 * 65536)
+    o = orc.Oracle(cfg)
+    with gpu_net(eng, cfg) as n:
+        for steps in (70, 33):
+            o.run(steps)
+            n.run(steps)
+            assert_same_run(o, n)
+        assert n.counters()["spikes"] > 100
