@@ -167,6 +167,7 @@ struct snn_net {
     int merged_grid = 0;            // blocks of the delivery and dense pass in one launch; 0: two launches
     int light_grid = 0;             // blocks of a dense step that defers its STDP (likewise)
     bool step_windows = false;      // the step kernels' steps take windows
+    uint32_t stdp_block = 0;        // threads per block of the windows' pass
     int res_grid = 0;               // blocks of the resident grid that runs this net's windows; 0: none does
     uint64_t version = 0;           // bumped whenever captured launches go stale
     // stimulus
@@ -700,9 +701,12 @@ int setup_windows(snn_net *net)
     net->stdp_grid = 0;
     net->res_grid = 0;
     net->step_windows = false;
-    const size_t bytes = stdp_smem_bytes(dn.npc, kStdpBlock);
     int optin = 0, parts = 1;
     SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
+    // 32 warps, fewer where their tables do not fit beside the trains
+    net->stdp_block = kStdpBlock;
+    while (net->stdp_block > 256 && stdp_smem_bytes(dn.npc, net->stdp_block) + 1024 > (size_t)optin) net->stdp_block /= 2;
+    const size_t bytes = stdp_smem_bytes(dn.npc, net->stdp_block);
     const bool lists = !net->tgt16;
     const bool can = !dn.tile && !(net->cfg.flags & (SNN_STDP_OFF | SNN_DELIVERY_OFF)) &&
                      (lists || bytes + 1024 <= (size_t)optin);
@@ -741,7 +745,7 @@ int setup_windows(snn_net *net)
     }
     SNN_CUDA(allow_smem((const void *)k_stdp, bytes));
     int per_sm = 0;
-    SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stdp, (int)kStdpBlock, bytes));
+    SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stdp, (int)net->stdp_block, bytes));
     if (per_sm < 1) {
         drop_windows(net);
         return SNN_OK;
@@ -1103,7 +1107,7 @@ void launch_stdp(snn_net *net, bool trains)
         return;
     }
     if (!trains) k_train<<<sized_grid(net, 8, dn.spk_words, 64), 256, 0, net->stream>>>(dn);
-    k_stdp<<<net->stdp_grid, kStdpBlock, stdp_smem_bytes(dn.npc, kStdpBlock), net->stream>>>(dn);
+    k_stdp<<<net->stdp_grid, net->stdp_block, stdp_smem_bytes(dn.npc, net->stdp_block), net->stream>>>(dn);
 }
 
 // after the window's last step; the kernels return at once when no step left
@@ -2016,11 +2020,14 @@ int batch_tables(snn_batch *b)
     // plasticity windows
     size_t smem_w = 0;
     size_t smem_l = 0;
+    uint32_t block_w = kStdpBlock;             // one that fits every net
+    for (const snn_net *n : b->nets)
+        if (n->step_windows) block_w = std::min(block_w, n->stdp_block);
     for (int k : {kBWinOpen, kBTrain, kBStdp, kBDenseLight}) cnt[k].assign(nn, 0);
     for (size_t i = 0; i < nn; ++i) {
         const snn_net *n = b->nets[i];
         if (!n->step_windows) continue;
-        smem_w = std::max(smem_w, stdp_smem_bytes(n->dn.npc, kStdpBlock));
+        smem_w = std::max(smem_w, stdp_smem_bytes(n->dn.npc, block_w));
         cnt[kBWinOpen][i] = (uint32_t)sized_grid(n, 8, n->N, 1024);
         cnt[kBTrain][i] = (uint32_t)sized_grid(n, 8, n->dn.spk_words, 64);
         cnt[kBStdp][i] = (uint32_t)n->stdp_grid;
@@ -2032,7 +2039,7 @@ int batch_tables(snn_batch *b)
     b->kind[kBDenseLight].smem = smem_l;
     if (smem_l) SNN_CUDA(allow_smem((const void *)k_dense_light_b, smem_l));
     b->kind[kBWinOpen].block = b->kind[kBTrain].block = 256;
-    b->kind[kBStdp].block = kStdpBlock;
+    b->kind[kBStdp].block = block_w;
     b->kind[kBStdp].smem = smem_w;
     if (smem_w) SNN_CUDA(allow_smem((const void *)k_stdp_b, smem_w));
     // one device buffer: DevNet[nn], parity[nn], then per kind first[nn],

@@ -828,7 +828,7 @@ constexpr uint32_t kDenseLightBlock = 1024;  // threads per block of a dense ste
 constexpr uint32_t kResBlock = 512;         // threads per block of a resident grid
 constexpr uint32_t kEmitBlock = 512;
 constexpr uint32_t kEmitWords = 2048;       // words of a step's spike bits per block
-constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's pass
+constexpr uint32_t kStdpBlock = 1024;       // threads per block of the window's pass, at most
 constexpr uint32_t kStdpListsBlock = 256;   // ... of nets with target lists
 // k_fold: as the step that closes a period runs it / always / before a
 // window's pass that closes a period

@@ -37,6 +37,8 @@ CASES = {
     "strong_drive": (_cfg(2, 1, 200, 20, seed=66, thal_per_col_per_ms=40, thal_amp_q16=4 * 65536), [53, 60]),
     # runs away: the resident grid stops, the step kernels go on and defer
     "runaway": (_cfg(2, 2, 400, 400, seed=67, w_exc0_q16=8 * 65536, thal_per_col_per_ms=2, deriv_period_ms=90), [40, 120, 70]),
+    # columns whose trains leave room for fewer warps' tables
+    "wide_columns": (_cfg(2, 1, 1801, 30, seed=74, thal_per_col_per_ms=9, deriv_period_ms=50), [60, 49]),
     # other STDP tables, the depression too wide for 15 bits
     "wide_depression": (_cfg(2, 2, 100, 50, seed=68, a_minus_mv=1.0, tau_plus_ms=12.0, thal_per_col_per_ms=2), [75, 75]),
 }
