@@ -360,7 +360,9 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
 // (its bulk prefetches would cost a third of the instructions here).  The
 // delay buckets are looked up once per 1024 synapses, each lane the flags of
 // 32 positions, and not at all when the source fired in each of the last D
-// steps; inside a chunk that has a due position the others add 0: a condition
+// steps; where some are due, the chunks of 8 that hold one are listed, so that
+// all lanes have one (a third of the synapses due 0.68 ms, 0.75 with the lanes
+// of the others idle; half 0.88 and 0.91).  Inside a chunk that has a due position the others add 0: a condition
 // around each addition costs a branch and a reconvergence, several times the
 // addition.  1.28 M neurons of 1125 synapses: 1.2 ms a step, 0.95 of the copy
 // bandwidth (1.5 ms inside the fused pass's kernel with 32 warps, 2.9 ms with
@@ -369,47 +371,71 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
 size_t dense_light_smem_bytes(uint32_t npc)
 {
     return (size_t)kSlots * npc * 4            // staged input
-           + (kDenseLightBlock / 32) * 32 * 4; // per-warp bucket offsets
+           + (kDenseLightBlock / 32) * 32 * 4  // per-warp bucket offsets
+           + (kDenseLightBlock / 32) * 128 * 2; // per-warp chunks that are due
 }
 
-__device__ __forceinline__ void light_row(const DevNet &n, int64_t base, bool exc, uint32_t fbits, uint32_t due,
-                                          const int32_t *w_off, uint32_t in0, int lane)
+// 8 synapses of a row into the staged input; those outside fmask add 0
+__device__ __forceinline__ void light_chunk(const DevNet &n, const uint4 *t4, const int4 *w4, bool exc, uint32_t fmask,
+                                            uint32_t in0)
 {
-    const int D = (int)n.D, m = (int)n.canon_m;
+    if (out_of_range(n, (const uint16_t *)(t4 + 1) <= n.tgt16 + n.S)) return;
+    const uint4 tv = *t4;
+    int4 wa, wb;
+    if (exc) {
+        wa = w4[0];
+        wb = w4[1];
+    } else {
+        wa = wb = make_int4(n.w_inh, n.w_inh, n.w_inh, n.w_inh);
+    }
+    const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
+    const int32_t wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const uint32_t v = (u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu);
+        if (out_of_range(n, v < kSlots * n.npc)) continue;
+        red_shared(in0 + 4u * v, (fmask >> u) & 1u ? wv[u] : 0);
+    }
+}
+
+// a row whose buckets are all due
+__device__ __forceinline__ void light_row(const DevNet &n, int64_t base, bool exc, uint32_t in0, int lane)
+{
+    const int m = (int)n.canon_m;
     const uint4 *t4 = reinterpret_cast<const uint4 *>(n.tgt16 + base) + lane;
     const int4 *w4 = reinterpret_cast<const int4 *>(n.w + base) + 2 * lane;
-    const bool full = fbits == due;                // the whole row is due
+    for (int left = m - 8 * lane; left > 0; left -= 256, t4 += 32, w4 += 64)
+        light_chunk(n, t4, w4, exc, left >= 8 ? 0xffu : (1u << left) - 1u, in0);
+}
+
+// A row with some buckets due: its chunks of 8 synapses that hold a due one
+// are listed first, so that every lane has one (a due bucket of 56 synapses is
+// 7 of a row's 141 chunks).
+__device__ __forceinline__ void light_row_part(const DevNet &n, int64_t base, bool exc, uint32_t fbits,
+                                               const int32_t *w_off, uint16_t *w_list, uint32_t in0, int lane)
+{
+    const int D = (int)n.D, m = (int)n.canon_m;
     const float scale = (float)D / (float)m;
-    uint32_t flags = 0;
-    for (int s = 0; 256 * s < m; ++s, t4 += 32, w4 += 64) {
-        const int left = m - 256 * s - 8 * lane;   // positions from the lane's chunk to the row's end
-        uint32_t fmask = left >= 8 ? 0xffu : left > 0 ? (1u << left) - 1u : 0u;
-        if (!full) {
-            if (!(s & 3)) {
-                const int q0 = 256 * s + 32 * lane;
-                flags = q0 < m ? word_flags(q0, m, D, scale, fbits, w_off) : 0u;
-            }
-            const uint32_t word = __shfl_sync(0xffffffffu, flags, 8 * (s & 3) + (lane >> 2));
-            fmask &= word >> (8 * (lane & 3));
-        }
-        if (!fmask || out_of_range(n, (const uint16_t *)(t4 + 1) <= n.tgt16 + n.S)) continue;
-        const uint4 tv = *t4;
-        int4 wa, wb;
-        if (exc) {
-            wa = w4[0];
-            wb = w4[1];
-        } else {
-            wa = wb = make_int4(n.w_inh, n.w_inh, n.w_inh, n.w_inh);
-        }
-        const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
-        const int32_t wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-        const bool all = full && 256 * (s + 1) <= m;   // warp-uniform
+    for (int s = 0; s < m; s += 1024) {
+        const int q0 = s + 32 * lane;
+        const uint32_t flags = q0 < m ? word_flags(q0, m, D, scale, fbits, w_off) : 0u;
+        const uint32_t any = ((flags & 0xffu) ? 1u : 0u) | ((flags & 0xff00u) ? 2u : 0u) | ((flags & 0xff0000u) ? 4u : 0u) |
+                             (flags >> 24 ? 8u : 0u);
+        const uint32_t own = __popc(any);
+        const uint32_t b0 = __ballot_sync(0xffffffffu, own & 1u), b1 = __ballot_sync(0xffffffffu, own & 2u),
+                       b2 = __ballot_sync(0xffffffffu, own & 4u), lt = lanemask_lt();
+        uint32_t at = __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const uint32_t v = (u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu);
-            if (out_of_range(n, v < kSlots * n.npc)) continue;
-            red_shared(in0 + 4u * v, all || ((fmask >> u) & 1u) ? wv[u] : 0);
+        for (int j = 0; j < 4; ++j)
+            if ((any >> j) & 1u) w_list[at++] = (uint16_t)((4 * lane + j) << 8 | ((flags >> (8 * j)) & 0xffu));
+        __syncwarp();
+        const uint32_t count = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+        for (uint32_t i = lane; i < count; i += 32) {
+            const uint32_t it = w_list[i], c = (uint32_t)s / 8u + (it >> 8);
+            light_chunk(n, reinterpret_cast<const uint4 *>(n.tgt16 + base) + c, reinterpret_cast<const int4 *>(n.w + base) + 2 * c,
+                        exc, it & 0xffu, in0);
         }
+        __syncwarp();
     }
 }
 
@@ -424,6 +450,7 @@ __device__ __forceinline__ void dense_light_body(const DevNet &n, const int *t_n
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, D = (int)n.D;
     int32_t *s_in = reinterpret_cast<int32_t *>(smem_i4);       // [kSlots * npc]
     int32_t *w_off = s_in + kSlots * npc + warp * 32;           // bucket end offsets
+    uint16_t *w_list = reinterpret_cast<uint16_t *>(s_in + kSlots * npc + nwarps * 32) + warp * 128;
     const uint32_t in0 = (uint32_t)__cvta_generic_to_shared(s_in);
     const uint32_t chunks = (npc + n.dense_rows - 1) / n.dense_rows;
     const uint32_t dmask = (2u << D) - 2u;
@@ -455,7 +482,8 @@ __device__ __forceinline__ void dense_light_body(const DevNet &n, const int *t_n
                 ev_all += (unsigned long long)events;
                 if (exc) ev_exc += (unsigned long long)events;
             }
-            light_row(n, row_base(n, p), exc, fbits, due, w_off, in0, lane);
+            if (fbits == due) light_row(n, row_base(n, p), exc, in0, lane);
+            else light_row_part(n, row_base(n, p), exc, fbits, w_off, w_list, in0, lane);
         }
         __syncthreads();
         for (int sl = 0; sl < kSlots; ++sl) {
