@@ -759,7 +759,7 @@ int setup_windows(snn_net *net)
     const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
     net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
     net->step_windows = net->n_rin >= kWinMinSynapses;
-    if (net->step_windows) {
+    if (net->step_windows && net->dense_ok) {
         const size_t light = dense_light_smem_bytes(dn.npc);
         SNN_CUDA(allow_smem((const void *)k_dense_light, light));
         SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dense_light, (int)kDenseLightBlock, light));

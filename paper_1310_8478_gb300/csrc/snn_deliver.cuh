@@ -17,9 +17,10 @@ namespace snn {
 // shared memory while this one is walked.  Bound by latency and instruction
 // issue (half of it) at 64 registers and two blocks of 512 threads per SM; with
 // three at 40 registers it spilled (busy 32x32 net: 142 against 129 us per
-// step), and five of 256 threads left a wave of 1024 columns two thirds full
-// (with depression, per step: busy 32x32 net 119 -> 90 us, onset of the 64x32
-// benchmark torus 83 -> 68, 64x64 torus of the paper's columns 91 -> 88).
+// step), and five of 256 threads left a wave of 1024 columns two thirds full.
+// Tried for steps without depression: all 13 columns' input in shared memory
+// in the deferred dense step's kernel, which needs no distinction of targets
+// but flushes 13 columns (70 us at any rate on the 32x32 net).
 template <bool kStdp>
 __device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Part &g)
 {
@@ -38,6 +39,12 @@ __device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Pa
     const uint32_t dmask = (2u << n.D) - 2u;
     const int64_t col_syn = (int64_t)npc * n.uniform_m;
     const int lg = bucket_lanes(n);
+    // buckets of more than 12 synapses, without depression of more than 6, go
+    // chunk by chunk: 32x32 net with buckets of 15, a tenth of the synapses due,
+    // 185 -> 88 us, with depression 169 -> 160; 64x32 with 56, with depression,
+    // onset 6.6 -> 6.4 ms; 64x64 with 10 100 -> 93 us, with depression 1 to 4 %
+    // slower
+    const bool chunked = !n.tile && lg >= (kStdp ? 5 : 4);
     if (kStdp)
         for (int i = threadIdx.x; i < kLut; i += blockDim.x) s_lut[i] = n.lut_m[i];
     drive(n, t, part_tid(g), part_threads(g));
@@ -91,32 +98,68 @@ __device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Pa
                 continue;
             }
             unsigned seen = 0;                                            // a tile's events on its own columns
-            const unsigned walked = walk_items(
-                blockDim.x, n, col, s_items, items, w_ab, lg, tg, n.w + cbase, col_syn,
-                [&] {
-                    if (begun) return;
-                    walk_inhibitory(blockDim.x, n, s_inh, s_inh_n, tg, col_syn, (uint32_t)__cvta_generic_to_shared(s_in));
-                    if (threadIdx.x == 0) ev_all += (unsigned long long)s_inh_n * n.canon_m;
-                },
-                [&](uint32_t v, int32_t w) -> int32_t {
-                    const uint32_t slot = __umulhi(v, n.npc_recip), loc = v - slot * npc;
-                    if (n.tile) {
-                        if (!owned_column(n, cols[slot])) return kNever;  // another tile's target
-                        ++seen;
+            unsigned walked;
+            auto inhibitory = [&] {
+                if (begun) return;
+                walk_inhibitory(blockDim.x, n, s_inh, s_inh_n, tg, col_syn, (uint32_t)__cvta_generic_to_shared(s_in));
+                if (threadIdx.x == 0) ev_all += (unsigned long long)s_inh_n * n.canon_m;
+            };
+            if (!chunked) {
+                walked = walk_items(
+                    blockDim.x, n, col, s_items, items, w_ab, lg, tg, n.w + cbase, col_syn, inhibitory,
+                    [&](uint32_t v, int32_t w) -> int32_t {
+                        const uint32_t slot = __umulhi(v, n.npc_recip), loc = v - slot * npc;
+                        if (n.tile) {
+                            if (!owned_column(n, cols[slot])) return kNever;  // another tile's target
+                            ++seen;
+                        }
+                        if ((local >> slot) & 1u) {
+                            atomicAdd(&s_in[loc], w);
+                            return kStdp ? last[loc] : 0;
+                        }
+                        const uint32_t gid = cols[slot] * npc + loc;
+                        red_add(&n.I[gid], w);
+                        return kStdp ? n.last_spike[gid] : 0;
+                    },
+                    [&](int32_t x, int at) {
+                        if (!kStdp) return;
+                        const int32_t amount = s_lut[min(t - x, kLut - 1)];   // lag >= 1
+                        if (amount) red_add(&sd[at], -amount);                // no load: most amounts are 0
+                    });
+            } else {
+                const uint32_t in0 = (uint32_t)__cvta_generic_to_shared(s_in);
+                const uint4 *t4 = reinterpret_cast<const uint4 *>(tg);
+                const int4 *w4 = reinterpret_cast<const int4 *>(n.w + cbase);
+                walked = walk_chunks(blockDim.x, n, col, s_items, items, w_ab, inhibitory, [&](uint32_t c, uint32_t mask) {
+                    if (out_of_range(n, 8 * (int64_t)c + 8 <= col_syn)) return;
+                    const uint4 tv = t4[c];
+                    const int4 wa = w4[2 * c], wb = w4[2 * c + 1];
+                    const uint32_t tw[4] = {tv.x, tv.y, tv.z, tv.w};
+                    const int32_t wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                    int32_t x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const uint32_t v = (u & 1) ? (tw[u >> 1] >> 16) : (tw[u >> 1] & 0xffffu);
+                        x[u] = kNever;
+                        if (out_of_range(n, v < kSlots * npc)) continue;
+                        const uint32_t slot = __umulhi(v, n.npc_recip), loc = v - slot * npc;
+                        const bool due = (mask >> u) & 1u, here = (local >> slot) & 1u;
+                        red_shared(in0 + 4u * loc, due && here ? wv[u] : 0);      // adds 0 elsewhere: no branch
+                        if (kStdp) x[u] = last[loc];
+                        if (due && !here) {
+                            const uint32_t gid = cols[slot] * npc + loc;
+                            red_add(&n.I[gid], wv[u]);
+                            if (kStdp) x[u] = n.last_spike[gid];
+                        }
                     }
-                    if ((local >> slot) & 1u) {
-                        atomicAdd(&s_in[loc], w);
-                        return kStdp ? last[loc] : 0;
-                    }
-                    const uint32_t gid = cols[slot] * npc + loc;
-                    red_add(&n.I[gid], w);
-                    return kStdp ? n.last_spike[gid] : 0;
-                },
-                [&](int32_t x, int at) {
                     if (!kStdp) return;
-                    const int32_t amount = s_lut[min(t - x, kLut - 1)];   // lag >= 1
-                    if (amount) red_add(&sd[at], -amount);                // no load: most amounts are 0
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int32_t amount = s_lut[min(t - x[u], kLut - 1)];    // lag >= 1
+                        if (amount && ((mask >> u) & 1u)) red_add(&sd[8 * c + u], -amount);   // no load: most are 0
+                    }
                 });
+            }
             if (n.tile) {
                 ev_all += seen;
                 ev_exc += seen;

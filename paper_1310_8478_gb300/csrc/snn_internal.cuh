@@ -715,6 +715,65 @@ __device__ __forceinline__ unsigned walk_items(uint32_t threads, const DevNet &n
     return walked;
 }
 
+// The same walk for events that only add their weight: the buckets' chunks of
+// 8 synapses one after another over the lanes, whatever the buckets' sizes and
+// alignment.  add(c, mask): the positions of chunk c of the column in mask.
+template <typename First, typename Add>
+__device__ __forceinline__ unsigned walk_chunks(uint32_t threads, const DevNet &n, uint32_t col, const uint32_t *items,
+                                                uint32_t count, int32_t *w_who, First first, Add add)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)(threads >> 5);
+    const uint32_t share = (count + warps - 1) / warps, lt = lanemask_lt();
+    const uint32_t i_hi = min(count, (warp + 1) * share);
+    uint32_t i_lo = warp * share, row = 0;
+    unsigned walked = 0;
+    uint32_t a = 0, b = 0;
+    auto fetch = [&]() {
+        a = b = 0;
+        if (i_lo + lane < i_hi) {
+            const uint32_t it = items[i_lo + lane];
+            row = it >> 5;
+            const uint16_t *off = n.doff + (size_t)(col * n.npc + row) * kDoffStride + (it & 31u);
+            a = off[-1];
+            b = off[0];
+        }
+    };
+    fetch();
+    first();
+    while (i_lo < i_hi) {
+        walked += (unsigned)__reduce_add_sync(0xffffffffu, b - a);
+        const uint32_t base = row * n.uniform_m, lo = base + a, hi = base + b;   // the bucket's synapses of the column
+        const uint32_t cnt = b > a ? ((hi - 1) >> 3) - (lo >> 3) + 1 : 0u;
+        i_lo += 32;
+        fetch();                                 // the next tile's buckets, under this tile's walk
+        uint32_t start = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, start, o);
+            if (lane >= o) start += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, start, 31);
+        start -= cnt;
+        // the lane of the k-th bucket that holds something
+        const uint32_t some = __ballot_sync(0xffffffffu, cnt != 0);
+        __syncwarp();
+        if (cnt) w_who[__popc(some & lt)] = lane;
+        __syncwarp();
+        int before = -1;
+        for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+            const uint32_t heads = __reduce_or_sync(0xffffffffu, cnt && start - e0 < 32u ? 1u << (start - e0) : 0u);
+            const int who = w_who[before + __popc(heads & (2u * lt + 1u))];
+            before += __popc(heads);
+            const uint32_t w_lo = __shfl_sync(0xffffffffu, lo, who), w_hi = __shfl_sync(0xffffffffu, hi, who);
+            const uint32_t c = (w_lo >> 3) + e0 + lane - __shfl_sync(0xffffffffu, start, who);
+            if (e0 + lane >= total) continue;
+            const int p = (int)(w_lo - 8 * c), q = (int)(w_hi - 8 * c);          // the bucket's positions in the chunk
+            add(c, (0xffu << max(p, 0)) & (0xffu >> (8 - min(q, 8))));
+        }
+    }
+    return walked;
+}
+
 // 4 bytes from global to shared memory, asynchronously
 __device__ __forceinline__ void copy4_async(void *shared, const void *global)
 {

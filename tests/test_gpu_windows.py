@@ -271,3 +271,20 @@ def test_resident_grid_of_a_big_column_equals_the_oracle(eng, orc):
             n.run(steps)
             assert_same_run(o, n)
         assert n.counters()["spikes"] > 100
+
+
+@pytest.mark.parametrize("stdp", [True, False], ids=["stdp", "static"])
+@pytest.mark.parametrize("npc,m,D", [(75, 300, 20), (130, 401, 31), (64, 13, 1), (33, 160, 16), (101, 60, 2)])
+def test_ordered_delivery_chunk_by_chunk_equals_the_oracle(eng, orc, npc, m, D, stdp):
+    """Event-driven steps of the step kernels: buckets of a few synapses to a
+    whole row, at any alignment, on a torus whose rings lead back."""
+    cfg = _cfg(2, 3, npc, m, seed=90, max_delay_ms=D, thal_per_col_per_ms=2, w_exc0_q16=4 * 65536, deriv_period_ms=60)
+    if not stdp:
+        cfg["flags"] = eng.snn.STDP_OFF
+    o = orc.Oracle(cfg, **({} if stdp else dict(flags=1)))
+    o.run(130)
+    with gpu_net(eng, cfg) as n:
+        n.set_launch(dense_permille=1001)
+        n.run(130)
+        assert_same_run(o, n)
+        assert n.counters()["spikes"] > 100
