@@ -204,10 +204,11 @@ class ClockSampler:
 
 def kernel_source_digest(kernel: str = "dense"):
     """sha256 of the sources a step kernel is compiled from (the dense pass
-    has its own file; the other step kernels share snn_step.cu)."""
+    in snn_dense.cu, the column-ordered delivery in snn_deliver.cuh, the
+    others in snn_step.cu)."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("snn_dense.cu" if kernel == "dense" else "snn_step.cu", "snn_internal.cuh"):
+    for f in (("snn_dense.cu",) if kernel == "dense" else ("snn_step.cu", "snn_deliver.cuh")) + ("snn_internal.cuh",):
         with open(os.path.join(ROOT, "paper_1310_8478_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -590,7 +591,7 @@ def main():
             ce1 = net.counters()
             e2e = {"value": (ce1["e_all"] - ce0["e_all"]) / el, "unit": "events/s",
                    "h2d_bytes_per_step": per_step * snn.STIM_DTYPE.itemsize,
-                   "d2h_bytes_per_step": 2 * DEVICE_COUNTERS_BYTES, "steps": KE,
+                   "d2h_bytes_per_step": DEVICE_COUNTERS_BYTES, "steps": KE,
                    "same_events_as_device_run": bool(ce1["e_all"] - ce0["e_all"] == c1["e_all"] - c0["e_all"]
                                                      and KE == K)}
             if KE == K and device_digest is not None and ce1["raster_dropped"] == 0:  # digest taken above
@@ -788,10 +789,28 @@ def timed_window(net, stream, n_steps: int, device: int = 0):
     return a0.elapsed_time(a1), p0, p1, c0, c1, clk
 
 
+def unprofiled_window(net, stream, n_steps: int):
+    """n_steps steps of one call between CUDA events, as a user's run has them."""
+    import torch
+    start, c0 = net.t, net.counters()
+    torch.cuda.synchronize()
+    a0 = torch.cuda.Event(enable_timing=True)
+    a1 = torch.cuda.Event(enable_timing=True)
+    a0.record(stream)
+    net.run(n_steps)
+    a1.record(stream)
+    torch.cuda.synchronize()
+    ms, events = a0.elapsed_time(a1), net.counters()["e_all"] - c0["e_all"]
+    return {"steps": [start, start + n_steps], "ms_per_step": ms / n_steps, "value": events / (ms / 1000.0),
+            "unit": "events/s"}
+
+
 def steady_leg(net, cfg, stream, n_neurons, args, dense_at: int = 60, n_dense: int = 10, period_from: int = 995,
                n_period: int = 10):
     """After the timed region: n_dense steps from step dense_at (the run-away
-    regime, dense pass), and n_period steps from period_from (they cross the
+    regime, dense pass), the 50 steps behind them in one call without the
+    profile (which has every step apply its STDP at once; without it one pass
+    per 50 steps does), and n_period steps from period_from (they cross the
     long-term update that closes step period - 1)."""
     peak, peak_kind = measured_peaks()
     out = {}
@@ -818,6 +837,8 @@ def steady_leg(net, cfg, stream, n_neurons, args, dense_at: int = 60, n_dense: i
             leg["dense_fused"] = {"bytes_per_step": fused_dense_bytes(cfg), "achieved": round(ach, 1), "peak": peak,
                                   "peak_kind": peak_kind, "unit": "GB/s", "frac": round(ach / peak, 4)}
         out[name] = leg
+        if name == "dense_regime" and net.t + 50 <= period_from:
+            out["dense_window"] = unprofiled_window(net, stream, 50)
     return out
 
 
@@ -825,7 +846,8 @@ def steady_leg(net, cfg, stream, n_neurons, args, dense_at: int = 60, n_dense: i
 RASTER_DIGEST_MAX_SPIKES = 500_000_000
 
 # bytes of the device counter block that snn_run_host copies to the host
-# before and after the steps it runs (its result: the spikes of the window)
+# after the steps it runs (its result: the spikes of the window, against the
+# block it read after the call before)
 DEVICE_COUNTERS_BYTES = 184
 
 

@@ -154,7 +154,8 @@ typedef struct {
     int64_t dense_deriv_steps;       /* of which closed a plasticity period */
     int64_t dense_events;            /* synaptic events delivered by the dense pass */
     int64_t dense_exc_events;
-    int64_t dense_ltp_visits;        /* potentiation visits done by the dense pass */
+    int64_t dense_ltp_visits;        /* potentiation visits done by the dense pass, or due in dense
+                                        steps and left to their window's pass */
     int64_t kernels;                 /* kernels launched by the profiled steps, every kind (a
                                         kind above may group two: k_fold + k_deriv, the
                                         column-ordered + column-staged deliveries) */
@@ -177,7 +178,9 @@ typedef struct snn_net snn_net;
  *   hbm_budget_bytes: upper bound of device memory the net may use (0: no bound).
  *   out: receives the handle.
  * Errors: SNN_EINVAL (bad cfg), SNN_ENOMEM (footprint above the budget or
- * allocation failure), SNN_EOVERFLOW (in-degree * wmax + drive may exceed
+ * allocation failure; the engine's optional arrays, 24 to 28 bytes per neuron
+ * for taking steps together, are left out or given back where they do not
+ * fit), SNN_EOVERFLOW (in-degree * wmax + drive may exceed
  * int32), SNN_ECUDA.
  */
 int snn_build_network(const snn_config *cfg, void *cuda_stream, size_t hbm_budget_bytes,
@@ -261,6 +264,12 @@ int snn_step(snn_net *net);
  * snn_run -- advance n_ms steps (CUDA-graph replays of graph_steps steps where
  * the alignment allows and no step of the chunk closes a plasticity period,
  * single steps otherwise); returns after completion and the error-word check.
+ * Inside a call the engine may take steps together, with the same results:
+ * nets whose blocks all fit the GPU at once run windows of up to 50 steps as
+ * one cooperative launch (calls of four steps or more, default
+ * dense_permille, staged_permille and ring_permille, no probe, no profile);
+ * nets of 8 M plastic synapses or more leave the STDP of busy steps to one pass
+ * over the synapses per window.  Nothing is left to do when the call returns.
  */
 int snn_run(snn_net *net, uint32_t n_ms);
 
@@ -273,7 +282,8 @@ int snn_run(snn_net *net, uint32_t n_ms);
  * *n_out = spikes emitted in the window.  SNN_ETRUNC if cap is too small (the
  * simulation still advanced) or the device raster overflowed.  Without
  * host_spikes the call synchronises with the stream once: the counters are
- * copied out before and after the steps into pinned memory on the stream.
+ * copied out behind the steps into pinned memory on the stream (before them
+ * too when the last call did not end with them).
  */
 int snn_run_host(snn_net *net, uint32_t n_ms, const snn_stimulus *host_stimulus, size_t n_stim,
                  snn_spike *host_spikes, size_t cap, size_t *n_out);
@@ -358,8 +368,9 @@ int snn_read_counters(snn_net *net, snn_counters *out);
 int snn_net_info(const snn_net *net, uint32_t *n_neurons, int64_t *n_synapses,
                  size_t *device_bytes);
 
-/* snn_set_profile -- 1: time every kernel with CUDA events (no graphs; the
- * kernels of a step run one after another on the net's stream); 0: off. */
+/* snn_set_profile -- 1: time every kernel with CUDA events (no graphs, no steps
+ * taken together; the kernels of a step run one after another on the net's
+ * stream and apply its STDP at once); 0: off. */
 int snn_set_profile(snn_net *net, int on);
 int snn_read_profile(snn_net *net, snn_profile *out);
 
