@@ -55,6 +55,7 @@ constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chu
 constexpr size_t kReadStage = 256 << 10;           // bytes of a net's pinned memory for small read-backs
 constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
 constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
+constexpr int64_t kLightMinSynapses = 64 << 20;    // deferred dense steps have their own launch from here on
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
 constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
 constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
@@ -321,6 +322,7 @@ void drop_windows(snn_net *net)
     dn.I2 = nullptr;
     net->res_grid = 0;
     net->step_windows = false;
+    net->light_grid = 0;
     dn.win = nullptr;
     dn.hl0 = nullptr;
     dn.spk = nullptr;
@@ -533,6 +535,12 @@ int alloc_common(snn_net *net)
     return SNN_OK;
 }
 
+// of k_dense, which may run both kinds of dense steps
+size_t dense_smem(uint32_t npc, uint32_t block)
+{
+    return std::max(dense_smem_bytes(npc, block), dense_light_smem_bytes(npc, block));
+}
+
 // whether the dense pass and the column-staged delivery can run with the
 // current launch shape (compact targets, shared memory)
 int setup_dense(snn_net *net)
@@ -582,7 +590,7 @@ int setup_dense(snn_net *net)
             net->dn.staged_min_events = pm == 0xffffffffu ? ~0ull : (unsigned long long)net->N * pm / 1000ull;
         }
     }
-    const size_t bytes = dense_smem_bytes(net->cfg.neurons_per_col, net->launch.dense_block);
+    const size_t bytes = dense_smem(net->cfg.neurons_per_col, net->launch.dense_block);
     if (bytes + 1024 > (size_t)optin) return SNN_OK;
     SNN_CUDA(allow_smem((const void *)k_dense, bytes));
     int per_sm = 0;
@@ -701,6 +709,7 @@ int setup_windows(snn_net *net)
     net->stdp_grid = 0;
     net->res_grid = 0;
     net->step_windows = false;
+    net->light_grid = 0;
     int optin = 0, parts = 1;
     SNN_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
     // 32 warps, fewer where their tables do not fit beside the trains
@@ -759,8 +768,13 @@ int setup_windows(snn_net *net)
     const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
     net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
     net->step_windows = net->n_rin >= kWinMinSynapses;
-    if (net->step_windows && net->dense_ok) {
-        const size_t light = dense_light_smem_bytes(dn.npc);
+    // Dense steps that defer their STDP have a kernel of their own from 64 M
+    // plastic synapses on: its launch costs every other step 3 us, its 64 warps
+    // per SM take a fifth off a dense step (42x11 columns with M = 67, 21
+    // sparse steps: 0.82 ms, 0.86 with the launch).
+    dn.light_in_dense = net->step_windows && net->dense_ok && net->n_rin < kLightMinSynapses;
+    if (net->step_windows && net->dense_ok && !dn.light_in_dense) {
+        const size_t light = dense_light_smem_bytes(dn.npc, kDenseLightBlock);
         SNN_CUDA(allow_smem((const void *)k_dense_light, light));
         SNN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dense_light, (int)kDenseLightBlock, light));
         const int64_t dense_units = (int64_t)dn.C * ((dn.npc + dn.dense_rows - 1) / dn.dense_rows);
@@ -993,7 +1007,10 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     // neurons of 100 synapses 32.5 us per step against 38.8)
     const bool idle = net->skip_ltp && !closes && !prof && exact_t;
     net->skip_ltp = false;
-    const bool fork = !idle && !closes && !prof && (dn.tgt16 || net->N >= kForkMinExplicit);
+    // (so do graphs whose delivery and dense pass are one launch: 4000 neurons of
+    // 1123 synapses, every one firing, 51 us per step against 73; steps launched
+    // one by one do not: one column in a closed loop 54.6 us against 52.6)
+    const bool fork = !idle && !closes && !prof && (exact_t || !net->merged_grid) && (dn.tgt16 || net->N >= kForkMinExplicit);
     cudaStream_t sl = fork ? net->side : s;        // the potentiation's stream
     auto mark = [&](int kind, cudaStream_t on) {
         if (prof) cudaEventRecord(next_event(net, kind), on);
@@ -1028,7 +1045,7 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     const bool both = net->merged_grid && !prof;
     if (both) {
         k_deliver_dense<<<net->merged_grid, L.dense_block,
-                          std::max(ordered_smem_bytes(dn.npc, L.dense_block), dense_smem_bytes(dn.npc, L.dense_block)),
+                          std::max(ordered_smem_bytes(dn.npc, L.dense_block), dense_smem(dn.npc, L.dense_block)),
                           s>>>(dn, t_now);
         ++launched;
     } else if (dn.ordered_ok) {
@@ -1047,10 +1064,10 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     mark(0, s);
     if (net->dense_ok) {
         mark(4, s);
-        if (!both) k_dense<<<net->dense_grid, L.dense_block, dense_smem_bytes(dn.npc, L.dense_block), s>>>(dn, t_now);
+        if (!both) k_dense<<<net->dense_grid, L.dense_block, dense_smem(dn.npc, L.dense_block), s>>>(dn, t_now);
         launched += both ? 0 : 1;
-        if (net->step_windows && !prof) {
-            k_dense_light<<<net->light_grid, kDenseLightBlock, dense_light_smem_bytes(dn.npc), s>>>(dn, t_now);
+        if (net->light_grid && !prof) {
+            k_dense_light<<<net->light_grid, kDenseLightBlock, dense_light_smem_bytes(dn.npc, kDenseLightBlock), s>>>(dn, t_now);
             ++launched;
         }
         mark(4, s);
@@ -1998,7 +2015,7 @@ int batch_tables(snn_batch *b)
         const snn_net *n = b->nets[i];
         w[i] = n->dense_ok ? (double)n->S : 0.0;
         cap[i] = (uint64_t)n->dn.C * ((n->dn.npc + n->dn.dense_rows - 1) / std::max(1u, n->dn.dense_rows));
-        if (n->dense_ok) smem_d = std::max(smem_d, dense_smem_bytes(n->dn.npc, L.dense_block));
+        if (n->dense_ok) smem_d = std::max(smem_d, dense_smem(n->dn.npc, L.dense_block));
     }
     b->kind[kBDense].block = L.dense_block;
     b->kind[kBDense].smem = smem_d;
@@ -2031,8 +2048,8 @@ int batch_tables(snn_batch *b)
         cnt[kBWinOpen][i] = (uint32_t)sized_grid(n, 8, n->N, 1024);
         cnt[kBTrain][i] = (uint32_t)sized_grid(n, 8, n->dn.spk_words, 64);
         cnt[kBStdp][i] = (uint32_t)n->stdp_grid;
-        if (!n->dense_ok) continue;
-        smem_l = std::max(smem_l, dense_light_smem_bytes(n->dn.npc));
+        if (!n->light_grid) continue;
+        smem_l = std::max(smem_l, dense_light_smem_bytes(n->dn.npc, kDenseLightBlock));
         cnt[kBDenseLight][i] = (uint32_t)n->light_grid;
     }
     b->kind[kBDenseLight].block = kDenseLightBlock;

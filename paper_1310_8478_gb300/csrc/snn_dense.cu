@@ -368,11 +368,11 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
 // bandwidth (1.5 ms inside the fused pass's kernel with 32 warps, 2.9 ms with
 // the STDP); 320 000: 0.34 ms, with the L1's shared-memory passes at 0.8.
 // ---------------------------------------------------------------------------
-size_t dense_light_smem_bytes(uint32_t npc)
+size_t dense_light_smem_bytes(uint32_t npc, uint32_t block)
 {
     return (size_t)kSlots * npc * 4            // staged input
-           + (kDenseLightBlock / 32) * 32 * 4  // per-warp bucket offsets
-           + (kDenseLightBlock / 32) * 128 * 2; // per-warp chunks that are due
+           + (block / 32) * 32 * 4             // per-warp bucket offsets
+           + (block / 32) * 128 * 2;           // per-warp chunks that are due
 }
 
 // 8 synapses of a row into the staged input; those outside fmask add 0
@@ -516,7 +516,14 @@ __device__ __forceinline__ void dense_light_body(const DevNet &n, const int *t_n
     }
 }
 
-__global__ void __launch_bounds__(1024) k_dense(DevNet n, const int *t_now) { dense_body(n, t_now, whole_grid()); }
+// the dense pass of nets whose deferred dense steps have no launch of their own
+__device__ __forceinline__ void dense_any(const DevNet &n, const int *t_now, const Part &g)
+{
+    if (n.light_in_dense && deferring(n, *t_now)) dense_light_body(n, t_now, g);
+    else dense_body(n, t_now, g);
+}
+
+__global__ void __launch_bounds__(1024) k_dense(DevNet n, const int *t_now) { dense_any(n, t_now, whole_grid()); }
 
 __global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered(DevNet n, const int *t_now)
 {
@@ -535,14 +542,14 @@ __global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_ordered_b(Batch
 __global__ void __launch_bounds__(kOrderedMaxBlock, 2) k_deliver_dense(DevNet n, const int *t_now)
 {
     if (ordered_selected(n, *t_now)) deliver_ordered(n, t_now, whole_grid());
-    else dense_body(n, t_now, whole_grid());
+    else dense_any(n, t_now, whole_grid());
 }
 
 __global__ void __launch_bounds__(1024) k_dense_b(BatchLaunch b)
 {
     const BatchBlock x = batch_block(b);
     const DevNet n = b.nets[x.net];
-    dense_body(n, x.t_now, x.part);
+    dense_any(n, x.t_now, x.part);
 }
 
 __global__ void __launch_bounds__(kDenseLightBlock, 2) k_dense_light(DevNet n, const int *t_now)

@@ -143,6 +143,7 @@ struct DevNet {
     unsigned long long defer_visits; // a step whose spikes, times the steps left in the window, reach
                                      //     this starts the deferral after it
     uint32_t stdp_rows;              // source rows per work unit of the window's pass
+    int light_in_dense;              // k_dense runs the dense steps that defer their STDP, not k_dense_light
     int32_t *I2;                     // [N] resident grids: the input of every other step (the others: I)
     uint32_t res_parts;              // resident grids: blocks per column
 };
@@ -882,7 +883,7 @@ size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
 size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists);
-size_t dense_light_smem_bytes(uint32_t npc);
+size_t dense_light_smem_bytes(uint32_t npc, uint32_t block);
 constexpr uint32_t kDenseLightBlock = 1024;  // threads per block of a dense step that defers its STDP
 constexpr uint32_t kResBlock = 512;         // threads per block of a resident grid
 constexpr uint32_t kEmitBlock = 512;
