@@ -268,7 +268,8 @@ int snn_step(snn_net *net);
  * nets whose blocks all fit the GPU at once run windows of up to 50 steps as
  * one cooperative launch (calls of four steps or more, default
  * dense_permille, staged_permille and ring_permille, no probe, no profile);
- * nets of 8 M plastic synapses or more leave the STDP of busy steps to one pass
+ * nets of 8 M plastic synapses or more (40 M when no such launch takes their
+ * sparse steps) leave the STDP of busy steps to one pass
  * over the synapses per window.  Nothing is left to do when the call returns.
  */
 int snn_run(snn_net *net, uint32_t n_ms);

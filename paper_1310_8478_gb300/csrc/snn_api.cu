@@ -51,6 +51,7 @@ void *g_alloc_ctx = nullptr;
     } while (0)
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
+constexpr int64_t kWinMinSparse = 40ll << 20;    // ... when its sparse steps run in the step kernels too
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
 constexpr size_t kReadStage = 256 << 10;           // bytes of a net's pinned memory for small read-backs
 constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
@@ -695,11 +696,14 @@ int resident_grid(snn_net *net, int *parts_out)
 
 // Plasticity windows (snn_window.cu): nets with compact targets whose 13
 // columns of train words fit shared memory, with STDP and delivery on, and
-// not tiles.  The step kernels take them from 8 M plastic synapses on: a
+// not tiles.  The step kernels take them from 8 M plastic synapses on, from 40 M
+// where no resident grid takes the sparse steps off them: a
 // window costs three launches (about 30 us with the change of the
 // shared-memory split, 0.6 us per step; the one-column workload ran 1.7 us
 // per step slower with windows) and a dense step of such a net saves 8 bytes
-// per synapse, about 10 us.  Resident grids take them at any size, also for
+// per synapse, about 10 us (33x21 columns with M = 61, quiet: 30.1 ms for 930
+// steps with windows, 28.7 without; 25x28 with M = 90, some activity: 9.85 and
+// 9.99).  Resident grids take them at any size, also for
 // nets with target lists, which have a pass of their own.  The
 // arrays (24 or 28 bytes per neuron) are taken only where the budget and the device
 // have room; without them every step applies its STDP at once.
@@ -721,7 +725,8 @@ int setup_windows(snn_net *net)
                      (lists || bytes + 1024 <= (size_t)optin);
     if (can && dn.win && !dn.I2 && resident_grid(net, &parts)) drop_windows(net);   // (a shape that lets one run now)
     const int res = can ? resident_grid(net, &parts) : 0;
-    if (!can || (!res && (lists || net->n_rin < kWinMinSynapses))) {
+    const int64_t win_min = res ? kWinMinSynapses : kWinMinSparse;
+    if (!can || (!res && (lists || net->n_rin < win_min))) {
         drop_windows(net);
         return SNN_OK;
     }
@@ -767,7 +772,7 @@ int setup_windows(snn_net *net)
     dn.stdp_rows = (dn.ne + chunks - 1) / chunks;
     const int64_t units = (int64_t)dn.C * ((dn.ne + dn.stdp_rows - 1) / dn.stdp_rows);
     net->stdp_grid = (int)std::min<int64_t>(units, (int64_t)per_sm * net->sm_count);
-    net->step_windows = net->n_rin >= kWinMinSynapses;
+    net->step_windows = net->n_rin >= win_min;
     // Dense steps that defer their STDP have a kernel of their own from 64 M
     // plastic synapses on: its launch costs every other step 3 us, its 64 warps
     // per SM take a fifth off a dense step (42x11 columns with M = 67, 21
