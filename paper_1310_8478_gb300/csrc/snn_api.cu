@@ -627,13 +627,17 @@ int setup_dense(snn_net *net)
     return SNN_OK;
 }
 
-// no window open (its steps are counted from a clock that a restart sets back)
+// no window open (its steps are counted from a clock that a restart sets back),
+// and nothing in the resident grids' second input, where a grid that gave up
+// leaves what it had delivered
 int clear_window(snn_net *net)
 {
     if (!net->dn.win) return SNN_OK;
     DevWindow none{};
     none.p1 = -1;
     none.defer_from = kNoDefer;
+    none.polls = kBarrierPolls;
+    if (net->dn.I2) SNN_CUDA(cudaMemsetAsync(net->dn.I2, 0, (size_t)net->N * 4, net->stream));
     SNN_CUDA(cudaMemcpyAsync(net->dn.win, &none, sizeof none, cudaMemcpyHostToDevice, net->stream));
     return SNN_OK;
 }
@@ -747,7 +751,6 @@ int setup_windows(snn_net *net)
         dn.spk = reinterpret_cast<uint32_t *>(block + 2 * N8);
         if (res) dn.I2 = reinterpret_cast<int32_t *>(block + 2 * N8 + bits);
         dn.win = win;
-        if (res) SNN_CUDA(cudaMemsetAsync(dn.I2, 0, (size_t)net->N * 4, net->stream));
         SNN_TRY(clear_window(net));
     }
     net->res_grid = res;

@@ -42,7 +42,6 @@ constexpr uint32_t kEmitList = 4096;         // spikes listed at a time
 constexpr uint32_t kResItems = 2048;         // pending (row, delay) items of a block
 constexpr int kResFlight = 4;                // buckets of a group of lanes in flight
 constexpr uint32_t kResThal = 512;           // thalamic events of a column drawn ahead
-constexpr int kBarrierPolls = 1 << 22;       // about two seconds, then the kernel gives up
 
 __host__ __device__ __forceinline__ uint32_t res_slice(uint32_t npc, uint32_t parts) { return (npc + parts - 1) / parts; }
 
@@ -58,15 +57,16 @@ size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists)
            + (size_t)(kResBlock / 32) * 64 * 4;                // per warp: a tile's buckets
 }
 
-// All blocks of the grid; false when one of them did not come.  The arrival
+// All blocks of the grid; false when one of them did not come within `polls`
+// looks.  The arrival
 // releases and the end acquires for the whole block (thread 0 behind and
 // before a block barrier); the polls between are relaxed.
-__device__ __forceinline__ bool grid_barrier(DevWindow *win, unsigned target, int *s_ok)
+__device__ __forceinline__ bool grid_barrier(DevWindow *win, unsigned target, int polls, int *s_ok)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&win->bar) : "memory");
-        int left = kBarrierPolls;
+        int left = polls;
         unsigned seen;
         do {
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&win->bar) : "memory");
@@ -111,6 +111,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
     const int D = (int)n.D;
     const uint32_t dmask = (2u << D) - 2u;
     const bool more = gridDim.x > 1;
+    const int polls = win->polls;
 
     F *const s_v = reinterpret_cast<F *>(smem_i4);
     F *const s_u = s_v + ns_max;
@@ -372,7 +373,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             s_fired[0] = s_fired[1] = 0;
         }
         if (more) {
-            if (!(ok = grid_barrier(win, (unsigned)(k + 1) * gridDim.x, &s_ok))) break;
+            if (!(ok = grid_barrier(win, (unsigned)(k + 1) * gridDim.x, polls, &s_ok))) break;
         } else {
             __syncthreads();
         }

@@ -1,0 +1,139 @@
+"""Restarts and long lives of a net: what a grid that gave up, a clock far from
+0, a refused allocation or a read-back on a full device leave behind.  Device
+state that no call can make is written into the net's own blocks, which the
+allocator hook knows."""
+import numpy as np
+import pytest
+
+import workloads
+from test_gpu_parity import assert_same_run
+
+pytestmark = pytest.mark.gpu
+
+WIN_POLLS = 7          # word of the window block that holds the barrier's limit
+WIN_BYTES = 768        # its header, rounded up
+
+
+@pytest.fixture(scope="module")
+def eng():
+    import paper_1310_8478_gb300 as e
+    e.build_engine()
+    return e
+
+
+class Blocks:
+    """The allocator hook on PyTorch's: remembers the blocks' sizes, refuses
+    what `refuse` says, and gives nothing back before the end, so that a stale
+    pointer reads old values."""
+
+    def __init__(self):
+        self.live, self.gone, self.asked = {}, [], []
+        self.refuse = lambda n: False
+
+    def __enter__(self):
+        from paper_1310_8478_gb300 import snn
+        alloc, self.free = snn.torch_allocator()
+
+        def take(n, stream):
+            self.asked.append(n)
+            if self.refuse(n):
+                return 0
+            p = alloc(n, stream)
+            self.live[p] = n
+            return p
+
+        def give(p):
+            self.gone.append(p)
+            del self.live[p]
+        snn.set_allocator(take, give)
+        return self
+
+    def __exit__(self, *exc):
+        from paper_1310_8478_gb300 import snn
+        snn.set_allocator(None)
+        for p in self.gone:
+            self.free(p)
+
+    def words(self, p):
+        """Block p as a tensor of 32-bit words."""
+        import torch
+
+        class Block:
+            __cuda_array_interface__ = dict(shape=(self.live[p] // 4,), typestr="<i4", data=(p, False), version=2)
+        return torch.as_tensor(Block(), device="cuda")
+
+
+def _up(x):
+    return (x + 255) & ~255
+
+
+def _window_block(blocks, n_neurons):
+    """Of a net with a resident grid: header, histories, trains, spike bits of
+    64 steps, second input."""
+    size = WIN_BYTES + 2 * _up(8 * n_neurons) + _up(64 * 4 * ((n_neurons + 31) // 32)) + _up(4 * n_neurons)
+    found = [p for p, n in blocks.live.items() if n == size]
+    assert len(found) == 1
+    return found[0]
+
+
+def _cfg(gx, gy, npc, m, **kw):
+    kw.setdefault("exc_per_col", npc * 4 // 5)
+    return workloads.custom(grid_x=gx, grid_y=gy, neurons_per_col=npc, fanout=m,
+                            pct_ring=(40, 30, 20, 10) if gx * gy > 1 else (100, 0, 0, 0), **kw)
+
+
+@pytest.mark.parametrize("restart", ["reset", "load"])
+def test_a_restart_clears_both_inputs_of_a_resident_grid(eng, orc, restart):
+    import torch
+    cfg = _cfg(3, 2, 130, 60, seed=91, thal_per_col_per_ms=2, deriv_period_ms=70)
+    o = orc.Oracle(cfg)
+    o.run(90)
+    with Blocks() as b, eng.Network(cfg, raster_capacity=1 << 20) as n:
+        N = n.n_neurons
+        n.run(30)
+        state = n.save_state()
+        n.run(20)
+        words = b.words(_window_block(b, N))
+        words[len(words) - _up(4 * N) // 4:] = 15 * 65536
+        torch.cuda.synchronize()
+        if restart == "reset":
+            n.reset()
+            n.run(90)
+            assert_same_run(o, n)
+        else:
+            n.load_state(state)
+            n.run(60)
+            s, x = o.synapses(), n.neurons()
+            w, sd = n.weights()
+            assert np.array_equal(w, s["w"]) and np.array_equal(sd, s["sd"])
+            assert np.array_equal(x["v"].view(np.int32), o.neurons()["v"].view(np.int32))
+            assert n.counters()["spikes"] == o.counters()["spikes"]
+
+
+def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
+    """A limit of one look: the first block at the barrier gives up, and none
+    waits longer."""
+    import torch
+    cfg = _cfg(4, 3, 130, 60, seed=92, thal_per_col_per_ms=2, deriv_period_ms=70)
+    o = orc.Oracle(cfg)
+    o.run(90)
+    with Blocks() as b, eng.Network(cfg, raster_capacity=1 << 20) as n:
+        n.run(30)
+        state = n.save_state()
+        for restart in ("reset", "load"):
+            b.words(_window_block(b, n.n_neurons))[WIN_POLLS] = 1
+            torch.cuda.synchronize()
+            for _ in range(2):
+                with pytest.raises(eng.snn.SnnError) as e:
+                    n.run(50)
+                assert e.value.code == eng.snn.ETIMEOUT
+            if restart == "reset":
+                n.reset()
+                n.run(90)
+                assert_same_run(o, n)
+            else:
+                n.load_state(state)
+                n.run(60)
+                w, sd = n.weights()
+                assert np.array_equal(w, o.synapses()["w"]) and np.array_equal(sd, o.synapses()["sd"])
+                assert n.counters()["spikes"] == o.counters()["spikes"] and n.counters()["error"] == 0
