@@ -154,7 +154,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         return c * n.npc +
                draw_below(philox10(make_uint4((uint32_t)t, c, 1u, e - c * n.thal_per_col), n.seed_lo, n.seed_hi).x, n.npc);
     };
-    const bool drawn = (uint32_t)steps * thal <= kResThal;
+    const bool drawn = (uint64_t)steps * thal <= kResThal;      // (thal: up to 2^31 - 1)
     if (drawn)
         for (uint32_t e = threadIdx.x; e < (uint32_t)steps * thal; e += kResBlock) {
             const uint32_t k = e / thal;

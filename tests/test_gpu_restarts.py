@@ -137,3 +137,16 @@ def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
                 w, sd = n.weights()
                 assert np.array_equal(w, o.synapses()["w"]) and np.array_equal(sd, o.synapses()["sd"])
                 assert n.counters()["spikes"] == o.counters()["spikes"] and n.counters()["error"] == 0
+
+
+def test_a_drive_whose_events_per_window_pass_32_bits(eng):
+    """50 steps of 85 899 346 events are 4 more than 2^32: too many to be drawn
+    ahead, in steps of a resident grid against the step kernels'."""
+    cfg = _cfg(1, 1, 300, 20, seed=93, thal_per_col_per_ms=85899346, thal_amp_q16=2, wmax_q16=65536, w_exc0_q16=65536)
+    with eng.Network(cfg, raster_capacity=1 << 16) as a, eng.Network(cfg, raster_capacity=1 << 16) as b:
+        a.run(50)
+        for _ in range(25):
+            b.run(2)
+        for x, y in zip(a.raster() + a.weights(), b.raster() + b.weights()):
+            assert np.array_equal(x, y)
+        assert a.counters() == b.counters() and a.counters()["spikes"] > 10
