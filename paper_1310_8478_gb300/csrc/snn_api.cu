@@ -668,8 +668,9 @@ int resident_grid(snn_net *net, int *parts_out)
     const bool f64 = dn.vd != nullptr;
     const void *kernel = resident_kernel(net);
     if (!net->tgt16) {
-        // target lists: slices of all neurons, one block per SM
-        if (dn.S > 0x7fffffffll || (uint64_t)dn.C * dn.thal_per_col > kResListsThal) return 0;
+        // target lists: slices of all neurons, one block per SM (the drive may
+        // be switched off just now)
+        if (dn.S > 0x7fffffffll || (uint64_t)dn.C * net->cfg.thal_per_col_per_ms > kResListsThal) return 0;
         const uint32_t blocks = std::min<uint32_t>((uint32_t)net->sm_count, (dn.N + 31u) / 32u);
         const size_t bytes = resident_smem_bytes(dn.N, blocks, f64, true);
         int per_sm = 0;

@@ -150,3 +150,17 @@ def test_a_drive_whose_events_per_window_pass_32_bits(eng):
         for x, y in zip(a.raster() + a.weights(), b.raster() + b.weights()):
             assert np.array_equal(x, y)
         assert a.counters() == b.counters() and a.counters()["spikes"] > 10
+
+
+def test_a_drive_switched_off_does_not_hide_its_events(eng):
+    """A net with target lists and more drive events per step than every block
+    should look at takes no grid, whether the drive is on or off."""
+    cfg = _cfg(1, 1, 300, 1, seed=94, thal_per_col_per_ms=5000, thal_amp_q16=100)
+    ex = dict(row_off=np.arange(301), tgt=np.arange(300)[::-1].copy(), delay=np.ones(300, np.int64), w=np.ones(300, np.int64))
+    with Blocks() as b, eng.Network(cfg, raster_capacity=1 << 16, explicit=ex) as n:
+        asked = len(b.asked)
+        n.set_thalamic(False)
+        n.set_launch(neuron_block=128)
+        n.set_thalamic(True)
+        assert len(b.asked) == asked
+        n.run(20)
