@@ -123,7 +123,7 @@ __device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Pa
                     },
                     [&](int32_t x, int at) {
                         if (!kStdp) return;
-                        const int32_t amount = s_lut[min(t - x, kLut - 1)];   // lag >= 1
+                        const int32_t amount = s_lut[lag_of(t, x)];   // lag >= 1
                         if (amount) red_add(&sd[at], -amount);                // no load: most amounts are 0
                     });
             } else {
@@ -155,7 +155,7 @@ __device__ __forceinline__ void deliver_columns(const DevNet &n, int t, const Pa
                     if (!kStdp) return;
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        const int32_t amount = s_lut[min(t - x[u], kLut - 1)];    // lag >= 1
+                        const int32_t amount = s_lut[lag_of(t, x[u])];    // lag >= 1
                         if (amount && ((mask >> u) & 1u)) red_add(&sd[8 * c + u], -amount);   // no load: most are 0
                     }
                 });

@@ -228,7 +228,7 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
             uint16_t *x_row = s_x + sl * npc;
             int32_t *in_row = s_in + sl * npc;
             for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                const int lag = min(t - ls[loc], 255);
+                const int lag = lag_of(t, ls[loc]);
                 x_row[loc] = (uint16_t)((lag == 1 ? kFiredLast : 0u) | (stdp ? (uint32_t)s_lutm[lag] : 0u));
                 in_row[loc] = 0;
             }
@@ -265,8 +265,7 @@ __device__ __forceinline__ void dense_body(const DevNet &n, const int *t_now, co
                 w_off[lane] = hi;
                 if (exc && ltp_on && len) {
                     const uint32_t recent = h & (0xffffffffu << lane);
-                    const int lag = recent ? (__ffs(recent) - 1 - lane) : (t - 1 - (int)hv.y - lane);
-                    amt = lag < kLut ? s_lutp[lag] : 0;
+                    amt = s_lutp[recent ? __ffs(recent) - 1 - lane : lag_of(t - 1 - lane, (int)hv.y)];
                 }
                 w_amt[lane] = amt;
             }

@@ -134,8 +134,8 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         n.hl0[g0 + i] = h;
         s_hist[i] = h.x;
         s_old[i] = (int32_t)h.y;
-        const int lag = h.x ? __ffs(h.x) : p0 - (int)h.y;       // of the latest spike before the window
-        s_train[i] = (unsigned long long)min(lag, kLut - 1) << kWinBits;
+        const int lag = h.x ? __ffs(h.x) : lag_of(p0, (int)h.y);       // of the latest spike before the window
+        s_train[i] = (unsigned long long)lag << kWinBits;
     }
     // empty spike bits: a slice's first and last words are also its
     // neighbours', which set bits in them behind the first barrier

@@ -161,11 +161,8 @@ __device__ __forceinline__ void deliver_ring(const DevNet &n, const int *t_now, 
 #pragma unroll
             for (int u = 0; u < kUnroll; ++u) {
                 if (k[u] < 0 || !((inf[u] & 1u) && stdp)) continue;
-                const int lag = t - ls[u];                     // >= 1
-                if (lag < kLut) {
-                    const int32_t a = s_lut[lag];
-                    if (a) red_add(&n.sd[k[u]], -a);
-                }
+                const int32_t a = s_lut[lag_of(t, ls[u])];     // lag >= 1
+                if (a) red_add(&n.sd[k[u]], -a);
             }
         }
         __syncwarp();
@@ -251,7 +248,7 @@ __device__ __forceinline__ void deliver_cols(const DevNet &n, int t, int32_t *s_
             uint16_t *x_row = s_x + sl * npc;
             int32_t *in_row = s_in + sl * npc;
             for (uint32_t loc = threadIdx.x; loc < npc; loc += blockDim.x) {
-                x_row[loc] = kStdp ? (uint16_t)s_lut[min(t - ls[loc], kLut - 1)] : (uint16_t)0;
+                x_row[loc] = kStdp ? (uint16_t)s_lut[lag_of(t, ls[loc])] : (uint16_t)0;
                 in_row[loc] = 0;
             }
         }
@@ -488,13 +485,10 @@ __device__ __forceinline__ bool ltp_walk(const DevNet &n, int64_t lo, int64_t hi
             if (!ok[u]) continue;
             const uint32_t d = dl[u];
             const uint32_t recent = h[u].x & (0xffffffffu << d);
-            const int lag = recent ? (__ffs(recent) - 1 - (int)d) : (tp - (int)h[u].y - (int)d);
-            if (lag < kLut) {
-                const int32_t a = s_lut[lag];
-                if (a) {
-                    red_add(&n.sd_rev[e0 + 32 * u], a);   // coalesced: the target's entries are contiguous
-                    wrote = true;
-                }
+            const int32_t a = s_lut[recent ? __ffs(recent) - 1 - (int)d : lag_of(tp - (int)d, (int)h[u].y)];
+            if (a) {
+                red_add(&n.sd_rev[e0 + 32 * u], a);       // coalesced: the target's entries are contiguous
+                wrote = true;
             }
         }
     }

@@ -97,9 +97,9 @@ __device__ __forceinline__ void train_body(const DevNet &n, const Part &g)
             const uint32_t i = (w0 + q) * 32u + lane;
             if (i < n.N) {
                 const uint2 h = n.hl0[i];
-                const int lag = h.x ? __ffs(h.x) : p0 - (int)h.y;      // bit j: fired at p0 - 1 - j
+                const int lag = h.x ? __ffs(h.x) : lag_of(p0, (int)h.y);      // bit j: fired at p0 - 1 - j
                 n.train[i] = (unsigned long long)lo | ((unsigned long long)hi << 32) |
-                             ((unsigned long long)min(lag, kLut - 1) << kWinBits);
+                             ((unsigned long long)lag << kWinBits);
             }
         }
         __syncwarp();
@@ -308,7 +308,7 @@ __device__ __forceinline__ void row_spikes(unsigned long long own, uint2 h, int 
         int lag = late ? sh - 31 + __clz((int)late)
                 : p1   ? sh + 1 + __clz((int)p1)
                 : p2   ? sh + 33 + __clz((int)p2)
-                       : 4 * lane + ((h.x >> 31) ? 1 : p0 - 31 - (int)h.y);
+                       : 4 * lane + ((h.x >> 31) ? 1 : lag_of(p0 - 31, (int)h.y));
         int32_t q[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -328,7 +328,7 @@ __device__ __forceinline__ void row_spikes(unsigned long long own, uint2 h, int 
 // a source without an arrival inside any amount's reach changes nothing
 __device__ __forceinline__ bool row_live(unsigned long long own, uint2 h, int p0, int D)
 {
-    return own || h.x || p0 - (int)h.y - D < kLut - 1;
+    return own || h.x || lag_of(p0 - D, (int)h.y) < kLut - 1;
 }
 
 // One row of a net with target lists (explicit targets: no alignment, no

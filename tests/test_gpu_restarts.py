@@ -164,3 +164,83 @@ def test_a_drive_switched_off_does_not_hide_its_events(eng):
         n.set_thalamic(True)
         assert len(b.asked) == asked
         n.run(20)
+
+
+# ---------------------------------------------------------------------------
+# a clock beyond 2^30: the distance to the time stamp of a neuron that never
+# fired, -2^30, is then beyond an int
+# ---------------------------------------------------------------------------
+NEVER = -(1 << 30)
+
+
+def _later(eng, cfg, state, n_stored, ahead):
+    """The checkpoint with its clock, and every spike's time, moved ahead."""
+    import ctypes
+    N, D = cfg["grid_x"] * cfg["grid_y"] * cfg["neurons_per_col"], cfg["max_delay_ms"]
+    b = bytearray(state)
+    head = 32 + ctypes.sizeof(eng.snn.SnnConfig)
+    assert len(b) == head + N * 24 + D * N * 4 + D * 8 + n_stored * 8 + 184
+    np.frombuffer(b, np.int32, 2, 24)[:] += ahead              # t, raster_t0
+    hl = np.frombuffer(b, np.int32, 2 * N, head + 12 * N)[1::2]
+    last = np.frombuffer(b, np.int32, N, head + 20 * N)
+    assert np.count_nonzero(last == NEVER) > 2 and np.count_nonzero(last != NEVER) > 2
+    for x in (hl, last):
+        x[x != NEVER] += ahead
+    return bytes(b)
+
+
+LATE = {  # launch shape, net, its calls from the checkpoint on
+    "resident": ({}, _cfg(3, 2, 110, 40, seed=95, deriv_period_ms=60, thal_per_col_per_ms=0), [50, 47]),
+    "single_steps": ({}, _cfg(2, 2, 110, 40, seed=95, deriv_period_ms=60, thal_per_col_per_ms=0), [1] * 70),
+    "explicit": ({}, _cfg(2, 1, 150, 1, seed=96, deriv_period_ms=60, thal_per_col_per_ms=0), [50, 3, 30]),
+    # windows of the step kernels, whose dense steps leave their STDP to them
+    "windows": ({}, _cfg(8, 8, 1000, 200, seed=97, deriv_period_ms=60, thal_per_col_per_ms=0), [90]),
+}
+for _mode, _shape in (("sparse", dict(dense_permille=1001)), ("staged", dict(dense_permille=1001, staged_permille=1)),
+                      ("dense", dict(dense_permille=1)), ("ring", dict(dense_permille=1001, ring_permille=0xffffffff))):
+    LATE[_mode] = (_shape, LATE["single_steps"][1], [70])
+
+
+@pytest.mark.parametrize("name", sorted(LATE))
+def test_a_clock_beyond_two_to_the_thirty_changes_nothing(eng, name):
+    shape, cfg, calls = LATE[name]
+    ahead = ((1 << 30) // 960 + 1) * 960                        # whole rings, periods and windows' slots
+    N, T = cfg["grid_x"] * cfg["grid_y"] * cfg["neurons_per_col"], 40 + sum(calls)
+    rng = np.random.default_rng(5)
+    ex = None
+    if name == "explicit":
+        off = np.arange(N + 1) * 30
+        exc = np.repeat(np.arange(N) % 150 < 120, 30)
+        ex = dict(row_off=off, tgt=rng.integers(0, N, off[-1]), delay=np.where(exc, rng.integers(1, 21, off[-1]), 1),
+                  w=np.where(exc, 6 * 65536, -5 * 65536))
+    # every step some of the first half fire; later, in every sixth step, nearly half of them at once
+    few = 4 * max(1, N // 400)
+    t = np.repeat(np.arange(T), few)
+    g = rng.integers(0, N // 2, len(t))
+    many = np.arange(60, T, 6)
+    t, g = np.concatenate([t, np.repeat(many, N // 2)]), np.concatenate([g, np.tile(np.arange(N // 2), len(many))])
+    order = np.argsort(t, kind="stable")
+    t, g, q = t[order], g[order], np.full(len(t), 90 * 65536)
+    with eng.Network(cfg, raster_capacity=1 << 22, explicit=ex) as a, \
+            eng.Network(cfg, raster_capacity=1 << 22, explicit=ex) as b:
+        for n in (a, b):
+            n.set_launch(**shape)
+        a.set_stimulus(t[t < 40], g[t < 40], q[t < 40])
+        a.run(40)
+        stored = N * ((cfg["fanout"] + 7) // 8 * 8) if ex is None else len(ex["tgt"])
+        b.load_state(_later(eng, cfg, a.save_state(), stored, ahead))
+        a.set_stimulus(t, g, q)
+        b.set_stimulus(t[t >= 40] + ahead, g[t >= 40], q[t >= 40])
+        for steps in calls:
+            a.run(steps)
+            b.run(steps)
+        assert b.t == a.t + ahead
+        for x, y in zip(a.weights() + tuple(a.neurons().values()), b.weights() + tuple(b.neurons().values())):
+            assert np.array_equal(x, y)
+        ta, ga = a.raster(40, T)
+        tb, gb = b.raster(40 + ahead, T + ahead)
+        assert np.array_equal(ta + ahead, tb) and np.array_equal(ga, gb) and len(ta) > 20
+        ca, cb = a.counters(), b.counters()
+        assert all(ca[k] == cb[k] for k in ("spikes", "e_all", "e_exc", "l_exc")) and cb["error"] == 0
+        if name in ("windows", "dense"):
+            assert a.profile()["dense_steps"] == b.profile()["dense_steps"] > 3
