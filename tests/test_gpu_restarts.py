@@ -220,7 +220,7 @@ def test_a_clock_beyond_two_to_the_thirty_changes_nothing(eng, name):
     many = np.arange(60, T, 6)
     t, g = np.concatenate([t, np.repeat(many, N // 2)]), np.concatenate([g, np.tile(np.arange(N // 2), len(many))])
     order = np.argsort(t, kind="stable")
-    t, g, q = t[order], g[order], np.full(len(t), 90 * 65536)
+    t, g, q = t[order], g[order], np.full(len(t), 300 * 65536)
     with eng.Network(cfg, raster_capacity=1 << 22, explicit=ex) as a, \
             eng.Network(cfg, raster_capacity=1 << 22, explicit=ex) as b:
         for n in (a, b):
