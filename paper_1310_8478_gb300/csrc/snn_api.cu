@@ -1408,6 +1408,7 @@ int set_stimulus_impl(snn_net *net, const snn_stimulus *ev, size_t n)
     for (size_t k = 1; k < n_off; ++k) off[k] += off[k - 1];
     if (stage > net->stim_cap) {
         dn.stim_t0 = dn.stim_t1 = 0;
+        drop_graphs(net);                  // they hold the buffer that goes, also when there is no other
         dfree(net, (void *)dn.stim_off);
         dn.stim_off = nullptr;
         net->stim_cap = 0;

@@ -244,3 +244,33 @@ def test_a_clock_beyond_two_to_the_thirty_changes_nothing(eng, name):
         assert all(ca[k] == cb[k] for k in ("spikes", "e_all", "e_exc", "l_exc")) and cb["error"] == 0
         if name in ("windows", "dense"):
             assert a.profile()["dense_steps"] == b.profile()["dense_steps"] > 3
+
+
+@pytest.mark.parametrize("batch", [False, True], ids=["alone", "batch"])
+def test_a_refused_stimulus_leaves_no_graph_with_the_old_one(eng, batch):
+    """The events of an earlier call are gone once a larger upload was refused,
+    also from the captured steps."""
+    cfg = _cfg(1, 1, 200, 30, seed=98, thal_per_col_per_ms=1)
+    t = np.repeat(np.arange(200), 3)
+    g, q = np.arange(len(t)) % 200, np.full(len(t), 40 * 65536)
+    more = np.repeat(np.arange(200), 50)
+    with Blocks() as b, eng.Network(cfg, raster_capacity=1 << 18) as n, eng.Network(cfg, raster_capacity=1 << 18) as ref:
+        runs = []
+        for x in (n, ref):
+            x.set_launch(dense_permille=1001, graph_steps=10)
+            runs.append(eng.Batch([x], graph_steps=10) if batch else x)
+            x.set_stimulus(t, g, q)
+            runs[-1].run(60)
+        b.refuse = lambda size: True
+        with pytest.raises(eng.snn.SnnError) as e:
+            n.set_stimulus(more, np.arange(len(more)) % 200, np.full(len(more), 40 * 65536))
+        assert e.value.code == eng.snn.ENOMEM
+        b.refuse = lambda size: False
+        ref.set_stimulus([], [], [])
+        for r in runs:
+            r.run(60)
+        for x, y in zip(n.raster() + n.weights(), ref.raster() + ref.weights()):
+            assert np.array_equal(x, y)
+        if batch:
+            for r in runs:
+                r.close()
