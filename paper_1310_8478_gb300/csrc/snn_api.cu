@@ -231,13 +231,14 @@ namespace {
 
 void drop_windows(snn_net *net);
 
-int dalloc(snn_net *net, size_t bytes, void **out)
+// evict: the plasticity windows' arrays, which are optional, make room
+int dalloc(snn_net *net, size_t bytes, void **out, bool evict = true)
 {
     *out = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~size_t(255);
-    // the plasticity windows' arrays are optional: they make room
-    if (net->budget && net->bytes_held + bytes > net->budget) drop_windows(net);
+    evict = evict && net->dn.win;
+    if (evict && net->budget && net->bytes_held + bytes > net->budget) drop_windows(net);
     if (net->budget && net->bytes_held + bytes > net->budget) {
         set_error("device budget exceeded: %zu + %zu > %zu bytes", net->bytes_held, bytes, net->budget);
         return SNN_ENOMEM;
@@ -245,7 +246,7 @@ int dalloc(snn_net *net, size_t bytes, void **out)
     void *p = nullptr;
     if (net->alloc) {
         p = net->alloc(bytes, (void *)net->stream, net->alloc_ctx);
-        if (!p && net->dn.win) {
+        if (!p && evict) {
             drop_windows(net);
             p = net->alloc(bytes, (void *)net->stream, net->alloc_ctx);
         }
@@ -260,7 +261,7 @@ int dalloc(snn_net *net, size_t bytes, void **out)
         }
     } else {
         cudaError_t e = cudaMalloc(&p, bytes);
-        if (e != cudaSuccess && net->dn.win) {
+        if (e != cudaSuccess && evict) {
             cudaGetLastError();
             drop_windows(net);
             e = cudaMalloc(&p, bytes);
@@ -292,10 +293,10 @@ void dfree(snn_net *net, void *p)
 }
 
 template <typename T>
-int dalloc_t(snn_net *net, size_t count, T **out)
+int dalloc_t(snn_net *net, size_t count, T **out, bool evict = true)
 {
     void *p = nullptr;
-    int r = dalloc(net, count * sizeof(T), &p);
+    int r = dalloc(net, count * sizeof(T), &p, evict);
     *out = (T *)p;
     return r;
 }
@@ -2535,9 +2536,14 @@ int snn_read_synapses(snn_net *net, uint32_t first, uint32_t count, int32_t *hos
                         : (uint32_t)std::min<int64_t>(count, std::max<int64_t>(few, kReadChunk / row_max));
     struct Scratch {
         snn_net *net;
+        bool windows;                    // held when the call began: taken again at its end
         int32_t *t = nullptr, *w = nullptr, *s = nullptr;
         uint8_t *d = nullptr;
-        ~Scratch() { drop(); }
+        ~Scratch()
+        {
+            drop();
+            if (windows && !net->dn.win) setup_windows(net);
+        }
         void drop()
         {
             dfree(net, t);
@@ -2547,21 +2553,17 @@ int snn_read_synapses(snn_net *net, uint32_t first, uint32_t count, int32_t *hos
             t = w = s = nullptr;
             d = nullptr;
         }
-    } x{net};
-    auto take = [&](size_t n) {
+    } x{net, net->dn.win != nullptr};
+    auto take = [&](size_t n, bool evict) {
         int r = SNN_OK;
-        if (host_tgt) r = dalloc_t(net, n, &x.t);
-        if (r == SNN_OK && host_delay) r = dalloc_t(net, n, &x.d);
-        if (r == SNN_OK && host_w) r = dalloc_t(net, n, &x.w);
-        if (r == SNN_OK && host_sd) r = dalloc_t(net, n, &x.s);
+        if (host_tgt) r = dalloc_t(net, n, &x.t, evict);
+        if (r == SNN_OK && host_delay) r = dalloc_t(net, n, &x.d, evict);
+        if (r == SNN_OK && host_w) r = dalloc_t(net, n, &x.w, evict);
+        if (r == SNN_OK && host_sd) r = dalloc_t(net, n, &x.s, evict);
         return r;
     };
-    auto room = [&](size_t n) {          // without pushing anything else out of the budget
-        const size_t bytes = n * ((host_tgt ? 4 : 0) + (host_delay ? 1 : 0) + (host_w ? 4 : 0) + (host_sd ? 4 : 0)) + 1024;
-        return !net->budget || net->bytes_held + bytes <= net->budget;
-    };
     const size_t big = (size_t)std::min<int64_t>(total, (int64_t)rows * row_max);
-    const bool once = rows > few && room(big) && take(big) == SNN_OK;
+    const bool once = rows > few && take(big, false) == SNN_OK;
     if (!once) {
         x.drop();
         rows = few;
@@ -2575,7 +2577,7 @@ int snn_read_synapses(snn_net *net, uint32_t first, uint32_t count, int32_t *hos
         if (n > 0) {
             if (!once) {
                 x.drop();
-                SNN_TRY(take((size_t)n));
+                SNN_TRY(take((size_t)n, true));
             }
             k_read_rows<<<sized_grid(net, 8, r1 - r0, 8), 256, 0, net->stream>>>(net->dn, net->gen, net->canon_delay, r0,
                                                                               r1 - r0, a, x.t, x.d, x.w, x.s);

@@ -274,3 +274,26 @@ def test_a_refused_stimulus_leaves_no_graph_with_the_old_one(eng, batch):
         if batch:
             for r in runs:
                 r.close()
+
+
+@pytest.mark.parametrize("pinch", ["large_blocks", "until_windows_go"])
+def test_a_read_back_keeps_or_returns_the_windows_arrays(eng, pinch):
+    """Where the large scratch of a read-back is not to be had, small chunks are
+    tried before the arrays of the plasticity windows make room; where those do,
+    they are taken again after the read."""
+    cfg = _cfg(2, 2, 1000, 100, seed=99, deriv_period_ms=60)
+    with Blocks() as b, eng.Network(cfg, raster_capacity=0) as n, eng.Network(cfg, raster_capacity=0) as ref:
+        n.run(70)
+        ref.run(70)
+        w, sd = ref.weights()
+        ref.close()
+        win = _window_block(b, n.n_neurons)
+        largest = 1024 * 100 * 4
+        b.refuse = (lambda size: size > largest) if pinch == "large_blocks" else (lambda size: win in b.live)
+        held = n.synapses(0, 4000, fields=("w", "sd"))
+        assert np.array_equal(held["w"], w) and np.array_equal(held["sd"], sd)
+        _window_block(b, n.n_neurons)
+        assert (win in b.live) == (pinch == "large_blocks")
+        b.refuse = lambda size: False
+        n.run(70)
+        assert n.counters()["spikes"] > 100
