@@ -406,7 +406,8 @@ int sized_grid(const snn_net *net, uint32_t blocks_per_sm, int64_t units, int64_
 }
 
 // blocks of the neuron update: one tile of 4 neurons per thread each, at most
-// one resident wave (32 warps per SM at the kernel's registers), which loops
+// one resident wave (32 warps per SM at the kernel's registers, whatever the
+// block: its shared memory follows its warps), which loops
 int neuron_blocks(const snn_net *net, uint32_t block)
 {
     return sized_grid(net, std::max(1u, 1024u / block), net->N, (int64_t)block * kNeuronsPerThread);
@@ -1086,8 +1087,9 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
     // [S2(t) S3(t)]
     const int nb_neuron = neuron_blocks(net, L.neuron_block);
     mark(1, s);
-    if (dn.vd) k_neuron_f64<<<nb_neuron, L.neuron_block, 0, s>>>(dn, t_now, t_next);
-    else k_neuron_f32<<<nb_neuron, L.neuron_block, 0, s>>>(dn, t_now, t_next);
+    const size_t neuron_smem = neuron_smem_bytes(L.neuron_block);
+    if (dn.vd) k_neuron_f64<<<nb_neuron, L.neuron_block, neuron_smem, s>>>(dn, t_now, t_next);
+    else k_neuron_f32<<<nb_neuron, L.neuron_block, neuron_smem, s>>>(dn, t_now, t_next);
     ++launched;
     if (dn.probe_n) {
         k_probe<<<(dn.probe_n + 255) / 256, 256, 0, s>>>(dn, t_now);
@@ -2044,6 +2046,7 @@ int batch_tables(snn_batch *b)
         cnt[kBProbe][i] = (n->dn.probe_n + 255) / 256;
     }
     b->kind[kBNeuron32].block = b->kind[kBNeuron64].block = L.neuron_block;
+    b->kind[kBNeuron32].smem = b->kind[kBNeuron64].smem = neuron_smem_bytes(L.neuron_block);
     b->kind[kBProbe].block = 256;
     // plasticity windows
     size_t smem_w = 0;

@@ -891,6 +891,7 @@ size_t dense_smem_bytes(uint32_t npc, uint32_t block);
 size_t staged_smem_bytes(uint32_t npc, uint32_t block);
 size_t ordered_smem_bytes(uint32_t npc, uint32_t block);
 size_t stdp_smem_bytes(uint32_t npc, uint32_t block);
+size_t neuron_smem_bytes(uint32_t block);
 size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists);
 size_t dense_light_smem_bytes(uint32_t npc, uint32_t block);
 constexpr uint32_t kDenseLightBlock = 1024;  // threads per block of a dense step that defers its STDP

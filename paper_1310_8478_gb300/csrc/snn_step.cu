@@ -736,11 +736,13 @@ __device__ __forceinline__ void store4(T *p, uint32_t i, uint32_t n, const T (&x
 // a warp's spikes not yet in the ring and raster
 constexpr int kWarpSpikes = 256;
 
+size_t neuron_smem_bytes(uint32_t block) { return (size_t)(block / 32) * kWarpSpikes * 4; }
+
 template <typename F>
 __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, int *t_next, const Part &g)
 {
     static_assert(kNeuronsPerThread == 4, "one 16-byte access per 4-byte array");
-    __shared__ int32_t s_spk[32][kWarpSpikes];       // per warp: exc ids from the front, inh ids from the back
+    extern __shared__ int4 smem_i4[];                // per warp: exc ids from the front, inh ids from the back
     __shared__ unsigned long long s_cnt[32];         // per warp: exc | inh << 32, then their block-wide prefix
     __shared__ unsigned long long s_base;
     __shared__ bool s_last;
@@ -757,7 +759,7 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     unsigned long long *const counts = reinterpret_cast<unsigned long long *>(&n.ctr->step_cnt[par][0]);
-    int32_t *const list = s_spk[warp];
+    int32_t *const list = reinterpret_cast<int32_t *>(smem_i4) + warp * kWarpSpikes;
     int we = 0, wi = 0;               // the warp's pending spikes
     unsigned long long indeg = 0;     // excitatory in-degree of the neurons that fired
     // the warp's pending spikes into the ring and the raster, at the positions
