@@ -58,6 +58,8 @@ constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's deliver
 constexpr uint32_t kForkMinExplicit = 100000;      // neurons from which an explicit net's step forks
 constexpr int64_t kLightMinSynapses = 64 << 20;    // deferred dense steps have their own launch from here on
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
+constexpr uint32_t kResQueue = 32;                 // windows that a call queues on a resident grid at first
+constexpr int64_t kResRetry = 200;                 // steps from one that was too busy to the next try
 constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
 constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
@@ -179,6 +181,7 @@ struct snn_net {
     // ([0]), and the staging of a stimulus upload
     DevCounters *host_ctr = nullptr;
     bool host_ctr_known = false;    // [1] is what the device holds
+    int64_t last_fired = 0;         // spikes of step t - 1 as the last read-back told; -1: not known
     char *read_stage = nullptr;     // kReadStage bytes of small read-backs
     char *stim_stage = nullptr;
     size_t stim_stage_cap = 0;
@@ -1213,6 +1216,13 @@ int read_counters_raw(snn_net *net, DevCounters *hc)
     return SNN_OK;
 }
 
+// the spikes of the last step before t, from counters read behind it
+int64_t fired_last(const DevCounters &c, int32_t t)
+{
+    const int32_t *x = c.step_cnt[(t - 1) & 1];
+    return t > 0 ? (int64_t)x[0] + x[1] : 0;
+}
+
 // end of a run: the counters are copied out behind the steps and read after
 // the one synchronisation (the device error word decides the return code)
 int finish_run(snn_net *net, bool copied)
@@ -1223,6 +1233,7 @@ int finish_run(snn_net *net, bool copied)
     }
     SNN_CUDA(cudaGetLastError());
     net->host_ctr_known = true;
+    net->last_fired = fired_last(net->host_ctr[1], net->t);
     net->stim_in_flight = false;
     if (net->profile && net->ev_used) {
         for (size_t i = 0; i + 1 < net->ev_used; i += 2) {
@@ -1253,9 +1264,8 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
                                  net->stream));
     // the last step of this net was a step kernel's, read back behind it, and
     // nothing fired in it: nothing to potentiate in the first one
-    const int32_t *fired = net->host_ctr[1].step_cnt[(net->t - 1) & 1];
-    net->skip_ltp = net->host_ctr_known && net->host_ctr[1].ltp_pending == net->t - 1 && net->t > 0 && fired[0] == 0 &&
-                    fired[1] == 0 && !net->dn.tile;
+    net->skip_ltp = net->host_ctr_known && net->host_ctr[1].ltp_pending == net->t - 1 && net->t > 0 &&
+                    net->last_fired == 0 && !net->dn.tile;
     net->host_ctr_known = false;
     const uint32_t L = effective_graph_len(net);
     if (L != net->graph_len) {
@@ -1267,18 +1277,40 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
     uint32_t window = 0;                       // steps left of the open window
     const bool resident = resident_call(net, left);
     int64_t resident_from = net->t;            // the step from which the resident grid is tried
+    uint32_t queue = kResQueue;                // windows of the next try
+    int64_t fired = net->last_fired;           // spikes of the step before t; -1: not known
     bool copied = false;                       // the counters have been read behind the last step
+    net->last_fired = -1;
+    bool stale = false;                        // this call's step kernels ran since `fired` was known
     while (left > 0) {
         const int32_t t = net->t;
         copied = false;
         if (resident && !window && t >= resident_from) {
-            // every window of the call at once; the one synchronisation says
-            // how far they came
+            // A step for the dense pass stops the grid, or keeps it from
+            // starting, and every window queued behind it costs three launches
+            // that return.  So none is queued when the last step is known to
+            // have fired that many (which the read-back of one synchronisation
+            // tells every kResRetry steps), and the queue of a try, whose
+            // synchronisation says how far it came, is bounded and doubles
+            // while all of it is taken (2x2 columns that stay saturated, us
+            // per step: 31.6 in a call of 20 000 and 39 in calls of four; 44 and
+            // 55 when every call tried, and every try queued the rest of it).
+            if (stale) {
+                SNN_TRY(read_counters_raw(net, &net->host_ctr[1]));
+                if (net->host_ctr[1].error) return finish_run(net, true);
+                fired = fired_last(net->host_ctr[1], t);
+                stale = false;
+            }
+            if (net->tgt16 && fired >= (int64_t)net->dn.dense_min_spikes) {
+                resident_from = t + kResRetry;
+                continue;
+            }
             if (net->ltp_owed) {
                 launch_flush(net);
                 net->ltp_owed = false;
             }
-            for (uint32_t ahead = 0; ahead < left;) {
+            uint32_t ahead = 0;
+            for (uint32_t q = 0; q < queue && ahead < left; ++q) {
                 const uint32_t at = (uint32_t)t + ahead;
                 uint32_t n = std::min<uint32_t>(left - ahead, kWinSteps);
                 if (P) n = std::min<uint32_t>(n, P - at % P);
@@ -1296,9 +1328,14 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             const int32_t now = std::max(t, hc.t_slot[(hc.t_slot[0] < hc.t_slot[1]) ? 1 : 0]);
             left -= (uint32_t)(now - t);
             net->t = now;
-            // a busy net goes on with the step kernels, 200 steps until the
-            // next try
-            resident_from = (int64_t)now + 200;
+            fired = fired_last(hc, now);
+            if (now == t + (int64_t)ahead) {
+                queue = std::min(2 * queue, 1u << 20);
+                resident_from = now;
+            } else {
+                queue = 1;
+                resident_from = now + kResRetry;
+            }
             copied = true;
             continue;
         }
@@ -1326,6 +1363,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             net->ltp_owed = true;
         }
         net->skip_ltp = false;                 // true of the call's first step at most
+        stale = true;
         if (window && (window -= before - left) == 0) {
             close_window(net);
             SNN_CUDA(cudaGetLastError());
@@ -2256,6 +2294,7 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
     for (snn_net *n : b->nets) {
         if (n->profile) { set_error("a net of the batch is profiling"); return SNN_ESTATE; }
         n->host_ctr_known = false;
+        n->last_fired = -1;
         n->skip_ltp = false;
         if ((int64_t)n->t + n_ms > 0x7fff0000ll) { set_error("time limit reached"); return SNN_ESTATE; }
         SNN_TRY(ensure_raster_steps(n, (int64_t)n->t + n_ms + 2 - n->dn.raster_t0));
@@ -2295,6 +2334,7 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
         n->ltp_owed = true;
         DevCounters hc{};
         SNN_TRY(read_counters_raw(n, &hc));
+        n->last_fired = fired_last(hc, n->t);
         if (hc.error && rc == SNN_OK) {
             set_error("device error word %d", hc.error);
             rc = (hc.error == SNN_ETIMEOUT || hc.error == SNN_EBOUNDS) ? hc.error : SNN_ECUDA;
@@ -2467,6 +2507,7 @@ int snn_reset(snn_net *net)
     SNN_CUDA(cudaStreamSynchronize(s));
     net->t = 0;
     net->host_ctr_known = false;
+    net->last_fired = 0;
     net->weights_moved = false;
     net->ltp_owed = false;
     net->dn.raster_t0 = 0;
@@ -2879,6 +2920,7 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     DevNet &dn = net->dn;
     net->weights_moved = true;
     net->host_ctr_known = false;
+    net->last_fired = -1;
     void *sv = dn.vd ? (void *)dn.vd : (void *)dn.v;
     void *su = dn.ud ? (void *)dn.ud : (void *)dn.u;
     void *dst[] = {sv, su, dn.I, dn.hl, dn.last_spike, dn.ring_ids, dn.ring_cnt, net->w, net->sd, net->ctr};

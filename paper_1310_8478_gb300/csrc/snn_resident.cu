@@ -609,7 +609,10 @@ __global__ void __launch_bounds__(kEmitBlock) k_emit(DevNet n)
     c->spikes = spikes;
     c->raster_dropped = dropped;
     c->raster_total = rt;
-    for (int q = 0; q < 8; ++q) c->step_cnt[q >> 2][q & 3] = 0;      // the last step kernel's, if any
+    // as the step kernels leave them: the last step's spikes, the next one's none
+    for (int q = 0; q < 8; ++q) c->step_cnt[q >> 2][q & 3] = 0;
+    c->step_cnt[(p0 + steps - 1) & 1][0] = (int)(s_cnt[steps - 1] & 0xffffffffull);
+    c->step_cnt[(p0 + steps - 1) & 1][1] = (int)(s_cnt[steps - 1] >> 32);
     c->l_exc_mark = __ldcg(&c->l_exc);
     c->ltp_pending = p0 + steps - 1;
     c->done_blocks = 0;

@@ -6,74 +6,16 @@ import numpy as np
 import pytest
 
 import workloads
+from device_blocks import Blocks, WIN_POLLS, up, window_block
 from test_gpu_parity import assert_same_run
 
 pytestmark = pytest.mark.gpu
-
-WIN_POLLS = 7          # word of the window block that holds the barrier's limit
-WIN_BYTES = 768        # its header, rounded up
-
 
 @pytest.fixture(scope="module")
 def eng():
     import paper_1310_8478_gb300 as e
     e.build_engine()
     return e
-
-
-class Blocks:
-    """The allocator hook on PyTorch's: remembers the blocks' sizes, refuses
-    what `refuse` says, and gives nothing back before the end, so that a stale
-    pointer reads old values."""
-
-    def __init__(self):
-        self.live, self.gone, self.asked = {}, [], []
-        self.refuse = lambda n: False
-
-    def __enter__(self):
-        from paper_1310_8478_gb300 import snn
-        alloc, self.free = snn.torch_allocator()
-
-        def take(n, stream):
-            self.asked.append(n)
-            if self.refuse(n):
-                return 0
-            p = alloc(n, stream)
-            self.live[p] = n
-            return p
-
-        def give(p):
-            self.gone.append(p)
-            del self.live[p]
-        snn.set_allocator(take, give)
-        return self
-
-    def __exit__(self, *exc):
-        from paper_1310_8478_gb300 import snn
-        snn.set_allocator(None)
-        for p in self.gone:
-            self.free(p)
-
-    def words(self, p):
-        """Block p as a tensor of 32-bit words."""
-        import torch
-
-        class Block:
-            __cuda_array_interface__ = dict(shape=(self.live[p] // 4,), typestr="<i4", data=(p, False), version=2)
-        return torch.as_tensor(Block(), device="cuda")
-
-
-def _up(x):
-    return (x + 255) & ~255
-
-
-def _window_block(blocks, n_neurons):
-    """Of a net with a resident grid: header, histories, trains, spike bits of
-    64 steps, second input."""
-    size = WIN_BYTES + 2 * _up(8 * n_neurons) + _up(64 * 4 * ((n_neurons + 31) // 32)) + _up(4 * n_neurons)
-    found = [p for p, n in blocks.live.items() if n == size]
-    assert len(found) == 1
-    return found[0]
 
 
 def _cfg(gx, gy, npc, m, **kw):
@@ -93,8 +35,8 @@ def test_a_restart_clears_both_inputs_of_a_resident_grid(eng, orc, restart):
         n.run(30)
         state = n.save_state()
         n.run(20)
-        words = b.words(_window_block(b, N))
-        words[len(words) - _up(4 * N) // 4:] = 15 * 65536
+        words = b.words(window_block(b, N))
+        words[len(words) - up(4 * N) // 4:] = 15 * 65536
         torch.cuda.synchronize()
         if restart == "reset":
             n.reset()
@@ -121,7 +63,7 @@ def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
         n.run(30)
         state = n.save_state()
         for restart in ("reset", "load"):
-            b.words(_window_block(b, n.n_neurons))[WIN_POLLS] = 1
+            b.words(window_block(b, n.n_neurons))[WIN_POLLS] = 1
             torch.cuda.synchronize()
             for _ in range(2):
                 with pytest.raises(eng.snn.SnnError) as e:
@@ -287,12 +229,12 @@ def test_a_read_back_keeps_or_returns_the_windows_arrays(eng, pinch):
         ref.run(70)
         w, sd = ref.weights()
         ref.close()
-        win = _window_block(b, n.n_neurons)
+        win = window_block(b, n.n_neurons)
         largest = 1024 * 100 * 4
         b.refuse = (lambda size: size > largest) if pinch == "large_blocks" else (lambda size: win in b.live)
         held = n.synapses(0, 4000, fields=("w", "sd"))
         assert np.array_equal(held["w"], w) and np.array_equal(held["sd"], sd)
-        _window_block(b, n.n_neurons)
+        window_block(b, n.n_neurons)
         assert (win in b.live) == (pinch == "large_blocks")
         b.refuse = lambda size: False
         n.run(70)

@@ -3,12 +3,11 @@ pick among resident grids, plasticity windows, captured graphs and single steps
 change no result, so they are held by what they leave on the device and by the
 time of one form against another, with a margin well below the ratio that a
 wrong choice gives."""
-import time
-
 import numpy as np
 import pytest
 
 import workloads
+from device_blocks import Blocks, WIN_P0, window_block
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +35,31 @@ def test_the_neuron_update_is_one_wave_at_any_block_size(eng):
                 ms[block] = min(ms.get(block, 1e9), n.profile()["neuron"][1])
                 n.set_profile(False)
         assert max(ms[128], ms[32]) < 1.3 * ms[256], ms
+
+
+def _saturated(**kw):
+    """2x2 columns of 400 neurons that run away, and stay so without a
+    long-term update."""
+    return workloads.custom(grid_x=2, grid_y=2, neurons_per_col=400, exc_per_col=320, fanout=400, pct_ring=(40, 30, 20, 10),
+                            seed=67, w_exc0_q16=8 * 65536, thal_per_col_per_ms=2, deriv_period_ms=0, **kw)
+
+
+def test_a_resident_grid_is_not_queued_for_a_net_that_stays_busy(eng):
+    """What the last window queued says where its steps begin: a call from rest
+    queues a bounded number of them, a call of a net known to be busy none,
+    however many steps are left."""
+    with Blocks() as b, eng.Network(_saturated(), raster_capacity=0) as n, eng.Network(_saturated(), raster_capacity=0) as ref:
+        N = n.n_neurons
+        ref.set_launch(dense_permille=251)             # no resident grid, no windows
+        n.run(3000)
+        last = int(b.words(window_block(b, N))[WIN_P0])
+        assert 0 <= last < 50 * 32
+        n.run(3000)
+        assert int(b.words(window_block(b, N))[WIN_P0]) == last
+        ref.run(6000)
+        assert n.counters() == ref.counters() and n.counters()["spikes"] > 1000 * N
+        for x, y in zip(n.weights() + tuple(n.neurons().values()), ref.weights() + tuple(ref.neurons().values())):
+            assert np.array_equal(x, y)
+        n.reset()
+        n.run(20)                                      # quiet again: tried from its first step
+        assert int(b.words(window_block(b, N))[WIN_P0]) == 0
