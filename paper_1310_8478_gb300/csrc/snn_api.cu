@@ -60,6 +60,7 @@ constexpr int64_t kLightMinSynapses = 64 << 20;    // deferred dense steps have 
 constexpr int kResMaxParts = 8;                    // blocks per column of a resident grid
 constexpr uint32_t kResQueue = 32;                 // windows that a call queues on a resident grid at first
 constexpr int64_t kResRetry = 200;                 // steps from one that was too busy to the next try
+constexpr uint32_t kResThalMax = 0xffffffffu / kWinSteps;   // drive events of a column per step: a window's fit 32 bits
 constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
 constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
@@ -641,7 +642,6 @@ int clear_window(snn_net *net)
     DevWindow none{};
     none.p1 = -1;
     none.defer_from = kNoDefer;
-    none.polls = kBarrierPolls;
     if (net->dn.I2) SNN_CUDA(cudaMemsetAsync(net->dn.I2, 0, (size_t)net->N * 4, net->stream));
     SNN_CUDA(cudaMemcpyAsync(net->dn.win, &none, sizeof none, cudaMemcpyHostToDevice, net->stream));
     return SNN_OK;
@@ -685,6 +685,9 @@ int resident_grid(snn_net *net, int *parts_out)
         *parts_out = (int)blocks;
         return per_sm >= 1 ? (int)blocks : 0;
     }
+    // (a product in 64 bits in the kernel cost its delivery a tenth: 16x16 torus
+    // of the paper's columns, 50 steps 826 us, 900)
+    if (net->cfg.thal_per_col_per_ms > kResThalMax) return 0;
     int parts = kResMaxParts;
     if (dn.C == 1 && !f64) parts = 1;
     for (; parts >= 1; --parts) {

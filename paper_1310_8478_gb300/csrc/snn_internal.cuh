@@ -26,7 +26,6 @@ constexpr int kWinSteps = 50;                // most steps of a plasticity windo
 constexpr int kWinBits = 56;                 // spike bits of a train word (the top 8 bits hold a lag)
 constexpr int kWinSlots = 64;                // steps of spike bits kept
 constexpr int kNoDefer = 0x7fffffff;         // DevWindow::defer_from while the plasticity is immediate
-constexpr int kBarrierPolls = 1 << 22;       // DevWindow::polls: about two seconds
 static_assert(kWinSteps <= kWinBits && kWinBits <= kWinSlots, "a window's steps must fit its train words");
 
 // Device counters and per-step bookkeeping (one struct, device memory).
@@ -62,7 +61,6 @@ struct DevWindow {
     // a window run by a resident grid (snn_resident.cu)
     int steps_done;                  // steps it ran
     unsigned bar;                    // arrivals at the grid barrier (0 between two grids)
-    int polls;                       // looks at it after which a block gives up
     unsigned long long cnt[kWinSlots];   // spikes of step p0 + k: exc | inh << 32
     unsigned long long last_deg;     // in-degrees of the last step's spikes (0 between two grids)
 };

@@ -42,6 +42,7 @@ constexpr uint32_t kEmitList = 4096;         // spikes listed at a time
 constexpr uint32_t kResItems = 2048;         // pending (row, delay) items of a block
 constexpr int kResFlight = 4;                // buckets of a group of lanes in flight
 constexpr uint32_t kResThal = 512;           // thalamic events of a column drawn ahead
+constexpr int kBarrierPolls = 1 << 22;       // about two seconds, then the kernel gives up
 
 __host__ __device__ __forceinline__ uint32_t res_slice(uint32_t npc, uint32_t parts) { return (npc + parts - 1) / parts; }
 
@@ -57,20 +58,20 @@ size_t resident_smem_bytes(uint32_t npc, uint32_t parts, bool fp64, bool lists)
            + (size_t)(kResBlock / 32) * 64 * 4;                // per warp: a tile's buckets
 }
 
-// All blocks of the grid; false when one of them did not come within `polls`
-// looks.  The arrival
-// releases and the end acquires for the whole block (thread 0 behind and
-// before a block barrier); the polls between are relaxed.
-__device__ __forceinline__ bool grid_barrier(DevWindow *win, unsigned target, int polls, int *s_ok)
+// All blocks of the grid; false when one of them did not come within
+// kBarrierPolls looks.  The arrival releases and the end acquires for the whole
+// block (thread 0 behind and before a block barrier); the polls between are
+// relaxed.  Arrivals count from 0; a test starts them below.
+__device__ __forceinline__ bool grid_barrier(DevWindow *win, unsigned target, int *s_ok)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&win->bar) : "memory");
-        int left = polls;
+        int left = kBarrierPolls;
         unsigned seen;
         do {
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&win->bar) : "memory");
-        } while (seen < target && --left);
+        } while ((int)(seen - target) < 0 && --left);
         *s_ok = left != 0;
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
     }
@@ -111,7 +112,6 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
     const int D = (int)n.D;
     const uint32_t dmask = (2u << D) - 2u;
     const bool more = gridDim.x > 1;
-    const int polls = win->polls;
 
     F *const s_v = reinterpret_cast<F *>(smem_i4);
     F *const s_u = s_v + ns_max;
@@ -154,7 +154,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
         return c * n.npc +
                draw_below(philox10(make_uint4((uint32_t)t, c, 1u, e - c * n.thal_per_col), n.seed_lo, n.seed_hi).x, n.npc);
     };
-    const bool drawn = (uint64_t)steps * thal <= kResThal;      // (thal: up to 2^31 - 1)
+    const bool drawn = (uint32_t)steps * thal <= kResThal;      // (no net has more than fit 32 bits: kResThalMax)
     if (drawn)
         for (uint32_t e = threadIdx.x; e < (uint32_t)steps * thal; e += kResBlock) {
             const uint32_t k = e / thal;
@@ -373,7 +373,7 @@ __device__ __forceinline__ void resident_body(const DevNet &n, int p0, int steps
             s_fired[0] = s_fired[1] = 0;
         }
         if (more) {
-            if (!(ok = grid_barrier(win, (unsigned)(k + 1) * gridDim.x, polls, &s_ok))) break;
+            if (!(ok = grid_barrier(win, (unsigned)(k + 1) * gridDim.x, &s_ok))) break;
         } else {
             __syncthreads();
         }

@@ -2,7 +2,7 @@
 
 WIN_BYTES = 768        # header of a window block, rounded up
 WIN_P0 = 0             # its words: first step of the last window opened
-WIN_POLLS = 7          # limit of the grid barrier
+WIN_BAR = 6            # arrivals at the grid barrier
 
 
 class Blocks:

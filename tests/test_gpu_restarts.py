@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import workloads
-from device_blocks import Blocks, WIN_POLLS, up, window_block
+from device_blocks import Blocks, WIN_BAR, up, window_block
 from test_gpu_parity import assert_same_run
 
 pytestmark = pytest.mark.gpu
@@ -53,8 +53,8 @@ def test_a_restart_clears_both_inputs_of_a_resident_grid(eng, orc, restart):
 
 
 def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
-    """A limit of one look: the first block at the barrier gives up, and none
-    waits longer."""
+    """Arrivals that start a million short: every block gives up at its first
+    barrier."""
     import torch
     cfg = _cfg(4, 3, 130, 60, seed=92, thal_per_col_per_ms=2, deriv_period_ms=70)
     o = orc.Oracle(cfg)
@@ -63,7 +63,7 @@ def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
         n.run(30)
         state = n.save_state()
         for restart in ("reset", "load"):
-            b.words(window_block(b, n.n_neurons))[WIN_POLLS] = 1
+            b.words(window_block(b, n.n_neurons))[WIN_BAR] = -1000000
             torch.cuda.synchronize()
             for _ in range(2):
                 with pytest.raises(eng.snn.SnnError) as e:
@@ -83,7 +83,7 @@ def test_a_grid_barrier_that_runs_out_is_an_error_until_a_restart(eng, orc):
 
 def test_a_drive_whose_events_per_window_pass_32_bits(eng):
     """50 steps of 85 899 346 events are 4 more than 2^32: too many to be drawn
-    ahead, in steps of a resident grid against the step kernels'."""
+    ahead by a resident grid; one call against short ones."""
     cfg = _cfg(1, 1, 300, 20, seed=93, thal_per_col_per_ms=85899346, thal_amp_q16=2, wmax_q16=65536, w_exc0_q16=65536)
     with eng.Network(cfg, raster_capacity=1 << 16) as a, eng.Network(cfg, raster_capacity=1 << 16) as b:
         a.run(50)
