@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -63,6 +64,9 @@ constexpr int64_t kResRetry = 200;                 // steps from one that was to
 constexpr uint32_t kResThalMax = 0xffffffffu / kWinSteps;   // drive events of a column per step: a window's fit 32 bits
 constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
 constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
+constexpr uint64_t kResPass = 2 << 20;             // plastic synapses likewise of a net with compact targets
+constexpr uint64_t kResPassClosing = 4 << 20;      // ... in windows that end with a period
+constexpr int kRecent = 8, kRecentMs = 40;         // a net's recent spikes: eight counts of 40 ms
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
 // Device staging of snn_read_synapses_noalloc: target, weight and sd words,
@@ -183,6 +187,9 @@ struct snn_net {
     DevCounters *host_ctr = nullptr;
     bool host_ctr_known = false;    // [1] is what the device holds
     int64_t last_fired = 0;         // spikes of step t - 1 as the last read-back told; -1: not known
+    int64_t seen_spikes = 0;        // spikes and step of the last read-back
+    int32_t seen_t = 0;
+    int64_t recent[kRecent] = {0};  // spikes by kRecentMs of the read-backs that told them, the last kRecent
     char *read_stage = nullptr;     // kReadStage bytes of small read-backs
     char *stim_stage = nullptr;
     size_t stim_stage_cap = 0;
@@ -1160,16 +1167,31 @@ void close_window(snn_net *net)
 
 // the steps of a call on a resident grid: false when the net takes the step
 // kernels (no such grid, a profile, a probe, or a call of fewer than four
-// steps, which would pay for a window's pass each)
+// steps, which would pay for a window's pass each, or windows too short for
+// the net)
 bool resident_call(const snn_net *net, uint32_t left)
 {
     if (!net->res_grid || net->profile || net->dn.probe_n || left < 4) return false;
-    if (net->tgt16) return true;
+    const uint32_t P = net->cfg.deriv_period_ms;
+    const uint64_t steps = std::min<uint32_t>({left, kWinSteps, P ? P : left});
     // with target lists nothing bounds the synapses: the passes (15 us per
     // million synapses and window) must cost less than the steps save (20 us
     // each)
-    const uint32_t P = net->cfg.deriv_period_ms;
-    return (uint64_t)std::min<uint32_t>({left, kWinSteps, P ? P : left}) * kResListsPass >= (uint64_t)net->dn.S;
+    if (!net->tgt16) return steps * kResListsPass >= (uint64_t)net->dn.S;
+    // Compact nets save 10 to 20 us per step for 8 us per million plastic
+    // synapses and pass.  us per step in calls of 4, 8, 16 and 25 steps, this
+    // grid and step kernels: 16x16 torus of the paper's columns 105 54 36 23
+    // and 41 29 33 26, 16x16 of the benchmark's with M = 100 71 48 27 22 and 29
+    // 28 27 26, 8x8 of the paper's 41 23 16 11 and 31 24 25 20.  A window that
+    // ends with a period does its long-term update, which the step kernels
+    // have to do too (periods of 2, 4, 7 and 10 ms: 16x16 217 113 71 52 and 173
+    // 97 68 59, 8x8 79 42 28 21 and 69 44 38 31, 4x4 with M = 1125 102 53 33 24
+    // and 75 51 40 34).
+    if (P && steps == P) return steps * kResPassClosing >= (uint64_t)net->n_rin;
+    // a row whose source has been silent for the reach of the amounts costs
+    // nothing: of a net that hardly fires few rows are walked
+    const int64_t live = std::min<int64_t>(net->N, std::accumulate(net->recent, net->recent + kRecent, (int64_t)0));
+    return (double)(steps * kResPass) >= (double)net->n_rin * live / net->N;
 }
 
 // `steps` more steps from t0 as one window on the resident grid (it runs as
@@ -1219,11 +1241,34 @@ int read_counters_raw(snn_net *net, DevCounters *hc)
     return SNN_OK;
 }
 
-// the spikes of the last step before t, from counters read behind it
+// The spikes of the last step before t, from counters read behind it.
 int64_t fired_last(const DevCounters &c, int32_t t)
 {
     const int32_t *x = c.step_cnt[(t - 1) & 1];
     return t > 0 ? (int64_t)x[0] + x[1] : 0;
+}
+
+// What counters read behind step t - 1 tell the rules on the next call's
+// steps: the last step's spikes, and those within the reach of the amounts.
+void note_activity(snn_net *net, const DevCounters &c)
+{
+    static_assert(kRecent * kRecentMs >= kLut + 31, "the largest lag and delay");
+    const int32_t now = net->t / kRecentMs;
+    for (int32_t k = std::max(net->seen_t / kRecentMs + 1, now - kRecent + 1); k <= now; ++k) net->recent[k % kRecent] = 0;
+    net->recent[now % kRecent] += (int64_t)c.spikes - net->seen_spikes;
+    net->last_fired = fired_last(c, net->t);
+    net->seen_spikes = (int64_t)c.spikes;
+    net->seen_t = net->t;
+}
+
+// of counters that start elsewhere, at step t, with `recent` spikes before
+void start_activity(snn_net *net, int32_t t, int64_t spikes, int64_t recent, int64_t last_fired)
+{
+    std::fill(net->recent, net->recent + kRecent, 0);
+    net->recent[t / kRecentMs % kRecent] = recent;
+    net->last_fired = last_fired;
+    net->seen_spikes = spikes;
+    net->seen_t = t;
 }
 
 // end of a run: the counters are copied out behind the steps and read after
@@ -1236,7 +1281,7 @@ int finish_run(snn_net *net, bool copied)
     }
     SNN_CUDA(cudaGetLastError());
     net->host_ctr_known = true;
-    net->last_fired = fired_last(net->host_ctr[1], net->t);
+    note_activity(net, net->host_ctr[1]);
     net->stim_in_flight = false;
     if (net->profile && net->ev_used) {
         for (size_t i = 0; i + 1 < net->ev_used; i += 2) {
@@ -2337,7 +2382,7 @@ int snn_batch_run(snn_batch *b, uint32_t n_ms)
         n->ltp_owed = true;
         DevCounters hc{};
         SNN_TRY(read_counters_raw(n, &hc));
-        n->last_fired = fired_last(hc, n->t);
+        note_activity(n, hc);
         if (hc.error && rc == SNN_OK) {
             set_error("device error word %d", hc.error);
             rc = (hc.error == SNN_ETIMEOUT || hc.error == SNN_EBOUNDS) ? hc.error : SNN_ECUDA;
@@ -2510,7 +2555,7 @@ int snn_reset(snn_net *net)
     SNN_CUDA(cudaStreamSynchronize(s));
     net->t = 0;
     net->host_ctr_known = false;
-    net->last_fired = 0;
+    start_activity(net, 0, 0, 0, 0);
     net->weights_moved = false;
     net->ltp_owed = false;
     net->dn.raster_t0 = 0;
@@ -2939,6 +2984,7 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     // the raster restarts at the checkpoint's step
     DevCounters hc{};
     std::memcpy(&hc, (const char *)host_buf + need - sizeof(DevCounters), sizeof hc);
+    start_activity(net, h.t, (int64_t)hc.spikes, net->N, -1);
     hc.raster_total = 0;
     hc.raster_dropped = 0;
     hc.raster_first_drop_t = 0x7fffffff;

@@ -3,6 +3,8 @@ pick among resident grids, plasticity windows, captured graphs and single steps
 change no result, so they are held by what they leave on the device and by the
 time of one form against another, with a margin well below the ratio that a
 wrong choice gives."""
+import time
+
 import numpy as np
 import pytest
 
@@ -63,3 +65,24 @@ def test_a_resident_grid_is_not_queued_for_a_net_that_stays_busy(eng):
         n.reset()
         n.run(20)                                      # quiet again: tried from its first step
         assert int(b.words(window_block(b, N))[WIN_P0]) == 0
+
+
+@pytest.mark.parametrize("steps,period", [(4, 1000), (200, 2)], ids=["short_calls", "short_periods"])
+def test_windows_too_short_for_a_net_take_the_step_kernels(eng, steps, period):
+    """16x16 torus of the paper's columns, 41 M plastic synapses: the pass of a
+    window of 4 steps takes ten times its steps (105 us per step, 41 with step
+    kernels), that of a period of 2 ms more than its steps' own update."""
+    cfg = workloads.workload("paper_16x16", deriv_period_ms=period)
+    with eng.Network(cfg, raster_capacity=0) as n, eng.Network(cfg, raster_capacity=0) as ref:
+        us = {}
+        for k, net in (("n", n), ("ref", ref)):
+            if k == "ref":
+                net.set_launch(dense_permille=251)     # no resident grid
+            net.run(300)
+            for _ in range(5):
+                t0 = time.perf_counter()
+                for _ in range(max(1, 60 // steps)):
+                    net.run(steps)
+                us[k] = min(us.get(k, 1e9), time.perf_counter() - t0)
+        assert us["n"] < 1.15 * us["ref"], us
+        assert n.counters() == ref.counters()
