@@ -64,8 +64,9 @@ constexpr int64_t kResRetry = 200;                 // steps from one that was to
 constexpr uint32_t kResThalMax = 0xffffffffu / kWinSteps;   // drive events of a column per step: a window's fit 32 bits
 constexpr uint32_t kResListsThal = 4096;           // drive events per step that every block of a net with lists may look at
 constexpr uint64_t kResListsPass = 1 << 20;        // synapses of a net with lists per step of its windows, at most
-constexpr uint64_t kResPass = 2 << 20;             // plastic synapses likewise of a net with compact targets
-constexpr uint64_t kResPassClosing = 4 << 20;      // ... in windows that end with a period
+constexpr double kResPass = 1.2e6;                 // plastic synapses likewise of a net with compact targets, in silence
+constexpr double kResPassBusy = 50e6;              // ... and for every spike per neuron and ms
+constexpr double kResPassClosing = 4e6;            // ... in windows that end with a period
 constexpr int kRecent = 8, kRecentMs = 40;         // a net's recent spikes: eight counts of 40 ms
 constexpr uint32_t kStateMagic = 0x534e4e31u;  // "SNN1"
 
@@ -1178,20 +1179,27 @@ bool resident_call(const snn_net *net, uint32_t left)
     // million synapses and window) must cost less than the steps save (20 us
     // each)
     if (!net->tgt16) return steps * kResListsPass >= (uint64_t)net->dn.S;
-    // Compact nets save 10 to 20 us per step for 8 us per million plastic
-    // synapses and pass.  us per step in calls of 4, 8, 16 and 25 steps, this
-    // grid and step kernels: 16x16 torus of the paper's columns 105 54 36 23
-    // and 41 29 33 26, 16x16 of the benchmark's with M = 100 71 48 27 22 and 29
-    // 28 27 26, 8x8 of the paper's 41 23 16 11 and 31 24 25 20.  A window that
-    // ends with a period does its long-term update, which the step kernels
-    // have to do too (periods of 2, 4, 7 and 10 ms: 16x16 217 113 71 52 and 173
-    // 97 68 59, 8x8 79 42 28 21 and 69 44 38 31, 4x4 with M = 1125 102 53 33 24
-    // and 75 51 40 34).
-    if (P && steps == P) return steps * kResPassClosing >= (uint64_t)net->n_rin;
+    // Compact nets save 10 to 30 us per step, the more the busier they are, for
+    // 8 us per million plastic synapses and pass.  As many steps per call at
+    // which both forms take the same: 8x8 torus of the paper's columns (10 M
+    // plastic synapses, 2.6 % firing) 7, with M = 300 (15 M, 3.8 %) 5, 16x16
+    // (41 M, 2.6 %) 16, with M = 300 (61 M, 3.8 %) 20, with M = 250 (51 M, 5.3 %)
+    // 12, 16x17 with M = 275 (60 M, 6.9 %) 13, 16x16 of the benchmark's columns
+    // with M = 100 (26 M, 0.5 %) 15.  us per step of the first 16x16 in calls of
+    // 4, 8, 16 and 25: 105 61 39 30 and 42 40 39 39.  A window that ends with a
+    // period does its long-term update, which the step kernels have to do too
+    // (periods of 2, 4, 7 and 10 ms: 16x16 217 113 71 52 and 173 97 68 59, 8x8
+    // 79 42 28 21 and 69 44 38 31, 4x4 with M = 1125 102 53 33 24 and 75 51 40
+    // 34).
+    if (P && steps == P) return (double)steps * kResPassClosing >= (double)net->n_rin;
     // a row whose source has been silent for the reach of the amounts costs
     // nothing: of a net that hardly fires few rows are walked
-    const int64_t live = std::min<int64_t>(net->N, std::accumulate(net->recent, net->recent + kRecent, (int64_t)0));
-    return (double)(steps * kResPass) >= (double)net->n_rin * live / net->N;
+    const double spikes = (double)std::accumulate(net->recent, net->recent + kRecent, (int64_t)0);
+    // (spikes per neuron and ms, not long after the net fell silent)
+    const int now = net->t / kRecentMs % kRecent, part = net->t % kRecentMs;
+    const double late = (double)(net->recent[now] + net->recent[(now + kRecent - 1) % kRecent]) / (kRecentMs + part);
+    const double rate = std::min(spikes / ((kRecent - 1) * kRecentMs + part), 4 * late) / net->N;
+    return (double)steps * (kResPass + kResPassBusy * rate) >= (double)net->n_rin * std::min(1.0, spikes / net->N);
 }
 
 // `steps` more steps from t0 as one window on the resident grid (it runs as
