@@ -53,6 +53,7 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int64_t kWinMinSynapses = 8ll << 20;   // plastic synapses from which a net takes plasticity windows
 constexpr int64_t kWinMinSparse = 40ll << 20;    // ... when its sparse steps run in the step kernels too
+constexpr uint32_t kWinShort = 16;                 // steps of a call below which they have to be dense ones
 constexpr int64_t kReadChunk = 16ll << 20;         // synapses read back per chunk
 constexpr size_t kReadStage = 256 << 10;           // bytes of a net's pinned memory for small read-backs
 constexpr uint32_t kMergeMaxNeurons = 300000;      // up to here a net's delivery and dense pass are one launch
@@ -1019,9 +1020,13 @@ void launch_flush(snn_net *net)
 // sd_rev, the other reads the weights and accumulates into I and sd.  While
 // profiling, every step runs its kernels one after another, so that each
 // kernel's CUDA-event time is its own.
-void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
+void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t, bool in_window = false)
 {
-    const DevNet &dn = net->dn;
+    DevNet dn = net->dn;
+    // outside a window no kernel asks for one, and none is launched for its dense
+    // steps (36x36 columns with M = 100, single steps 64.9 us, 58.8 without)
+    const bool windows = in_window || !exact_t;
+    if (!windows) dn.win = nullptr;
     const int *t_now = &net->ctr->t_slot[t & 1];
     int *t_next = &net->ctr->t_slot[(t & 1) ^ 1];
     const snn_launch &L = net->launch;
@@ -1091,7 +1096,7 @@ void launch_step(snn_net *net, int32_t t, cudaStream_t s, bool exact_t)
         mark(4, s);
         if (!both) k_dense<<<net->dense_grid, L.dense_block, dense_smem(dn.npc, L.dense_block), s>>>(dn, t_now);
         launched += both ? 0 : 1;
-        if (net->light_grid && !prof) {
+        if (net->light_grid && windows && !prof) {
             k_dense_light<<<net->light_grid, kDenseLightBlock, dense_light_smem_bytes(dn.npc, kDenseLightBlock), s>>>(dn, t_now);
             ++launched;
         }
@@ -1122,13 +1127,25 @@ uint32_t effective_graph_len(const snn_net *net)
     return L & ~1u;
 }
 
+// Whether the step kernels' steps of a call take windows.  A short one costs
+// its launches and, when it defers, a pass for few steps: it has to be known to
+// be dense (us per step in calls of 4, 8 and 12 steps, with windows and without
+// them: 25x28 columns with M = 90, quiet, 42 50 37 and 38 47 35; 36x36 with M =
+// 100 75 53 54 and 67 47 47; saturated nets 18x18 with M = 1125 549 449 414 and
+// 837 835 834).  From 16 steps on the busy ones gain more than the others lose
+// (23x23 with M = 100, 8 % firing, 71 and 80; 36x36 55 and 53).
+bool windows_call(const snn_net *net, uint32_t left)
+{
+    if (!net->step_windows || net->profile) return false;
+    return left >= kWinShort || net->last_fired < 0 || net->last_fired >= (int64_t)net->dn.dense_min_spikes;
+}
+
 // The next steps of a call as a plasticity window, at most to the end of the
 // period (the window's pass then runs the long-term update); 0: no window
 // (fewer than four steps could not share the pass with an immediate first
 // one; while profiling, every step's kernels do their own work).
 uint32_t window_steps(const snn_net *net, uint32_t left)
 {
-    if (!net->step_windows || net->profile) return 0;
     const uint32_t P = net->cfg.deriv_period_ms;
     uint32_t n = std::min<uint32_t>(left, kWinSteps);
     if (P) n = std::min<uint32_t>(n, P - (uint32_t)net->t % P);
@@ -1331,7 +1348,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
     uint32_t left = n_ms;
     const uint32_t P = net->cfg.deriv_period_ms;
     uint32_t window = 0;                       // steps left of the open window
-    const bool resident = resident_call(net, left);
+    const bool resident = resident_call(net, left), windows = windows_call(net, left);
     int64_t resident_from = net->t;            // the step from which the resident grid is tried
     uint32_t queue = kResQueue;                // windows of the next try
     int64_t fired = net->last_fired;           // spikes of the step before t; -1: not known
@@ -1395,7 +1412,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             copied = true;
             continue;
         }
-        if (!window && (window = window_steps(net, left)) != 0) open_window(net, window);
+        if (windows && !window && (window = window_steps(net, left)) != 0) open_window(net, window);
         const uint32_t ahead = window ? window : left;
         // the first step from t on that closes a period (t' > 0, t' % P == 0)
         const int64_t closing = P ? std::max<int64_t>((int64_t)P, ((int64_t)t + P - 1) / P * P) : INT64_MAX;
@@ -1412,7 +1429,7 @@ int run_steps(snn_net *net, uint32_t n_ms, bool count_before = false)
             left -= L;
             net->ltp_owed = true;
         } else {
-            launch_step(net, t, net->stream, true);
+            launch_step(net, t, net->stream, true, window != 0);
             SNN_CUDA(cudaGetLastError());
             net->t += 1;
             left -= 1;

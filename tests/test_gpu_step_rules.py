@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import workloads
-from device_blocks import Blocks, WIN_P0, window_block
+from device_blocks import Blocks, WIN_BYTES, WIN_P0, up, window_block
 
 pytestmark = pytest.mark.gpu
 
@@ -86,3 +86,28 @@ def test_windows_too_short_for_a_net_take_the_step_kernels(eng, steps, period):
                 us[k] = min(us.get(k, 1e9), time.perf_counter() - t0)
         assert us["n"] < 1.15 * us["ref"], us
         assert n.counters() == ref.counters()
+
+
+def _blocks_opened(eng, cfg, calls):
+    """First steps of the windows that a net's calls opened (of those that left
+    a trace), in a net whose steps run in the step kernels."""
+    seen = []
+    with Blocks() as b, eng.Network(cfg, raster_capacity=0) as n:
+        N = n.n_neurons
+        size = WIN_BYTES + 2 * up(8 * N) + up(64 * 4 * ((N + 31) // 32))
+        win = b.words([p for p, x in b.live.items() if x == size][0])
+        for steps in calls:
+            n.run(steps)
+            seen.append(int(win[WIN_P0]))
+        return seen, n.counters()
+
+
+def test_short_calls_open_windows_for_dense_steps_only(eng):
+    """42 M plastic synapses, too many columns for a resident grid: a quiet net's
+    calls of fewer than 16 steps open no window, a saturated one's do."""
+    mix = dict(grid_x=23, grid_y=23, neurons_per_col=1000, exc_per_col=800, fanout=100, pct_ring=(76, 12, 8, 4), seed=7)
+    quiet, c = _blocks_opened(eng, workloads.custom(**mix), [16, 4, 15, 1, 17])
+    assert quiet == [0, 0, 0, 0, 36] and c["spikes"] > 1000
+    busy, c = _blocks_opened(eng, workloads.custom(**mix, w_exc0_q16=10 * 65536, thal_per_col_per_ms=400,
+                                                   thal_amp_q16=60 * 65536), [20, 4, 4])
+    assert busy == [0, 20, 24] and c["spikes"] > 28 * 529000 // 4
