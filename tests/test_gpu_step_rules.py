@@ -21,22 +21,33 @@ def eng():
     return e
 
 
+def _soon_below(limit, ratio, rounds=8):
+    """A ratio of two times, measured in turn until it is below the limit (a
+    machine's noise goes away, a wrong choice does not)."""
+    seen = []
+    for _ in range(rounds):
+        seen.append(ratio())
+        if seen[-1] < limit:
+            return
+    raise AssertionError((limit, seen))
+
+
 def test_the_neuron_update_is_one_wave_at_any_block_size(eng):
     """ms of the update of 5.1 M neurons, small blocks against the default
     (blocks that hold the spike lists of 32 warps each take 1.5 times as long at
     128 threads and 2.4 times at 32; blocks of their own size 1.0 and 1.1)."""
     with eng.Network(workloads.workload("grid64_m16"), raster_capacity=0) as n:
         n.run(20)
-        ms = {}
-        for _ in range(3):
-            for block in (256, 128, 32):
-                n.set_launch(neuron_block=block)
-                n.step()
-                n.set_profile(True)
-                n.run(10)
-                ms[block] = min(ms.get(block, 1e9), n.profile()["neuron"][1])
-                n.set_profile(False)
-        assert max(ms[128], ms[32]) < 1.3 * ms[256], ms
+
+        def ms(block):
+            n.set_launch(neuron_block=block)
+            n.step()
+            n.set_profile(True)
+            n.run(10)
+            t = n.profile()["neuron"][1]
+            n.set_profile(False)
+            return t
+        _soon_below(1.3, lambda: max(ms(128), ms(32)) / ms(256))
 
 
 def _saturated(**kw):
@@ -74,21 +85,22 @@ def test_windows_too_short_for_a_net_take_the_step_kernels(eng, steps, period):
     kernels), that of a period of 2 ms more than its steps' own update."""
     cfg = workloads.workload("paper_16x16", deriv_period_ms=period)
     with eng.Network(cfg, raster_capacity=0) as n, eng.Network(cfg, raster_capacity=0) as ref:
-        us = {}
-        for k, net in (("n", n), ("ref", ref)):
-            if k == "ref":
-                net.set_launch(dense_permille=251)     # no resident grid
-            net.run(300)
-            for _ in range(5):
-                t0 = time.perf_counter()
-                for _ in range(max(1, 60 // steps)):
-                    net.run(steps)
-                us[k] = min(us.get(k, 1e9), time.perf_counter() - t0)
-        assert us["n"] < 1.15 * us["ref"], us
+        ref.set_launch(dense_permille=251)             # no resident grid
+
+        def run(net):
+            t0 = time.perf_counter()
+            for _ in range(max(1, 200 // steps)):
+                net.run(steps)
+            return time.perf_counter() - t0
+        n.run(300)
+        ref.run(300)
+        _soon_below(1.1, lambda: run(n) / run(ref))
+        while ref.counters()["t"] < n.counters()["t"]:
+            ref.run(steps)
         assert n.counters() == ref.counters()
 
 
-def _blocks_opened(eng, cfg, calls):
+def _windows_opened(eng, cfg, calls):
     """First steps of the windows that a net's calls opened (of those that left
     a trace), in a net whose steps run in the step kernels."""
     seen = []
@@ -106,8 +118,46 @@ def test_short_calls_open_windows_for_dense_steps_only(eng):
     """42 M plastic synapses, too many columns for a resident grid: a quiet net's
     calls of fewer than 16 steps open no window, a saturated one's do."""
     mix = dict(grid_x=23, grid_y=23, neurons_per_col=1000, exc_per_col=800, fanout=100, pct_ring=(76, 12, 8, 4), seed=7)
-    quiet, c = _blocks_opened(eng, workloads.custom(**mix), [16, 4, 15, 1, 17])
+    quiet, c = _windows_opened(eng, workloads.custom(**mix), [16, 4, 15, 1, 17])
     assert quiet == [0, 0, 0, 0, 36] and c["spikes"] > 1000
-    busy, c = _blocks_opened(eng, workloads.custom(**mix, w_exc0_q16=10 * 65536, thal_per_col_per_ms=400,
+    busy, c = _windows_opened(eng, workloads.custom(**mix, w_exc0_q16=10 * 65536, thal_per_col_per_ms=400,
                                                    thal_amp_q16=60 * 65536), [20, 4, 4])
     assert busy == [0, 20, 24] and c["spikes"] > 28 * 529000 // 4
+
+
+M61 = dict(grid_x=33, grid_y=21, fanout=61, pct_ring=(40, 30, 20, 10), seed=7)      # 42 M plastic synapses, 1.4 Hz
+
+
+def test_windows_from_an_odd_step_come_back_to_even_ones(eng):
+    """Captured chunks begin at even steps: a quiet net's odd step runs alone, an
+    unknown one's window ends before an even step."""
+    cfg = workloads.custom(**M61)
+    quiet, _ = _windows_opened(eng, cfg, [1, 201])
+    assert quiet == [0, 152]                           # 1 alone, 2, 52, 102, 152
+    with Blocks() as b, eng.Network(cfg, raster_capacity=0) as n, eng.Network(cfg, raster_capacity=0) as other:
+        N = n.n_neurons
+        other.run(201)
+        n.load_state(other.save_state())
+        size = WIN_BYTES + 2 * up(8 * N) + up(64 * 4 * ((N + 31) // 32))
+        first = [p for p, x in b.live.items() if x == size][0]
+        n.run(103)
+        assert int(b.words(first)[WIN_P0]) == 300      # 201, 250, 300
+        other.run(103)
+        assert all(n.counters()[k] == other.counters()[k] for k in ("t", "spikes", "e_all", "e_exc", "l_exc"))
+        for x, y in zip(n.neurons().values(), other.neurons().values()):
+            assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("steps", [30, 40])
+def test_a_graph_length_that_does_not_divide_a_window_costs_no_single_steps(eng, steps):
+    """us per step against the default length: 34.1 and 33.4 to 30.8 to 32.4 with
+    the rest of a window launched step by step, 30.8 to 30.7 as a graph."""
+    with eng.Network(workloads.custom(**M61, deriv_period_ms=0), raster_capacity=0) as n:
+        def us(length):
+            n.reset()
+            n.set_launch(graph_steps=length)
+            n.run(400)
+            t0 = time.perf_counter()
+            n.run(500)
+            return time.perf_counter() - t0
+        _soon_below(1.02, lambda: us(steps) / us(50))
