@@ -5,6 +5,9 @@ WIN_P0 = 0             # its words: first step of the last window opened
 WIN_BAR = 6            # arrivals at the grid barrier
 
 
+_hooks = []
+
+
 class Blocks:
     """The allocator hook on PyTorch's: remembers the blocks' sizes, refuses
     what `refuse` says, and gives nothing back before the end, so that a stale
@@ -30,6 +33,7 @@ class Blocks:
             self.gone.append(p)
             del self.live[p]
         snn.set_allocator(take, give)
+        _hooks.append(snn._allocator_refs)             # of nets that a failed test leaves open
         return self
 
     def __exit__(self, *exc):
