@@ -201,6 +201,7 @@ struct snn_net {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // chunks of graph_len steps, and of what they leave of a window
     uint32_t graph_len = 0;
     bool graphs_dirty = true;
+    bool tuning = false;            // launch shapes are being timed
     bool profile = false;
     std::vector<cudaEvent_t> ev_pool;
     std::vector<int> ev_kind;
@@ -1192,12 +1193,12 @@ void close_window(snn_net *net)
 }
 
 // the steps of a call on a resident grid: false when the net takes the step
-// kernels (no such grid, a profile, a probe, or a call of fewer than four
+// kernels (no such grid, launch shapes being timed, a profile, a probe, or a call of fewer than four
 // steps, which would pay for a window's pass each, or windows too short for
 // the net)
 bool resident_call(const snn_net *net, uint32_t left)
 {
-    if (!net->res_grid || net->profile || net->dn.probe_n || left < 4) return false;
+    if (!net->res_grid || net->tuning || net->profile || net->dn.probe_n || left < 4) return false;
     const uint32_t P = net->cfg.deriv_period_ms;
     const uint64_t steps = std::min<uint32_t>({left, kWinSteps, P ? P : left});
     // with target lists nothing bounds the synapses: the passes (15 us per
@@ -2540,6 +2541,7 @@ int snn_autotune(snn_net *net, uint32_t probe_ms, snn_launch *best)
     float best_ms = 1e30f;
     size_t best_i = 0;
     int rc = SNN_OK;
+    net->tuning = true;                  // the step kernels: a resident grid takes no shape from the candidates
     for (size_t i = 0; i < cand.size() && rc == SNN_OK; ++i) {
         net->launch = cand[i];
         net->dn.dense_min_spikes = dense_threshold(net->N, cand[i].dense_permille);
@@ -2556,6 +2558,7 @@ int snn_autotune(snn_net *net, uint32_t probe_ms, snn_launch *best)
         cudaEventElapsedTime(&ms, e0, e1);
         if (ms < best_ms) { best_ms = ms; best_i = i; }
     }
+    net->tuning = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != SNN_OK) return rc;

@@ -161,3 +161,21 @@ def test_a_graph_length_that_does_not_divide_a_window_costs_no_single_steps(eng,
             n.run(500)
             return time.perf_counter() - t0
         _soon_below(1.02, lambda: us(steps) / us(50))
+
+
+def test_autotuning_times_the_step_kernels(eng):
+    """A resident grid has one shape, so that its windows would tell nothing of
+    the candidates: it leaves trains in the window block, which stay untouched
+    here."""
+    import torch
+    cfg = workloads.custom(grid_x=2, grid_y=2, fanout=60, pct_ring=(40, 30, 20, 10), seed=8)
+    with Blocks() as b, eng.Network(cfg, raster_capacity=0) as n:
+        N = n.n_neurons
+        at = (WIN_BYTES + up(8 * N)) // 4
+        trains = b.words(window_block(b, N))[at:at + 2 * N]
+        trains[:] = 12345
+        torch.cuda.synchronize()
+        n.autotune(probe_ms=50)
+        assert int((trains != 12345).sum()) == 0
+        n.run(50)
+        assert int((trains == 12345).sum()) == 0
