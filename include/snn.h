@@ -266,11 +266,13 @@ int snn_step(snn_net *net);
  * single steps otherwise); returns after completion and the error-word check.
  * Inside a call the engine may take steps together, with the same results:
  * nets whose blocks all fit the GPU at once run windows of up to 50 steps as
- * one cooperative launch (calls of four steps or more, default
+ * one cooperative launch (calls of four steps or more, and of as many as pay for
+ * the windows' passes over the net's plastic synapses; default
  * dense_permille, staged_permille and ring_permille, no probe, no profile);
  * nets of 8 M plastic synapses or more (40 M when no such launch takes their
  * sparse steps) leave the STDP of busy steps to one pass
- * over the synapses per window.  Nothing is left to do when the call returns.
+ * over the synapses per window (calls of fewer than 16 steps only when the step
+ * before them was a dense one).  Nothing is left to do when the call returns.
  */
 int snn_run(snn_net *net, uint32_t n_ms);
 
@@ -390,8 +392,8 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n);
 /*
  * snn_autotune -- pick the fastest launch shape for this net: every candidate
  * shape (rows per dense block, resident blocks of the event-driven kernels,
- * neuron block, steps per graph) runs probe_ms steps from a reset, timed with
- * CUDA events; the best is kept and the net is left reset at t = 0.  Results
+ * neuron block, steps per graph) runs probe_ms steps from a reset in the step
+ * kernels, timed with CUDA events; the best is kept and the net is left reset at t = 0.  Results
  * never depend on the shape.  Generated nets only (SNN_ESTATE otherwise).
  * *best (may be NULL) receives the chosen shape.
  */

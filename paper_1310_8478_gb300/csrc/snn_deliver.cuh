@@ -16,8 +16,9 @@ namespace snn {
 // claimed two columns ahead, and its histories and last spikes are copied into
 // shared memory while this one is walked.  Bound by latency and instruction
 // issue (half of it) at 64 registers and two blocks of 512 threads per SM; with
-// three at 40 registers it spilled (busy 32x32 net: 142 against 129 us per
-// step), and five of 256 threads left a wave of 1024 columns two thirds full.
+// three at 40 registers it spilled (busy 32x32 net, before the walk by chunks:
+// 142 us per step, 129 with two), and five of 256 threads left a wave of 1024
+// columns two thirds full.
 // Tried for steps without depression: all 13 columns' input in shared memory
 // in the deferred dense step's kernel, which needs no distinction of targets
 // but flushes 13 columns (70 us at any rate on the 32x32 net).

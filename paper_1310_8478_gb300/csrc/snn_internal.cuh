@@ -646,9 +646,11 @@ __device__ __forceinline__ int bucket_lanes(const DevNet &n)
 
 // The warp's share of a block's `items`, tile by tile: a lane fetches an
 // item's bucket, then a lane takes a synapse, a group of 2^lg lanes a bucket,
-// kFlight buckets of every group in flight.  (A lane per 8-synapse chunk, with
-// a branch per synapse, took 2.5 times the instructions at M = 200, whose
-// buckets of 10 fill 0.6 of their chunks.)  Per synapse: x = begin(target word,
+// kFlight buckets of every group in flight.  (A lane per 8-synapse chunk with
+// a branch per synapse took 2.5 times the instructions at M = 200, whose
+// buckets of 10 fill 0.6 of their chunks; walk_chunks below adds zeros instead
+// of branching, and is the faster one there without depression.)  Per synapse:
+// x = begin(target word,
 // weight), then, behind the other synapses in flight, end(x, position).
 // `first` runs once under the first fetch.  w_ab: 64 words of the warp's own.
 // Returns the synapses walked (lane 0).

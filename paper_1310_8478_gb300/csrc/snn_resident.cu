@@ -17,11 +17,14 @@
 //
 // Bound by latency: per step a chain of a list, the buckets' bounds, their
 // synapses, the reductions' way to L2 under the barrier (1.6 us alone) and the
-// update.  us per step, with the step kernels before: one column of 1250
-// neurons 4.3 (21), in FP64 5.7 (33), 8x8 torus of the paper's columns 9.8
-// (54), 16x16 21 (62).  Tried without gain: delivering the next step's
+// update.  us per step of long calls, emission and pass included (in brackets
+// the step kernels before there were grids): one column of 1250 neurons 4.3
+// (21), in FP64 5.7 (33), 8x8 torus of the paper's columns 9.8 (54), 16x16 23
+// (62); of the last the grid itself takes 13 in the mean of the first 200 steps
+// and 16.6 in their busiest 50.  Tried without gain: delivering the next step's
 // arrivals from earlier spikes while the barrier fills, with three inputs in
-// turn (8x8 10.1, one column 4.9).
+// turn (8x8 10.1, one column 4.9).  The kernels need all of their 64 registers:
+// one more value held through a step shows in the delivery (see resident_grid).
 //
 // Nets with target lists have no columns in this sense: a block owns a slice of
 // all neurons, inhibitory rows are walked by delay like the others, and every

@@ -783,8 +783,11 @@ __device__ __forceinline__ void neuron_body(const DevNet &n, const int *t_now, i
     // while this one is updated (not in double: the registers spill, and the
     // FP64 units are the bound); its spikes collect in shared memory and leave
     // with one atomic per block.  HBM bound: 40 bytes per neuron, 4.1 M
-    // neurons in 29 us (41 us with a block per 2048 neurons, each waiting for
-    // its loads, its prefix, its atomics and its fence in turn).
+    // neurons in 26.6 us (41 us with a block per 2048 neurons, each waiting for
+    // its loads, its prefix, its atomics and its fence in turn).  The lists are
+    // as large as the block: with 32 warps' in every one, blocks of 128 threads
+    // and fewer did not all fit (5.1 M neurons, us at 256, 128, 64 and 32
+    // threads: 33 51 53 82; now 34 34 35 37).
     constexpr bool kAhead = sizeof(F) == 4;
     const uint32_t stride = part_threads(g) * 4u;
     __align__(16) int32_t iq[4], iq_n[4];
