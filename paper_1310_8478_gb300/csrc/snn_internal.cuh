@@ -328,12 +328,12 @@ __device__ __forceinline__ bool dense_selected(const DevNet &n, int t)
     return (uint32_t)(n.ring_cnt[2 * slot] + n.ring_cnt[2 * slot + 1]) >= n.dense_min_spikes;
 }
 
-// ms from `last` to t >= last, kLut - 1 at most (no amount there).  Without a
-// sign: from t = 2^30 on an int does not hold the distance to kNever.
-__device__ __forceinline__ int lag_of(int t, int last)
-{
-    return (int)min((uint32_t)t - (uint32_t)last, (uint32_t)(kLut - 1));
-}
+// ms from `last` to t >= last.  Without a sign: from t = 2^30 on an int does not
+// hold the distance to kNever.
+__device__ __forceinline__ uint32_t ms_since(int t, int last) { return (uint32_t)t - (uint32_t)last; }
+
+// ... kLut - 1 at most (no amount there)
+__device__ __forceinline__ int lag_of(int t, int last) { return (int)min(ms_since(t, last), (uint32_t)(kLut - 1)); }
 
 // the STDP of step t (depression at its arrivals, potentiation owed by step
 // t - 1) is left to the window's pass
