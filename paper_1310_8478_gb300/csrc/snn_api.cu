@@ -776,6 +776,10 @@ int setup_windows(snn_net *net)
     }
     net->res_grid = res;
     dn.res_parts = (uint32_t)parts;
+    // the kernels that a first window would have to load (some 0.1 ms)
+    cudaFuncAttributes loaded;
+    for (const void *f : {(const void *)k_win_open, (const void *)k_train, (const void *)k_emit, (const void *)k_stdp_lists})
+        SNN_CUDA(cudaFuncGetAttributes(&loaded, f));
     if (lists) {
         // a warp per row, one wave
         net->stdp_grid = sized_grid(net, 2048 / kStdpListsBlock, (int64_t)dn.C * dn.ne, kStdpListsBlock / 32);
