@@ -643,16 +643,13 @@ int setup_dense(snn_net *net)
     return SNN_OK;
 }
 
-// no window open (its steps are counted from a clock that a restart sets back),
-// and nothing in the resident grids' second input, where a grid that gave up
-// leaves what it had delivered
+// no window open (its steps are counted from a clock that a restart sets back)
 int clear_window(snn_net *net)
 {
     if (!net->dn.win) return SNN_OK;
     DevWindow none{};
     none.p1 = -1;
     none.defer_from = kNoDefer;
-    if (net->dn.I2) SNN_CUDA(cudaMemsetAsync(net->dn.I2, 0, (size_t)net->N * 4, net->stream));
     SNN_CUDA(cudaMemcpyAsync(net->dn.win, &none, sizeof none, cudaMemcpyHostToDevice, net->stream));
     return SNN_OK;
 }
@@ -772,6 +769,7 @@ int setup_windows(snn_net *net)
         dn.spk = reinterpret_cast<uint32_t *>(block + 2 * N8);
         if (res) dn.I2 = reinterpret_cast<int32_t *>(block + 2 * N8 + bits);
         dn.win = win;
+        if (res) SNN_CUDA(cudaMemsetAsync(dn.I2, 0, (size_t)net->N * 4, net->stream));
         SNN_TRY(clear_window(net));
     }
     net->res_grid = res;
@@ -3046,6 +3044,8 @@ int snn_load_state(snn_net *net, const void *host_buf, size_t n)
     hc.fold_cursor = 0;
     SNN_CUDA(cudaMemcpyAsync(net->ctr, &hc, sizeof hc, cudaMemcpyHostToDevice, s));
     if (dn.raster_step_off) SNN_CUDA(cudaMemsetAsync(dn.raster_step_off, 0, 8, s));
+    // (a grid that gave up leaves what it had delivered in the second input)
+    if (dn.I2) SNN_CUDA(cudaMemsetAsync(dn.I2, 0, N * 4, s));
     SNN_TRY(clear_window(net));
     SNN_CUDA(cudaStreamSynchronize(s));
     dn.raster_t0 = h.t;

@@ -260,6 +260,7 @@ __global__ void k_init_state(DevNet n)
             n.ud[i] = __dmul_rn(0.2, -65.0);
         }
         n.I[i] = 0;
+        if (n.I2) n.I2[i] = 0;
         n.hl[i] = make_uint2(0u, (uint32_t)kNever);
         n.last_spike[i] = kNever;
     }
